@@ -745,7 +745,7 @@ def run_gpu(args):
         cpu = _cpu_baseline(args.cpu_rows)
 
     if rank == 0:
-        chosen = splits or 4  # the automatic choice at this size is 4 (pick_splits)
+        chosen = splits or 4  # the automatic choice (lm_plan)
         traffic = LMHEAD_DRAM_BYTES_PER_ROW.get((WORKLOAD, chosen))
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": K,

@@ -547,8 +547,9 @@ typedef enum {
  * faster).  From now on, in this process, batches with enough rows to give
  * every resident cluster at least four items use `splits` (clamped to the
  * number of 256-column vocabulary tiles); smaller batches and splits = 0 use
- * the automatic choice (the first of 4, 2, 3, 6, 8 that keeps rounds of items
- * at least 90 % full; 4 reads the vocabulary from HBM about once per round).
+ * the automatic choice (4, which reads the vocabulary from HBM about once per
+ * round; 2 or 1 for a vocabulary of a few uneven tiles).  Row pairs that do not
+ * fill a last round of items are dealt to the clusters tile by tile instead.
  * Returns PACE_ERR_INVALID_ARG unless 0 <= splits <= 8. */
 PACE_API pace_status pace_set_lmhead_splits(int32_t splits);
 

@@ -35,11 +35,16 @@
 //                     target's logit.
 // No operand is multicast: every CTA reads only its own tiles; the pair shares
 // the vocabulary tile through the 2-CTA MMA itself.
-// A work item is a pair of 128-row blocks (one per CTA of the cluster) and one
-// of S contiguous vocabulary splits; each CTA writes one (max, sum) pair per row
-// and split.  Consecutive items share a row pair, so the hidden tiles re-read
-// for every vocabulary tile stay in L2 while the vocabulary streams.  S is
-// chosen on the device from the rows actually present (pick_splits).  A soft
+// Work is cut in two (lm_plan, evaluated on the device from the rows actually
+// present).  Rounds: an item is a pair of 128-row blocks (one per CTA of the
+// cluster) and one of S contiguous vocabulary splits, and every round gives each
+// cluster one item; consecutive items share a row pair, so the hidden tiles re-read
+// for every vocabulary tile stay in L2 while the vocabulary streams.  Tail: the
+// row pairs that would not fill a last round (all of them in a small batch) are
+// dealt to the clusters tile by tile (TailSpan), so that every cluster gets the
+// same number of tiles, give or take one, and all of them walk the vocabulary
+// together.  Each CTA writes one (max, sum) pair per row and split (rounds) or per
+// row and cluster that shares the row (tail).  A soft
 // barrier at item boundaries (wait_round) keeps the clusters of a split
 // together, so each vocabulary tile is fetched from DRAM about once per round:
 // left alone, the clusters' small speed differences add up over the hundreds
@@ -48,7 +53,7 @@
 // power-capped SMs their clock (a 1.01M-row launch of the 7B head read the
 // vocabulary 8.7 times per round; paced, 1.02 times).
 //
-// lse_merge_kernel: per row, merges the S partial pairs into the log-sum-exp
+// lse_merge_kernel: per row, merges its partial pairs into the log-sum-exp
 //   and writes lp = z_y / tau - lse.
 //
 // Every mbarrier wait is bounded (2 s); on timeout the CTA reports
@@ -102,42 +107,95 @@ struct AMaps {
   CUtensorMap box[kBoxLevels];  // box[j]: 2^j rows
 };
 constexpr int kMaxSplits = 8;
+constexpr int kMaxClusters = 128;  // clusters launched at most (bounds the tail's partials)
 
-// Number of vocabulary splits S for row_pairs row pairs on n_clusters persistent
-// clusters.  With S = 4 the 19 clusters sweeping one split stay close enough
-// for L2 to serve each vocabulary tile to all of them: the vocabulary is read
-// from HBM about once per round of items.  With S = 2 the 38 clusters of a
-// split drift apart over its 545 MB and it is read ~4 times per round (18.9 GB
-// of DRAM reads for four 9,728-row rounds of the 7B head), yet on some GPUs the
-// power-capped clock still comes out 2-10 % higher, on others as much lower;
-// S = 1 is far slower.  Small batches need more splits to give
-// every cluster an item.  So: the first of 4, 2, 3, 6, 8 whose rounds of items
-// are at least 90 % full, else whichever fills its rounds best (the earlier on
-// ties); a preferred count (pace_set_lmhead_splits, from a measurement on this
-// GPU) replaces the choice when it still gives every cluster at least four
-// items.  Evaluated identically on the device by the LM head and the merge,
-// from the device-side row count.
-__host__ __device__ inline int pick_splits(int64_t row_pairs, int64_t n_clusters, int n_vtiles,
-                                           int pref) {
-  if (pref > 0) {
-    const int sp = pref < n_vtiles ? pref : (n_vtiles > 0 ? n_vtiles : 1);
-    if (row_pairs * sp >= 4 * n_clusters) return sp;
+// How row_pairs row pairs over n_vtiles vocabulary tiles are dealt to n_clusters
+// persistent clusters.
+//
+// Rounds: the first `rounds_rp` row pairs in items of (row pair, one of S
+// contiguous splits of tiles_per_split tiles), as many as make whole rounds of one
+// item per cluster.  With S = 4 the 19 clusters sweeping one split stay close
+// enough for L2 to serve each vocabulary tile to all of them; S = 2 is 2-10 %
+// faster on some GPUs and as much slower on others (the power-capped clock), S = 1
+// far slower, so a preferred count (pace_set_lmhead_splits, from a measurement on
+// this GPU) replaces 4 when it still gives every cluster at least four items.  A
+// vocabulary of so few tiles that 4 splits are over 5 % uneven takes 2 or 1.
+//
+// Tail: the other row pairs, fewer than n_clusters, whose tiles are dealt one by
+// one (TailSpan).  Split into equal items instead (the best of 2, 3, 4, 6 and 8
+// splits), they left part of the chip idle in the last round; with the tail, one
+// launch on the H 2048 / V 151,936 head went from 866 to 276 us on 290 rows, 1016 to
+// 967 on 2,582 (rows of one run a block) and 4060 to 3650-3760 on 10,589, and from
+// 1260 to 1178 us on 20,506 rows of H 1024 / V 50,001.  Dealing every batch of fewer
+// than n_clusters pairs this way (no rounds at all) is as fast up to about 40 pairs
+// but 17 % slower on 57 pairs of the H 3584 head, where the 76 clusters drift apart
+// over the vocabulary (9.1 against 10.6 ms), so whole rounds come first.
+//
+// Evaluated identically by the LM head and the merge, from the device-side count.
+struct LmPlan {
+  int64_t rounds_rp;
+  int splits, tiles_per_split;
+  int tail_rp;     // row pairs of the tail, 0 .. n_clusters - 1
+  int tail_slots;  // partials per row of the tail: clusters that may share its tiles
+};
+
+__host__ __device__ inline LmPlan lm_plan(int64_t row_pairs, int n_clusters, int n_vtiles,
+                                          int pref) {
+  LmPlan p;
+  int sp = 4;
+  if (pref > 0 && row_pairs * (pref < n_vtiles ? pref : n_vtiles) >= 4 * int64_t{n_clusters}) {
+    sp = pref < n_vtiles ? pref : n_vtiles;
+  } else {
+    while (sp > 1 && (n_vtiles + sp - 1) / sp * sp * 20 > n_vtiles * 21) sp /= 2;
   }
-  const int cand[5] = {4, 2, 3, 6, kMaxSplits};
-  int best = 1;
-  int64_t best_items = 0, best_rounds = 1;
-  for (int i = 0; i < 5; ++i) {
-    const int sp = cand[i] < n_vtiles ? cand[i] : (n_vtiles > 0 ? n_vtiles : 1);
-    const int64_t items = row_pairs * sp;
-    const int64_t rounds = (items + n_clusters - 1) / n_clusters;
-    if (items * 10 >= 9 * rounds * n_clusters) return sp;
-    if (best_items == 0 || items * best_rounds > best_items * rounds) {
-      best = sp;
-      best_items = items;
-      best_rounds = rounds;
-    }
+  int g = n_clusters, r = sp;  // gcd
+  while (r) {
+    const int q = g % r;
+    g = r;
+    r = q;
   }
-  return best;
+  const int64_t unit = n_clusters / g;  // row pairs of the smallest whole number of rounds
+  p.splits = sp;
+  p.tiles_per_split = (n_vtiles + sp - 1) / sp;
+  p.rounds_rp = row_pairs / unit * unit;
+  p.tail_rp = static_cast<int>(row_pairs - p.rounds_rp);
+  p.tail_slots = p.tail_rp ? n_clusters / p.tail_rp + 2 : 0;
+  return p;
+}
+
+// The tail's tiles of one cluster.  Row pair i of R covers [i C, (i + 1) C) of a
+// line and cluster c of C the stretch [c R, (c + 1) R) of it, so a cluster shares
+// at most two row pairs (R < C) and a row pair at most C / R + 2 clusters.  Tile t
+// of row pair i sits at i C + (t R mod C): successive tiles step from cluster to
+// cluster, every cluster gets floor or ceil of the mean number of tiles, its k-th
+// tile is tile k C / R to within one, whatever its row pairs (so all clusters walk
+// the vocabulary together and each tile is fetched from DRAM once), and no tile
+// number comes to it twice.
+struct TailSpan {
+  int R, C;
+  int rp;    // first of its row pairs (of the tail's)
+  int a0;    // its stretch starts at rp * C + a0
+  bool two;  // the stretch reaches into row pair rp + 1
+  __device__ TailSpan(int tail_rp, int n_clusters, int c) : R(tail_rp), C(n_clusters) {
+    const int64_t x = static_cast<int64_t>(c) * R;
+    rp = static_cast<int>(x / C);
+    a0 = static_cast<int>(x - static_cast<int64_t>(rp) * C);
+    two = a0 + R > C;
+  }
+  // y = t R mod C, advanced by step() from tile to tile; 0 or 1: tile t of row
+  // pair rp or rp + 1 is this cluster's; -1: no tile t is
+  __device__ int which(int y) const {
+    return y >= a0 && y < a0 + R ? 0 : (y < a0 + R - C ? 1 : -1);
+  }
+  __device__ int step(int y) const {
+    y += R;
+    return y >= C ? y - C : y;
+  }
+};
+
+// First cluster that shares row pair i of the tail (its slot is 0).
+__device__ __forceinline__ int tail_first_cluster(int i, int tail_rp, int n_clusters) {
+  return static_cast<int>(static_cast<int64_t>(i) * n_clusters / tail_rp);
 }
 
 struct LmArgs {
@@ -151,8 +209,8 @@ struct LmArgs {
   const int32_t* rowidx;        // compact row -> original row, or null (identity)
   int32_t gather;               // 1: rows read by index (rowidx), in planned boxes
   int32_t max_level;            // largest box level no taller than the hidden-state tensor
-  float* part_m;                // [rows_cap * kMaxSplits], row r's splits at r * S
-  float* part_s;
+  float* part_m;                // the rounds' rows: row r's splits at r * S; then the
+  float* part_s;                // tail's rows, tail_slots each
   float* tgt_logit;             // [rows_cap]
   unsigned* round_ctr;          // pacing counter, zero at launch (or null: no pacing)
   int32_t* status;
@@ -164,17 +222,61 @@ __device__ __forceinline__ uint64_t make_policy_evict_normal() {
   return pol;
 }
 
-// A work item is (row pair, vocabulary split): the two CTAs of a cluster take
-// the two 128-row blocks of the pair and sweep the same vocabulary tiles, each
-// loading its half of every 256-row vocabulary tile.  Clusters are persistent
-// and take items round-robin, so all clusters sweep their splits in step and
-// each vocabulary tile is read from HBM about once per round of items.
-struct ItemCursor {
+// One cluster's work in order: its items of the rounds (taken round-robin by the
+// persistent clusters, so all of them sweep their splits in step), then its share
+// of the tail.  The two CTAs of a cluster take the two 128-row blocks of a row pair
+// and sweep the same vocabulary tiles, each loading its half of every 256-row tile.
+// A segment's tiles are those of [tile0, tile1) for which tile() says 0 or 1 (of
+// which of its row pairs); tile() is called once for each of them, in order.
+struct Segments {
+  const LmPlan& w;
+  const TailSpan& span;
+  int n_vtiles;
   int64_t item, n_items;
   int n_clusters;
-  __device__ ItemCursor(int cid, int nc, int64_t ni) : item(cid), n_items(ni), n_clusters(nc) {}
-  __device__ bool valid() const { return item < n_items; }
-  __device__ void next() { item += n_clusters; }
+  bool is_tail;  // the current segment is the tail's
+  int64_t rp;    // its first row pair
+  int split, tile0, tile1;
+  int y;
+  __device__ Segments(const LmPlan& w_, const TailSpan& s_, int nt, int cid, int nc)
+      : w(w_), span(s_), n_vtiles(nt), item(cid), n_items(w_.rounds_rp * w_.splits),
+        n_clusters(nc), is_tail(false), rp(0), split(0), tile0(0), tile1(0), y(0) {}
+  // loads the current segment; false when there is none left
+  __device__ bool load() {
+    if (is_tail) return false;
+    if (item < n_items) {
+      rp = item / w.splits;
+      split = static_cast<int>(item % w.splits);
+      tile0 = split * w.tiles_per_split;
+      tile1 = min(tile0 + w.tiles_per_split, n_vtiles);
+      item += n_clusters;
+      return true;
+    }
+    if (w.tail_rp == 0) return false;
+    is_tail = true;
+    rp = w.rounds_rp + span.rp;
+    tile0 = 0;
+    tile1 = n_vtiles;
+    return true;
+  }
+  __device__ bool two() const { return is_tail && span.two; }
+  __device__ int tile() {
+    if (!is_tail) return 0;
+    const int r = span.which(y);
+    y = span.step(y);
+    return r;
+  }
+};
+
+// One lane's part of a 128-row block's loads: lane 0 the vocabulary half-tile,
+// lanes 1..n the n boxes of the hidden tile.
+struct BlockLoads {
+  int n;             // boxes
+  uint32_t a_bytes;  // the block's hidden-tile bytes per K step
+  int32_t psrc;      // this lane's box: first source row
+  int pdst, plev;    // first block row (-127..127), box level
+  int32_t g4[4];     // scattered blocks: this lane's four source rows
+  bool scattered;
 };
 
 // The loads of one 128-row block whose rows are read by index.  Block row r is
@@ -292,12 +394,12 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
   const int cid = static_cast<int>(blockIdx.x) / CLUSTER;
   const int64_t n_valid = p.n_valid_dev ? static_cast<int64_t>(*p.n_valid_dev) : p.rows_cap;
   const int64_t row_pairs = (n_valid + 2 * BM - 1) / (2 * BM);
-  const int n_splits = pick_splits(row_pairs, n_clusters, p.n_vtiles, p.split_pref);
-  const int tiles_per_split = (p.n_vtiles + n_splits - 1) / n_splits;
-  const int64_t n_items = row_pairs * n_splits;
-  // both CTAs of a cluster read the same n_valid and cid: the exit is uniform,
-  // and comes before the pair's collective tensor-memory allocation
-  if (cid >= n_items) return;
+  const LmPlan plan_w = lm_plan(row_pairs, n_clusters, p.n_vtiles, p.split_pref);
+  // every CTA reads the same n_valid: the exit is uniform, and comes before the
+  // pair's collective tensor-memory allocation
+  if (row_pairs == 0) return;
+  const TailSpan span(plan_w.tail_rp > 0 ? plan_w.tail_rp : 1, n_clusters, cid);
+  Segments seg(plan_w, span, p.n_vtiles, cid, n_clusters);  // each role walks its own copy
   const int nkb = p.H / BK;
 
   if (threadIdx.x == 0) {
@@ -344,44 +446,50 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t it = 0;
     bool ok = true;
     unsigned round = 0;  // this cluster's items so far (the round of the current one)
-    for (ItemCursor c(cid, n_clusters, n_items); c.valid() && ok; c.next(), ++round) {
-      const int64_t rp = c.item / n_splits;
-      const int split = static_cast<int>(c.item % n_splits);
+    // the loads of row pair rp's block of this CTA
+    auto plan_block = [&](int64_t rp, BlockLoads& bl) {
       const int64_t row0 = (rp * CLUSTER + crank) * BM;
-      // this lane's load: lane 0 the vocabulary half-tile (its coordinates are
-      // set per tile below), lane 1 + q the hidden tile's box q
-      int n = 1;
-      uint32_t a_bytes = kStageA;  // this CTA's hidden-tile bytes per K step
-      int32_t psrc = static_cast<int32_t>(row0);
-      int pdst = 0, plev = kBoxLevels - 1;
-      int32_t g4[4] = {0, 0, 0, 0};
-      bool scattered = false;
-      if (gather) {
-        plan_block_loads(p.rowidx, row0, n_valid, p.max_level, lane, row_src, piece, plan);
-        n = plan[0];
-        scattered = n > kMaxBoxes;
-        if (!scattered) {
-          a_bytes = static_cast<uint32_t>(plan[1]);
-          if (lane >= 1 && lane <= n) {
-            const int2 pc = piece[lane - 1];
-            psrc = pc.x;
-            pdst = (pc.y & 0x1ff) - BM;  // first block row, -127..127
-            plev = pc.y >> 9;
-          }
-        } else {
+      bl.n = 1;
+      bl.a_bytes = kStageA;
+      bl.psrc = static_cast<int32_t>(row0);
+      bl.pdst = 0;
+      bl.plev = kBoxLevels - 1;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) g4[j] = row_src[4 * lane + j];  // row 0 past the end
+      for (int j = 0; j < 4; ++j) bl.g4[j] = 0;
+      bl.scattered = false;
+      if (!gather) return;
+      plan_block_loads(p.rowidx, row0, n_valid, p.max_level, lane, row_src, piece, plan);
+      bl.n = plan[0];
+      bl.scattered = bl.n > kMaxBoxes;
+      if (!bl.scattered) {
+        bl.a_bytes = static_cast<uint32_t>(plan[1]);
+        if (lane >= 1 && lane <= bl.n) {
+          const int2 pc = piece[lane - 1];
+          bl.psrc = pc.x;
+          bl.pdst = (pc.y & 0x1ff) - BM;
+          bl.plev = pc.y >> 9;
         }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bl.g4[j] = row_src[4 * lane + j];  // row 0 past the end
       }
-      // every round before the last is full, so round k starts once all
-      // clusters issued their round k-1 loads (the even CTA paces the pair)
+      __syncwarp();  // row_src and piece are rewritten by the next plan
+    };
+    for (; ok && seg.load(); ++round) {
+      BlockLoads b0, b1;
+      plan_block(seg.rp, b0);
+      b1 = b0;
+      if (seg.two()) plan_block(seg.rp + 1, b1);
+      // every round is full, so round k (or the tail) starts once all clusters
+      // issued their round k-1 loads (the even CTA paces the pair)
       if (leader && lane == 0 && round > 0 && p.round_ctr)
         wait_round(p.round_ctr, round * static_cast<unsigned>(n_clusters));
       __syncwarp();
-      const int tile0 = split * tiles_per_split;
-      const int tile1 = min(tile0 + tiles_per_split, p.n_vtiles);
-      const int issuers = scattered ? 1 : n + 1;
-      for (int t = tile0; t < tile1 && ok; ++t) {
+      for (int t = seg.tile0; t < seg.tile1 && ok; ++t) {
+        const int which = seg.tile();
+        if (which < 0) continue;
+        const BlockLoads bl = which ? b1 : b0;
+        const int issuers = bl.scattered ? 1 : bl.n + 1;
         const int32_t nb = t * BN + static_cast<int32_t>(crank) * (BN / CLUSTER);
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           const uint32_t s = it % STAGES;
@@ -398,23 +506,26 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
             // this CTA's bytes of the stage, announced with its arrival on the
             // even CTA's barrier (which completes once both CTAs' bytes land)
             if (leader)
-              mbar_arrive_expect_tx(&full[s], a_bytes + kStageB);
+              mbar_arrive_expect_tx(&full[s], bl.a_bytes + kStageB);
             else
-              mbar_arrive_expect_tx_cluster(bar, a_bytes + kStageB);
+              mbar_arrive_expect_tx_cluster(bar, bl.a_bytes + kStageB);
           }
+          // Reconverge, so that the lanes' loads below are one TMA instruction:
+          // when lane 0 comes out of the arrival alone and issues its load by
+          // itself, every launch is 20-25 % slower.
+          __syncwarp();
           if (lane < issuers) {
             const void* desc = lane == 0 ? static_cast<const void*>(&tm_b)
-                                         : static_cast<const void*>(&am.box[plev]);
-            unsigned char* dst = lane == 0 ? sb : sa + pdst * (BK * 2);
-            tma_load_2d_pair(dst, desc, bar, kb * BK, lane == 0 ? nb : psrc, pol);
+                                         : static_cast<const void*>(&am.box[bl.plev]);
+            unsigned char* dst = lane == 0 ? sb : sa + bl.pdst * (BK * 2);
+            tma_load_2d_pair(dst, desc, bar, kb * BK, lane == 0 ? nb : bl.psrc, pol);
           }
-          if (scattered)
-            tma_gather4_pair(sa + lane * 4 * (BK * 2), &am.box[0], bar, kb * BK, g4[0], g4[1],
-                             g4[2], g4[3], pol);
+          if (bl.scattered)
+            tma_gather4_pair(sa + lane * 4 * (BK * 2), &am.box[0], bar, kb * BK, bl.g4[0],
+                             bl.g4[1], bl.g4[2], bl.g4[3], pol);
         }
       }
       if (leader && lane == 0 && ok && p.round_ctr) atomicAdd(p.round_ctr, 1u);
-      __syncwarp();  // row_src and piece are rewritten for the next item
     }
     if (lane == 0) {
       if (!ok) give_up();
@@ -437,13 +548,12 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
       // ------------------------------------------------ MMA issuer (even CTA)
       uint32_t it = 0, tcount = 0;
       bool ok = true;
-      for (ItemCursor c(cid, n_clusters, n_items); c.valid() && ok; c.next()) {
-        const int split = static_cast<int>(c.item % n_splits);
-        const int tile0 = split * tiles_per_split;
-        const int tile1 = min(tile0 + tiles_per_split, p.n_vtiles);
-        for (int t = tile0; t < tile1 && ok; ++t, ++tcount) {
+      while (ok && seg.load()) {
+        for (int t = seg.tile0; t < seg.tile1 && ok; ++t) {
+          if (seg.tile() < 0) continue;
           const uint32_t acc = tcount & 1u;
           const uint32_t acc_ph = (tcount >> 1) & 1u;
+          ++tcount;
           if (!mbar_wait_bounded_cluster(&tmem_empty[acc], acc_ph ^ 1u, abort_flag)) {
             ok = false;
             break;
@@ -488,23 +598,43 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t empty1 = cluster_addr(&tmem_empty[1], 0);
     uint32_t tcount = 0;
     bool ok = true;
-    for (ItemCursor c(cid, n_clusters, n_items); c.valid() && ok; c.next()) {
-      const int64_t rp = c.item / n_splits;
-      const int split = static_cast<int>(c.item % n_splits);
-      const int tile0 = split * tiles_per_split;
-      const int tile1 = min(tile0 + tiles_per_split, p.n_vtiles);
-      const int64_t row = (rp * CLUSTER + crank) * BM + r_local;
-      const bool row_ok = row < n_valid;
-      int32_t y = -1;
-      if (row_ok) {
-        const int64_t orig = p.rowidx ? static_cast<int64_t>(p.rowidx[row]) : row;
-        y = p.targets[orig];
+    // a row's running state over its vocabulary tiles
+    struct RowState {
+      int64_t row;
+      bool row_ok, have_tgt;
+      int32_t y;
+      float m, s, tgt;
+    };
+    auto start_row = [&](int64_t rp, RowState& rs) {
+      rs.row = (rp * CLUSTER + crank) * BM + r_local;
+      rs.row_ok = rs.row < n_valid;
+      rs.y = -1;
+      if (rs.row_ok) {
+        const int64_t orig = p.rowidx ? static_cast<int64_t>(p.rowidx[rs.row]) : rs.row;
+        rs.y = p.targets[orig];
       }
-      float m = -INFINITY, s = 0.0f, tgt = 0.0f;
-      bool have_tgt = false;
-      for (int t = tile0; t < tile1; ++t, ++tcount) {
+      rs.m = -INFINITY;
+      rs.s = 0.0f;
+      rs.tgt = 0.0f;
+      rs.have_tgt = false;
+    };
+    auto finish_row = [&](const RowState& rs, int64_t o) {
+      if (!rs.row_ok) return;
+      p.part_m[o] = rs.m;
+      p.part_s[o] = rs.s;
+      if (rs.have_tgt) p.tgt_logit[rs.row] = rs.tgt;
+    };
+    while (ok && seg.load()) {
+      RowState r0, r1;
+      start_row(seg.rp, r0);
+      r1 = r0;
+      if (seg.two()) start_row(seg.rp + 1, r1);
+      for (int t = seg.tile0; t < seg.tile1; ++t) {
+        const int which = seg.tile();
+        if (which < 0) continue;
         const uint32_t acc = tcount & 1u;
         const uint32_t acc_ph = (tcount >> 1) & 1u;
+        ++tcount;
         // one outcome for the whole warp: tcgen05.ld below is warp-collective,
         // and a lane that saw the peer's abort must not leave its warp behind
         const bool got = __all_sync(0xffffffffu,
@@ -517,6 +647,9 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
         tc_fence_after();
         const int32_t n0 = t * BN;
         const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + acc * BN;
+        const int32_t y = which ? r1.y : r0.y;
+        float m = which ? r1.m : r0.m, s = which ? r1.s : r0.s, tgt = which ? r1.tgt : r0.tgt;
+        bool have_tgt = which ? r1.have_tgt : r0.have_tgt;
 #pragma unroll 1
         for (int cc = 0; cc < BN; cc += 32) {
           float v[32];
@@ -550,12 +683,30 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acc ? empty1 : empty0);
+        if (which) {
+          r1.m = m;
+          r1.s = s;
+          r1.tgt = tgt;
+          r1.have_tgt = have_tgt;
+        } else {
+          r0.m = m;
+          r0.s = s;
+          r0.tgt = tgt;
+          r0.have_tgt = have_tgt;
+        }
       }
-      if (row_ok && ok) {
-        const int64_t o = row * n_splits + split;
-        p.part_m[o] = m;
-        p.part_s[o] = s;
-        if (have_tgt) p.tgt_logit[row] = tgt;
+      if (!ok) break;
+      if (!seg.is_tail) {
+        finish_row(r0, r0.row * plan_w.splits + seg.split);
+      } else {  // a cluster that got none of a row pair's tiles writes an empty partial
+        const int64_t row_base = plan_w.rounds_rp * (CLUSTER * BM);
+        const int64_t base = row_base * plan_w.splits;
+        const int R = plan_w.tail_rp;
+        finish_row(r0, base + (r0.row - row_base) * plan_w.tail_slots + cid -
+                           tail_first_cluster(span.rp, R, n_clusters));
+        if (span.two)
+          finish_row(r1, base + (r1.row - row_base) * plan_w.tail_slots + cid -
+                             tail_first_cluster(span.rp + 1, R, n_clusters));
       }
     }
   }
@@ -581,16 +732,25 @@ __global__ void lse_merge_kernel(int64_t rows_cap, const long long* __restrict__
                                  const int32_t* __restrict__ rowidx, float* __restrict__ logprob,
                                  float* __restrict__ lse_out, int32_t* status) {
   const int64_t n_valid = n_valid_dev ? static_cast<int64_t>(*n_valid_dev) : rows_cap;
-  // the split count the LM head used for these rows
-  const int splits =
-      pick_splits((n_valid + 2 * BM - 1) / (2 * BM), lm_clusters, n_vtiles, split_pref);
+  // how the LM head dealt these rows
+  const LmPlan plan = lm_plan((n_valid + 2 * BM - 1) / (2 * BM), lm_clusters, n_vtiles, split_pref);
+  const int64_t tail_row0 = plan.rounds_rp * (2 * BM);
   for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < n_valid;
        r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t orig = rowidx ? static_cast<int64_t>(rowidx[r]) : r;
+    int64_t o = r * plan.splits;
+    int splits = plan.splits;
+    if (r >= tail_row0) {  // the clusters whose stretch meets the row pair's
+      o = tail_row0 * plan.splits + (r - tail_row0) * plan.tail_slots;
+      const int i = static_cast<int>((r - tail_row0) / (2 * BM));
+      const int64_t x1 = static_cast<int64_t>(i + 1) * lm_clusters - 1;
+      splits = static_cast<int>(x1 / plan.tail_rp) -
+               tail_first_cluster(i, plan.tail_rp, lm_clusters) + 1;
+    }
     float mm = -INFINITY;
-    for (int s = 0; s < splits; ++s) mm = fmaxf(mm, part_m[r * splits + s]);
+    for (int s = 0; s < splits; ++s) mm = fmaxf(mm, part_m[o + s]);
     float ss = 0.0f;
-    for (int s = 0; s < splits; ++s) ss += part_s[r * splits + s] * ex2_approx(part_m[r * splits + s] - mm);
+    for (int s = 0; s < splits; ++s) ss += part_s[o + s] * ex2_approx(part_m[o + s] - mm);
     const float lse = (mm + lg2_approx(ss)) * 0.69314718055994531f;
     const int32_t y = targets[orig];
     float lp;
@@ -639,7 +799,7 @@ pace_status lm_launch_info(LmLaunchInfo* out) {
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, lmhead_lse_kernel, &cfg) != cudaSuccess || n < 1)
       n = sm_count() / CLUSTER;
-    info[dev].max_clusters = n;
+    info[dev].max_clusters = n < kMaxClusters ? n : kMaxClusters;
   }
   *out = info[dev];
   return PACE_OK;
@@ -655,8 +815,13 @@ void carve_lm_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, bool dense_ro
   w->hidden_c =
       dense_rows ? static_cast<void*>(cv.take<uint16_t>(static_cast<size_t>(rows_cap) * H))
                  : nullptr;
-  w->part_m = cv.take<float>(static_cast<size_t>(rows_cap) * kMaxSplits);
-  w->part_s = cv.take<float>(static_cast<size_t>(rows_cap) * kMaxSplits);
+  // partials: kMaxSplits a row, and the tail's C / R + 2 a row for 256 R rows, R < C
+  const int64_t rp = (rows_cap + 2 * BM - 1) / (2 * BM);
+  const size_t parts =
+      static_cast<size_t>(rows_cap) * kMaxSplits +
+      2 * BM * (kMaxClusters + 2 * static_cast<size_t>(rp < kMaxClusters ? rp : kMaxClusters));
+  w->part_m = cv.take<float>(parts);
+  w->part_s = cv.take<float>(parts);
   w->tgt = cv.take<float>(static_cast<size_t>(rows_cap));
   w->round_ctr = cv.take<unsigned>(1);
 }
@@ -733,9 +898,9 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   a.round_ctr = ws.round_ctr;
   a.status = status_dev;
   // persistent: at most one wave of 2-CTA clusters, never more clusters than the
-  // most items the rows could make (the split count is chosen on the device)
-  const int64_t items = (rows_cap + 2 * BM - 1) / (2 * BM) * kMaxSplits;
-  const int64_t clusters = items < li.max_clusters ? items : li.max_clusters;
+  // rows could make tiles
+  const int64_t tiles = (rows_cap + 2 * BM - 1) / (2 * BM) * n_vtiles;
+  const int64_t clusters = tiles < li.max_clusters ? tiles : li.max_clusters;
   const int64_t grid = clusters * CLUSTER;
   PACE_TRY_CUDA(cudaMemsetAsync(ws.round_ctr, 0, sizeof(unsigned), st));
   const ProfileEvents& pe = profile_events(PACE_PROFILE_LMHEAD);

@@ -88,6 +88,31 @@ def test_masks_of_runs(rows, H, V, max_run):
     assert (lp[~sel] == 0).all() and (lse[~sel] == 0).all()
 
 
+@pytest.mark.parametrize("pairs,extra", [(1, 0), (2, -200), (18, 0), (19, 0), (20, -1), (38, 1),
+                                         (75, -128), (76, 0), (77, -255), (96, 0)])
+@pytest.mark.parametrize("V", [200, 600, 1300, 2048, 5000])
+def test_row_pairs_around_whole_rounds(pairs, extra, V):
+    """Batches of `pairs` 256-row pairs (give or take some rows) around the sizes at
+    which whole rounds of items and the tile-by-tile tail meet (19 and 76 pairs on
+    76 clusters), over vocabularies of 1, 3, 6, 8 and 20 tiles: a tile dealt twice or
+    not at all would move every log-sum-exp by at least log(20 / 19).  The bound is
+    that of 32-bit sums of 64 products and V terms (|z| < 12)."""
+    rows, H = 256 * pairs + extra, 64
+    g = torch.Generator(device=DEV)
+    g.manual_seed(pairs * 1000 + V)
+    h = torch.randn(rows, H, device=DEV, generator=g).to(torch.bfloat16)
+    w = (torch.randn(V, H, device=DEV, generator=g) / 4).to(torch.bfloat16)
+    y = torch.randint(0, V, (rows,), device=DEV, generator=g, dtype=torch.int32)
+    z = h.double() @ w.double().T
+    olse = torch.logsumexp(z, 1)
+    olp = z.gather(1, y.long()[:, None])[:, 0] - olse
+    tol = 12 * 64 * 2.0 ** -24 + 16 * 2.0 ** -22  # the products' sum; ex2 / lg2 approximations
+    for mask in (None, torch.ones(rows, dtype=torch.uint8, device=DEV)):
+        lp, lse = _run(h, w, y, mask=mask)
+        assert np.abs(lse - as_np(olse)).max() <= tol
+        assert np.abs(lp - as_np(olp)).max() <= 2 * tol
+
+
 def test_vocab_smaller_than_one_tile():
     rng = np.random.default_rng(1)
     rows, H, V = 200, 64, 100
