@@ -107,7 +107,7 @@ struct AMaps {
   CUtensorMap box[kBoxLevels];  // box[j]: 2^j rows
 };
 constexpr int kMaxSplits = 8;
-constexpr int kMaxClusters = 128;  // clusters launched at most (bounds the tail's partials)
+constexpr int kMaxClusters = 76;  // clusters launched at most (bounds the tail's partials)
 
 // How row_pairs row pairs over n_vtiles vocabulary tiles are dealt to n_clusters
 // persistent clusters.
@@ -815,11 +815,10 @@ void carve_lm_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, bool dense_ro
   w->hidden_c =
       dense_rows ? static_cast<void*>(cv.take<uint16_t>(static_cast<size_t>(rows_cap) * H))
                  : nullptr;
-  // partials: kMaxSplits a row, and the tail's C / R + 2 a row for 256 R rows, R < C
+  // partials: of rp row pairs, kMaxSplits a row in the rounds, and C / R + 2 a row
+  // for the R row pairs of the tail
   const int64_t rp = (rows_cap + 2 * BM - 1) / (2 * BM);
-  const size_t parts =
-      static_cast<size_t>(rows_cap) * kMaxSplits +
-      2 * BM * (kMaxClusters + 2 * static_cast<size_t>(rp < kMaxClusters ? rp : kMaxClusters));
+  const size_t parts = 2 * BM * (kMaxClusters + static_cast<size_t>(rp) * kMaxSplits);
   w->part_m = cv.take<float>(parts);
   w->part_s = cv.take<float>(parts);
   w->tgt = cv.take<float>(static_cast<size_t>(rows_cap));
