@@ -17,9 +17,9 @@
 //                     through the compact-row index.  Per work item the warp
 //                     splits the block's 128 rows into runs of consecutive
 //                     source rows (plan_block_loads) and the runs into boxes of
-//                     2^j rows (one box for a block inside a response; the
-//                     first and last of several runs spill into 16 KB regions
-//                     around the tile).  A block of more than 31 boxes is
+//                     1, 2, 4 or a multiple of 8 rows (one box for a block inside
+//                     a response; the first and last of several runs, rounded up
+//                     to one box, spill into 16 KB regions around the tile).  A block of more than 31 boxes is
 //                     fetched by four-row TMA gathers (tile::gather4), one per
 //                     lane.  No copy of the rows is made.
 //   warp 1 / lane 0   MMA issuer, even CTA only: tcgen05.mma.cta_group::2
@@ -99,12 +99,29 @@ __host__ __device__ constexpr uint32_t a_tile_off(uint32_t s) {
   return kSpill + s * (kStageA + kSpill);
 }
 __host__ __device__ constexpr uint32_t b_tile_off(uint32_t s) { return kARegion + s * kStageB; }
-// Tensor maps of the hidden states with boxes of 1, 2, 4, ..., 128 rows (64
-// columns, 128-byte swizzle).
-constexpr int kBoxLevels = 8;
+// Tensor maps of the hidden states with boxes of 1, 2, 4, 8, 16, 24, ..., 128 rows
+// (64 columns, 128-byte swizzle).  An SM takes in operand tiles at close to the
+// rate the tensor cores use them, so the rows a block's boxes load beyond its 128
+// cost their share of time: with heights of 2^j only, a block of two runs loaded 192
+// rows on average, with multiples of 8 it loads 135.  Micro-batches whose blocks
+// straddle two or three sequences (H 2048, V 151,936), one launch: 1,455 rows 605-654
+// -> 558-575 us, 2,582 rows 1135 -> 1054, 6,186 rows 2484 -> 2222; 37k rows of
+// multi-turn sequences (H 3584) 24.1 -> 23.7-24.1 ms (power-capped).
+constexpr int kBoxLevels = 19;
 constexpr int kMaxBoxes = 31;  // more boxes in a block: four-row gathers instead
+__host__ __device__ constexpr int box_rows(int level) {
+  return level < 3 ? 1 << level : 8 * (level - 2);
+}
+// the lowest box of at least n rows, the tallest of at most n (n in 1..128)
+__host__ __device__ constexpr int box_covering(int n) {
+  return n <= 2 ? n - 1 : (n <= 4 ? 2 : 2 + (n + 7) / 8);
+}
+__host__ __device__ constexpr int box_within(int n) {
+  return n >= 8 ? 2 + n / 8 : (n >= 4 ? 2 : n - 1 < 1 ? 0 : 1);
+}
+static_assert(box_rows(kBoxLevels - 1) == BM, "the tallest box is a block");
 struct AMaps {
-  CUtensorMap box[kBoxLevels];  // box[j]: 2^j rows
+  CUtensorMap box[kBoxLevels];  // box[j]: box_rows(j) rows
 };
 constexpr int kMaxSplits = 8;
 constexpr int kMaxClusters = 76;  // clusters launched at most (bounds the tail's partials)
@@ -283,15 +300,13 @@ struct BlockLoads {
 // compact row row0 + r; its source row is rowidx[row0 + r] while that is below
 // n_valid.  A run is a maximal stretch of block rows with consecutive source
 // rows; the rows past n_valid (loaded, never written back) belong to the last
-// run.  A block of one run is loaded as one box per set bit of its length (one
-// 128-row box when the tensor has 128 rows or more).  Of several runs, the
-// first is one box of the smallest power of two rows that covers it, ending at
-// the run's end (its earlier rows land in the spill region before the tile),
-// the last one such box starting at the run's start (its later rows land in the
-// spill region after the tile), and a run in between one box per set bit of
-// its length, largest first.  Boxes never overlap inside the tile, and no box
-// is taller than 2^max_level rows (the tallest map the hidden-state tensor
-// allows).  Writes the source rows to row_src[BM], the boxes to piece[] as
+// run.  A block of one run is loaded exactly, tallest boxes first (one 128-row box
+// when the tensor has 128 rows or more).  Of several runs, the first is the lowest
+// box that covers it, ending at the run's end (its earlier rows land in the spill
+// region before the tile), the last one such box starting at the run's start (its
+// later rows land in the spill region after the tile), and a run in between is
+// loaded exactly.  Boxes never overlap inside the tile, and no box is taller than
+// box_rows(max_level) (the tallest map the hidden-state tensor allows).  Writes the source rows to row_src[BM], the boxes to piece[] as
 // (first source row, (first block row + 128) | level << 9), their number to
 // plan[0] and their bytes per K step to plan[1].  All 32 lanes call it.
 __device__ void plan_block_loads(const int32_t* __restrict__ rowidx, int64_t row0,
@@ -336,25 +351,26 @@ __device__ void plan_block_loads(const int32_t* __restrict__ rowidx, int64_t row
       }
       const int32_t s0 = row_src[r];
       const int len = e - r;
-      const int cl = len <= 1 ? 0 : 32 - __clz(len - 1);  // smallest level that covers the run
+      const int cl = box_covering(len);
       if (m > 1 && (k == 0 || k == m - 1) && cl <= max_level) {
-        // first or last of several runs: one box of 2^cl rows, ending at the
+        // first or last of several runs: one box that covers it, ending at the
         // first run's end (spilling before the tile) or starting at the last
         // run's start (spilling after it)
-        const int at = k == 0 ? len - (1 << cl) : r;
+        const int at = k == 0 ? len - box_rows(cl) : r;
         piece[n++] = make_int2(s0 + (at - r), (at + BM) | (cl << 9));
-        rows += 1u << cl;
-      } else {  // the only run, or one in between: one box per set bit of its length
+        rows += box_rows(cl);
+      } else {  // the only run, or one in between: exactly
         int at = r, left_rows = len;
         int32_t src = s0;
         while (left_rows > 0) {
-          int lev = 31 - __clz(left_rows);
+          int lev = box_within(left_rows);
           if (lev > max_level) lev = max_level;
+          const int h = box_rows(lev);
           piece[n++] = make_int2(src, (at + BM) | (lev << 9));
-          rows += 1u << lev;
-          at += 1 << lev;
-          src += 1 << lev;
-          left_rows -= 1 << lev;
+          rows += h;
+          at += h;
+          src += h;
+          left_rows -= h;
         }
       }
       r = e;
@@ -441,7 +457,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
     // more than kMaxBoxes boxes is gathered four rows a lane instead.
     const bool gather = p.gather != 0;
     if (lane == 0) tma_prefetch_desc(&tm_b);
-    if (lane < kBoxLevels) tma_prefetch_desc(&am.box[lane]);
+    if (gather ? lane < kBoxLevels : lane == kBoxLevels - 1) tma_prefetch_desc(&am.box[lane]);
     const uint64_t pol = make_policy_evict_normal();
     uint32_t it = 0;
     bool ok = true;
@@ -867,14 +883,17 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   const int n_vtiles = (V + BN - 1) / BN;
   AMaps am;
   CUtensorMap tm_b;
-  // boxes of 2^j hidden rows for j up to the tensor's height (at most 128);
-  // taller levels repeat the tallest valid map and are never used
+  // boxes up to the tensor's height (at most 128 rows); taller levels repeat the
+  // tallest valid map and are never used, nor are the others without a row index
   int max_level = 0;
-  while (max_level + 1 < kBoxLevels && (int64_t{1} << (max_level + 1)) <= n_rows) ++max_level;
+  while (max_level + 1 < kBoxLevels && box_rows(max_level + 1) <= n_rows) ++max_level;
   if (!compact && max_level != kBoxLevels - 1) return PACE_ERR_INVALID_ARG;  // n_rows >= 128
+  PACE_TRY(encode_bf16_2d(&am.box[max_level], hidden, n_rows, H, H, BK, box_rows(max_level)));
   for (int j = 0; j < kBoxLevels; ++j) {
-    if (j <= max_level) PACE_TRY(encode_bf16_2d(&am.box[j], hidden, n_rows, H, H, BK, 1 << j));
-    else am.box[j] = am.box[max_level];
+    if (compact && j < max_level)
+      PACE_TRY(encode_bf16_2d(&am.box[j], hidden, n_rows, H, H, BK, box_rows(j)));
+    else
+      am.box[j] = am.box[max_level];
   }
   PACE_TRY(encode_bf16_2d(&tm_b, w_vocab, V, H, H, BK, BN / CLUSTER));  // one CTA's half tile
   LmLaunchInfo li;
