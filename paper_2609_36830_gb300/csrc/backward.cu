@@ -11,9 +11,13 @@
 //                             GEMMs read it in long contiguous runs (a K step of
 //                             dH is one 16 KB run, a K step of dW 8 KB);
 //   2. gemm_kernel<EPI_ROWS>: dH_c = G W (A = G K-major, B = W read MN-major),
-//                             fp32 rows scattered back to their original row;
+//                             fp32 rows scattered back to their original row.  The
+//                             tiles that would not fill a last round are split
+//                             along K (tail_split) into partial tiles, which
+//                             reduce_tail_kernel adds in a fixed order;
 //   3. gemm_kernel<EPI_ACC>:  dW += G^T H_c (A = G and B = H_c, both read
-//                             MN-major), fp32 accumulation in place.
+//                             MN-major), fp32 accumulation in place; the first
+//                             chunk stores, so dW needs no clearing.
 // The GEMM is one warp-specialised tcgen05 kernel on CTA pairs: in each CTA
 // warp 0 issues TMA for the CTA's own A tile and its own half of the B tile
 // into a 4-stage ring (128-byte swizzle), both CTAs' bytes completing on the
@@ -49,6 +53,15 @@ constexpr uint32_t kGTmemCols = 2 * GBN;
 constexpr size_t kGSmemBytes = 1024 + GSTAGES * kGStageBytes + 256;
 constexpr int64_t kChunkRows = 32768;         // rows of G held at once (bf16 M x V)
 constexpr int kGroupM = 38;                   // M tiles per raster group
+// The clusters meet (wait_round) about every kPaceSteps K steps, at a round
+// boundary: meeting costs 1-2 us, the time of a few K steps, and the clusters drift
+// slowly.  Whole calls meeting at every round / 512 / 4096 steps / never: 2,582 rows
+// of the H 2048 head 3.31 / 3.22 / 3.18-3.30 / 3.18-3.23 ms, two 32k chunks of the
+// H 1024 / V 50,001 head 14.92 / 14.76 / 14.68 / 14.65 ms, 21k rows of the H 3584 head
+// 42.2 / 42.1 / 42.0 / 42.3 ms.
+constexpr int kPaceSteps = 4096;
+constexpr int kMaxKSplits = 8;                // parts a tail tile is split into at most
+constexpr int kMaxGemmClusters = 76;          // clusters launched at most (bounds the partial tiles)
 
 enum { EPI_G = 0, EPI_ROWS = 1, EPI_ACC = 2 };
 enum { TRIM_NONE = 0, TRIM_M = 1, TRIM_K = 2 };
@@ -77,8 +90,11 @@ struct GemmArgs {
   // EPI_ROWS
   float* rows_out;              // fp32 [orig rows][ldo]
   int64_t ldo;
+  // partial tiles of the tail, or null: fp32 [part * items + item][2 GBM][GBN]
+  float* part;
   // EPI_ACC
   float* acc_out;               // fp32 [M][ldo]
+  int acc_first;                // 1: store (the first chunk), 0: add
   unsigned* round_ctr;          // pacing counter, zeroed before the launch (or null)
   int32_t* status;
 };
@@ -102,6 +118,35 @@ __device__ __forceinline__ void item_of(const GemmArgs& p, int64_t m_tiles, int6
   const int64_t gm = (pairs - g0) < gp ? (pairs - g0) : gp;
   *mp = g0 + r % gm;
   *n = r / gm;
+}
+
+// The last, partial round of items items on n_clusters clusters: its tail items are
+// split along K into `splits` parts each, so that together they fill the clusters
+// for 1 / splits of a round instead of leaving most of them idle for a whole one
+// (the dH of a micro-batch, 88 tiles on 76 clusters, took two rounds and takes
+// 1 + 1/6).  Whole rounds are not split, so the partial tiles stay below kMaxKSplits
+// a cluster.  splits = 1: no split pays (a full round, a short K).
+struct TailSplit {
+  int64_t full;  // items before the tail
+  int tail;      // items of the tail
+  int splits;
+};
+
+__host__ __device__ inline TailSplit tail_split(int64_t items, int n_clusters, int nkb) {
+  TailSplit s;
+  s.full = items / n_clusters * n_clusters;
+  s.tail = static_cast<int>(items - s.full);
+  s.splits = 1;
+  int best = nkb;  // the tail's K steps
+  for (int k = 2; k <= kMaxKSplits; ++k) {
+    const int rounds = (s.tail * k + n_clusters - 1) / n_clusters;
+    const int steps = rounds * ((nkb + k - 1) / k);
+    if (nkb >= 32 * k && steps < best) {
+      best = steps;
+      s.splits = k;
+    }
+  }
+  return s;
 }
 
 // 128-byte-swizzled operand tiles.  K-major: rows of 64 K elements (128 B),
@@ -170,11 +215,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       K = v;
     }
   }
-  const int64_t n_items = (m_tiles + 1) / 2 * p.n_tiles;
+  const int64_t base_items = (m_tiles + 1) / 2 * p.n_tiles;
   const int64_t cid = blockIdx.x / 2, n_clusters = gridDim.x / 2;
-  const int nkb = static_cast<int>((K + GBK - 1) / GBK);
+  const int nkb_all = static_cast<int>((K + GBK - 1) / GBK);
   // uniform over the grid, and before the pair's collective TMEM allocation
-  if (nkb == 0 || n_items == 0) return;
+  if (nkb_all == 0 || base_items == 0) {
+    if (EPI == EPI_ACC && p.acc_first)  // no rows in the loss: dW = 0
+      for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+           i < p.M * p.N / 4; i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        reinterpret_cast<float4*>(p.acc_out)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    return;
+  }
+  TailSplit ts{base_items, 0, 1};
+  if (EPI == EPI_ROWS && p.part)
+    ts = tail_split(base_items, static_cast<int>(n_clusters), nkb_all);
+  const int64_t n_items = ts.splits > 1 ? ts.full + static_cast<int64_t>(ts.tail) * ts.splits
+                                        : base_items;
+  // item t's tile and K steps [k0, k1); a tail item's part (-1: the whole K)
+  auto work_of = [&](int64_t t, int* k0, int* k1, int* part) -> int64_t {
+    *k0 = 0;
+    *k1 = nkb_all;
+    *part = -1;
+    if (EPI != EPI_ROWS || ts.splits == 1 || t < ts.full) return t;
+    const int u = static_cast<int>(t - ts.full);
+    *part = u / ts.tail;
+    *k0 = nkb_all * *part / ts.splits;
+    *k1 = nkb_all * (*part + 1) / ts.splits;
+    return ts.full + u % ts.tail;
+  };
+  const int pace_rounds = max(1, kPaceSteps / nkb_all);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < GSTAGES; ++s) {
@@ -217,13 +286,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       unsigned round = 0;  // this cluster's items so far
       for (int64_t t = cid; t < n_items && ok; t += n_clusters, ++round) {
         int64_t mp, nt;
-        item_of(p, m_tiles, t, &mp, &nt);
+        int kb0, kb1, part;
+        item_of(p, m_tiles, work_of(t, &kb0, &kb1, &part), &mp, &nt);
         const int32_t m0 = static_cast<int32_t>((2 * mp + crank) * GBM);
         const int32_t n0 = static_cast<int32_t>(nt * GBN);
-        // the clusters start each round together (every round but the last is full)
-        if (leader && round > 0 && p.round_ctr)
+        // the clusters start this round together (every round but the last is full)
+        if (leader && round > 0 && round % pace_rounds == 0 && p.round_ctr)
           wait_round(p.round_ctr, round * static_cast<unsigned>(n_clusters));
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % GSTAGES, ph = (it / GSTAGES) & 1u;
           if (!mbar_wait_bounded(&empty[s], ph ^ 1u, abort_flag)) {
             ok = false;
@@ -278,6 +348,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       uint32_t it = 0, tc = 0;
       bool ok = true;
       for (int64_t t = cid; t < n_items && ok; t += n_clusters, ++tc) {
+        int kb0, kb1, part;
+        work_of(t, &kb0, &kb1, &part);
         const uint32_t acc = tc & 1u, acc_ph = (tc >> 1) & 1u;
         if (!mbar_wait_bounded_cluster(&tmem_empty[acc], acc_ph ^ 1u, abort_flag)) {
           ok = false;
@@ -285,7 +357,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * GBN;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % GSTAGES, ph = (it / GSTAGES) & 1u;
           if (!mbar_wait_bounded(&full[s], ph, abort_flag)) {
             ok = false;
@@ -299,7 +371,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
             const uint32_t ka = A_MN ? sa + k * 2048 : sa + k * 32;
             const uint32_t kbb = B_MN ? sb + k * 2048 : sb + k * 32;
             tc_mma_f16_pair(d_tmem, operand_desc(ka, A_MN), operand_desc(kbb, B_MN), kIdesc,
-                            (kb > 0 || k > 0) ? 1u : 0u);
+                            (kb > kb0 || k > 0) ? 1u : 0u);
           }
           tc_commit_pair(cluster_addr(&empty[s], 0));
           tc_commit_pair(cluster_addr(&empty[s], 1));
@@ -320,7 +392,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     uint32_t tc = 0;
     for (int64_t t = cid; t < n_items; t += n_clusters, ++tc) {
       int64_t mp, nt;
-      item_of(p, m_tiles, t, &mp, &nt);
+      int kb0, kb1, part;
+      item_of(p, m_tiles, work_of(t, &kb0, &kb1, &part), &mp, &nt);
       const int64_t mt = 2 * mp + crank;
       const uint32_t acc = tc & 1u, acc_ph = (tc >> 1) & 1u;
       // one outcome for the whole warp (tcgen05.ld below is warp-collective)
@@ -381,7 +454,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
                                  packed[4 * q + 3]);
           }
         } else if (EPI == EPI_ROWS) {
-          if (row_ok) {
+          if (part >= 0) {  // a partial tile, whole (its rows outside the loss are not read)
+            float4* d4 = reinterpret_cast<float4*>(
+                p.part + ((t - ts.full) * (2 * GBM) + crank * GBM + r_local) * GBN + c);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              d4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          } else if (row_ok) {
             float* dst = p.rows_out + orig * p.ldo + col0;
             if (col0 + 32 <= p.N) {
               float4* d4 = reinterpret_cast<float4*>(dst);
@@ -397,17 +476,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
             float* dst = p.acc_out + row * p.ldo + col0;
             if (col0 + 32 <= p.N) {
               float4* d4 = reinterpret_cast<float4*>(dst);
+              if (p.acc_first) {
 #pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                float4 o = d4[q];
-                o.x += v[4 * q];
-                o.y += v[4 * q + 1];
-                o.z += v[4 * q + 2];
-                o.w += v[4 * q + 3];
-                d4[q] = o;
+                for (int q = 0; q < 8; ++q)
+                  d4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+              } else {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                  float4 o = d4[q];
+                  o.x += v[4 * q];
+                  o.y += v[4 * q + 1];
+                  o.z += v[4 * q + 2];
+                  o.w += v[4 * q + 3];
+                  d4[q] = o;
+                }
               }
             } else {
-              for (int i = 0; i < 32 && col0 + i < p.N; ++i) dst[i] += v[i];
+              for (int i = 0; i < 32 && col0 + i < p.N; ++i)
+                dst[i] = p.acc_first ? v[i] : dst[i] + v[i];
             }
           }
         }
@@ -427,6 +513,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   tc_fence_after();
   if (warp == 1) tmem_dealloc_pair(tmem_base, kGTmemCols);
   cluster_sync();  // the collective release is complete in both CTAs
+}
+
+// Adds the partial tiles of the tail of a dH GEMM (the same geometry as the GEMM's,
+// from the same device-side count), part 0 first, and writes their rows in the loss:
+// a warp per row of 256 columns.
+__global__ void __launch_bounds__(256)
+    reduce_tail_kernel(GemmArgs p, int n_clusters) {
+  int64_t v = static_cast<int64_t>(*p.n_valid) - p.chunk_row0;
+  v = v < 0 ? 0 : (v > p.M ? p.M : v);
+  const int64_t m_tiles = (v + GBM - 1) / GBM;
+  const int nkb = static_cast<int>((p.K + GBK - 1) / GBK);
+  const TailSplit ts = tail_split((m_tiles + 1) / 2 * p.n_tiles, n_clusters, nkb);
+  if (ts.splits == 1) return;
+  const int lane = threadIdx.x & 31;
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < ts.tail * 2 * GBM; u += warps) {
+    const int i = u / (2 * GBM), r = u % (2 * GBM);
+    int64_t mp, nt;
+    item_of(p, m_tiles, ts.full + i, &mp, &nt);
+    const int64_t row = mp * (2 * GBM) + r;
+    if (row >= v) continue;
+    float* dst = p.rows_out + static_cast<int64_t>(p.rowidx[p.chunk_row0 + row]) * p.ldo;
+    const int64_t n0 = nt * GBN;
+    for (int c = lane * 4; c < GBN && n0 + c < p.N; c += 128) {  // N is a multiple of 64
+      float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int s = 0; s < ts.splits; ++s) {
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(
+            p.part + ((static_cast<int64_t>(s) * ts.tail + i) * (2 * GBM) + r) * GBN + c));
+        a.x += x.x;
+        a.y += x.y;
+        a.z += x.z;
+        a.w += x.w;
+      }
+      *reinterpret_cast<float4*>(dst + n0 + c) = a;
+    }
+  }
 }
 
 // Zero the gathered rows from n_valid up to the next multiple of GBM (at most
@@ -499,6 +621,11 @@ __global__ void count_used_seqs_kernel(const long long* __restrict__ seq_in, int
 
 // ---------------------------------------------------------------- host side
 
+int gemm_clusters() {
+  const int n = sm_count() / 2;
+  return n < kMaxGemmClusters ? (n > 0 ? n : 1) : kMaxGemmClusters;
+}
+
 template <bool A_MN, bool B_MN, int EPI>
 pace_status launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, GemmArgs a,
                         unsigned* round_ctr, cudaStream_t st) {
@@ -521,13 +648,20 @@ pace_status launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, GemmArgs a
   a.n_tiles = (a.N + GBN - 1) / GBN;
   const int64_t items = (a.m_tiles + 1) / 2 * a.n_tiles;
   if (items == 0) return PACE_OK;
-  const int64_t max_clusters = sm_count() / 2;
-  const int64_t grid = 2 * (items < max_clusters ? items : max_clusters);
+  // with partial tiles every cluster is launched: a short tail is spread over all
+  const int64_t max_clusters = gemm_clusters();
+  const int64_t grid = 2 * (items < max_clusters && !a.part ? items : max_clusters);
   PACE_TRY_CUDA(cudaMemsetAsync(round_ctr, 0, sizeof(unsigned), st));
   a.round_ctr = round_ctr;
   gemm_kernel<A_MN, B_MN, EPI><<<static_cast<unsigned>(grid), kGemmThreads, kGSmemBytes, st>>>(
       ta, tb, a);
-  return last_launch_status();
+  PACE_TRY(last_launch_status());
+  if (EPI == EPI_ROWS && a.part) {
+    reduce_tail_kernel<<<static_cast<unsigned>(sm_count() * 4), 256, 0, st>>>(
+        a, static_cast<int>(max_clusters));
+    return last_launch_status();
+  }
+  return PACE_OK;
 }
 
 struct BwWs {
@@ -535,6 +669,7 @@ struct BwWs {
   uint16_t* g;        // bf16 G of one chunk, 64-column blocks [ceil(V / 64)][chunk][64]
   int* n_seq_used;
   unsigned* round_ctr;  // the GEMMs' pacing counter
+  float* part;          // dH's partial tiles
 };
 
 int64_t chunk_rows(int64_t n_rows) {
@@ -548,6 +683,12 @@ void carve_bw_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, int V, BwWs* 
   w->g = cv.take<uint16_t>(static_cast<size_t>(chunk_rows(n_rows > 0 ? n_rows : 1)) * g_cols);
   w->n_seq_used = cv.take<int>(1);
   w->round_ctr = cv.take<unsigned>(1);
+  // a tail of R < kMaxGemmClusters tiles in kMaxKSplits parts at most, and no more
+  // tiles than the rows have
+  const int64_t tiles = (chunk_rows(n_rows > 0 ? n_rows : 1) + 2 * GBM - 1) / (2 * GBM) *
+                        ((H + GBN - 1) / GBN);
+  const int64_t tail = tiles < kMaxGemmClusters ? tiles : kMaxGemmClusters - 1;
+  w->part = cv.take<float>(static_cast<size_t>(tail) * kMaxKSplits * 2 * GBM * GBN);
 }
 
 }  // namespace
@@ -627,8 +768,10 @@ extern "C" pace_status pace_token_logprob_backward(
   if (!cv.fits()) return PACE_ERR_WORKSPACE;
   cudaStream_t st = as_stream(stream);
   const int64_t n_rows = batch->n_rows;
-  PACE_TRY_CUDA(cudaMemsetAsync(grad_w, 0, static_cast<size_t>(V) * H * 4, st));
-  if (n_rows == 0) return PACE_OK;
+  if (n_rows == 0) {
+    PACE_TRY_CUDA(cudaMemsetAsync(grad_w, 0, static_cast<size_t>(V) * H * 4, st));
+    return PACE_OK;
+  }
   PACE_TRY_CUDA(cudaMemsetAsync(grad_hidden, 0, static_cast<size_t>(n_rows) * H * 4, st));
   // the rows in the loss, gathered densely (always compacted here)
   PACE_TRY(run_compaction(batch, ws.lm.cw, status_dev, st));
@@ -693,6 +836,7 @@ extern "C" pace_status pace_token_logprob_backward(
       a.rowidx = ws.lm.cw.rowidx;
       a.rows_out = grad_hidden;
       a.ldo = H;
+      a.part = ws.part;
       a.status = status_dev;
       PACE_TRY((launch_gemm<false, true, EPI_ROWS>(ta, tb, a, ws.round_ctr, st)));
     }
@@ -711,6 +855,7 @@ extern "C" pace_status pace_token_logprob_backward(
       a.chunk_row0 = c0;
       a.n_valid = ws.lm.cw.total;
       a.acc_out = grad_w;
+      a.acc_first = c0 == 0 ? 1 : 0;
       a.ldo = H;
       a.status = status_dev;
       PACE_TRY((launch_gemm<true, true, EPI_ACC>(ta, tb, a, ws.round_ctr, st)));

@@ -175,3 +175,40 @@ def test_lmhead_backward_multi_chunk_trimmed(rows, frac):
     assert _rel(as_np(dh), odh) <= REL, _rel(as_np(dh), odh)
     assert _rel(as_np(dw), odw) <= REL, _rel(as_np(dw), odw)
     assert (as_np(dh)[mask == 0] == 0).all()
+
+
+@pytest.mark.parametrize("rows,H,V,keep", [(300, 256, 4097, 1.0), (257, 64, 20000, 1.0),
+                                           (2600, 320, 8200, 0.9), (5000, 1024, 4700, 1.0),
+                                           (19000, 256, 4160, 0.97), (300, 128, 4097, 0.0),
+                                           (33000, 64, 4097, 0.999)])
+def test_split_tail_and_first_chunk_store(rows, H, V, keep):
+    """dH tiles that do not fill a round split along the vocabulary (2 to 80 tiles on 76
+    clusters, 64 to 313 K steps), dW stored by the first chunk and added to by the next,
+    into gradients that held NaN before, with rows of zero dlp and no rows at all; the
+    per-element bounds of the module, against 64-bit torch."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(rows + V)
+    h = torch.randn(rows, H, device=DEV, generator=g).to(torch.bfloat16)
+    w = (torch.randn(V, H, device=DEV, generator=g) * 2 / math.sqrt(H)).to(torch.bfloat16)
+    y = torch.randint(0, V, (rows,), device=DEV, generator=g, dtype=torch.int32)
+    mask = (torch.rand(rows, device=DEV, generator=g) < keep).to(torch.uint8)
+    d = torch.randn(rows, device=DEV, generator=g) * mask
+    d[::7] = 0.0
+    b = pace.make_batch(to_dev(np.array([0, rows], np.int64)), rows, mask=mask)
+    hd, wd = h.double(), w.double()
+    z = hd @ wd.T
+    lse = torch.logsumexp(z, 1)
+    G = -torch.exp(z - lse[:, None])
+    G[torch.arange(rows, device=DEV), y.long()] += 1.0
+    G *= d.double()[:, None]
+    del z
+    gh = torch.full((rows, H), math.nan, device=DEV)
+    gw = torch.full((V, H), math.nan, device=DEV)
+    status = pace.new_status(DEV)
+    pace.token_logprob_backward(b, h, w, y, lse.float(), d, grad_hidden=gh, grad_w=gw,
+                                status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    for got, ref, mag in ((gh, G @ wd, G.abs() @ wd.abs()), (gw, G.T @ hd, G.abs().T @ hd.abs())):
+        assert torch.isfinite(got).all()
+        assert ((got.double() - ref).abs() <= ELEM * mag).all()
