@@ -34,8 +34,10 @@
 
 #include <mutex>
 
+#include "pace_block.cuh"
 #include "pace_internal.cuh"
 #include "pace_loss.cuh"
+#include "pace_rows.cuh"
 #include "pace_tma.cuh"
 
 namespace pace {
@@ -575,58 +577,86 @@ __global__ void zero_tail_rows_kernel(uint4* __restrict__ buf, int64_t row_vecs,
     buf[start * row_vecs + i] = make_uint4(0, 0, 0, 0);
 }
 
-// dLoss/dlp per row of the clipped surrogate (oracle: oracle_surrogate_grad).
-__global__ void surrogate_grad_kernel(const int64_t* __restrict__ seq_offsets,
-                                      const uint8_t* __restrict__ seq_accepted,
-                                      const uint8_t* __restrict__ mask,
-                                      const float* __restrict__ logprob,
-                                      const float* __restrict__ behav,
-                                      const float* __restrict__ adv,
-                                      const long long* __restrict__ seq_in,
-                                      const long long* __restrict__ total, int64_t n_seq,
-                                      int64_t n_rows, float eps_low, float eps_high, float dual,
-                                      int agg, const int* __restrict__ n_seq_used,
-                                      float* __restrict__ dlp) {
-  for (int64_t i = blockIdx.x; i < n_seq; i += gridDim.x) {
-    const int64_t r0 = seq_offsets[i], r1 = seq_offsets[i + 1];
-    if (r1 < r0 || r0 < 0 || r1 > n_rows) continue;
-    const bool acc = seq_accepted ? seq_accepted[i] != 0 : true;
-    const float a = adv[i];
-    const double scale = agg == PACE_AGG_TOKEN_MEAN
-                             ? 1.0 / static_cast<double>(*total)
-                             : 1.0 / (static_cast<double>(*n_seq_used) *
-                                      static_cast<double>(seq_in[i]));
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-      const bool in = acc && (mask ? mask[r] != 0 : true);
-      float g = 0.0f;
-      if (in) {
-        const float d = logprob[r] - behav[r];
-        const float dc = fminf(fmaxf(d, -20.0f), 20.0f);
-        const float rho = expf(dc);
-        const float rc = fminf(fmaxf(rho, 1.0f - eps_low), 1.0f + eps_high);
-        const float p1 = -a * rho, p2 = -a * rc;
-        const float l = fmaxf(p1, p2);
-        if (d > -20.0f && d < 20.0f && p1 >= p2) g = -a * rho;
-        if (a < 0.0f && -dual * a < l) g = 0.0f;
-        g = static_cast<float>(static_cast<double>(g) * scale);
+// dLoss/dlp per row of the clipped surrogate (oracle: oracle_surrogate_grad), 0
+// outside the loss.  The scale (1 / rows in the loss, or 1 / (sequences x rows of
+// the sequence)) is an fp64 quotient; a row's product with it is rounded once to
+// fp32 as g * hi + g * lo, scale = hi + lo in two floats (48 bits), because one
+// conversion to fp64, product and conversion back per row would bound the kernel on
+// GB300's narrow fp64 pipe.
+struct GradArgs {
+  const int64_t* seq_offsets;
+  const uint8_t* seq_accepted;
+  const uint8_t* mask;
+  const float* logprob;
+  const float* behav;
+  const float* adv;
+  int64_t n_seq, n_rows;
+  RowGeom geom;
+  float eps_low, eps_high, dual;
+  int agg;
+  const int* block_in;  // TOKEN_MEAN: rows in the loss per block of the count
+  const unsigned long long* seq_in;  // SEQ_MEAN: rows in the loss per sequence,
+  const int* n_used;                 // sequences that have any
+  float* dlp;
+};
+
+__global__ void __launch_bounds__(kRowThreads) surrogate_grad_kernel(GradArgs p) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * p.geom.per_warp;
+  double scale = 0.0;
+  if (p.agg == PACE_AGG_TOKEN_MEAN) {
+    __shared__ double s_scale;
+    long long mine = 0, total = 0;
+    for (int i = threadIdx.x; i < p.geom.blocks; i += kRowThreads) mine += p.block_in[i];
+    block_exclusive_scan<long long>(mine, &total);
+    if (threadIdx.x == 0) s_scale = 1.0 / static_cast<double>(total);
+    __syncthreads();
+    scale = s_scale;
+  }
+  for (int64_t w = w0; w < w0 + p.geom.per_warp && w < p.geom.n_tiles; ++w) {
+    const int64_t t0 = w * kRowTile;
+    const int64_t t1 = t0 + kRowTile < p.n_rows ? t0 + kRowTile : p.n_rows;
+    float lp[kRowsPerLane], bh[kRowsPerLane], g[kRowsPerLane];
+    unsigned m = 0u;
+#pragma unroll
+    for (int u = 0; u < kRowsPerLane; ++u) {
+      const int64_t r = t0 + 32 * u + lane;
+      const bool ok = r < t1;
+      lp[u] = ok ? p.logprob[r] : 0.0f;
+      bh[u] = ok ? p.behav[r] : 0.0f;
+      m |= (ok && (p.mask ? p.mask[r] != 0 : true) ? 1u : 0u) << u;
+      g[u] = 0.0f;
+    }
+    walk_pieces(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0, t1,
+                [&](int64_t seq, int64_t lo, int64_t hi, float a) {
+      const int l = static_cast<int>(lo - t0), h = static_cast<int>(hi - t0);
+      if (p.agg != PACE_AGG_TOKEN_MEAN)
+        scale = 1.0 / (static_cast<double>(*p.n_used) * static_cast<double>(p.seq_in[seq]));
+      const float s_hi = static_cast<float>(scale);
+      const float s_lo = static_cast<float>(scale - static_cast<double>(s_hi));
+#pragma unroll
+      for (int u = 0; u < kRowsPerLane; ++u) {
+        const int r = 32 * u + lane;
+        if (r >= l && r < h && (m >> u & 1u)) {
+          const float d = lp[u] - bh[u];
+          const float dc = fminf(fmaxf(d, -20.0f), 20.0f);
+          const float rho = expf(dc);
+          const float rc = fminf(fmaxf(rho, 1.0f - p.eps_low), 1.0f + p.eps_high);
+          const float p1 = -a * rho, p2 = -a * rc;
+          const float lm = fmaxf(p1, p2);
+          float x = 0.0f;
+          if (d > -20.0f && d < 20.0f && p1 >= p2) x = -a * rho;
+          if (a < 0.0f && -p.dual * a < lm) x = 0.0f;
+          g[u] = fmaf(x, s_hi, x * s_lo);
+        }
       }
-      dlp[r] = g;
+    });
+#pragma unroll
+    for (int u = 0; u < kRowsPerLane; ++u) {
+      const int64_t r = t0 + 32 * u + lane;
+      if (r < t1) p.dlp[r] = g[u];
     }
   }
-}
-
-__global__ void count_used_seqs_kernel(const long long* __restrict__ seq_in, int64_t n_seq,
-                                       int* __restrict__ out) {
-  __shared__ int sh[256];
-  int c = 0;
-  for (int64_t i = threadIdx.x; i < n_seq; i += blockDim.x) c += seq_in[i] > 0;
-  sh[threadIdx.x] = c;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = sh[0];
 }
 
 // ---------------------------------------------------------------- host side
@@ -677,7 +707,6 @@ pace_status launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, GemmArgs a
 struct BwWs {
   LmWs lm;            // compaction + gathered rows (hidden_c)
   uint16_t* g;        // bf16 G of one chunk, 64-column blocks [ceil(V / 64)][chunk][64]
-  int* n_seq_used;
   unsigned* round_ctr;  // the GEMMs' pacing counter
   float* part;          // dH's partial tiles
 };
@@ -691,7 +720,6 @@ void carve_bw_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, int V, BwWs* 
   carve_lm_ws(cv, n_rows, n_seq, H, true, &w->lm);
   const int64_t g_cols = (static_cast<int64_t>(V) + 63) / 64 * 64;
   w->g = cv.take<uint16_t>(static_cast<size_t>(chunk_rows(n_rows > 0 ? n_rows : 1)) * g_cols);
-  w->n_seq_used = cv.take<int>(1);
   w->round_ctr = cv.take<unsigned>(1);
   // a tail of R < kMaxGemmClusters tiles in kMaxKSplits parts at most, and no more
   // tiles than the rows have
@@ -706,13 +734,33 @@ void carve_bw_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, int V, BwWs* 
 
 using namespace pace;
 
+namespace pace {
+namespace {
+
+struct SurBwWs {
+  int* block_in;
+  unsigned long long* seq_in;
+  int* n_used;
+  float* adv;
+};
+
+SurBwWs carve_sur_bw_ws(Carver& cv, int64_t n_rows, int64_t n_seq) {
+  SurBwWs w;
+  const RowGeom g = row_geom(n_rows);
+  w.block_in = cv.take<int>(g.blocks > 0 ? g.blocks : 1);
+  w.seq_in = cv.take<unsigned long long>(n_seq > 0 ? n_seq : 1);
+  w.n_used = cv.take<int>(1);
+  w.adv = cv.take<float>(n_seq > 0 ? n_seq : 1);
+  return w;
+}
+
+}  // namespace
+}  // namespace pace
+
 extern "C" size_t pace_surrogate_backward_workspace_size(int64_t n_rows, int64_t n_seq) {
+  if (n_rows < 0 || n_seq < 0) return 0;
   Carver cv;
-  CompactWs cw;
-  SurrogateWs sw;
-  carve_compact_ws(cv, n_seq, n_rows, &cw);
-  carve_surrogate_ws(cv, n_seq, &sw);
-  cv.take<int>(1);
+  carve_sur_bw_ws(cv, n_rows, n_seq);
   return cv.used;
 }
 
@@ -725,30 +773,47 @@ extern "C" pace_status pace_surrogate_backward(const PaceBatch* batch, const flo
   if (batch->n_rows > 0 && (!logprob || !dlp)) return PACE_ERR_INVALID_ARG;
   if (!workspace || !aligned(workspace, 256)) return PACE_ERR_WORKSPACE;
   Carver cv(workspace, workspace_bytes);
-  CompactWs cw;
-  SurrogateWs sw;
-  carve_compact_ws(cv, batch->n_seq, batch->n_rows, &cw);
-  carve_surrogate_ws(cv, batch->n_seq, &sw);
-  int* n_used = cv.take<int>(1);
+  const SurBwWs ws = carve_sur_bw_ws(cv, batch->n_rows, batch->n_seq);
   if (!cv.fits()) return PACE_ERR_WORKSPACE;
   cudaStream_t st = as_stream(stream);
-  if (batch->n_rows > 0)
-    PACE_TRY_CUDA(cudaMemsetAsync(dlp, 0, static_cast<size_t>(batch->n_rows) * 4, st));
-  if (batch->n_seq == 0) return PACE_OK;
-  float* adv = loss->adv ? loss->adv : sw.adv;
-  PACE_TRY(launch_group_adv(loss->reward, batch->seq_accepted, batch->n_seq,
-                                   loss->group_size, loss->params.adv_eps,
-                                   loss->params.std_unbiased, adv, st));
-  PACE_TRY(run_compaction(batch, cw, status_dev, st));  // rows in the loss per sequence
-  count_used_seqs_kernel<<<1, 256, 0, st>>>(cw.seq_in, batch->n_seq, n_used);
-  PACE_TRY(last_launch_status());
-  int64_t grid = batch->n_seq;
-  const int64_t cap = static_cast<int64_t>(sm_count()) * 8;
-  if (grid > cap) grid = cap;
-  surrogate_grad_kernel<<<static_cast<unsigned>(grid), 256, 0, st>>>(
-      batch->seq_offsets, batch->seq_accepted, batch->mask, logprob, loss->behav_lp, adv,
-      cw.seq_in, cw.total, batch->n_seq, batch->n_rows, loss->params.eps_low,
-      loss->params.eps_high, loss->params.dual_clip, loss->params.agg, n_used, dlp);
+  if (batch->n_seq == 0) {
+    if (batch->n_rows > 0)
+      PACE_TRY_CUDA(cudaMemsetAsync(dlp, 0, static_cast<size_t>(batch->n_rows) * 4, st));
+    return PACE_OK;
+  }
+  float* adv = loss->adv ? loss->adv : ws.adv;
+  const AdvJob job =
+      adv_job(loss->reward, batch->seq_accepted, batch->n_seq, loss->group_size,
+              loss->params.adv_eps, loss->params.std_unbiased, adv);
+  if (batch->n_rows == 0) return launch_group_adv(job, batch, nullptr, status_dev, st);
+  const bool seq_mean = loss->params.agg != PACE_AGG_TOKEN_MEAN;
+  if (seq_mean) {
+    PACE_TRY_CUDA(cudaMemsetAsync(ws.seq_in, 0,
+                                  static_cast<size_t>(batch->n_seq) * sizeof(*ws.seq_in), st));
+    PACE_TRY_CUDA(cudaMemsetAsync(ws.n_used, 0, sizeof(int), st));
+  }
+  // rows in the loss (per block, per sequence) and the advantages, then the rows
+  PACE_TRY(launch_count_rows(batch, ws.block_in, seq_mean ? ws.seq_in : nullptr, ws.n_used, job,
+                             nullptr, nullptr, status_dev, st));
+  GradArgs a;
+  a.seq_offsets = batch->seq_offsets;
+  a.seq_accepted = batch->seq_accepted;
+  a.mask = batch->mask;
+  a.logprob = logprob;
+  a.behav = loss->behav_lp;
+  a.adv = adv;
+  a.n_seq = batch->n_seq;
+  a.n_rows = batch->n_rows;
+  a.geom = row_geom(batch->n_rows);
+  a.eps_low = loss->params.eps_low;
+  a.eps_high = loss->params.eps_high;
+  a.dual = loss->params.dual_clip;
+  a.agg = loss->params.agg;
+  a.block_in = ws.block_in;
+  a.seq_in = ws.seq_in;
+  a.n_used = ws.n_used;
+  a.dlp = dlp;
+  surrogate_grad_kernel<<<static_cast<unsigned>(a.geom.blocks), kRowThreads, 0, st>>>(a);
   return last_launch_status();
 }
 
@@ -784,7 +849,7 @@ extern "C" pace_status pace_token_logprob_backward(
   }
   PACE_TRY_CUDA(cudaMemsetAsync(grad_hidden, 0, static_cast<size_t>(n_rows) * H * 4, st));
   // the rows in the loss, gathered densely (always compacted here)
-  PACE_TRY(run_compaction(batch, ws.lm.cw, status_dev, st));
+  PACE_TRY(run_compaction(batch, ws.lm.cw, AdvJob{}, nullptr, nullptr, nullptr, nullptr, status_dev, st));
   PACE_TRY(run_gather(hidden, H, n_rows, ws.lm.cw, ws.lm.hidden_c, st));
   const int64_t rows_cap = n_rows > 128 ? n_rows : 128;
   const int64_t row_vecs = static_cast<int64_t>(H) * 2 / 16;

@@ -826,8 +826,8 @@ pace_status lm_launch_info(LmLaunchInfo* out) {
 void carve_lm_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, bool dense_rows,
                  LmWs* w) {
   const int64_t rows_cap = n_rows > BM ? n_rows : BM;
-  carve_compact_ws(cv, n_seq, n_rows, &w->cw);
-  carve_surrogate_ws(cv, n_seq, &w->sw);
+  carve_compact_ws(cv, n_rows, &w->cw);
+  carve_surrogate_ws(cv, n_rows, n_seq, &w->sw);
   w->hidden_c =
       dense_rows ? static_cast<void*>(cv.take<uint16_t>(static_cast<size_t>(rows_cap) * H))
                  : nullptr;
@@ -859,22 +859,20 @@ pace_status check_lm_args(const PaceBatch* batch, const void* hidden, const void
 }
 
 // Compaction, fused LM head and merge: lp (and lse) for every row in
-// the batch's loss, 0 elsewhere.
+// the batch's loss, 0 elsewhere.  When the rows are compacted, the same launches also
+// compute the advantages of `adv` and clear `counter` (the caller does otherwise).
 pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* w_vocab,
                         const int32_t* targets, int H, int V, float temperature, float* logprob,
-                        float* lse, const LmWs& ws, int32_t* status_dev, cudaStream_t st) {
+                        float* lse, const LmWs& ws, const AdvJob& adv, unsigned* counter,
+                        int32_t* status_dev, cudaStream_t st) {
   const int64_t n_rows = batch->n_rows;
   const bool compact = lm_needs_compaction(batch);
-  if (n_rows > 0) {
-    PACE_TRY_CUDA(cudaMemsetAsync(logprob, 0, static_cast<size_t>(n_rows) * sizeof(float), st));
-    if (lse) PACE_TRY_CUDA(cudaMemsetAsync(lse, 0, static_cast<size_t>(n_rows) * sizeof(float), st));
-  }
   const long long* n_valid_dev = nullptr;
   const int32_t* rowidx = nullptr;
   int64_t rows_cap = n_rows;
   if (compact) {
     // the LM head reads the rows in the loss through rowidx (no dense copy)
-    PACE_TRY(run_compaction(batch, ws.cw, status_dev, st));
+    PACE_TRY(run_compaction(batch, ws.cw, adv, counter, ws.round_ctr, logprob, lse, status_dev, st));
     n_valid_dev = ws.cw.total;
     rowidx = ws.cw.rowidx;
     rows_cap = n_rows > BM ? n_rows : BM;
@@ -920,7 +918,7 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   const int64_t tiles = (rows_cap + 2 * BM - 1) / (2 * BM) * n_vtiles;
   const int64_t clusters = tiles < li.max_clusters ? tiles : li.max_clusters;
   const int64_t grid = clusters * CLUSTER;
-  PACE_TRY_CUDA(cudaMemsetAsync(ws.round_ctr, 0, sizeof(unsigned), st));
+  if (!compact) PACE_TRY_CUDA(cudaMemsetAsync(ws.round_ctr, 0, sizeof(unsigned), st));
   const ProfileEvents& pe = profile_events(PACE_PROFILE_LMHEAD);
   if (pe.begin) PACE_TRY_CUDA(cudaEventRecord(pe.begin, st));
   lmhead_lse_kernel<<<static_cast<unsigned>(grid), kThreads, kSmemBytes, st>>>(am, tm_b, a);
@@ -966,8 +964,15 @@ extern "C" pace_status pace_token_logprob(const PaceBatch* batch, const void* hi
   carve_lm_ws(cv, batch->n_rows, batch->n_seq, hidden_size, false, &ws);
   if (!cv.fits()) return PACE_ERR_WORKSPACE;
   cudaStream_t st = as_stream(stream);
+  AdvJob adv{};
+  if (loss)
+    adv = adv_job(loss->reward, batch->seq_accepted, batch->n_seq, loss->group_size,
+                  loss->params.adv_eps, loss->params.std_unbiased,
+                  loss->adv ? loss->adv : ws.sw.adv);
   PACE_TRY(run_logprob(batch, hidden, w_vocab, targets, hidden_size, vocab_size, temperature,
-                       logprob, lse, ws, status_dev, st));
-  if (loss) PACE_TRY(run_surrogate(batch, logprob, loss, ws.sw, status_dev, st));
+                       logprob, lse, ws, adv, loss ? ws.sw.counter : nullptr, status_dev, st));
+  if (loss)
+    PACE_TRY(run_surrogate(batch, logprob, loss, ws.sw, lm_needs_compaction(batch), status_dev,
+                           st));
   return PACE_OK;
 }

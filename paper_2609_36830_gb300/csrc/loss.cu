@@ -10,19 +10,57 @@
 #include "pace_block.cuh"
 #include "pace_internal.cuh"
 #include "pace_loss.cuh"
+#include "pace_rows.cuh"
 
 namespace pace {
 
 // ------------------------------------------------------------ advantages
 
-// One thread per prompt group: mean and standard deviation of the accepted
-// members' rewards in fp64, summed from the lowest index up, then
-// A_i = (R_i - mean) / (std + eps).
-__global__ void group_adv_kernel(const float* __restrict__ reward,
-                                 const uint8_t* __restrict__ accepted, int64_t n_groups, int G,
-                                 double eps, int unbiased, float* __restrict__ adv) {
-  const int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (g >= n_groups) return;
+// Prompt groups of at most 32: L = 2^m >= G lanes per group (32 / L groups a warp),
+// lane k holding member k.  Mean and standard deviation of the accepted members'
+// rewards in fp64, summed from the lowest index up (the same order as one thread
+// would take), then A_i = (R_i - mean) / (std + eps), each lane its own division:
+// with a thread per group, its chain of 2 G loads and G divisions took 8-11 us.
+__device__ void group_adv_lanes(const float* __restrict__ reward,
+                                const uint8_t* __restrict__ accepted, int64_t n_groups, int G,
+                                int L, double eps, int unbiased, float* __restrict__ adv,
+                                int64_t warp) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int k = lane & (L - 1);
+  const int64_t g = warp * (32 / L) + lane / L;
+  const bool mine = g < n_groups && k < G;
+  const int64_t i = g * G + k;
+  const bool in = mine && (accepted ? accepted[i] != 0 : true);
+  const float rf = mine ? reward[i] : 0.0f;
+  const double r = static_cast<double>(rf);
+  const unsigned bal = __ballot_sync(full, in);
+  const int first = lane & ~(L - 1);
+  const unsigned members = bal >> first & (L == 32 ? full : (1u << L) - 1u);
+  const int n = __popc(members);
+  double sum = 0.0;
+  for (int m = 0; m < G; ++m) {
+    const double x = __shfl_sync(full, r, first + m);
+    if (members >> m & 1u) sum = __dadd_rn(sum, x);
+  }
+  const double mean = n > 0 ? __ddiv_rn(sum, static_cast<double>(n)) : 0.0;
+  const double d = __dsub_rn(r, mean);
+  const double dd = __dmul_rn(d, d);
+  double ss = 0.0;
+  for (int m = 0; m < G; ++m) {
+    const double x = __shfl_sync(full, dd, first + m);
+    if (members >> m & 1u) ss = __dadd_rn(ss, x);
+  }
+  const int div = unbiased ? n - 1 : n;
+  const double sd = div > 0 ? __dsqrt_rn(__ddiv_rn(ss, static_cast<double>(div))) : 0.0;
+  const double den = __dadd_rn(sd, eps);
+  if (mine) adv[i] = static_cast<float>(in && d != 0.0 ? __ddiv_rn(d, den) : 0.0);
+}
+
+// Larger groups: a thread per group, in the same order.
+__device__ void group_adv_thread(const float* __restrict__ reward,
+                                 const uint8_t* __restrict__ accepted, int64_t g, int G, double eps,
+                                 int unbiased, float* __restrict__ adv) {
   const int64_t i0 = g * G;
   int64_t n = 0;
   double sum = 0.0;
@@ -51,19 +89,53 @@ __global__ void group_adv_kernel(const float* __restrict__ reward,
   }
 }
 
-pace_status launch_group_adv(const float* reward, const uint8_t* accepted, int64_t n_seq, int G,
-                             float eps, int unbiased, float* adv, cudaStream_t st) {
-  const int64_t n_groups = n_seq / G;
-  if (n_groups == 0) return PACE_OK;
-  const int threads = 128;
-  group_adv_kernel<<<static_cast<unsigned>((n_groups + threads - 1) / threads), threads, 0, st>>>(
-      reward, accepted, n_groups, G, static_cast<double>(eps), unbiased, adv);
-  return last_launch_status();
+constexpr int kAdvThreads = 128;
+
+// The advantages a launch computes, by `blocks` of its blocks (0: none).
+AdvJob adv_job(const float* reward, const uint8_t* accepted, int64_t n_seq, int G, float eps,
+               int unbiased, float* adv) {
+  AdvJob j{};
+  j.reward = reward;
+  j.accepted = accepted;
+  j.n_groups = n_seq / G;
+  j.G = G;
+  j.L = 1;
+  while (j.L < G && j.L < 32) j.L *= 2;
+  j.eps = static_cast<double>(eps);
+  j.unbiased = unbiased;
+  j.adv = adv;
+  // warps (or threads, for groups of more than 32) over the groups
+  const int64_t per_block = G <= 32 ? kAdvThreads / j.L : kAdvThreads;
+  j.blocks = static_cast<int>((j.n_groups + per_block - 1) / per_block);
+  return j;
+}
+
+// Block b of the job's blocks (threads from kAdvThreads on have no part in it).
+__device__ void adv_block(const AdvJob& j, int64_t b) {
+  if (threadIdx.x >= kAdvThreads) return;
+  if (j.G <= 32) {
+    group_adv_lanes(j.reward, j.accepted, j.n_groups, j.G, j.L, j.eps, j.unbiased, j.adv,
+                    b * (kAdvThreads / 32) + (threadIdx.x >> 5));
+  } else {
+    const int64_t g = b * kAdvThreads + threadIdx.x;
+    if (g < j.n_groups) group_adv_thread(j.reward, j.accepted, g, j.G, j.eps, j.unbiased, j.adv);
+  }
+}
+
+// Also checks the sequence offsets and clears a counter, for the launch that follows
+// (offsets / counter may be null).
+__global__ void __launch_bounds__(kAdvThreads)
+    group_adv_kernel(AdvJob j, const int64_t* __restrict__ seq_offsets, int64_t n_seq,
+                     int64_t n_rows, unsigned* counter, int32_t* status) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (counter && t == 0) *counter = 0u;
+  if (seq_offsets)
+    for (int64_t i = t; i < n_seq; i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+      check_seq(seq_offsets, i, n_rows, status);
+  if (blockIdx.x < static_cast<unsigned>(j.blocks)) adv_block(j, blockIdx.x);
 }
 
 // ------------------------------------------------------------ surrogate
-
-constexpr int kSurThreads = 256;
 
 __device__ __forceinline__ float clipped_term(float lp, float behav, float a, float eps_low,
                                               float eps_high, float dual, float* rho_out) {
@@ -79,71 +151,162 @@ __device__ __forceinline__ float clipped_term(float lp, float behav, float a, fl
   return l;
 }
 
-// One block per sequence (grid-stride): per-token terms in fp32, the
-// sequence's sum and count in fp64 with a fixed reduction shape.
-__global__ void __launch_bounds__(kSurThreads)
-    surrogate_seq_kernel(const int64_t* __restrict__ seq_offsets,
-                         const uint8_t* __restrict__ seq_accepted,
-                         const uint8_t* __restrict__ mask, const float* __restrict__ logprob,
-                         const float* __restrict__ behav, const float* __restrict__ adv,
-                         int64_t n_seq, float eps_low, float eps_high, float dual,
-                         int64_t n_rows, float* __restrict__ ratio,
-                         double* __restrict__ seq_sum, double* __restrict__ seq_cnt,
-                         int32_t* status) {
-  __shared__ double sh[kSurThreads];
-  for (int64_t i = blockIdx.x; i < n_seq; i += gridDim.x) {
-    int64_t r0 = seq_offsets[i], r1 = seq_offsets[i + 1];
-    if (r1 < r0 || r0 < 0 || r1 > n_rows || (i == 0 && r0 != 0)) {
-      if (threadIdx.x == 0) report(status, PACE_ERR_INVALID_ARG);
-      r0 = r1 = 0;
+// The batch's numerator and denominator.  Per-token terms in fp32, every sum in
+// fp64 and in a fixed order.  TOKEN_MEAN needs the whole sums only: a lane adds its
+// rows, a warp its lanes, a block its warps, and the block that finishes last (the
+// counter, cleared by the launch before) adds the blocks' sums and divides.
+// SEQ_MEAN needs each sequence's: a warp writes the part of a sequence that begins
+// in its tile to the sequence's slot and the part of one that began earlier to the
+// tile's head slot, and the last block adds a sequence's slot and head slots.
+struct SurrogateArgs {
+  const int64_t* seq_offsets;
+  const uint8_t* seq_accepted;
+  const uint8_t* mask;
+  const float* logprob;
+  const float* behav;
+  const float* adv;
+  int64_t n_seq, n_rows;
+  RowGeom geom;
+  int agg;
+  float eps_low, eps_high, dual;
+  float* ratio;
+  SurrogateWs ws;
+  double* loss;
+  double* partial;
+};
+
+__device__ __forceinline__ double warp_sum_fixed(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+__device__ void surrogate_finish(const SurrogateArgs& p) {
+  __shared__ double sh[kRowThreads];
+  double a = 0.0, b = 0.0;
+  if (p.agg == PACE_AGG_TOKEN_MEAN) {
+    for (int i = threadIdx.x; i < p.geom.blocks; i += kRowThreads) {
+      a = __dadd_rn(a, __ldcg(p.ws.block_sum + i));
+      b = __dadd_rn(b, __ldcg(p.ws.block_cnt + i));
     }
-    const bool acc = seq_accepted ? seq_accepted[i] != 0 : true;
-    const float a = adv[i];
-    double tot = 0.0, cnt = 0.0;
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += kSurThreads) {
-      const bool in = acc && (mask ? mask[r] != 0 : true);
-      float rho = 0.0f;
-      if (in) {
-        const float l = clipped_term(logprob[r], behav[r], a, eps_low, eps_high, dual, &rho);
-        tot = __dadd_rn(tot, static_cast<double>(l));
-        cnt = __dadd_rn(cnt, 1.0);
+  } else {  // a warp per sequence
+    const int lane = threadIdx.x & 31;
+    for (int64_t i = threadIdx.x >> 5; i < p.n_seq; i += kRowWarps) {
+      const int64_t r0 = p.seq_offsets[i], r1 = p.seq_offsets[i + 1];
+      if (r0 < 0 || r1 > p.n_rows || r1 <= r0 || (p.seq_accepted && !p.seq_accepted[i])) continue;
+      double s = 0.0, c = 0.0;
+      const int64_t w0 = r0 / kRowTile, w1 = (r1 - 1) / kRowTile;
+      for (int64_t w = w0 + lane; w <= w1; w += 32) {
+        s = __dadd_rn(s, __ldcg(w == w0 ? p.ws.seq_sum + i : p.ws.head_sum + w));
+        c = __dadd_rn(c, __ldcg(w == w0 ? p.ws.seq_cnt + i : p.ws.head_cnt + w));
       }
-      if (ratio) ratio[r] = in ? rho : 0.0f;
+      s = warp_sum_fixed(s);
+      c = warp_sum_fixed(c);
+      if (lane == 0 && c > 0.0) {
+        a = __dadd_rn(a, __ddiv_rn(s, c));
+        b = __dadd_rn(b, 1.0);
+      }
     }
-    const double ts = block_sum_fixed<kSurThreads>(tot, sh);
-    const double tc = block_sum_fixed<kSurThreads>(cnt, sh);
-    if (threadIdx.x == 0) {
-      seq_sum[i] = ts;
-      seq_cnt[i] = tc;
+  }
+  const double ta = block_sum_fixed<kRowThreads>(a, sh);
+  const double tb = block_sum_fixed<kRowThreads>(b, sh);
+  if (threadIdx.x == 0) {
+    *p.loss = tb > 0.0 ? __ddiv_rn(ta, tb) : 0.0;
+    if (p.partial) {
+      p.partial[0] = ta;
+      p.partial[1] = tb;
     }
   }
 }
 
-// One block: the aggregate over sequences in a fixed order.
-__global__ void __launch_bounds__(kSurThreads)
-    surrogate_reduce_kernel(const double* __restrict__ seq_sum,
-                            const double* __restrict__ seq_cnt, int64_t n_seq, int agg,
-                            double* __restrict__ loss, double* __restrict__ partial) {
-  __shared__ double sh[kSurThreads];
-  double a = 0.0, b = 0.0;
-  for (int64_t i = threadIdx.x; i < n_seq; i += kSurThreads) {
-    if (agg == PACE_AGG_TOKEN_MEAN) {
-      a = __dadd_rn(a, seq_sum[i]);
-      b = __dadd_rn(b, seq_cnt[i]);
-    } else if (seq_cnt[i] > 0.0) {
-      a = __dadd_rn(a, __ddiv_rn(seq_sum[i], seq_cnt[i]));
-      b = __dadd_rn(b, 1.0);
+__global__ void __launch_bounds__(kRowThreads) surrogate_kernel(SurrogateArgs p) {
+  __shared__ double sh_sum[kRowWarps], sh_cnt[kRowWarps];
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * p.geom.per_warp;
+  double tot = 0.0;
+  int cnt = 0;
+  for (int64_t w = w0; w < w0 + p.geom.per_warp && w < p.geom.n_tiles; ++w) {
+    const int64_t t0 = w * kRowTile;
+    const int64_t t1 = t0 + kRowTile < p.n_rows ? t0 + kRowTile : p.n_rows;
+    float lp[kRowsPerLane], bh[kRowsPerLane], rho[kRowsPerLane];
+    unsigned m = 0u;
+#pragma unroll
+    for (int u = 0; u < kRowsPerLane; ++u) {
+      const int64_t r = t0 + 32 * u + lane;
+      const bool ok = r < t1;
+      lp[u] = ok ? p.logprob[r] : 0.0f;
+      bh[u] = ok ? p.behav[r] : 0.0f;
+      m |= (ok && (p.mask ? p.mask[r] != 0 : true) ? 1u : 0u) << u;
+      rho[u] = 0.0f;
+    }
+    double head_s = 0.0, head_c = 0.0;
+    walk_pieces(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0, t1,
+                [&](int64_t seq, int64_t lo, int64_t hi, float a) {
+      const int l = static_cast<int>(lo - t0), h = static_cast<int>(hi - t0);
+      double s = 0.0;
+      int c = 0;
+#pragma unroll
+      for (int u = 0; u < kRowsPerLane; ++u) {
+        const int r = 32 * u + lane;
+        if (r >= l && r < h && (m >> u & 1u)) {
+          const float x = clipped_term(lp[u], bh[u], a, p.eps_low, p.eps_high, p.dual, &rho[u]);
+          s = __dadd_rn(s, static_cast<double>(x));
+          ++c;
+        }
+      }
+      if (p.agg == PACE_AGG_TOKEN_MEAN) {
+        tot = __dadd_rn(tot, s);
+        cnt += c;
+        return;
+      }
+      s = warp_sum_fixed(s);
+      const double cd = static_cast<double>(__reduce_add_sync(0xffffffffu, c));
+      if (p.seq_offsets[seq] < t0) {  // the sequence began in an earlier tile
+        head_s = s;
+        head_c = cd;
+      } else if (lane == 0) {
+        p.ws.seq_sum[seq] = s;
+        p.ws.seq_cnt[seq] = cd;
+      }
+    });
+    if (p.agg != PACE_AGG_TOKEN_MEAN && lane == 0) {
+      p.ws.head_sum[w] = head_s;
+      p.ws.head_cnt[w] = head_c;
+    }
+    if (p.ratio) {
+#pragma unroll
+      for (int u = 0; u < kRowsPerLane; ++u) {
+        const int64_t r = t0 + 32 * u + lane;
+        if (r < t1) p.ratio[r] = rho[u];
+      }
     }
   }
-  const double ta = block_sum_fixed<kSurThreads>(a, sh);
-  const double tb = block_sum_fixed<kSurThreads>(b, sh);
-  if (threadIdx.x == 0) {
-    *loss = tb > 0.0 ? __ddiv_rn(ta, tb) : 0.0;
-    if (partial) {
-      partial[0] = ta;
-      partial[1] = tb;
+  if (p.agg == PACE_AGG_TOKEN_MEAN) {
+    tot = warp_sum_fixed(tot);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) {
+      sh_sum[wid] = tot;
+      sh_cnt[wid] = static_cast<double>(cnt);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double s = sh_sum[0], c = sh_cnt[0];
+      for (int i = 1; i < kRowWarps; ++i) {
+        s = __dadd_rn(s, sh_sum[i]);
+        c = __dadd_rn(c, sh_cnt[i]);
+      }
+      p.ws.block_sum[blockIdx.x] = s;
+      p.ws.block_cnt[blockIdx.x] = c;
     }
   }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(p.ws.counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  surrogate_finish(p);
 }
 
 // loss = numerator / denominator of partials summed over the parts of a batch
@@ -154,10 +317,18 @@ __global__ void loss_from_partial_kernel(const double* __restrict__ partial,
     *loss = partial[1] > 0.0 ? __ddiv_rn(partial[0], partial[1]) : 0.0;
 }
 
-void carve_surrogate_ws(Carver& cv, int64_t n_seq, SurrogateWs* w) {
+void carve_surrogate_ws(Carver& cv, int64_t n_rows, int64_t n_seq, SurrogateWs* w) {
+  const RowGeom g = row_geom(n_rows);
+  const size_t blocks = g.blocks > 0 ? g.blocks : 1;
+  const size_t tiles = g.n_tiles > 0 ? static_cast<size_t>(g.n_tiles) : 1;
   w->seq_sum = cv.take<double>(n_seq > 0 ? n_seq : 1);
   w->seq_cnt = cv.take<double>(n_seq > 0 ? n_seq : 1);
+  w->head_sum = cv.take<double>(tiles);
+  w->head_cnt = cv.take<double>(tiles);
+  w->block_sum = cv.take<double>(blocks);
+  w->block_cnt = cv.take<double>(blocks);
   w->adv = cv.take<float>(n_seq > 0 ? n_seq : 1);
+  w->counter = cv.take<unsigned>(1);
 }
 
 pace_status check_batch(const PaceBatch* b) {
@@ -180,129 +351,152 @@ pace_status check_loss_args(const PaceBatch* b, const PaceLossArgs* l) {
   return PACE_OK;
 }
 
-// Advantages, per-token terms and the aggregate; logprob is [n_rows].
+pace_status launch_group_adv(const AdvJob& j, const PaceBatch* b, unsigned* counter,
+                             int32_t* status, cudaStream_t st) {
+  if (j.blocks == 0 && !counter) return PACE_OK;
+  group_adv_kernel<<<static_cast<unsigned>(j.blocks > 0 ? j.blocks : 1), kAdvThreads, 0, st>>>(
+      j, b ? b->seq_offsets : nullptr, b ? b->n_seq : 0, b ? b->n_rows : 0, counter, status);
+  return last_launch_status();
+}
+
+// Advantages, per-token terms and the aggregate; logprob is [n_rows].  adv_done: an
+// earlier launch of the call has computed the advantages, checked the offsets and
+// cleared the counter.
 pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLossArgs* l,
-                          const SurrogateWs& ws, int32_t* status, cudaStream_t st) {
+                          const SurrogateWs& ws, bool adv_done, int32_t* status,
+                          cudaStream_t st) {
   float* adv = l->adv ? l->adv : ws.adv;
-  PACE_TRY(launch_group_adv(l->reward, b->seq_accepted, b->n_seq, l->group_size,
-                            l->params.adv_eps, l->params.std_unbiased, adv, st));
-  if (b->n_seq > 0) {
-    int64_t grid = b->n_seq;
-    const int64_t cap = static_cast<int64_t>(sm_count()) * 8;
-    if (grid > cap) grid = cap;
-    surrogate_seq_kernel<<<static_cast<unsigned>(grid), kSurThreads, 0, st>>>(
-        b->seq_offsets, b->seq_accepted, b->mask, logprob, l->behav_lp, adv, b->n_seq,
-        l->params.eps_low, l->params.eps_high, l->params.dual_clip, b->n_rows, l->ratio,
-        ws.seq_sum, ws.seq_cnt, status);
-    PACE_TRY(last_launch_status());
-  }
-  surrogate_reduce_kernel<<<1, kSurThreads, 0, st>>>(ws.seq_sum, ws.seq_cnt, b->n_seq,
-                                                     l->params.agg, l->loss, l->partial);
+  if (!adv_done)
+    PACE_TRY(launch_group_adv(adv_job(l->reward, b->seq_accepted, b->n_seq, l->group_size,
+                                      l->params.adv_eps, l->params.std_unbiased, adv),
+                              b, ws.counter, status, st));
+  SurrogateArgs a;
+  a.seq_offsets = b->seq_offsets;
+  a.seq_accepted = b->seq_accepted;
+  a.mask = b->mask;
+  a.logprob = logprob;
+  a.behav = l->behav_lp;
+  a.adv = adv;
+  a.n_seq = b->n_seq;
+  a.n_rows = b->n_rows;
+  a.geom = row_geom(b->n_rows);
+  a.agg = l->params.agg;
+  a.eps_low = l->params.eps_low;
+  a.eps_high = l->params.eps_high;
+  a.dual = l->params.dual_clip;
+  a.ratio = l->ratio;
+  a.ws = ws;
+  a.loss = l->loss;
+  a.partial = l->partial;
+  surrogate_kernel<<<static_cast<unsigned>(a.geom.blocks > 0 ? a.geom.blocks : 1), kRowThreads, 0,
+                     st>>>(a);
   return last_launch_status();
 }
 
 // ------------------------------------------------------------ compaction
 
-constexpr int kCompThreads = 256;
-
-// Per sequence: number of rows in the loss.
-__global__ void __launch_bounds__(kCompThreads)
+// Rows in the loss per block of the flat row walk; the first blocks also check the
+// offsets, and the blocks after the walk's compute the advantages of a call that
+// needs them.  Clears the two counters of the launches that follow (either may be
+// null).  seq_in (or null): rows in the loss per sequence, added to, and n_used the
+// sequences that have any.
+__global__ void __launch_bounds__(kRowThreads)
     count_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
-                      int64_t n_seq, int64_t n_rows, long long* __restrict__ seq_in,
-                      int32_t* status) {
-  __shared__ long long sh[kCompThreads];
-  for (int64_t i = blockIdx.x; i < n_seq; i += gridDim.x) {
-    const int64_t r0 = seq_offsets[i], r1 = seq_offsets[i + 1];
-    if (r1 < r0 || r0 < 0 || r1 > n_rows || (i == 0 && r0 != 0)) {
-      if (threadIdx.x == 0) {
-        report(status, PACE_ERR_INVALID_ARG);
-        seq_in[i] = 0;
-      }
-      continue;
-    }
-    const bool acc = seq_accepted ? seq_accepted[i] != 0 : true;
-    long long c = 0;
-    if (acc)
-      for (int64_t r = r0 + threadIdx.x; r < r1; r += kCompThreads) c += mask ? (mask[r] != 0) : 1;
-    sh[threadIdx.x] = c;
-    __syncthreads();
-    for (int o = kCompThreads / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) seq_in[i] = sh[0];
-    __syncthreads();
+                      int64_t n_seq, int64_t n_rows, RowGeom geom, int* __restrict__ block_in,
+                      unsigned long long* __restrict__ seq_in, int* __restrict__ n_used,
+                      AdvJob adv, unsigned* counter0, unsigned* counter1, int32_t* status) {
+  if (static_cast<int>(blockIdx.x) >= geom.blocks) {
+    adv_block(adv, blockIdx.x - geom.blocks);
+    return;
   }
-}
-
-// One block: exclusive scan of the per-sequence counts; total rows in M.
-__global__ void __launch_bounds__(1024)
-    scan_rows_kernel(const long long* __restrict__ seq_in, int64_t n_seq, int64_t n_rows,
-                     long long* __restrict__ seq_base, long long* __restrict__ total) {
-  __shared__ long long warp_sums[32];
-  __shared__ long long carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
+  __shared__ int sh[kRowWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t i0 = 0; i0 < n_seq; i0 += blockDim.x) {
-    const int64_t i = i0 + threadIdx.x;
-    const long long v = i < n_seq ? seq_in[i] : 0;
-    long long x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sums[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-      long long w = warp_sums[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      warp_sums[lane] = w;
-    }
-    __syncthreads();
-    const long long before = (wid > 0 ? warp_sums[wid - 1] : 0) + x - v;
-    if (i < n_seq) seq_base[i] = carry + before;
-    __syncthreads();
-    if (threadIdx.x == 0) carry += warp_sums[31];
-    __syncthreads();
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t == 0) {
+    if (counter0) *counter0 = 0u;
+    if (counter1) *counter1 = 0u;
   }
-  // overlapping sequences (reported by count_rows_kernel) must not overflow rowidx
-  if (threadIdx.x == 0) *total = carry < n_rows ? carry : n_rows;
+  const int64_t threads = static_cast<int64_t>(geom.blocks) * blockDim.x;
+  for (int64_t i = t; i < n_seq; i += threads) check_seq(seq_offsets, i, n_rows, status);
+  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * geom.per_warp;
+  int c = 0;
+  for (int64_t w = w0; w < w0 + geom.per_warp && w < geom.n_tiles; ++w) {
+    const int64_t t0 = w * kRowTile;
+    const unsigned in = rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, t0);
+    c += __popc(in);
+    if (seq_in) {
+      const int64_t t1 = t0 + kRowTile < n_rows ? t0 + kRowTile : n_rows;
+      walk_pieces(seq_offsets, seq_accepted, nullptr, n_seq, t0, t1,
+                  [&](int64_t seq, int64_t lo, int64_t hi, float) {
+        int k = 0;
+#pragma unroll
+        for (int u = 0; u < kRowsPerLane; ++u) {
+          const int64_t r = t0 + 32 * u + lane;
+          k += r >= lo && r < hi && (in >> u & 1u);
+        }
+        k = __reduce_add_sync(0xffffffffu, k);
+        if (lane == 0 && k > 0 && atomicAdd(seq_in + seq, static_cast<unsigned long long>(k)) == 0)
+          atomicAdd(n_used, 1);
+      });
+    }
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) sh[wid] = c;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int s = 0;
+    for (int i = 0; i < kRowWarps; ++i) s += sh[i];
+    block_in[blockIdx.x] = s;
+  }
 }
 
-// Per sequence: write the original row index of every row in the loss, in
-// row order, at the sequence's base offset.
-__global__ void __launch_bounds__(kCompThreads)
+// The row indices of the rows in the loss, in row order; their number in *total.
+// Every block adds up the counts of the blocks before it itself (at most
+// kMaxRowBlocks of them), so there is no launch for a scan.  lp and lse (or null) of
+// rows outside the loss are set to 0 here.
+__global__ void __launch_bounds__(kRowThreads)
     write_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
-                      int64_t n_seq, int64_t n_rows, const long long* __restrict__ seq_base,
-                      int32_t* __restrict__ rowidx) {
-  __shared__ int warp_sums[kCompThreads / 32];
+                      int64_t n_seq, int64_t n_rows, RowGeom geom,
+                      const int* __restrict__ block_in, int32_t* __restrict__ rowidx,
+                      long long* __restrict__ total, float* __restrict__ lp,
+                      float* __restrict__ lse) {
+  __shared__ int sh[kRowWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t i = blockIdx.x; i < n_seq; i += gridDim.x) {
-    const int64_t r0 = seq_offsets[i], r1 = seq_offsets[i + 1];
-    if (r1 < r0 || r0 < 0 || r1 > n_rows) continue;
-    if (seq_accepted && !seq_accepted[i]) continue;
-    long long base = seq_base[i];
-    for (int64_t c0 = r0; c0 < r1; c0 += kCompThreads) {
-      const int64_t r = c0 + threadIdx.x;
-      const int in = (r < r1) && (mask ? mask[r] != 0 : 1);
-      const unsigned bal = __ballot_sync(0xffffffffu, in);
-      if (lane == 0) warp_sums[wid] = __popc(bal);
-      __syncthreads();
-      int before = 0, tot = 0;
-      for (int w = 0; w < kCompThreads / 32; ++w) {
-        before += w < wid ? warp_sums[w] : 0;
-        tot += warp_sums[w];
+  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * geom.per_warp;
+  // this warp's rows in the loss (the last tile's bits are kept: mostly the only one)
+  unsigned in = 0u;
+  int c = 0;
+  for (int64_t w = w0; w < w0 + geom.per_warp && w < geom.n_tiles; ++w) {
+    in = rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w * kRowTile);
+    c += __popc(in);
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) sh[wid] = c;
+  long long mine = 0;
+  for (int i = threadIdx.x; i < static_cast<int>(blockIdx.x); i += kRowThreads) mine += block_in[i];
+  long long before = 0;
+  block_exclusive_scan<long long>(mine, &before);  // its barriers publish sh too
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1)
+    *total = before + block_in[blockIdx.x];
+  for (int i = 0; i < wid; ++i) before += sh[i];
+  for (int64_t w = w0; w < w0 + geom.per_warp && w < geom.n_tiles; ++w) {
+    const int64_t t0 = w * kRowTile;
+    if (geom.per_warp > 1)
+      in = rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, t0);
+#pragma unroll
+    for (int u = 0; u < kRowsPerLane; ++u) {
+      const int64_t r = t0 + 32 * u + lane;
+      const bool k = in >> u & 1u;
+      const unsigned bal = __ballot_sync(0xffffffffu, k);
+      if (k) {
+        rowidx[before + __popc(bal & ((1u << lane) - 1u))] = static_cast<int32_t>(r);
+      } else if (r < n_rows) {
+        if (lp) lp[r] = 0.0f;
+        if (lse) lse[r] = 0.0f;
       }
-      before += __popc(bal & ((1u << lane) - 1u));
-      if (in && base + before < n_rows) rowidx[base + before] = static_cast<int32_t>(r);
-      base += tot;
-      __syncthreads();
+      before += __popc(bal);
     }
   }
 }
@@ -323,29 +517,39 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ hidden, int64_t row
   }
 }
 
-void carve_compact_ws(Carver& cv, int64_t n_seq, int64_t n_rows, CompactWs* w) {
-  w->seq_in = cv.take<long long>(n_seq > 0 ? n_seq : 1);
-  w->seq_base = cv.take<long long>(n_seq > 0 ? n_seq : 1);
+void carve_compact_ws(Carver& cv, int64_t n_rows, CompactWs* w) {
+  const RowGeom g = row_geom(n_rows);
+  w->block_in = cv.take<int>(g.blocks > 0 ? g.blocks : 1);
   w->total = cv.take<long long>(1);
   w->rowidx = cv.take<int32_t>(n_rows > 0 ? n_rows : 1);
 }
 
-pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, int32_t* status,
-                           cudaStream_t st) {
-  if (b->n_seq == 0) {
+pace_status launch_count_rows(const PaceBatch* b, int* block_in, unsigned long long* seq_in,
+                              int* n_used, const AdvJob& adv, unsigned* counter0,
+                              unsigned* counter1, int32_t* status, cudaStream_t st) {
+  const RowGeom g = row_geom(b->n_rows);
+  count_rows_kernel<<<static_cast<unsigned>(g.blocks + adv.blocks), kRowThreads, 0, st>>>(
+      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, block_in, seq_in, n_used,
+      adv, counter0, counter1, status);
+  return last_launch_status();
+}
+
+pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob& adv,
+                           unsigned* counter0, unsigned* counter1, float* lp, float* lse,
+                           int32_t* status, cudaStream_t st) {
+  if (b->n_seq == 0 || b->n_rows == 0) {
     PACE_TRY_CUDA(cudaMemsetAsync(ws.total, 0, sizeof(long long), st));
-    return PACE_OK;
+    const size_t bytes = static_cast<size_t>(b->n_rows) * sizeof(float);
+    if (lp && bytes) PACE_TRY_CUDA(cudaMemsetAsync(lp, 0, bytes, st));
+    if (lse && bytes) PACE_TRY_CUDA(cudaMemsetAsync(lse, 0, bytes, st));
+    if (counter1) PACE_TRY_CUDA(cudaMemsetAsync(counter1, 0, sizeof(unsigned), st));
+    return launch_group_adv(adv, b, counter0, status, st);
   }
-  int64_t grid = b->n_seq;
-  const int64_t cap = static_cast<int64_t>(sm_count()) * 8;
-  if (grid > cap) grid = cap;
-  count_rows_kernel<<<static_cast<unsigned>(grid), kCompThreads, 0, st>>>(
-      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, ws.seq_in, status);
-  PACE_TRY(last_launch_status());
-  scan_rows_kernel<<<1, 1024, 0, st>>>(ws.seq_in, b->n_seq, b->n_rows, ws.seq_base, ws.total);
-  PACE_TRY(last_launch_status());
-  write_rows_kernel<<<static_cast<unsigned>(grid), kCompThreads, 0, st>>>(
-      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, ws.seq_base, ws.rowidx);
+  PACE_TRY(launch_count_rows(b, ws.block_in, nullptr, nullptr, adv, counter0, counter1, status, st));
+  const RowGeom g = row_geom(b->n_rows);
+  write_rows_kernel<<<static_cast<unsigned>(g.blocks), kRowThreads, 0, st>>>(
+      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, ws.block_in, ws.rowidx,
+      ws.total, lp, lse);
   return last_launch_status();
 }
 
@@ -382,15 +586,16 @@ extern "C" pace_status pace_group_advantages(const float* reward, const uint8_t*
   if (n_seq < 0 || group_size < 1 || n_seq % group_size != 0) return PACE_ERR_INVALID_ARG;
   if (n_seq > 0 && (!reward || !adv)) return PACE_ERR_INVALID_ARG;
   if (!(adv_eps >= 0.0f)) return PACE_ERR_INVALID_ARG;
-  return launch_group_adv(reward, seq_accepted, n_seq, group_size, adv_eps, std_unbiased, adv,
-                          as_stream(stream));
+  return launch_group_adv(
+      adv_job(reward, seq_accepted, n_seq, group_size, adv_eps, std_unbiased, adv), nullptr,
+      nullptr, nullptr, as_stream(stream));
 }
 
 extern "C" size_t pace_surrogate_loss_workspace_size(int64_t n_rows, int64_t n_seq) {
-  (void)n_rows;
+  if (n_rows < 0 || n_seq < 0) return 0;
   Carver cv;
   SurrogateWs w;
-  carve_surrogate_ws(cv, n_seq, &w);
+  carve_surrogate_ws(cv, n_rows, n_seq, &w);
   return cv.used;
 }
 
@@ -404,9 +609,9 @@ extern "C" pace_status pace_surrogate_loss(const PaceBatch* batch, const float* 
   if (!workspace || !aligned(workspace, 256)) return PACE_ERR_WORKSPACE;
   Carver cv(workspace, workspace_bytes);
   SurrogateWs ws;
-  carve_surrogate_ws(cv, batch->n_seq, &ws);
+  carve_surrogate_ws(cv, batch->n_rows, batch->n_seq, &ws);
   if (!cv.fits()) return PACE_ERR_WORKSPACE;
-  return run_surrogate(batch, logprob, loss, ws, status_dev, as_stream(stream));
+  return run_surrogate(batch, logprob, loss, ws, false, status_dev, as_stream(stream));
 }
 
 extern "C" pace_status pace_loss_from_partial(const double* partial, double* loss,

@@ -7,16 +7,32 @@
 namespace pace {
 
 struct SurrogateWs {
-  double* seq_sum;
+  double* seq_sum;    // SEQ_MEAN: per sequence, the part in the tile it begins in
   double* seq_cnt;
+  double* head_sum;   // SEQ_MEAN: per tile, the part of a sequence that began earlier
+  double* head_cnt;
+  double* block_sum;  // TOKEN_MEAN: per block
+  double* block_cnt;
   float* adv;
+  unsigned* counter;  // finished blocks
 };
 
 struct CompactWs {
-  long long* seq_in;    // rows in the loss per sequence
-  long long* seq_base;  // exclusive scan of seq_in
-  long long* total;     // M, the number of rows in the loss (clamped to n_rows)
+  int* block_in;        // rows in the loss per block of the row walk
+  long long* total;     // M, the number of rows in the loss
   int32_t* rowidx;      // [n_rows]: compact row -> original row
+};
+
+// The group advantages of a call, computed by `blocks` blocks of some launch.
+struct AdvJob {
+  const float* reward;
+  const uint8_t* accepted;
+  int64_t n_groups;
+  int G, L;
+  double eps;
+  int unbiased;
+  float* adv;
+  int blocks;
 };
 
 // Workspace of the log-prob pipeline (compaction, gathered rows, split partials).
@@ -31,9 +47,11 @@ struct LmWs {
   unsigned* round_ctr;  // the LM head's pacing counter (items whose loads were issued)
 };
 
-void carve_surrogate_ws(Carver& cv, int64_t n_seq, SurrogateWs* w);
-pace_status launch_group_adv(const float* reward, const uint8_t* accepted, int64_t n_seq, int G,
-                             float eps, int unbiased, float* adv, cudaStream_t st);
+void carve_surrogate_ws(Carver& cv, int64_t n_rows, int64_t n_seq, SurrogateWs* w);
+AdvJob adv_job(const float* reward, const uint8_t* accepted, int64_t n_seq, int G, float eps,
+               int unbiased, float* adv);
+pace_status launch_group_adv(const AdvJob& j, const PaceBatch* b, unsigned* counter,
+                             int32_t* status, cudaStream_t st);
 void carve_lm_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, bool dense_rows,
                  LmWs* w);
 bool lm_needs_compaction(const PaceBatch* b);
@@ -42,14 +60,21 @@ pace_status check_lm_args(const PaceBatch* batch, const void* hidden, const void
                           const float* logprob);
 pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* w_vocab,
                         const int32_t* targets, int H, int V, float temperature, float* logprob,
-                        float* lse, const LmWs& ws, int32_t* status_dev, cudaStream_t st);
-void carve_compact_ws(Carver& cv, int64_t n_seq, int64_t n_rows, CompactWs* w);
+                        float* lse, const LmWs& ws, const AdvJob& adv, unsigned* counter,
+                        int32_t* status_dev, cudaStream_t st);
+void carve_compact_ws(Carver& cv, int64_t n_rows, CompactWs* w);
 pace_status check_batch(const PaceBatch* b);
 pace_status check_loss_args(const PaceBatch* b, const PaceLossArgs* l);
 pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLossArgs* l,
-                          const SurrogateWs& ws, int32_t* status, cudaStream_t st);
-pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, int32_t* status,
-                           cudaStream_t st);
+                          const SurrogateWs& ws, bool adv_done, int32_t* status, cudaStream_t st);
+// Counts the rows in the loss and lists them; clears counter0 and counter1 and lp /
+// lse of the rows outside the loss (any may be null), and computes the advantages.
+pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob& adv,
+                           unsigned* counter0, unsigned* counter1, float* lp, float* lse,
+                           int32_t* status, cudaStream_t st);
+pace_status launch_count_rows(const PaceBatch* b, int* block_in, unsigned long long* seq_in,
+                              int* n_used, const AdvJob& adv, unsigned* counter0,
+                              unsigned* counter1, int32_t* status, cudaStream_t st);
 pace_status run_gather(const void* hidden, int H, int64_t n_rows, const CompactWs& ws,
                        void* out, cudaStream_t st);
 

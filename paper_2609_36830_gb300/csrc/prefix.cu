@@ -142,7 +142,7 @@ extern "C" pace_status pace_prefix_score(const PaceBatch* batch, const void* hid
   scored.seq_accepted = nullptr;
   scored.mask = ws.mask_c;
   PACE_TRY(run_logprob(&scored, hidden, w_vocab, targets, hidden_size, vocab_size, temperature,
-                       lp, nullptr, ws.lm, status_dev, st));
+                       lp, nullptr, ws.lm, AdvJob{}, nullptr, status_dev, st));
   prefix_reduce_kernel<<<static_cast<unsigned>(grid), kThreads, 0, st>>>(
       batch->seq_offsets, ws.mask_c, ws.n_elig, lp, behav_lp, batch->n_seq, batch->n_rows,
       min_tokens, cap_tokens, s_pre);
