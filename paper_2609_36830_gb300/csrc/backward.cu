@@ -594,15 +594,20 @@ struct GradArgs {
   RowGeom geom;
   float eps_low, eps_high, dual;
   int agg;
-  const int* block_in;  // TOKEN_MEAN: rows in the loss per block of the count
+  const long long* block_in;  // TOKEN_MEAN: rows in the loss per block of the count
   const unsigned long long* seq_in;  // SEQ_MEAN: rows in the loss per sequence,
   const int* n_used;                 // sequences that have any
   float* dlp;
 };
 
-__global__ void __launch_bounds__(kRowThreads) surrogate_grad_kernel(GradArgs p) {
+__global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_kernel(GradArgs p) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * p.geom.per_warp;
+  const int64_t w1 = w0 + p.geom.per_warp < p.geom.n_tiles ? w0 + p.geom.per_warp : p.geom.n_tiles;
+  int64_t t0 = w0 * kRowTile;
+  RowLoads cur, nxt;
+  // the first rows' loads are in flight while the counts are added up
+  if (w0 < w1) cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows));
   double scale = 0.0;
   if (p.agg == PACE_AGG_TOKEN_MEAN) {
     __shared__ double s_scale;
@@ -613,32 +618,23 @@ __global__ void __launch_bounds__(kRowThreads) surrogate_grad_kernel(GradArgs p)
     __syncthreads();
     scale = s_scale;
   }
-  for (int64_t w = w0; w < w0 + p.geom.per_warp && w < p.geom.n_tiles; ++w) {
-    const int64_t t0 = w * kRowTile;
-    const int64_t t1 = t0 + kRowTile < p.n_rows ? t0 + kRowTile : p.n_rows;
-    float lp[kRowsPerLane], bh[kRowsPerLane], g[kRowsPerLane];
-    unsigned m = 0u;
-#pragma unroll
-    for (int u = 0; u < kRowsPerLane; ++u) {
-      const int64_t r = t0 + 32 * u + lane;
-      const bool ok = r < t1;
-      lp[u] = ok ? p.logprob[r] : 0.0f;
-      bh[u] = ok ? p.behav[r] : 0.0f;
-      m |= (ok && (p.mask ? p.mask[r] != 0 : true) ? 1u : 0u) << u;
-      g[u] = 0.0f;
-    }
-    walk_pieces(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0, t1,
-                [&](int64_t seq, int64_t lo, int64_t hi, float a) {
-      const int l = static_cast<int>(lo - t0), h = static_cast<int>(hi - t0);
+  if (w0 >= w1) return;
+  PieceWalker pw(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0);
+  for (int64_t w = w0; w < w1; ++w) {
+    const int64_t t1 = tile_end(t0, p.n_rows);
+    if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows));
+    unsigned in = 0u;
+    pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t) {
+      const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
+      in |= rows;
       if (p.agg != PACE_AGG_TOKEN_MEAN)
         scale = 1.0 / (static_cast<double>(*p.n_used) * static_cast<double>(p.seq_in[seq]));
       const float s_hi = static_cast<float>(scale);
       const float s_lo = static_cast<float>(scale - static_cast<double>(s_hi));
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) {
-        const int r = 32 * u + lane;
-        if (r >= l && r < h && (m >> u & 1u)) {
-          const float d = lp[u] - bh[u];
+        if (rows >> u & 1u) {
+          const float d = cur.lp[u] - cur.bh[u];
           const float dc = fminf(fmaxf(d, -20.0f), 20.0f);
           const float rho = expf(dc);
           const float rc = fminf(fmaxf(rho, 1.0f - p.eps_low), 1.0f + p.eps_high);
@@ -647,15 +643,17 @@ __global__ void __launch_bounds__(kRowThreads) surrogate_grad_kernel(GradArgs p)
           float x = 0.0f;
           if (d > -20.0f && d < 20.0f && p1 >= p2) x = -a * rho;
           if (a < 0.0f && -p.dual * a < lm) x = 0.0f;
-          g[u] = fmaf(x, s_hi, x * s_lo);
+          cur.lp[u] = fmaf(x, s_hi, x * s_lo);  // the derivative, once the row is used
         }
       }
     });
 #pragma unroll
     for (int u = 0; u < kRowsPerLane; ++u) {
       const int64_t r = t0 + 32 * u + lane;
-      if (r < t1) p.dlp[r] = g[u];
+      if (r < t1) p.dlp[r] = in >> u & 1u ? cur.lp[u] : 0.0f;
     }
+    cur = nxt;
+    t0 = t1;
   }
 }
 
@@ -738,7 +736,7 @@ namespace pace {
 namespace {
 
 struct SurBwWs {
-  int* block_in;
+  RowCounts counts;
   unsigned long long* seq_in;
   int* n_used;
   float* adv;
@@ -746,8 +744,7 @@ struct SurBwWs {
 
 SurBwWs carve_sur_bw_ws(Carver& cv, int64_t n_rows, int64_t n_seq) {
   SurBwWs w;
-  const RowGeom g = row_geom(n_rows);
-  w.block_in = cv.take<int>(g.blocks > 0 ? g.blocks : 1);
+  w.counts = carve_row_counts(cv, n_rows);
   w.seq_in = cv.take<unsigned long long>(n_seq > 0 ? n_seq : 1);
   w.n_used = cv.take<int>(1);
   w.adv = cv.take<float>(n_seq > 0 ? n_seq : 1);
@@ -793,7 +790,7 @@ extern "C" pace_status pace_surrogate_backward(const PaceBatch* batch, const flo
     PACE_TRY_CUDA(cudaMemsetAsync(ws.n_used, 0, sizeof(int), st));
   }
   // rows in the loss (per block, per sequence) and the advantages, then the rows
-  PACE_TRY(launch_count_rows(batch, ws.block_in, seq_mean ? ws.seq_in : nullptr, ws.n_used, job,
+  PACE_TRY(launch_count_rows(batch, ws.counts, seq_mean ? ws.seq_in : nullptr, ws.n_used, job,
                              nullptr, nullptr, status_dev, st));
   GradArgs a;
   a.seq_offsets = batch->seq_offsets;
@@ -809,7 +806,7 @@ extern "C" pace_status pace_surrogate_backward(const PaceBatch* batch, const flo
   a.eps_high = loss->params.eps_high;
   a.dual = loss->params.dual_clip;
   a.agg = loss->params.agg;
-  a.block_in = ws.block_in;
+  a.block_in = ws.counts.block;
   a.seq_in = ws.seq_in;
   a.n_used = ws.n_used;
   a.dlp = dlp;

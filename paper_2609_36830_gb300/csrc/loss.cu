@@ -89,7 +89,7 @@ __device__ void group_adv_thread(const float* __restrict__ reward,
   }
 }
 
-constexpr int kAdvThreads = 128;
+constexpr int kAdvThreads = 32;  // a warp: the groups' fp64 divisions spread over the SMs
 
 // The advantages a launch computes, by `blocks` of its blocks (0: none).
 AdvJob adv_job(const float* reward, const uint8_t* accepted, int64_t n_seq, int G, float eps,
@@ -157,7 +157,8 @@ __device__ __forceinline__ float clipped_term(float lp, float behav, float a, fl
 // counter, cleared by the launch before) adds the blocks' sums and divides.
 // SEQ_MEAN needs each sequence's: a warp writes the part of a sequence that begins
 // in its tile to the sequence's slot and the part of one that began earlier to the
-// tile's head slot, and the last block adds a sequence's slot and head slots.
+// tile's head slot; seq_mean_kernel adds a sequence's slot and head slots, a warp
+// per sequence, and its last block adds the means.
 struct SurrogateArgs {
   const int64_t* seq_offsets;
   const uint8_t* seq_accepted;
@@ -175,138 +176,182 @@ struct SurrogateArgs {
   double* partial;
 };
 
+// A lane's running sum of a tile's terms, exact to well past fp64's 53 bits, in three
+// floats: each addition's rounding error is itself added, and that addition's error
+// kept (Knuth's two-sum, twice).  Eight terms cost one conversion to fp64 instead of
+// eight conversions and additions, which held the kernel to GB300's narrow fp64 pipe
+// (61 % busy).  Terms are below 2^60 in magnitude (|A| <= sqrt(G), rho <= e^20), so
+// no sum overflows; NaN stays NaN.
+struct Sum3 {
+  float s, e, f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(s, x);
+    const float z = __fsub_rn(t, s);
+    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
+    s = t;
+    const float t2 = __fadd_rn(e, err);
+    const float z2 = __fsub_rn(t2, e);
+    f = __fadd_rn(f, __fadd_rn(__fsub_rn(e, __fsub_rn(t2, z2)), __fsub_rn(err, z2)));
+    e = t2;
+  }
+  __device__ __forceinline__ double value() const {
+    return __dadd_rn(static_cast<double>(s),
+                     __dadd_rn(static_cast<double>(e), static_cast<double>(f)));
+  }
+};
+
 __device__ __forceinline__ double warp_sum_fixed(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 
-__device__ void surrogate_finish(const SurrogateArgs& p) {
-  __shared__ double sh[kRowThreads];
+// By the block of a launch that finishes last (uniform over each block): the sums of
+// s[0, n) and c[0, n) and the aggregate.  Every thread of every block calls it once.
+__device__ void finish_in_last_block(unsigned* counter, const double* s, const double* c,
+                                     int64_t n, double* loss, double* partial) {
+  __shared__ bool s_last;
+  __shared__ double sh_a[kRowWarps], sh_b[kRowWarps];
+  __threadfence();  // this thread's sums before the block's arrival
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
   double a = 0.0, b = 0.0;
-  if (p.agg == PACE_AGG_TOKEN_MEAN) {
-    for (int i = threadIdx.x; i < p.geom.blocks; i += kRowThreads) {
-      a = __dadd_rn(a, __ldcg(p.ws.block_sum + i));
-      b = __dadd_rn(b, __ldcg(p.ws.block_cnt + i));
+#pragma unroll 4
+  for (int64_t i = threadIdx.x; i < n; i += kRowThreads) {
+    a = __dadd_rn(a, __ldcg(s + i));
+    b = __dadd_rn(b, __ldcg(c + i));
+  }
+  a = warp_sum_fixed(a);
+  b = warp_sum_fixed(b);
+  if ((threadIdx.x & 31) == 0) {
+    sh_a[threadIdx.x >> 5] = a;
+    sh_b[threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < kRowWarps; ++i) {
+      a = __dadd_rn(a, sh_a[i]);
+      b = __dadd_rn(b, sh_b[i]);
     }
-  } else {  // a warp per sequence
-    const int lane = threadIdx.x & 31;
-    for (int64_t i = threadIdx.x >> 5; i < p.n_seq; i += kRowWarps) {
-      const int64_t r0 = p.seq_offsets[i], r1 = p.seq_offsets[i + 1];
-      if (r0 < 0 || r1 > p.n_rows || r1 <= r0 || (p.seq_accepted && !p.seq_accepted[i])) continue;
-      double s = 0.0, c = 0.0;
+    *loss = b > 0.0 ? __ddiv_rn(a, b) : 0.0;
+    if (partial) {
+      partial[0] = a;
+      partial[1] = b;
+    }
+  }
+}
+
+// SEQ_MEAN: per sequence its mean (0 without rows in the loss) and whether it has any.
+__global__ void __launch_bounds__(kRowThreads) seq_mean_kernel(SurrogateArgs p) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * kRowWarps;
+  for (int64_t i = static_cast<int64_t>(blockIdx.x) * kRowWarps + (threadIdx.x >> 5); i < p.n_seq;
+       i += warps) {
+    const int64_t r0 = p.seq_offsets[i], r1 = p.seq_offsets[i + 1];
+    const bool any = r0 >= 0 && r1 <= p.n_rows && r1 > r0 &&
+                     (p.seq_accepted ? p.seq_accepted[i] != 0 : true);
+    double s = 0.0, c = 0.0;
+    if (any) {
       const int64_t w0 = r0 / kRowTile, w1 = (r1 - 1) / kRowTile;
       for (int64_t w = w0 + lane; w <= w1; w += 32) {
         s = __dadd_rn(s, __ldcg(w == w0 ? p.ws.seq_sum + i : p.ws.head_sum + w));
         c = __dadd_rn(c, __ldcg(w == w0 ? p.ws.seq_cnt + i : p.ws.head_cnt + w));
       }
-      s = warp_sum_fixed(s);
-      c = warp_sum_fixed(c);
-      if (lane == 0 && c > 0.0) {
-        a = __dadd_rn(a, __ddiv_rn(s, c));
-        b = __dadd_rn(b, 1.0);
-      }
+    }
+    s = warp_sum_fixed(s);
+    c = warp_sum_fixed(c);
+    if (lane == 0) {
+      p.ws.seq_sum[i] = c > 0.0 ? __ddiv_rn(s, c) : 0.0;
+      p.ws.seq_cnt[i] = c > 0.0 ? 1.0 : 0.0;
     }
   }
-  const double ta = block_sum_fixed<kRowThreads>(a, sh);
-  const double tb = block_sum_fixed<kRowThreads>(b, sh);
-  if (threadIdx.x == 0) {
-    *p.loss = tb > 0.0 ? __ddiv_rn(ta, tb) : 0.0;
-    if (p.partial) {
-      p.partial[0] = ta;
-      p.partial[1] = tb;
-    }
-  }
+  finish_in_last_block(p.ws.counter, p.ws.seq_sum, p.ws.seq_cnt, p.n_seq, p.loss, p.partial);
 }
 
-__global__ void __launch_bounds__(kRowThreads) surrogate_kernel(SurrogateArgs p) {
+__global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(SurrogateArgs p) {
   __shared__ double sh_sum[kRowWarps], sh_cnt[kRowWarps];
-  __shared__ bool s_last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * p.geom.per_warp;
+  const int64_t w1 = w0 + p.geom.per_warp < p.geom.n_tiles ? w0 + p.geom.per_warp : p.geom.n_tiles;
   double tot = 0.0;
   int cnt = 0;
-  for (int64_t w = w0; w < w0 + p.geom.per_warp && w < p.geom.n_tiles; ++w) {
-    const int64_t t0 = w * kRowTile;
-    const int64_t t1 = t0 + kRowTile < p.n_rows ? t0 + kRowTile : p.n_rows;
-    float lp[kRowsPerLane], bh[kRowsPerLane], rho[kRowsPerLane];
-    unsigned m = 0u;
+  if (w0 < w1) {
+    int64_t t0 = w0 * kRowTile;
+    RowLoads cur, nxt;
+    cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows));
+    PieceWalker pw(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0);
+    for (int64_t w = w0; w < w1; ++w) {
+      const int64_t t1 = tile_end(t0, p.n_rows);
+      if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows));
+      unsigned in = 0u;
+      double head_s = 0.0, head_c = 0.0;
+      pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t begin) {
+        const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
+        in |= rows;
+        Sum3 sum{0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int u = 0; u < kRowsPerLane; ++u) {
-      const int64_t r = t0 + 32 * u + lane;
-      const bool ok = r < t1;
-      lp[u] = ok ? p.logprob[r] : 0.0f;
-      bh[u] = ok ? p.behav[r] : 0.0f;
-      m |= (ok && (p.mask ? p.mask[r] != 0 : true) ? 1u : 0u) << u;
-      rho[u] = 0.0f;
-    }
-    double head_s = 0.0, head_c = 0.0;
-    walk_pieces(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0, t1,
-                [&](int64_t seq, int64_t lo, int64_t hi, float a) {
-      const int l = static_cast<int>(lo - t0), h = static_cast<int>(hi - t0);
-      double s = 0.0;
-      int c = 0;
+        for (int u = 0; u < kRowsPerLane; ++u) {
+          if (rows >> u & 1u) {
+            float rho;
+            const float x =
+                clipped_term(cur.lp[u], cur.bh[u], a, p.eps_low, p.eps_high, p.dual, &rho);
+            cur.bh[u] = rho;  // the ratio, once the row is used
+            sum.add(x);
+          }
+        }
+        double s = sum.value();
+        const int c = __popc(rows);
+        if (p.agg == PACE_AGG_TOKEN_MEAN) {
+          tot = __dadd_rn(tot, s);
+          cnt += c;
+          return;
+        }
+        s = warp_sum_fixed(s);
+        const double cd = static_cast<double>(__reduce_add_sync(0xffffffffu, c));
+        if (begin < t0) {  // the sequence began in an earlier tile
+          head_s = s;
+          head_c = cd;
+        } else if (lane == 0) {
+          p.ws.seq_sum[seq] = s;
+          p.ws.seq_cnt[seq] = cd;
+        }
+      });
+      if (p.agg != PACE_AGG_TOKEN_MEAN && lane == 0) {
+        p.ws.head_sum[w] = head_s;
+        p.ws.head_cnt[w] = head_c;
+      }
+      if (p.ratio) {
 #pragma unroll
-      for (int u = 0; u < kRowsPerLane; ++u) {
-        const int r = 32 * u + lane;
-        if (r >= l && r < h && (m >> u & 1u)) {
-          const float x = clipped_term(lp[u], bh[u], a, p.eps_low, p.eps_high, p.dual, &rho[u]);
-          s = __dadd_rn(s, static_cast<double>(x));
-          ++c;
+        for (int u = 0; u < kRowsPerLane; ++u) {
+          const int64_t r = t0 + 32 * u + lane;
+          if (r < t1) p.ratio[r] = in >> u & 1u ? cur.bh[u] : 0.0f;
         }
       }
-      if (p.agg == PACE_AGG_TOKEN_MEAN) {
-        tot = __dadd_rn(tot, s);
-        cnt += c;
-        return;
-      }
-      s = warp_sum_fixed(s);
-      const double cd = static_cast<double>(__reduce_add_sync(0xffffffffu, c));
-      if (p.seq_offsets[seq] < t0) {  // the sequence began in an earlier tile
-        head_s = s;
-        head_c = cd;
-      } else if (lane == 0) {
-        p.ws.seq_sum[seq] = s;
-        p.ws.seq_cnt[seq] = cd;
-      }
-    });
-    if (p.agg != PACE_AGG_TOKEN_MEAN && lane == 0) {
-      p.ws.head_sum[w] = head_s;
-      p.ws.head_cnt[w] = head_c;
-    }
-    if (p.ratio) {
-#pragma unroll
-      for (int u = 0; u < kRowsPerLane; ++u) {
-        const int64_t r = t0 + 32 * u + lane;
-        if (r < t1) p.ratio[r] = rho[u];
-      }
+      cur = nxt;
+      t0 = t1;
     }
   }
-  if (p.agg == PACE_AGG_TOKEN_MEAN) {
-    tot = warp_sum_fixed(tot);
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if (lane == 0) {
-      sh_sum[wid] = tot;
-      sh_cnt[wid] = static_cast<double>(cnt);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = sh_sum[0], c = sh_cnt[0];
-      for (int i = 1; i < kRowWarps; ++i) {
-        s = __dadd_rn(s, sh_sum[i]);
-        c = __dadd_rn(c, sh_cnt[i]);
-      }
-      p.ws.block_sum[blockIdx.x] = s;
-      p.ws.block_cnt[blockIdx.x] = c;
-    }
+  if (p.agg != PACE_AGG_TOKEN_MEAN) return;
+  tot = warp_sum_fixed(tot);
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) {
+    sh_sum[wid] = tot;
+    sh_cnt[wid] = static_cast<double>(cnt);
   }
-  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(p.ws.counter, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  surrogate_finish(p);
+  if (threadIdx.x == 0) {
+    double s = sh_sum[0], c = sh_cnt[0];
+    for (int i = 1; i < kRowWarps; ++i) {
+      s = __dadd_rn(s, sh_sum[i]);
+      c = __dadd_rn(c, sh_cnt[i]);
+    }
+    p.ws.block_sum[blockIdx.x] = s;
+    p.ws.block_cnt[blockIdx.x] = c;
+  }
+  finish_in_last_block(p.ws.counter, p.ws.block_sum, p.ws.block_cnt, gridDim.x, p.loss, p.partial);
 }
 
 // loss = numerator / denominator of partials summed over the parts of a batch
@@ -390,12 +435,18 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
   a.partial = l->partial;
   surrogate_kernel<<<static_cast<unsigned>(a.geom.blocks > 0 ? a.geom.blocks : 1), kRowThreads, 0,
                      st>>>(a);
+  PACE_TRY(last_launch_status());
+  if (a.agg == PACE_AGG_TOKEN_MEAN) return PACE_OK;
+  int64_t blocks = (b->n_seq + kRowWarps - 1) / kRowWarps;
+  const int64_t most = static_cast<int64_t>(sm_count()) * 8;
+  if (blocks > most) blocks = most;
+  seq_mean_kernel<<<static_cast<unsigned>(blocks > 0 ? blocks : 1), kRowThreads, 0, st>>>(a);
   return last_launch_status();
 }
 
 // ------------------------------------------------------------ compaction
 
-// Rows in the loss per block of the flat row walk; the first blocks also check the
+// Rows in the loss per warp and per block of the row walk; the same blocks check the
 // offsets, and the blocks after the walk's compute the advantages of a call that
 // needs them.  Clears the two counters of the launches that follow (either may be
 // null).  seq_in (or null): rows in the loss per sequence, added to, and n_used the
@@ -403,14 +454,14 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
 __global__ void __launch_bounds__(kRowThreads)
     count_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
-                      int64_t n_seq, int64_t n_rows, RowGeom geom, int* __restrict__ block_in,
+                      int64_t n_seq, int64_t n_rows, RowGeom geom, RowCounts counts,
                       unsigned long long* __restrict__ seq_in, int* __restrict__ n_used,
                       AdvJob adv, unsigned* counter0, unsigned* counter1, int32_t* status) {
   if (static_cast<int>(blockIdx.x) >= geom.blocks) {
     adv_block(adv, blockIdx.x - geom.blocks);
     return;
   }
-  __shared__ int sh[kRowWarps];
+  __shared__ long long sh[kRowWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t == 0) {
@@ -419,35 +470,36 @@ __global__ void __launch_bounds__(kRowThreads)
   }
   const int64_t threads = static_cast<int64_t>(geom.blocks) * blockDim.x;
   for (int64_t i = t; i < n_seq; i += threads) check_seq(seq_offsets, i, n_rows, status);
-  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * geom.per_warp;
+  const int64_t warp = static_cast<int64_t>(blockIdx.x) * kRowWarps + wid;
+  const int64_t w0 = warp * geom.per_warp;
+  const int64_t w1 = w0 + geom.per_warp < geom.n_tiles ? w0 + geom.per_warp : geom.n_tiles;
   int c = 0;
-  for (int64_t w = w0; w < w0 + geom.per_warp && w < geom.n_tiles; ++w) {
-    const int64_t t0 = w * kRowTile;
-    const unsigned in = rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, t0);
-    c += __popc(in);
-    if (seq_in) {
-      const int64_t t1 = t0 + kRowTile < n_rows ? t0 + kRowTile : n_rows;
-      walk_pieces(seq_offsets, seq_accepted, nullptr, n_seq, t0, t1,
-                  [&](int64_t seq, int64_t lo, int64_t hi, float) {
-        int k = 0;
-#pragma unroll
-        for (int u = 0; u < kRowsPerLane; ++u) {
-          const int64_t r = t0 + 32 * u + lane;
-          k += r >= lo && r < hi && (in >> u & 1u);
-        }
-        k = __reduce_add_sync(0xffffffffu, k);
+  if (seq_in && w0 < w1) {
+    PieceWalker pw(seq_offsets, seq_accepted, nullptr, n_seq, w0 * kRowTile);
+    for (int64_t w = w0; w < w1; ++w) {
+      const int64_t t0 = w * kRowTile, t1 = tile_end(t0, n_rows);
+      const unsigned bits = load_mask_bits(mask, t0, t1);
+      pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float, int64_t) {
+        const int k = __reduce_add_sync(0xffffffffu, __popc(piece_bits(t0, lo, hi) & bits));
         if (lane == 0 && k > 0 && atomicAdd(seq_in + seq, static_cast<unsigned long long>(k)) == 0)
           atomicAdd(n_used, 1);
+        c += k;
       });
     }
+  } else {
+    walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1,
+                      [&](int64_t, int64_t, unsigned in) { c += __popc(in); });
+    c = __reduce_add_sync(0xffffffffu, c);
   }
-  c = __reduce_add_sync(0xffffffffu, c);
-  if (lane == 0) sh[wid] = c;
+  if (lane == 0) {
+    sh[wid] = c;
+    counts.warp[warp] = c;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int s = 0;
+    long long s = 0;
     for (int i = 0; i < kRowWarps; ++i) s += sh[i];
-    block_in[blockIdx.x] = s;
+    counts.block[blockIdx.x] = s;
   }
 }
 
@@ -458,33 +510,24 @@ __global__ void __launch_bounds__(kRowThreads)
 __global__ void __launch_bounds__(kRowThreads)
     write_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
-                      int64_t n_seq, int64_t n_rows, RowGeom geom,
-                      const int* __restrict__ block_in, int32_t* __restrict__ rowidx,
-                      long long* __restrict__ total, float* __restrict__ lp,
-                      float* __restrict__ lse) {
-  __shared__ int sh[kRowWarps];
+                      int64_t n_seq, int64_t n_rows, RowGeom geom, RowCounts counts,
+                      int32_t* __restrict__ rowidx, long long* __restrict__ total,
+                      float* __restrict__ lp, float* __restrict__ lse) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * geom.per_warp;
-  // this warp's rows in the loss (the last tile's bits are kept: mostly the only one)
-  unsigned in = 0u;
-  int c = 0;
-  for (int64_t w = w0; w < w0 + geom.per_warp && w < geom.n_tiles; ++w) {
-    in = rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w * kRowTile);
-    c += __popc(in);
-  }
-  c = __reduce_add_sync(0xffffffffu, c);
-  if (lane == 0) sh[wid] = c;
+  const int64_t warp = static_cast<int64_t>(blockIdx.x) * kRowWarps + wid;
+  const int64_t w0 = warp * geom.per_warp;
+  const int64_t w1 = w0 + geom.per_warp < geom.n_tiles ? w0 + geom.per_warp : geom.n_tiles;
   long long mine = 0;
-  for (int i = threadIdx.x; i < static_cast<int>(blockIdx.x); i += kRowThreads) mine += block_in[i];
+  for (int i = threadIdx.x; i < static_cast<int>(blockIdx.x); i += kRowThreads)
+    mine += counts.block[i];
+  const int wc = lane < wid ? counts.warp[warp - wid + lane] : 0;
   long long before = 0;
-  block_exclusive_scan<long long>(mine, &before);  // its barriers publish sh too
+  block_exclusive_scan<long long>(mine, &before);
   if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1)
-    *total = before + block_in[blockIdx.x];
-  for (int i = 0; i < wid; ++i) before += sh[i];
-  for (int64_t w = w0; w < w0 + geom.per_warp && w < geom.n_tiles; ++w) {
-    const int64_t t0 = w * kRowTile;
-    if (geom.per_warp > 1)
-      in = rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, t0);
+    *total = before + counts.block[blockIdx.x];
+  before += __reduce_add_sync(0xffffffffu, wc);
+  walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1,
+                    [&](int64_t t0, int64_t t1, unsigned in) {
 #pragma unroll
     for (int u = 0; u < kRowsPerLane; ++u) {
       const int64_t r = t0 + 32 * u + lane;
@@ -492,13 +535,13 @@ __global__ void __launch_bounds__(kRowThreads)
       const unsigned bal = __ballot_sync(0xffffffffu, k);
       if (k) {
         rowidx[before + __popc(bal & ((1u << lane) - 1u))] = static_cast<int32_t>(r);
-      } else if (r < n_rows) {
+      } else if (r < t1) {
         if (lp) lp[r] = 0.0f;
         if (lse) lse[r] = 0.0f;
       }
       before += __popc(bal);
     }
-  }
+  });
 }
 
 // Copy the hidden rows listed in rowidx into a dense buffer, one warp per row,
@@ -517,19 +560,27 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ hidden, int64_t row
   }
 }
 
-void carve_compact_ws(Carver& cv, int64_t n_rows, CompactWs* w) {
+RowCounts carve_row_counts(Carver& cv, int64_t n_rows) {
   const RowGeom g = row_geom(n_rows);
-  w->block_in = cv.take<int>(g.blocks > 0 ? g.blocks : 1);
+  const size_t blocks = g.blocks > 0 ? g.blocks : 1;
+  RowCounts c;
+  c.block = cv.take<long long>(blocks);
+  c.warp = cv.take<int>(blocks * kRowWarps);
+  return c;
+}
+
+void carve_compact_ws(Carver& cv, int64_t n_rows, CompactWs* w) {
+  w->counts = carve_row_counts(cv, n_rows);
   w->total = cv.take<long long>(1);
   w->rowidx = cv.take<int32_t>(n_rows > 0 ? n_rows : 1);
 }
 
-pace_status launch_count_rows(const PaceBatch* b, int* block_in, unsigned long long* seq_in,
+pace_status launch_count_rows(const PaceBatch* b, RowCounts counts, unsigned long long* seq_in,
                               int* n_used, const AdvJob& adv, unsigned* counter0,
                               unsigned* counter1, int32_t* status, cudaStream_t st) {
   const RowGeom g = row_geom(b->n_rows);
   count_rows_kernel<<<static_cast<unsigned>(g.blocks + adv.blocks), kRowThreads, 0, st>>>(
-      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, block_in, seq_in, n_used,
+      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, counts, seq_in, n_used,
       adv, counter0, counter1, status);
   return last_launch_status();
 }
@@ -545,10 +596,10 @@ pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob
     if (counter1) PACE_TRY_CUDA(cudaMemsetAsync(counter1, 0, sizeof(unsigned), st));
     return launch_group_adv(adv, b, counter0, status, st);
   }
-  PACE_TRY(launch_count_rows(b, ws.block_in, nullptr, nullptr, adv, counter0, counter1, status, st));
+  PACE_TRY(launch_count_rows(b, ws.counts, nullptr, nullptr, adv, counter0, counter1, status, st));
   const RowGeom g = row_geom(b->n_rows);
   write_rows_kernel<<<static_cast<unsigned>(g.blocks), kRowThreads, 0, st>>>(
-      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, ws.block_in, ws.rowidx,
+      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, ws.counts, ws.rowidx,
       ws.total, lp, lse);
   return last_launch_status();
 }

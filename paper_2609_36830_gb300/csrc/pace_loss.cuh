@@ -17,8 +17,13 @@ struct SurrogateWs {
   unsigned* counter;  // finished blocks
 };
 
+struct RowCounts {
+  long long* block;  // rows in the loss per block of the row walk,
+  int* warp;         // and per warp
+};
+
 struct CompactWs {
-  int* block_in;        // rows in the loss per block of the row walk
+  RowCounts counts;
   long long* total;     // M, the number of rows in the loss
   int32_t* rowidx;      // [n_rows]: compact row -> original row
 };
@@ -72,7 +77,8 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
 pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob& adv,
                            unsigned* counter0, unsigned* counter1, float* lp, float* lse,
                            int32_t* status, cudaStream_t st);
-pace_status launch_count_rows(const PaceBatch* b, int* block_in, unsigned long long* seq_in,
+RowCounts carve_row_counts(Carver& cv, int64_t n_rows);
+pace_status launch_count_rows(const PaceBatch* b, RowCounts counts, unsigned long long* seq_in,
                               int* n_used, const AdvJob& adv, unsigned* counter0,
                               unsigned* counter1, int32_t* status, cudaStream_t st);
 pace_status run_gather(const void* hidden, int H, int64_t n_rows, const CompactWs& ws,

@@ -355,3 +355,29 @@ def test_concurrent_launches_on_two_streams():
     assert all(int(st.item()) == 0 for st in statuses)
     for lp, r in zip(outs, ref):
         np.testing.assert_array_equal(as_np(lp), r)
+
+
+def test_row_list_of_several_tiles_a_warp():
+    """A million rows (more than one 256-row tile a warp of the row walk), masked at
+    random and in runs, over sequences of many lengths: every row in the loss gets its
+    own log-prob and the others 0.  Bound: 32-bit sums of 64 products (|z| < 12)."""
+    H, V, n = 64, 96, 1_000_003
+    g = torch.Generator(device=DEV)
+    g.manual_seed(9)
+    h = torch.randn(n, H, device=DEV, generator=g).to(torch.bfloat16)
+    w = (torch.randn(V, H, device=DEV, generator=g) / 4).to(torch.bfloat16)
+    y = torch.randint(0, V, (n,), device=DEV, generator=g, dtype=torch.int32)
+    rng = np.random.default_rng(2)
+    cuts = np.sort(rng.choice(n, size=3000, replace=False))
+    so = to_dev(np.concatenate([[0], cuts, [n]]).astype(np.int64))
+    acc = to_dev((rng.random(3001) < 0.8).astype(np.uint8))
+    mask = torch.rand(n, device=DEV, generator=g) < 0.9
+    mask[400_000:600_000] = True
+    lp, _ = _run(h, w, y, seq_offsets=so, seq_accepted=acc, mask=mask.to(torch.uint8))
+    sel = mask & (torch.repeat_interleave(acc, torch.diff(so)) == 1)
+    z = h.float() @ w.float().T
+    ref = as_np(z.gather(1, y.long()[:, None])[:, 0] - torch.logsumexp(z, 1))
+    sel = as_np(sel)
+    tol = 4 * 12 * 64 * 2.0 ** -24
+    assert np.abs(lp - ref)[sel].max() <= tol
+    assert (lp[~sel] == 0).all()

@@ -109,3 +109,64 @@ def test_empty_loss_is_zero_and_bad_offsets_reported():
     pace.surrogate_loss(b, to_dev(np.zeros(5, np.float32)), la, status=status)
     torch.cuda.synchronize()
     assert int(status.item()) == pace.ERR_INVALID_ARG
+
+
+def _layout(kind, rng):
+    if kind == "short":      # more sequences than a walker holds, in every tile, and empty ones
+        return rng.integers(0, 6, size=1200)
+    if kind == "edges":      # tile edges on sequence edges, empties there too
+        return np.array([256, 0, 0, 255, 1, 0, 512, 257, 0, 511, 1, 1, 0, 2, 254, 0])
+    if kind == "one":
+        return np.array([1])
+    if kind == "gap":        # long sequences between short ones
+        return np.array([0, 3000, 1, 5000, 0, 1, 2, 4097, 31, 0])
+    return rng.integers(0, 4000, size=608)  # several tiles a warp
+
+
+@pytest.mark.parametrize("kind,G", [("short", 40), ("short", 5), ("edges", 8), ("one", 1),
+                                    ("gap", 2), ("long", 32), ("long", 1)])
+@pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
+@pytest.mark.parametrize("masked", [False, True])
+def test_row_tiles_of_any_layout(kind, G, agg, masked):
+    """The loss, the ratios and the derivative over sequences of every length relative to
+    the 256-row tiles.  Ratios lie off the clip edges, so fp32 and fp64 take the same
+    branch; a term is within 16 roundings of fp32 (expf 2 ulp), sums are fp64."""
+    rng = np.random.default_rng(G)
+    lens = _layout(kind, rng)
+    so = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    n_seq, n = lens.size, int(so[-1])
+    lp = (-3.0 * rng.random(n)).astype(np.float32)
+    d = rng.choice([-25.0, -0.5, -0.1, 0.0, 0.1, 0.2, 0.4, 2.0, 3.0], size=n)
+    behav = (lp - d).astype(np.float32)
+    mask = (rng.random(n) < 0.6).astype(np.uint8) if masked else None
+    acc = (rng.random(n_seq) < 0.7).astype(np.uint8) if masked else None
+    reward = rng.choice([0.0, 0.5, 1.0], size=n_seq).astype(np.float32)
+    params = pace.loss_params(agg=agg)
+    loss = torch.full((1,), 7.0, dtype=torch.float64, device=DEV)
+    ratio = torch.full((n,), 7.0, dtype=torch.float32, device=DEV)
+    adv = torch.empty(n_seq, dtype=torch.float32, device=DEV)
+    la = pace.make_loss_args(to_dev(behav), to_dev(reward), G, params, loss, adv_out=adv,
+                             ratio_out=ratio)
+    b = pace.make_batch(to_dev(so), n, seq_accepted=None if acc is None else to_dev(acc),
+                        mask=None if mask is None else to_dev(mask))
+    status = pace.new_status(DEV)
+    dlp = torch.full((n,), 7.0, dtype=torch.float32, device=DEV)
+    pace.surrogate_loss(b, to_dev(lp), la, status=status)
+    pace.surrogate_backward(b, to_dev(lp), la, dlp=dlp, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    _, oadv = oracle.group_advantages(reward, G, seq_accepted=acc, eps=float(np.float32(1e-6)))
+    np.testing.assert_array_equal(as_np(adv), oadv.astype(np.float32))
+    # the oracle takes the rounded differences the kernel sees
+    kw = dict(mask=mask, seq_accepted=acc, eps_low=float(np.float32(0.2)),
+              eps_high=float(np.float32(0.28)), agg=agg)
+    a32 = oadv.astype(np.float32)
+    d32 = (lp - behav).astype(np.float64)
+    st, oloss, oratio, oterm = oracle.surrogate(d32, np.zeros(n), so, a32, **kw)
+    assert st == 0
+    st, odlp = oracle.surrogate_grad(d32, np.zeros(n), so, a32, **kw)
+    assert st == 0
+    unit = 16 * 2.0 ** -24
+    assert abs(float(loss.item()) - oloss) <= unit * max(np.abs(oterm).max(initial=0.0), 1e-30)
+    assert (np.abs(as_np(ratio) - oratio) <= unit * oratio).all()
+    assert (np.abs(as_np(dlp) - odlp) <= unit * np.abs(odlp)).all()
