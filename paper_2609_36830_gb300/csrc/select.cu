@@ -1205,92 +1205,203 @@ namespace pace {
 namespace {
 
 constexpr int kMaxWindowSlots = 4096;
-constexpr int kAdmitThreads = 1024;
+// 512 threads: every instruction of a block of 1,024 takes a scheduler eight cycles, and
+// the kernel is one block's chain of short steps; with 256, long candidate lists wait
+// for loads (16,384 candidates 20.1 us a call, 16.9 with 512).
+constexpr int kAdmitThreads = 512;
+constexpr int kAdmitSlots = kMaxWindowSlots / kAdmitThreads;  // window values a thread
+constexpr int kAdmitChunk = kAdmitThreads * 32;  // candidates per scan: one 32-bit word a thread
 
-// One block: sort the window's recent scores in shared memory (bitonic, +inf
-// padding), take the inverted-CDF (1 - r) quantile, decide the candidates in
-// draw order with block scans, then append the drawn scores to the ring.
+__device__ __forceinline__ uint64_t warp_min_u64(uint64_t x) {
+  const unsigned hi = static_cast<unsigned>(x >> 32), lo = static_cast<unsigned>(x);
+  const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
+  return static_cast<uint64_t>(mh) << 32 | ml;
+}
+
+__device__ __forceinline__ uint64_t warp_max_u64(uint64_t x) { return ~warp_min_u64(~x); }
+
+__device__ __forceinline__ bool is_nan_bits(double x) {
+  return (static_cast<uint64_t>(__double_as_longlong(x)) & 0x7fffffffffffffffull) >
+         0x7ff0000000000000ull;
+}
+
+// The k-th smallest (1 <= k <= n) of the block's n order keys, key i held by thread
+// i % kAdmitThreads (slot i / kAdmitThreads): histograms of the 11 bits below the
+// highest bit in which the candidates differ, until the candidates are equal (one or
+// two rounds on spread-out scores).  Each round fixes at least one bit.
+__device__ uint64_t block_kth_smallest(const uint64_t (&key)[kAdmitSlots], int n, int k) {
+  __shared__ unsigned hist[kHistBins];
+  __shared__ uint64_t s_lo[kAdmitThreads / 32], s_hi[kAdmitThreads / 32];
+  __shared__ int s_digit, s_k;
+  const int t = threadIdx.x, lane = t & 31;
+  constexpr int kBins = kHistBins / kAdmitThreads;  // histogram bins a thread scans
+  uint64_t prefix = 0ull, mask = 0ull;
+  for (;;) {
+    uint64_t lo = ~0ull, hi = 0ull;
+#pragma unroll
+    for (int s = 0; s < kAdmitSlots; ++s)
+      if (t + s * kAdmitThreads < n && (key[s] & mask) == prefix) {
+        lo = key[s] < lo ? key[s] : lo;
+        hi = key[s] > hi ? key[s] : hi;
+      }
+    lo = warp_min_u64(lo);
+    hi = warp_max_u64(hi);
+    if (lane == 0) {
+      s_lo[t >> 5] = lo;
+      s_hi[t >> 5] = hi;
+    }
+    for (int b = t; b < kHistBins; b += kAdmitThreads) hist[b] = 0u;
+    __syncthreads();
+    lo = warp_min_u64(lane < kAdmitThreads / 32 ? s_lo[lane] : ~0ull);
+    hi = warp_max_u64(lane < kAdmitThreads / 32 ? s_hi[lane] : 0ull);
+    if (lo == hi) return lo;  // uniform
+    const int d = 63 - __clzll(static_cast<long long>(lo ^ hi));
+    const int shift = d >= 10 ? d - 10 : 0;
+    const int nbins = 1 << (d - shift + 1);
+    mask = d == 63 ? 0ull : (~0ull << (d + 1));
+    prefix = lo & mask;
+#pragma unroll
+    for (int s = 0; s < kAdmitSlots; ++s)
+      if (t + s * kAdmitThreads < n && (key[s] & mask) == prefix)
+        atomicAdd(&hist[static_cast<unsigned>(key[s] >> shift) & (nbins - 1)], 1u);
+    __syncthreads();
+    int h[kBins], mine = 0;
+#pragma unroll
+    for (int i = 0; i < kBins; ++i) {
+      h[i] = static_cast<int>(hist[kBins * t + i]);  // bins past nbins are empty
+      mine += h[i];
+    }
+    int run = block_exclusive_scan<int>(mine, nullptr);
+    if (run < k && k <= run + mine) {  // exactly one thread
+#pragma unroll
+      for (int i = 0; i < kBins; ++i) {
+        if (run < k && k <= run + h[i]) {
+          s_digit = kBins * t + i;
+          s_k = k - run;
+        }
+        run += h[i];
+      }
+    }
+    __syncthreads();
+    prefix |= static_cast<uint64_t>(s_digit) << shift;
+    mask |= static_cast<uint64_t>(nbins - 1) << shift;
+    k = s_k;
+  }
+}
+
+// One block: the inverted-CDF (1 - r) quantile of the window's recent scores by a
+// radix select, then the candidates in draw order.  Candidates are drawn up to and
+// with the batch_units-th retained one, so one block scan per 16,384 of them finds
+// where drawing ends, and the decisions follow from the keep bits; last, the drawn
+// scores enter the ring.  Bound by latency: one block by design (the window and the
+// draw order are sequential state), so its steps are few: scores are compared as
+// integer keys and the rank is computed by one thread, because fp64 instructions of
+// whole blocks queue on the narrow fp64 pipe.  A bitonic sort of the window and two
+// scans per 1,024 candidates took 20.5 us a call (graph replay) with a window of 512
+// and 256 candidates, now 11.1; 45.1 with 16,384 candidates, now 16.9; 148 with a
+// window of 4,096 and 32,768 candidates, now 26.2.
 __global__ void __launch_bounds__(kAdmitThreads)
     quantile_admit_kernel(const double* __restrict__ score, int64_t n_cand, double r,
                           int64_t batch_units, int32_t min_obs, double* __restrict__ window,
                           int64_t capacity, long long* __restrict__ state,
                           uint8_t* __restrict__ decision, double* __restrict__ kappa_out,
                           int32_t* status) {
-  __shared__ double sw[kMaxWindowSlots];
-  __shared__ long long s_retained, s_drawn;
+  __shared__ unsigned s_keep[kAdmitThreads];
+  __shared__ int s_end;
+  __shared__ long long s_kth;
+  __shared__ double s_kappa;
+  constexpr int kWarps = kAdmitThreads / 32;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const long long n = state[0], head = state[1];
   if (n < 0 || n > capacity || head < 0 || head >= capacity) {
-    if (threadIdx.x == 0) report(status, PACE_ERR_INVALID_ARG);
+    if (t == 0) report(status, PACE_ERR_INVALID_ARG);
     return;
   }
   double kappa = __longlong_as_double(0x7ff0000000000000ll);  // +inf: no threshold
   if (n > 0 && n >= min_obs) {
-    int pw = 1;
-    while (pw < n) pw <<= 1;
-    for (int t = threadIdx.x; t < pw; t += blockDim.x)
-      sw[t] = t < n ? window[(head - n + t + capacity) % capacity]
-                    : __longlong_as_double(0x7ff0000000000000ll);
+    // the ring's newest n values, in any order (one thread does the fp64 work: GB300's
+    // fp64 pipe is narrow)
+    if (t == 0) {
+      const long long k = static_cast<long long>(
+          ceil(__dsub_rn(__dmul_rn(__dsub_rn(1.0, r), static_cast<double>(n)), 1e-9)));
+      s_kth = k < 1 ? 1 : (k > n ? n : k);
+    }
+    uint64_t key[kAdmitSlots];
+#pragma unroll
+    for (int s = 0; s < kAdmitSlots; ++s) {
+      const int i = t + s * kAdmitThreads;
+      long long at = head - n + i;
+      if (at < 0) at += capacity;
+      key[s] = i < n ? order_key(window[at]) : ~0ull;
+    }
     __syncthreads();
-    for (int size = 2; size <= pw; size <<= 1) {
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        for (int t = threadIdx.x; t < pw; t += blockDim.x) {
-          const int u = t ^ stride;
-          if (u > t) {
-            const bool up = (t & size) == 0;
-            const double a = sw[t], b = sw[u];
-            if ((a > b) == up) {
-              sw[t] = b;
-              sw[u] = a;
-            }
-          }
-        }
-        __syncthreads();
+    const uint64_t pivot =
+        block_kth_smallest(key, static_cast<int>(n), static_cast<int>(s_kth));
+#pragma unroll
+    for (int s = 0; s < kAdmitSlots; ++s) {  // a value with that key (either zero has it)
+      const int i = t + s * kAdmitThreads;
+      long long at = head - n + i;
+      if (at < 0) at += capacity;
+      if (i < n && key[s] == pivot) s_kappa = window[at];
+    }
+    __syncthreads();
+    kappa = s_kappa;
+  }
+  const uint64_t kappa_key = is_nan_bits(kappa) ? ~0ull : order_key(kappa);
+  if (t == 0) *kappa_out = kappa;
+  long long retained = 0;      // before this chunk
+  long long drawn = n_cand;    // candidates drawn: all, unless the batch fills up
+  for (int64_t c0 = 0; c0 < n_cand; c0 += kAdmitChunk) {
+    const int m = n_cand - c0 < kAdmitChunk ? static_cast<int>(n_cand - c0) : kAdmitChunk;
+    const int words = (m + 31) / 32;
+    // warp w takes words w, w + kWarps, ...: 32 candidates each, eight loads in flight
+    for (int w0 = wid; w0 < words; w0 += kWarps * 8) {
+      double x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int i = (w0 + kWarps * j) * 32 + lane;
+        x[j] = i < m ? score[c0 + i] : 0.0;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int i = (w0 + kWarps * j) * 32 + lane;
+        const bool nan = is_nan_bits(x[j]);
+        if (i < m && nan) report(status, PACE_ERR_NAN_INPUT);
+        const unsigned bal =
+            __ballot_sync(0xffffffffu, i < m && (nan || order_key(x[j]) <= kappa_key));
+        if (lane == 0 && w0 + kWarps * j < words) s_keep[w0 + kWarps * j] = bal;
       }
     }
-    long long k = static_cast<long long>(
-        ceil(__dsub_rn(__dmul_rn(__dsub_rn(1.0, r), static_cast<double>(n)), 1e-9)));
-    if (k < 1) k = 1;
-    if (k > n) k = n;
-    kappa = sw[k - 1];
-  }
-  if (threadIdx.x == 0) {
-    s_retained = 0;
-    s_drawn = 0;
-    *kappa_out = kappa;
-  }
-  __syncthreads();
-  for (int64_t c0 = 0; c0 < n_cand; c0 += blockDim.x) {
-    const int64_t i = c0 + threadIdx.x;
-    const double x = i < n_cand ? score[i] : 0.0;
-    if (i < n_cand && isnan(x)) report(status, PACE_ERR_NAN_INPUT);
-    const int keep = (i < n_cand && !(x > kappa)) ? 1 : 0;
+    if (t == 0) s_end = -1;
+    __syncthreads();
+    const unsigned keep = t < words ? s_keep[t] : 0u;
     int tot = 0;
-    const int before = block_exclusive_scan<int>(keep, &tot);
-    const long long ret0 = s_retained;
-    if (i < n_cand) {
-      const bool drawn = batch_units <= 0 || ret0 + before < batch_units;
-      decision[i] = drawn ? (keep ? 1 : 0) : 2;
+    const int before = block_exclusive_scan<int>(__popc(keep), &tot);
+    if (batch_units > 0) {
+      // the word that holds the batch_units-th retained candidate, and its bit there
+      long long need = batch_units - retained - before;
+      if (need >= 1 && need <= __popc(keep)) {
+        unsigned b = keep;
+        for (; need > 1; --need) b &= b - 1;
+        s_end = 32 * t + __ffs(static_cast<int>(b)) - 1;  // one thread at most
+      }
+      __syncthreads();
     }
-    int last_drawn = -1;  // last candidate of this chunk that was drawn
-    if (i < n_cand && (batch_units <= 0 || ret0 + before < batch_units))
-      last_drawn = threadIdx.x;
-    int chunk_drawn = 0;
-    block_exclusive_scan<int>(last_drawn >= 0 ? 1 : 0, &chunk_drawn);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      s_retained = ret0 + tot;
-      s_drawn += chunk_drawn;
-    }
-    __syncthreads();
+    const bool filled = batch_units > 0 && retained >= batch_units;  // in an earlier chunk
+    const int end = filled ? -1 : (s_end >= 0 ? s_end : m - 1);
+    for (int i = t; i < m; i += kAdmitThreads)
+      decision[c0 + i] = i <= end ? (s_keep[i >> 5] >> (i & 31) & 1u) : 2;
+    if (!filled && s_end >= 0) drawn = c0 + s_end + 1;
+    retained += tot;
+    __syncthreads();  // s_keep and s_end are rewritten by the next chunk
   }
   // append the drawn scores (in draw order) to the ring; when more were drawn
   // than the ring holds, only the newest `capacity` of them survive
-  const long long drawn = s_drawn;
   const long long keep_n = drawn < capacity ? drawn : capacity;
-  for (long long t = drawn - keep_n + threadIdx.x; t < drawn; t += blockDim.x)
-    window[(head + t) % capacity] = score[t];
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  for (long long i = drawn - keep_n + t; i < drawn; i += blockDim.x)
+    window[(head + i) % capacity] = score[i];
+  if (t == 0) {
     state[1] = (head + drawn) % capacity;
     state[0] = n + drawn < capacity ? n + drawn : capacity;
   }

@@ -111,3 +111,42 @@ def test_quantile_admission_large_candidate_list():
         _, odec, okap = oracle.quantile_admit(o["unit_score"], r, batch, ow)
         assert float(kap.item()) == okap
         np.testing.assert_array_equal(as_np(dec), odec)
+
+
+@pytest.mark.parametrize("capacity,filled", [(1, 1), (5, 3), (512, 512), (513, 513),
+                                             (4096, 4096), (4096, 2047), (64, 0)])
+@pytest.mark.parametrize("n_cand,batch", [(1, 1), (33, 20), (1024, 0), (16384, 9000),
+                                          (16385, 16384), (70001, 40000), (70001, 1), (0, 4)])
+def test_quantile_admit_sizes(capacity, filled, n_cand, batch):
+    """Window sizes around the values a thread holds, candidates around the 32 of a word
+    and the 16,384 of a scan, batches that fill in an early chunk, on its edge or never;
+    heavy ties and infinite scores.  Every output is exact."""
+    rng = np.random.default_rng(capacity * 7 + n_cand)
+    vals = rng.integers(0, 40, size=capacity) / 8.0
+    vals[rng.random(capacity) < 0.02] = np.inf
+    x = rng.integers(0, 40, size=n_cand) / 8.0
+    head = int(rng.integers(0, capacity))
+    if filled < capacity:
+        head = max(head, filled) % capacity
+    for r in (0.0, 1.0 / 3.0, 1.0):
+        win = pace.ScoreWindow(capacity, DEV)
+        win.values.copy_(to_dev(vals))
+        win.state.copy_(torch.tensor([filled, head]))
+        status = pace.new_status(DEV)
+        dec, kappa = pace.quantile_admit(to_dev(x), r, batch, win, min_obs=2, status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        recent = np.sort(vals[(head - filled + np.arange(filled)) % capacity])
+        k = min(max(int(np.ceil((1.0 - r) * filled - 1e-9)), 1), max(filled, 1))
+        okappa = recent[k - 1] if filled >= 2 else np.inf
+        assert float(kappa.item()) == okappa
+        keep = ~(x > okappa)
+        before = np.cumsum(keep) - keep
+        drawn = before < batch if batch > 0 else np.ones(n_cand, bool)
+        np.testing.assert_array_equal(as_np(dec), np.where(drawn, keep, 2).astype(np.uint8))
+        nd = int(drawn.sum())
+        ring = vals.copy()
+        for i in range(max(0, nd - capacity), nd):
+            ring[(head + i) % capacity] = x[i]
+        np.testing.assert_array_equal(as_np(win.values), ring)
+        assert win.state.tolist() == [min(filled + nd, capacity), (head + nd) % capacity]
