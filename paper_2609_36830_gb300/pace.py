@@ -148,26 +148,38 @@ def _check(st: int, where: str):
         raise PaceError(st, where)
 
 
+# The current device's index without torch.cuda.current_device()'s checks that CUDA is
+# initialised (a CUDA tensor at hand says so): 13 tensors of a scoring call asked it.
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
+
+
 def _arg(t: Optional[torch.Tensor], dtype, n: Optional[int] = None, name: str = "tensor"):
-    """Device pointer of a contiguous tensor of `dtype` with at least `n` elements on
-    the current CUDA device; None passes as NULL.  Anything else raises here, before
-    the library sees a pointer its kernels could not use."""
+    """Device pointer (an int) of a contiguous tensor of `dtype` with at least `n`
+    elements on the current CUDA device; None passes as NULL.  Anything else raises
+    here, before the library sees a pointer its kernels could not use."""
     if t is None:
         return None
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.get_device() == _current_device()
+            and t.is_contiguous() and (dtype is None or t.dtype is dtype)
+            and (n is None or t.numel() >= n)):
+        return t.data_ptr()
+    return _refuse(t, dtype, n, name)
+
+
+def _refuse(t, dtype, n, name):
+    """Raises for the first requirement of _arg that `t` misses."""
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name}: expected a torch.Tensor, got {type(t).__name__}")
     if not t.is_cuda:
         raise ValueError(f"{name}: expected a CUDA tensor")
-    if t.get_device() != torch.cuda.current_device():
+    if t.get_device() != _current_device():
         raise ValueError(f"{name}: on cuda:{t.get_device()}, the current device is "
-                         f"cuda:{torch.cuda.current_device()}")
+                         f"cuda:{_current_device()}")
     if not t.is_contiguous():
         raise ValueError(f"{name}: expected a contiguous tensor")
     if dtype is not None and t.dtype != dtype:
         raise ValueError(f"{name}: expected {dtype}, got {t.dtype}")
-    if n is not None and t.numel() < n:
-        raise ValueError(f"{name}: needs at least {n} elements, has {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{name}: needs at least {n} elements, has {t.numel()}")
 
 
 _U8, _I32T, _I64T = torch.uint8, torch.int32, torch.int64
@@ -182,10 +194,10 @@ _raw_current_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 def _stream(stream=None):
     if stream is not None:
-        return ctypes.c_void_p(stream.cuda_stream)
+        return stream.cuda_stream
     if _raw_current_stream is not None:
-        return ctypes.c_void_p(_raw_current_stream(torch.cuda.current_device()))
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return _raw_current_stream(_current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def workspace(nbytes: int, device) -> torch.Tensor:
