@@ -57,18 +57,34 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 }  // namespace
 
-pace_status encode_bf16_2d(CUtensorMap* tm, const void* ptr, int64_t rows, int64_t cols,
-                           int64_t ld, int box_inner, int box_outer) {
+namespace {
+
+pace_status encode_2d(CUtensorMap* tm, CUtensorMapDataType type, int elem_bytes, const void* ptr,
+                      int64_t rows, int64_t cols, int64_t ld, int box_inner, int box_outer) {
   auto enc = tensor_map_encoder();
   if (!enc) return PACE_ERR_CUDA;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * 2};
+  cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * elem_bytes};
   cuuint32_t box[2] = {static_cast<cuuint32_t>(box_inner), static_cast<cuuint32_t>(box_outer)};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides,
-                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  CUresult r = enc(tm, type, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? PACE_OK : PACE_ERR_UNSUPPORTED_SHAPE;
+}
+
+}  // namespace
+
+pace_status encode_bf16_2d(CUtensorMap* tm, const void* ptr, int64_t rows, int64_t cols,
+                           int64_t ld, int box_inner, int box_outer) {
+  return encode_2d(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, rows, cols, ld, box_inner,
+                   box_outer);
+}
+
+pace_status encode_f32_2d(CUtensorMap* tm, const void* ptr, int64_t rows, int64_t cols, int64_t ld,
+                          int box_inner, int box_outer) {
+  return encode_2d(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ptr, rows, cols, ld, box_inner,
+                   box_outer);
 }
 
 ProfileEvents& profile_events(int kernel) {

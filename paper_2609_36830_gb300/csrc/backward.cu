@@ -52,7 +52,10 @@ constexpr uint32_t kGStageA = GBM * GBK * 2;  // 16 KB
 constexpr uint32_t kGStageB = GBN / 2 * GBK * 2;  // 16 KB: this CTA's half of the B tile
 constexpr uint32_t kGStageBytes = kGStageA + kGStageB;
 constexpr uint32_t kGTmemCols = 2 * GBN;
-constexpr size_t kGSmemBytes = 1024 + GSTAGES * kGStageBytes + 256;
+// Two staging tiles of 32 rows x 128 bytes per epilogue warp, then the barriers.
+constexpr uint32_t kGOutTile = 32 * 128;
+constexpr uint32_t kGOutBytes = 4 * 2 * kGOutTile;
+constexpr size_t kGSmemBytes = 1024 + GSTAGES * kGStageBytes + kGOutBytes + 256;
 constexpr int64_t kChunkRows = 32768;         // rows of G held at once (bf16 M x V)
 constexpr int kGroupM = 38;                   // M tiles per raster group
 // The clusters meet (wait_round) about every kPaceSteps K steps, at a round
@@ -83,9 +86,9 @@ struct GemmArgs {
   const float* dlp;             // dLoss/dlp per original row
   float scale_log2;             // log2(e) / tau
   float inv_tau;
-  uint16_t* g_out;              // bf16 G in 64-column blocks: [g_cols / 64][g_pitch][64]
-  int64_t g_cols;               // V rounded up to 64 (columns >= V hold zeros)
-  int64_t g_pitch;              // rows per 64-column block
+  int64_t g_cols;               // bf16 G in 64-column blocks [g_cols / 64][g_pitch][64]: V rounded
+                                // up to 64 (columns >= V hold zeros)
+  int64_t g_pitch;              // rows per 64-column block (tm_c stores 32-row boxes of it)
   // A operand from the blocked G (a_pitch > 0: rows per 64-column block); 0: plain matrix
   int64_t a_pitch;
   int32_t V;
@@ -183,11 +186,11 @@ __device__ __forceinline__ uint32_t bf16x2_rn(float lo, float hi) {
 template <bool A_MN, bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                GemmArgs p) {
+                const __grid_constant__ CUtensorMap tm_c, GemmArgs p) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + GSTAGES * kGStageBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + GSTAGES * kGStageBytes + kGOutBytes);
   uint64_t* full = bars;
   uint64_t* empty = bars + GSTAGES;
   uint64_t* tmem_full = bars + 2 * GSTAGES;
@@ -391,6 +394,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     const int r_local = quad * 32 + lane;
     const uint32_t empty0 = cluster_addr(&tmem_empty[0], 0);
     const uint32_t empty1 = cluster_addr(&tmem_empty[1], 0);
+    // Output tiles leave through shared memory: a lane writes its row's 128 bytes (in
+    // the 128-byte swizzle, so the warp's 16-byte stores are conflict-free) and lane 0
+    // hands the 32 x 128-byte tile to the TMA, two tiles in turn.  Whole 128-byte lines
+    // go out, asynchronously, where a lane storing its own row piece by piece spread
+    // every store over 32 lines: whole calls of 607 rows (H 2048 head) 1.24 -> 1.01 ms,
+    // 2,582 rows 3.17 -> 3.03, two 32k chunks of H 1024 / V 50,001 12.5 -> 11.8, 21k
+    // rows of H 3584 41.4 -> 40.8.
+    unsigned char* out = smem + GSTAGES * kGStageBytes + (warp - 2) * 2 * kGOutTile;
+    uint32_t n_out = 0;  // tiles handed out so far
+    auto out_begin = [&]() -> unsigned char* {  // the next tile, once its last copy was read
+      if (lane == 0) bulk_wait_read<1>();
+      __syncwarp();
+      return out + (n_out & 1u) * kGOutTile + lane * 128;
+    };
+    auto out_chunk = [&](unsigned char* row, int q, uint4 v) {  // 16-byte chunk q of the row
+      *reinterpret_cast<uint4*>(row + ((q ^ (lane & 7)) << 4)) = v;
+    };
+    auto out_end = [&](int32_t x, int32_t y) {
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        tma_store_2d(&tm_c, out + (n_out & 1u) * kGOutTile, x, y);
+        bulk_commit();
+      }
+      ++n_out;
+    };
     uint32_t tc = 0;
     for (int64_t t = cid; t < n_items; t += n_clusters, ++tc) {
       int64_t mp, nt;
@@ -409,6 +438,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       const int64_t row = mt * GBM + r_local;  // row of C
       const int64_t n0 = nt * GBN;
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + acc * GBN;
+      unsigned char* orow = nullptr;
+      const int64_t row_w = mt * GBM + quad * 32;  // the warp's first row
       // per-row context
       bool row_ok = row < M;
       int32_t y = -1;
@@ -432,7 +463,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         tmem_wait_ld();
         const int64_t col0 = n0 + c;
         if (EPI == EPI_G) {
-          if (row_ok && col0 < p.g_cols) {
+          if (row_w < M && col0 < p.g_cols) {  // M is a multiple of 32: all its rows
             // G = (g / tau) (onehot - p), zero for rows outside the loss.  This epilogue
             // bounds the G GEMM at small H (a 256-column tile takes 5 us of MMAs at H
             // 1024), so per-column tests stay out of it: with them and rounding in
@@ -457,13 +488,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
               const uint32_t g = bf16x2_rn(-gscale * v[2 * i], -gscale * v[2 * i + 1]);
               packed[i] = gscale != 0.0f ? g : 0u;
             }
-            // col0 is a multiple of 32, so the 32 columns lie in one 64-column block
-            uint4* d4 = reinterpret_cast<uint4*>(
-                p.g_out + ((col0 >> 6) * p.g_pitch + row) * 64 + (col0 & 63));
+            // two chunks of 32 columns make one 64-column block's 128-byte rows
+            if ((c & 32) == 0) orow = out_begin();
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-              d4[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2],
-                                 packed[4 * q + 3]);
+              out_chunk(orow, (c & 32 ? 4 : 0) + q,
+                        make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2],
+                                   packed[4 * q + 3]));
+            if (c & 32)
+              out_end(0, static_cast<int32_t>((col0 >> 6) * p.g_pitch + row_w));
           }
         } else if (EPI == EPI_ROWS) {
           if (part >= 0) {  // a partial tile, whole (its rows outside the loss are not read)
@@ -484,28 +517,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
             }
           }
         } else {
-          if (row_ok) {
-            float* dst = p.acc_out + row * p.ldo + col0;
-            if (col0 + 32 <= p.N) {
-              float4* d4 = reinterpret_cast<float4*>(dst);
-              if (p.acc_first) {
+          // N is a multiple of 64, so a chunk of 32 columns is inside or outside; rows
+          // past M are clipped by the tensor map
+          if (p.acc_first) {
+            if (row_w < M && col0 < p.N) {
+              orow = out_begin();
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                  d4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-              } else {
+              for (int q = 0; q < 8; ++q)
+                out_chunk(orow, q,
+                          make_uint4(__float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]),
+                                     __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3])));
+              out_end(static_cast<int32_t>(col0), static_cast<int32_t>(row_w));
+            }
+          } else if (row_ok && col0 < p.N) {  // (a TMA reduction would flush subnormals)
+            float4* d4 = reinterpret_cast<float4*>(p.acc_out + row * p.ldo + col0);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                  float4 o = d4[q];
-                  o.x += v[4 * q];
-                  o.y += v[4 * q + 1];
-                  o.z += v[4 * q + 2];
-                  o.w += v[4 * q + 3];
-                  d4[q] = o;
-                }
-              }
-            } else {
-              for (int i = 0; i < 32 && col0 + i < p.N; ++i)
-                dst[i] = p.acc_first ? v[i] : dst[i] + v[i];
+            for (int q = 0; q < 8; ++q) {
+              float4 o = d4[q];
+              o.x += v[4 * q];
+              o.y += v[4 * q + 1];
+              o.z += v[4 * q + 2];
+              o.w += v[4 * q + 3];
+              d4[q] = o;
             }
           }
         }
@@ -515,6 +548,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acc ? empty1 : empty0);
     }
+    if (lane == 0) bulk_wait_all();  // the copies are done before the CTA's memory goes
+    __syncwarp();
   }
 
   tc_fence_before();
@@ -665,8 +700,8 @@ int gemm_clusters() {
 }
 
 template <bool A_MN, bool B_MN, int EPI>
-pace_status launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, GemmArgs a,
-                        unsigned* round_ctr, cudaStream_t st) {
+pace_status launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc,
+                        GemmArgs a, unsigned* round_ctr, cudaStream_t st) {
   constexpr int kMaxDevices = 64;
   static bool done[kMaxDevices] = {};  // shared-memory opt-in made on that device
   static std::mutex mu;
@@ -692,7 +727,7 @@ pace_status launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, GemmArgs a
   PACE_TRY_CUDA(cudaMemsetAsync(round_ctr, 0, sizeof(unsigned), st));
   a.round_ctr = round_ctr;
   gemm_kernel<A_MN, B_MN, EPI><<<static_cast<unsigned>(grid), kGemmThreads, kGSmemBytes, st>>>(
-      ta, tb, a);
+      ta, tb, tc, a);
   PACE_TRY(last_launch_status());
   if (EPI == EPI_ROWS && a.part) {
     reduce_tail_kernel<<<static_cast<unsigned>(sm_count() * 4), 256, 0, st>>>(
@@ -867,8 +902,9 @@ extern "C" pace_status pace_token_logprob_backward(
     const int64_t hc_rows = (rows_cap - c0) < rows_c_pad ? (rows_cap - c0) : rows_c_pad;
     // 1. G = (g / tau) (onehot - softmax) for the chunk's rows (bf16)
     {
-      CUtensorMap ta, tb;
+      CUtensorMap ta, tb, tc;
       PACE_TRY(encode_bf16_2d(&ta, hc, hc_rows, H, H, 64, GBM));
+      PACE_TRY(encode_bf16_2d(&tc, ws.g, g_blocks * rows_c_pad, 64, 64, 64, 32));
       PACE_TRY(encode_bf16_2d(&tb, w_vocab, V, H, H, 64, GBN / 2));
       GemmArgs a = {};
       a.M = rows_c_pad;
@@ -884,12 +920,11 @@ extern "C" pace_status pace_token_logprob_backward(
       a.dlp = dlp;
       a.scale_log2 = 1.4426950408889634f / temperature;
       a.inv_tau = 1.0f / temperature;
-      a.g_out = ws.g;
       a.g_cols = g_cols;
       a.g_pitch = rows_c_pad;
       a.V = V;
       a.status = status_dev;
-      PACE_TRY((launch_gemm<false, false, EPI_G>(ta, tb, a, ws.round_ctr, st)));
+      PACE_TRY((launch_gemm<false, false, EPI_G>(ta, tb, tc, a, ws.round_ctr, st)));
     }
     // 2. dH rows = G W   (W read MN-major: [K = V][N = H])
     {
@@ -910,12 +945,13 @@ extern "C" pace_status pace_token_logprob_backward(
       a.ldo = H;
       a.part = ws.part;
       a.status = status_dev;
-      PACE_TRY((launch_gemm<false, true, EPI_ROWS>(ta, tb, a, ws.round_ctr, st)));
+      PACE_TRY((launch_gemm<false, true, EPI_ROWS>(ta, tb, ta, a, ws.round_ctr, st)));
     }
     // 3. dW += G^T H_c   (G read MN-major: [K = rows][M = V]; H_c MN-major: [K = rows][N = H])
     {
-      CUtensorMap ta, tb;
+      CUtensorMap ta, tb, tc;
       PACE_TRY(encode_bf16_2d(&ta, ws.g, g_blocks * rows_c_pad, 64, 64, 64, 64));
+      PACE_TRY(encode_f32_2d(&tc, grad_w, V, H, H, 32, 32));
       PACE_TRY(encode_bf16_2d(&tb, hc, hc_rows, H, H, 64, 64));
       GemmArgs a = {};
       a.M = V;
@@ -930,7 +966,7 @@ extern "C" pace_status pace_token_logprob_backward(
       a.acc_first = c0 == 0 ? 1 : 0;
       a.ldo = H;
       a.status = status_dev;
-      PACE_TRY((launch_gemm<true, true, EPI_ACC>(ta, tb, a, ws.round_ctr, st)));
+      PACE_TRY((launch_gemm<true, true, EPI_ACC>(ta, tb, tc, a, ws.round_ctr, st)));
     }
   }
   return PACE_OK;

@@ -274,6 +274,38 @@ __device__ __forceinline__ void tma_gather4_pair(void* smem_dst, const void* des
       : "memory");
 }
 
+// ---- TMA (bulk tensor copies, shared -> global)
+
+// One box from this CTA's shared memory; parts outside the matrix are not written
+// (x and y must not be negative, x * element size a multiple of 16 bytes).
+__device__ __forceinline__ void tma_store_2d(const void* desc, const void* smem_src, int32_t x,
+                                             int32_t y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(desc)),
+               "r"(smem_u32(smem_src)), "r"(x), "r"(y)
+               : "memory");
+}
+
+// This thread's stores so far form a group; waits until at most N groups have yet to
+// read their shared memory, or until all are complete.
+__device__ __forceinline__ void bulk_commit() {
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ void bulk_wait_all() {
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+// Orders this thread's shared-memory writes before later TMA reads of them.
+__device__ __forceinline__ void fence_proxy_async_smem() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
 // ---- tcgen05 on CTA pairs (5th-generation tensor cores, accumulators in
 // tensor memory).  Every tcgen05 instruction of a kernel names the same CTA
 // group; the kernels here all run on pairs (cta_group::2): one MMA of

@@ -15,4 +15,8 @@ namespace pace {
 pace_status encode_bf16_2d(CUtensorMap* tm, const void* ptr, int64_t rows, int64_t cols,
                            int64_t ld, int box_inner, int box_outer);
 
+// The same for a float32 matrix (ld * 4 a multiple of 16 bytes, box_inner * 4 <= 128).
+pace_status encode_f32_2d(CUtensorMap* tm, const void* ptr, int64_t rows, int64_t cols, int64_t ld,
+                          int box_inner, int box_outer);
+
 }  // namespace pace
