@@ -5,7 +5,7 @@
 // Order: score descending, then unit id ascending.  The k first units in that
 // order are rejected; outputs list trajectory ids ascending.
 //
-//   small pools (U <= 512): one block ranks every unit against every other
+//   small pools (U <= 288): one block ranks every unit against every other
 //     unit in shared memory and compacts the ids (one launch).
 //   mid-size pools (U <= 131,072): one cluster of up to 8 CTAs holds every key
 //     in shared memory (16,384 per CTA), finds the pivot by a radix select that
@@ -36,8 +36,14 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kSmallMax = 512;
-constexpr int kSmallThreads = 512;
+// Ranking takes U^2 comparisons on one SM, the radix select a nearly constant time: per
+// call (graph of 20) 128 units 3.7 against 7.2 us, 256 units 6.5 / 8.2, 320 units 9.1 /
+// 8.3, 512 units 15.8 / 8.7.
+constexpr int kSmallMax = 288;
+constexpr int kSmallThreads = 288;
+// Pools up to this size take one CTA whatever their outputs and stay within the shared
+// memory that needs no attribute, so their first call may be inside a stream capture.
+constexpr int kOneCtaMax = 512;
 constexpr int kHistBins = 2048;
 constexpr int kTile = 256;  // units per compaction block of the radix path
 constexpr int kTileThreads = 256;
@@ -53,6 +59,17 @@ __device__ __forceinline__ uint64_t order_key(double x) {
   if (b == 0x8000000000000000ull) b = 0;
   return (b & 0x8000000000000000ull) ? ~b : (b | 0x8000000000000000ull);
 }
+
+// Two 32-bit warp reductions: the high halves, then the low halves of the lanes that
+// hold the extreme high half.
+__device__ __forceinline__ uint64_t warp_min_u64(uint64_t x) {
+  const unsigned hi = static_cast<unsigned>(x >> 32), lo = static_cast<unsigned>(x);
+  const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
+  return static_cast<uint64_t>(mh) << 32 | ml;
+}
+
+__device__ __forceinline__ uint64_t warp_max_u64(uint64_t x) { return ~warp_min_u64(~x); }
 
 struct SelectState {
   unsigned long long prefix;
@@ -133,7 +150,7 @@ __device__ __forceinline__ void write_unit(int64_t u, bool rejected, int64_t rej
   }
 }
 
-// U <= 512: rank of u = number of units ordered before it.  The ranks compare
+// U <= kSmallMax: rank of u = number of units ordered before it.  The ranks compare
 // order keys, not doubles: the same order (-0.0 equals +0.0), on the integer
 // pipe instead of GB300's narrow fp64 pipe.
 __global__ void __launch_bounds__(kSmallThreads)
@@ -164,7 +181,7 @@ __global__ void __launch_bounds__(kSmallThreads)
     write_unit(u, rejected, rej_before, u - rej_before, G, 0, accepted_ids, rejected_ids, flags);
 }
 
-// 512 < U <= 131,072: one launch of one thread-block cluster of C CTAs (1, 2,
+// kSmallMax < U <= 131,072: one launch of one thread-block cluster of C CTAs (1, 2,
 // 4 or 8; 1024 threads each).  CTA r owns the contiguous units
 // [r * B, r * B + B) with B = ceil(U / C) <= 16,384; its thread t owns the
 // contiguous units t * per .. t * per + per - 1 of that range (per, a power of
@@ -176,9 +193,10 @@ __global__ void __launch_bounds__(kSmallThreads)
 // candidates over the whole cluster, stops when they are equal, and otherwise
 // histograms the (up to 11) bits just below the highest bit where they differ;
 // each CTA counts its own keys and sums the C histograms through distributed
-// shared memory.  Candidates in one round share every bit above that one, so a
-// round fixes at least one bit and there are at most 64 rounds (two to four for
-// spread-out scores).  Every CTA computes the same values from the same shared
+// shared memory.  Once the pivot's digit holds at most kSelList candidates (after one
+// round, on spread-out scores), no further round is taken: every CTA lists its own,
+// and one warp of each ranks them all against each other (finish_list).  Candidates in one round share every bit above that one, so a
+// round fixes at least one bit and there are at most 64 rounds.  Every CTA computes the same values from the same shared
 // data, so all of them take the same branches and pass the same sequence of
 // cluster barriers.
 //
@@ -219,28 +237,16 @@ __host__ __device__ inline size_t sel_smem_bytes(int b) {
 __device__ __forceinline__ void cta_min_max_to_slot(uint64_t lo, uint64_t hi, uint64_t* s_wlo,
                                                     uint64_t* s_whi, uint64_t* s_mm) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t a = __shfl_xor_sync(0xffffffffu, lo, o);
-    const uint64_t b = __shfl_xor_sync(0xffffffffu, hi, o);
-    lo = a < lo ? a : lo;
-    hi = b > hi ? b : hi;
-  }
+  lo = warp_min_u64(lo);
+  hi = warp_max_u64(hi);
   if (lane == 0) {
     s_wlo[wid] = lo;
     s_whi[wid] = hi;
   }
   __syncthreads();
   if (wid == 0) {  // one warp folds the 32 warp results into this CTA's slot
-    lo = s_wlo[lane];
-    hi = s_whi[lane];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t a = __shfl_xor_sync(0xffffffffu, lo, o);
-      const uint64_t b = __shfl_xor_sync(0xffffffffu, hi, o);
-      lo = a < lo ? a : lo;
-      hi = b > hi ? b : hi;
-    }
+    lo = warp_min_u64(s_wlo[lane]);
+    hi = warp_max_u64(s_whi[lane]);
     if (lane == 0) {
       s_mm[0] = lo;
       s_mm[1] = hi;
@@ -269,13 +275,8 @@ __device__ __forceinline__ void cluster_fold_slots(cg::cluster_group& cluster, u
       lo = peer[0];
       hi = peer[1];
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t a = __shfl_xor_sync(0xffffffffu, lo, o);
-      const uint64_t b = __shfl_xor_sync(0xffffffffu, hi, o);
-      lo = a < lo ? a : lo;
-      hi = b > hi ? b : hi;
-    }
+    lo = warp_min_u64(lo);
+    hi = warp_max_u64(hi);
     if (lane == 0) {
       s_g[0] = lo;
       s_g[1] = hi;
@@ -284,6 +285,49 @@ __device__ __forceinline__ void cluster_fold_slots(cg::cluster_group& cluster, u
   __syncthreads();
   lo = s_g[0];
   hi = s_g[1];
+}
+
+// Candidates that one warp ranks.  The list saves a round and the extremes before it:
+// per call (graph replay) 2,048 units 14.5 -> 12.3 us, 16,384 units on 4 CTAs 24.6 ->
+// 20.5, 131,072 on 8 CTAs 61.5 -> 56.7.
+constexpr int kSelList = 64;
+
+// The pivot and the number of keys equal to it that are rejected, from the cluster's
+// lists of candidates (list / n_list: this CTA's; at most kSelList in all, k-th
+// largest wanted), by warp 0; the caller's barriers publish the lists before and
+// out[] after.
+template <bool kMulti>
+__device__ __forceinline__ void finish_list(cg::cluster_group& cluster, uint64_t* list, int* n_list,
+                                            uint64_t* all, long long k, uint64_t* out) {
+  const int lane = threadIdx.x & 31;
+  int total = 0;
+  if (kMulti) {
+    const int nc = static_cast<int>(cluster.num_blocks());
+    const int mine = lane < nc ? *cluster.map_shared_rank(n_list, static_cast<unsigned>(lane)) : 0;
+    for (int r = 0; r < nc; ++r) {
+      const int n = __shfl_sync(0xffffffffu, mine, r);
+      const uint64_t* peer = cluster.map_shared_rank(list, static_cast<unsigned>(r));
+      for (int i = lane; i < n; i += 32) all[total + i] = peer[i];
+      total += n;
+    }
+    __syncwarp();
+  } else {
+    all = list;
+    total = *n_list;
+  }
+  for (int i = lane; i < total; i += 32) {
+    const uint64_t x = all[i];
+    int above = 0, equal = 0;
+    for (int w = 0; w < total; ++w) {
+      const uint64_t y = all[w];
+      above += y > x;
+      equal += y == x;
+    }
+    if (above < k && k <= above + equal) {  // the pivot (the same from each of its copies)
+      out[0] = x;
+      out[1] = static_cast<uint64_t>(k - above);
+    }
+  }
 }
 
 // kMulti = false: a cluster of one CTA, with block barriers and plain shared
@@ -299,8 +343,10 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   __shared__ uint64_t s_mm[2], s_g[2];
   __shared__ long long s_cnt[2];  // this CTA's keys equal to / above the pivot (peers read)
   __shared__ long long s_off[2];  // ties and rejections in lower-ranked CTAs
-  __shared__ int s_digit;
+  __shared__ int s_digit, s_here;
   __shared__ long long s_left;
+  __shared__ uint64_t s_list[kSelList], s_all[kSelList], s_out[2];
+  __shared__ int s_n_list;
   cg::cluster_group cluster = cg::this_cluster();
   const int nc = static_cast<int>(cluster.num_blocks());
   const int rank = static_cast<int>(cluster.block_rank());
@@ -357,7 +403,10 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     mask = d == 63 ? 0ull : (~0ull << (d + 1));
     prefix = lo & mask;
     for (int b = t; b < nbins; b += kSelThreads) hist[b] = 0u;
-    if (t == 0) s_digit = -1;
+    if (t == 0) {
+      s_digit = -1;
+      s_n_list = 0;
+    }
     __syncthreads();
     for (int i = 0; i < n_mine; ++i) {
       const uint64_t key = keys[i * kSelRow + t];
@@ -398,11 +447,13 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     if (top >= 0 && run < k_rem && k_rem <= run + h0) {
       s_digit = top;
       s_left = k_rem - run;
+      s_here = static_cast<int>(h0);
     }
     run += h0;
     if (top >= 1 && run < k_rem && k_rem <= run + h1) {
       s_digit = top - 1;
       s_left = k_rem - run;
+      s_here = static_cast<int>(h1);
     }
     __syncthreads();  // s_digit and s_left are set
     if (s_digit < 0) {  // the same in every CTA: the histograms summed are the same
@@ -412,6 +463,19 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     prefix |= static_cast<uint64_t>(s_digit) << shift;
     mask |= static_cast<uint64_t>(nbins - 1) << shift;
     k_rem = s_left;
+    if (s_here <= kSelList) {  // the same in every CTA
+      for (int i = 0; i < n_mine; ++i) {
+        const uint64_t key = keys[i * kSelRow + t];
+        if ((key & mask) == prefix) s_list[atomicAdd(&s_n_list, 1)] = key;
+      }
+      if (kMulti) cluster.sync();  // every CTA's list is complete
+      else __syncthreads();
+      if (t < 32) finish_list<kMulti>(cluster, s_list, &s_n_list, s_all, k_rem, s_out);
+      __syncthreads();
+      lo = s_out[0];
+      k_rem = static_cast<long long>(s_out[1]);
+      break;
+    }
     lo = ~0ull;
     hi = 0ull;
     for (int i = 0; i < n_mine; ++i) {
@@ -931,6 +995,10 @@ extern "C" pace_status pace_select_k(const double* unit_score, int64_t n_units, 
                                                      status_dev);
     return last_launch_status();
   }
+  if (n_units <= kOneCtaMax)
+    return launch_select_cluster(unit_score, static_cast<int>(n_units), G,
+                                 static_cast<long long>(k), 1, accepted_ids, rejected_ids,
+                                 traj_accepted, status_dev, st);
   if (n_units <= kSelMaxUnits) {
     int limit = 1;
     PACE_TRY(sel_cluster_limit(&limit));
@@ -1211,15 +1279,6 @@ constexpr int kMaxWindowSlots = 4096;
 constexpr int kAdmitThreads = 512;
 constexpr int kAdmitSlots = kMaxWindowSlots / kAdmitThreads;  // window values a thread
 constexpr int kAdmitChunk = kAdmitThreads * 32;  // candidates per scan: one 32-bit word a thread
-
-__device__ __forceinline__ uint64_t warp_min_u64(uint64_t x) {
-  const unsigned hi = static_cast<unsigned>(x >> 32), lo = static_cast<unsigned>(x);
-  const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
-  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
-  return static_cast<uint64_t>(mh) << 32 | ml;
-}
-
-__device__ __forceinline__ uint64_t warp_max_u64(uint64_t x) { return ~warp_min_u64(~x); }
 
 __device__ __forceinline__ bool is_nan_bits(double x) {
   return (static_cast<uint64_t>(__double_as_longlong(x)) & 0x7fffffffffffffffull) >

@@ -231,3 +231,36 @@ def test_select_outputs_at_unaligned_addresses(U, G):
         np.testing.assert_array_equal(as_np(acc)[off_ids:off_ids + (U - k) * G], oacc)
         np.testing.assert_array_equal(as_np(rej)[off_ids:off_ids + k * G], orej)
         np.testing.assert_array_equal(as_np(flags)[off_flags:off_flags + n], oflag)
+
+
+@pytest.mark.parametrize("U", [600, 3000, 20000, 131072])
+@pytest.mark.parametrize("m", [1, 2, 31, 63, 64, 65, 200])
+@pytest.mark.parametrize("dist", ["equal", "ulps", "near"])
+def test_candidate_list_sizes(U, m, dist):
+    """m scores share the pivot's digit (m around the 64 candidates that one warp ranks
+    and the 32 lanes it has), equal, an ulp apart or spread over the digit, spread over
+    the pool's ids so that every CTA of the cluster holds some; ids exact."""
+    rng = np.random.default_rng(U + m)
+    s = np.concatenate([rng.random(U // 2) * 10.0, 30.0 + rng.random(U - U // 2) * 10.0])
+    at = rng.choice(U, size=m, replace=False)
+    if dist == "equal":
+        s[at] = 20.0
+    elif dist == "ulps":
+        s[at] = 20.0 + rng.integers(0, 2 * m, size=m) * np.spacing(20.0)
+    else:
+        s[at] = 20.0 + rng.random(m) * 1e-4
+    s = s[rng.permutation(U)]
+    above = int((s > 25.0).sum())
+    for k in sorted({above + 1, above + (m + 1) // 2, above + m}):
+        _check_k(s, 8, k)
+
+
+@pytest.mark.parametrize("U", [31, 32, 33, 287, 288, 289, 511, 512, 513])
+@pytest.mark.parametrize("G", [1, 3, 8, 100])
+def test_small_pools_around_the_rank_kernel(U, G):
+    """Pools around the largest that are ranked all against all and the largest that take
+    one CTA whatever their outputs; ids exact."""
+    rng = np.random.default_rng(U * G)
+    for s in (rng.random(U) * 20.0, rng.integers(0, 5, size=U) / 2.0):
+        for k in (1, U // 3, U - 1):
+            _check_k(s, G, k)
