@@ -578,9 +578,9 @@ PACE_API int64_t pace_score_fused_min_traj_default(void);
  * the caller.  Returns PACE_ERR_INVALID_ARG for an unknown kernel. */
 PACE_API pace_status pace_set_profile_events(int32_t kernel, void* begin, void* end);
 
-/* Not part of the method: checks the integer construction of the doubles the
- * scoring writes.  For every i, with T[i] >= 1:
- *   q_int[i]  = S[i] / T[i] as the scoring kernels build it on the integer pipe,
+/* Not part of the method: checks the integer construction of the quotients that
+ * pace_stale_k writes.  For every i, with T[i] >= 1:
+ *   q_int[i]  = S[i] / T[i] as its kernel builds it on the integer pipe,
  *   q_fp64[i] = the same quotient from the fp64 pipe, __ll2double_rn(S[i]) then
  *               a correctly rounded division (the rounding the oracle's
  *               (double)S / (double)T performs),

@@ -96,11 +96,10 @@ __device__ __forceinline__ void l2_prefetch_bulk(const void* p, uint32_t bytes) 
 
 // ---- exact integer quotients without the fp64 pipe
 //
-// GB300's fp64 pipe is narrow, and the finalisation is bound by it (one int64
-// to double conversion and one correctly rounded division per trajectory).  The
-// functions below build the same doubles from integer arithmetic: the result
-// of __ddiv_rn(__ll2double_rn(S), T) for 64-bit S and 32-bit T > 0, and of
-// __ll2double_rn(x), bit for bit.
+// GB300's fp64 pipe is narrow.  The functions below build the same doubles from
+// integer arithmetic: the result of __ddiv_rn(__ll2double_rn(S), T) for 64-bit S and
+// 32-bit T > 0, and of __ll2double_rn(x), bit for bit.  pace_stale_k's quotients are
+// built this way (as fast as in fp64 there); the scores' finalisation divides in fp64.
 
 // (double)x rounded to nearest even, from its bits (every int64 is in range).
 __device__ __forceinline__ double i64_to_double_rn(long long x) {
@@ -616,6 +615,7 @@ struct FinalizeArgs {
   int32_t mode;
   int32_t gamma;
   int32_t group_size;
+  double inv_group;             // 1 / G for G a power of two (exact), else 0
   int32_t lanes;                // threads per trajectory for the direct count
   double f_missing;
   double* kgen;
@@ -780,9 +780,10 @@ __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, 
       report(p.status, PACE_ERR_VERSION_ORDER);
     // Lemma 1: K_gen = (1/T) sum (c - v_t) = (c T - sum v_t) / T, exact integers
     const long long gen_sum = static_cast<long long>(c) * static_cast<long long>(t_count) - tag_sum;
-    // the correctly rounded K_gen and K_wait, built on the integer pipe
-    const double kgen = t_count > 0u ? i64_div_u32_rn(gen_sum, t_count) : 0.0;
-    const double kwait = i64_to_double_rn(static_cast<long long>(p.j) - c);
+    // the correctly rounded K_gen and K_wait
+    const double kgen = t_count > 0u ? __ddiv_rn(__ll2double_rn(gen_sum), __uint2double_rn(t_count))
+                                     : 0.0;
+    const double kwait = __ll2double_rn(static_cast<long long>(p.j) - c);
     double f;
     if (!p.window_ready) {
       f = 1.0;
@@ -815,14 +816,25 @@ __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, 
     m.sscore[slot] = sc;
   }
   __syncthreads();
+  // The groups' means, a thread per group, the groups in consecutive threads: a chain of
+  // G additions holds the narrow fp64 pipe for as many warps as have a group, which with
+  // the first thread of each group working was every warp (half of the kernel's time).
+  // With the pipe free of them, K_gen's quotient is faster in fp64 than from integer
+  // divisions: whole calls (graph replay) 1k pool 24.6 -> 23.7 us, 16k 62.8 -> 61.9, 20k in
+  // groups of 12 73.3 -> 72.6, 128k 319.9 -> 317.9, 1M 2229 -> 2214.
   const int G = p.group_size;
-  if (p.unit_score && lead && i < i_end && (slot % G) == 0) {
-    double acc = 0.0;
-    for (int g = 0; g < G; ++g) acc = __dadd_rn(acc, m.sscore[slot + g]);
-    // for G = 2^m, acc * 2^-m is the same correctly rounded value as acc / G
-    // (2^-m is exact), one multiplication instead of a division
-    p.unit_score[i / G] = (G & (G - 1)) == 0 ? __dmul_rn(acc, 1.0 / static_cast<double>(G))
-                                             : __ddiv_rn(acc, static_cast<double>(G));
+  if (p.unit_score) {
+    const int64_t n = i_end - i0 < tpb ? i_end - i0 : tpb;  // whole groups
+    const int units = static_cast<int>(n) / G;
+    for (int u = tid; u < units; u += static_cast<int>(blockDim.x)) {
+      const double* s = m.sscore + u * G;
+      double acc = 0.0;
+      for (int g = 0; g < G; ++g) acc = __dadd_rn(acc, s[g]);
+      // for G = 2^m, acc * 2^-m is the same correctly rounded value as acc / G
+      // (2^-m is exact), one multiplication instead of a division
+      p.unit_score[i0 / G + u] = p.inv_group != 0.0 ? __dmul_rn(acc, p.inv_group)
+                                                    : __ddiv_rn(acc, static_cast<double>(G));
+    }
   }
 }
 
@@ -1263,6 +1275,7 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
   a.mode = params->mode;
   a.gamma = params->gamma;
   a.group_size = G;
+  a.inv_group = (G & (G - 1)) == 0 ? 1.0 / static_cast<double>(G) : 0.0;
   a.f_missing = params->f_missing;
   a.kgen = kgen;
   a.kwait = kwait;
