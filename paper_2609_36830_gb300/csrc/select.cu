@@ -71,6 +71,11 @@ __device__ __forceinline__ uint64_t warp_min_u64(uint64_t x) {
 
 __device__ __forceinline__ uint64_t warp_max_u64(uint64_t x) { return ~warp_min_u64(~x); }
 
+__device__ __forceinline__ bool is_nan_bits(double x) {
+  return (static_cast<uint64_t>(__double_as_longlong(x)) & 0x7fffffffffffffffull) >
+         0x7ff0000000000000ull;
+}
+
 struct SelectState {
   unsigned long long prefix;
   unsigned long long mask;
@@ -1218,27 +1223,45 @@ namespace {
 
 constexpr int kMaxHistBins = 4096;
 
+// Bound by the narrow fp64 pipe: the bin is floor(((x - lo) / width) * n_bins) with each
+// operation rounded, about 17 fp64 instructions a value with the division and the
+// comparisons.  The comparisons are made on integer keys, and the division only where
+// it can matter: t = (x - lo) * (n_bins / width) differs from the exact sequence's
+// result by at most 4 roundings of a number below 4096, less than 2^-38, so where t is
+// further than 2^-36 from an integer its floor is the bin.  Per call (graph of 20), 64
+// bins: 131,072 values 10.4 -> 8.4 us, 1M values 37.5 -> 20.6.
 __global__ void staleness_hist_kernel(const double* __restrict__ values,
                                       const uint8_t* __restrict__ flags, int64_t n, double lo,
-                                      double hi, int n_bins, unsigned* __restrict__ hist,
-                                      int32_t* status) {
+                                      double hi, double per_bin, int n_bins,
+                                      unsigned* __restrict__ hist, int32_t* status) {
   extern __shared__ unsigned h[];  // [2 * n_bins]
   for (int b = threadIdx.x; b < 2 * n_bins; b += blockDim.x) h[b] = 0;
   __syncthreads();
   const double width = __dsub_rn(hi, lo);
+  const double bins = static_cast<double>(n_bins);
+  const uint64_t lo_key = order_key(lo), hi_key = order_key(hi);
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const double x = values[i];
-    if (isnan(x)) {
+    if (is_nan_bits(x)) {
       report(status, PACE_ERR_NAN_INPUT);
       continue;
     }
+    const uint64_t key = order_key(x);
     int b;
-    if (x < lo) b = 0;
-    else if (x >= hi) b = n_bins - 1;
+    if (key < lo_key) b = 0;
+    else if (key >= hi_key) b = n_bins - 1;
     else {
-      const double f = floor(__dmul_rn(__ddiv_rn(__dsub_rn(x, lo), width), (double)n_bins));
-      b = f > (double)(n_bins - 1) ? n_bins - 1 : static_cast<int>(f);
+      const double d = __dsub_rn(x, lo);
+      const double t = __dmul_rn(d, per_bin);
+      b = __double2int_rd(t);
+      // t - b in [0, 1), compared as bits with 2^-36 and 1 - 2^-36
+      const int64_t frac = __double_as_longlong(__dsub_rn(t, static_cast<double>(b)));
+      if (per_bin == 0.0 || frac < 0x3DB0000000000000ll || frac > 0x3FEFFFFFFFFE0000ll) {
+        const double f = floor(__dmul_rn(__ddiv_rn(d, width), bins));
+        b = f > bins - 1.0 ? n_bins - 1 : static_cast<int>(f);
+      }
+      if (b > n_bins - 1) b = n_bins - 1;
     }
     atomicAdd(&h[(flags && flags[i] ? n_bins : 0) + b], 1u);
   }
@@ -1260,8 +1283,12 @@ extern "C" pace_status pace_staleness_histogram(const double* values, const uint
   cudaStream_t st = as_stream(stream);
   PACE_TRY_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * 2 * n_bins, st));
   if (n == 0) return PACE_OK;
-  staleness_hist_kernel<<<grid_for(n, 256, 4), 256, sizeof(unsigned) * 2 * n_bins, st>>>(
-      values, flags, n, lo, hi, n_bins, hist, status_dev);
+  // bins per unit of x for the quick path (0: off, where it is not a normal number)
+  double per_bin = static_cast<double>(n_bins) / (hi - lo);
+  if (!isnormal(per_bin)) per_bin = 0.0;
+  // two values a thread at least: fewer blocks' bins to clear and add up
+  staleness_hist_kernel<<<grid_for(n, 512, 2), 256, sizeof(unsigned) * 2 * n_bins, st>>>(
+      values, flags, n, lo, hi, per_bin, n_bins, hist, status_dev);
   return last_launch_status();
 }
 
@@ -1279,11 +1306,6 @@ constexpr int kMaxWindowSlots = 4096;
 constexpr int kAdmitThreads = 512;
 constexpr int kAdmitSlots = kMaxWindowSlots / kAdmitThreads;  // window values a thread
 constexpr int kAdmitChunk = kAdmitThreads * 32;  // candidates per scan: one 32-bit word a thread
-
-__device__ __forceinline__ bool is_nan_bits(double x) {
-  return (static_cast<uint64_t>(__double_as_longlong(x)) & 0x7fffffffffffffffull) >
-         0x7ff0000000000000ull;
-}
 
 // The k-th smallest (1 <= k <= n) of the block's n order keys, key i held by thread
 // i % kAdmitThreads (slot i / kAdmitThreads): histograms of the 11 bits below the

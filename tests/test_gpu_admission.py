@@ -150,3 +150,31 @@ def test_quantile_admit_sizes(capacity, filled, n_cand, batch):
             ring[(head + i) % capacity] = x[i]
         np.testing.assert_array_equal(as_np(win.values), ring)
         assert win.state.tolist() == [min(filled + nd, capacity), (head + nd) % capacity]
+
+
+@pytest.mark.parametrize("lo,hi,n_bins", [(0.0, 32.0, 1000), (0.1, 0.7, 77), (-3.0, 1e-3, 4096),
+                                          (0.0, 5e-324, 3), (-1e308, 1.5e308, 10),
+                                          (1e-310, 1e-308, 50), (0.3, np.nextafter(0.3, 1), 2)])
+def test_histogram_at_bin_edges(lo, hi, n_bins):
+    """Values at every bin edge and a few ulps around it, on ranges up to the smallest and
+    largest that doubles hold, where a shorter computation of the bin could go astray;
+    counts exact (the oracle's division, product and floor)."""
+    rng = np.random.default_rng(n_bins)
+    with np.errstate(over="ignore", invalid="ignore"):
+        e = lo + (hi - lo) * (np.arange(n_bins + 1) / n_bins)
+        x = [rng.uniform(0, 1, 5000) * (hi / 2 - lo / 2) * 2 + lo]
+    e = e[np.isfinite(e)]
+    x += [e, np.array([lo, hi, np.inf, -np.inf])]
+    for step in (1, 2, 3):
+        y = e.copy()
+        z = e.copy()
+        for _ in range(step):
+            y, z = np.nextafter(y, np.inf), np.nextafter(z, -np.inf)
+        x += [y, z]
+    x = np.concatenate(x)
+    x = x[~np.isnan(x)]
+    flags = (rng.random(x.size) < 0.5).astype(np.uint8)
+    hist = pace.staleness_histogram(to_dev(x), to_dev(flags), lo, hi, n_bins)
+    st, oh = oracle.histogram(x, flags, lo, hi, n_bins)
+    assert st == 0
+    np.testing.assert_array_equal(as_np(hist).astype(np.uint32), oh)
