@@ -30,15 +30,17 @@ namespace {
 
 constexpr int kReduceThreads = 256;  // 8 warps
 constexpr int kTileTokens = 128;     // one int4 per lane
-// Tiles per warp batch (128 tokens each) and resident blocks per SM, by pool
-// size.  Large pools: 8 tiles (1024 tokens, 4 KB in flight per register set),
-// 126 registers, 2 blocks per SM.  Pools of up to kSmallPoolTokens tags: 4
-// tiles, 79 registers, 3 blocks per SM; more warps with half the work each
-// shorten the ramp and the tail where those dominate (16k sweep pool, 55 M
-// tags: 62 -> 52 us), and cost ~0.5 % on long streams (128k and 1M pools).
-constexpr int kTilesLarge = 8, kBlocksLarge = 2;
-constexpr int kTilesSmall = 4, kBlocksSmall = 3;
-constexpr int64_t kSmallPoolTokens = int64_t(1) << 27;
+// Tiles of a warp's batch (128 tokens each), two register sets of them in flight in
+// turn, and resident blocks per SM: 24 warps with 80 registers keep 48-96 KB of loads
+// in flight per SM, which is what the memory needs.  No L2 prefetch runs beside them:
+// one of four batches ahead held every pool back (the prefetched lines compete with the
+// loads).  Whole scoring + selection calls, graph replay: 20k pool 72.0 -> 66.7 us, 128k
+// 316 -> 282, 1M 2203 -> 2129; pace_stale_k on 128k 293 -> 257.  Measured without the
+// prefetch (tiles x blocks per SM, 128k / 1M pool): 8 x 2 337 us / 2.51 ms, 6 x 3 288 /
+// 2.13, 4 x 4 296 / 2.16 (spills), 3 x 4 289 / 2.13, 2 x 6 367 / 3.0, one register set
+// 4 x 6 595 / 4.6.  A plain read of the same bytes takes 239 us / 1.95 ms.
+constexpr int kTiles = 4, kBlocksPerSm = 3;
+constexpr int64_t kBatchTokens = kTileTokens * kTiles;
 // Short streams get fewer warps rather than fewer batches a warp: below this
 // many batches a warp, trajectories spread over several warps' ranges and their
 // totals need more head slots.  On the 1k sweep pool (3.6 M tags, ~3,500 a
@@ -85,7 +87,8 @@ __device__ __forceinline__ int4 ld_stream_v4(const int32_t* p) {
   return v;
 }
 
-constexpr int64_t kPrefetchAhead = 4;
+// Batches of a range asked into L2 before the search for its first trajectory.
+constexpr int kFirstBatches = 2;
 
 // Bulk prefetch of a 16-byte-aligned range into L2 (no data returned).
 __device__ __forceinline__ void l2_prefetch_bulk(const void* p, uint32_t bytes) {
@@ -237,7 +240,6 @@ struct TagTotals {
 // Geometry of one tag-reduction launch: warp w streams batches
 // [n_batches w / n_warps, n_batches (w + 1) / n_warps).
 struct StreamGeom {
-  int64_t batch_tokens;
   int64_t n_batches;
   int64_t n_warps;
 };
@@ -253,23 +255,28 @@ __host__ __device__ __forceinline__ int64_t warp_of_batch(const StreamGeom& g, i
 __device__ __forceinline__ void emit(LaneAcc& a, int64_t traj, bool continues, bool head,
                                      int64_t warp, const TagTotals& tt) {
   const unsigned full = 0xffffffffu;
-  long long s = a.sum;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
+  // the lanes' 64-bit sums in three digits of 26, 26 and 12 bits, each a 32-bit warp
+  // reduction that cannot overflow (the top one wraps like the 64-bit sum would)
+  const unsigned long long u = static_cast<unsigned long long>(a.sum);
+  const unsigned d0 = __reduce_add_sync(full, static_cast<unsigned>(u) & 0x3ffffffu);
+  const unsigned d1 = __reduce_add_sync(full, static_cast<unsigned>(u >> 26) & 0x3ffffffu);
+  const unsigned d2 = __reduce_add_sync(full, static_cast<unsigned>(u >> 52));
+  const unsigned long long s = d0 + (static_cast<unsigned long long>(d1) << 26) +
+                               (static_cast<unsigned long long>(d2) << 52);
   const unsigned c = __reduce_add_sync(full, a.cnt);
   const unsigned m = __reduce_max_sync(full, a.maxp1);
   if ((threadIdx.x & 31) == 0) {
     if (head) {
       HeadSlot h;
       h.traj = traj;
-      h.sum = static_cast<unsigned long long>(s);
+      h.sum = s;
       h.cnt = c;
       h.maxp1 = m;
       h.pad = 0;
       tt.head[warp] = h;
     } else {
       ulonglong2 v;
-      v.x = static_cast<unsigned long long>(s) | (continues ? kContinues : 0ull);
+      v.x = s | (continues ? kContinues : 0ull);
       v.y = static_cast<unsigned long long>(c) | (static_cast<unsigned long long>(m) << 32);
       tt.slot[traj] = v;
     }
@@ -298,8 +305,8 @@ __device__ __forceinline__ void traj_totals(const TagTotals& tt, const StreamGeo
   maxp1 = static_cast<unsigned>(v.y >> 32);
   if (v.x & kContinues) {
     const int64_t last = (o1 < n_tokens ? o1 : n_tokens) - 1;
-    const int64_t w0 = warp_of_batch(g, o0 / g.batch_tokens);
-    const int64_t w1 = warp_of_batch(g, last / g.batch_tokens);
+    const int64_t w0 = warp_of_batch(g, o0 / kBatchTokens);
+    const int64_t w1 = warp_of_batch(g, last / kBatchTokens);
     for (int64_t w = w0 + 1; w <= w1; w += 2) {
       longlong2 h0[2], h1[2];
 #pragma unroll
@@ -335,18 +342,17 @@ __device__ __forceinline__ bool small_policy(int bits_or) {
 // Sum, count and max of a batch that lies inside one trajectory and holds only
 // policy tags below 2^26.  Returns false (and leaves acc untouched) when the
 // batch needs the per-group path.
-template <int kTilesPerBatch>
-__device__ __forceinline__ bool acc_batch_fast(LaneAcc& a, const int4 (&v)[kTilesPerBatch]) {
+__device__ __forceinline__ bool acc_batch_fast(LaneAcc& a, const int4 (&v)[kTiles]) {
   int o = 0, mx = 0, s = 0;
 #pragma unroll
-  for (int u = 0; u < kTilesPerBatch; ++u) {
+  for (int u = 0; u < kTiles; ++u) {
     o |= (v[u].x | v[u].y) | (v[u].z | v[u].w);
     mx = __vimax3_s32(__vimax3_s32(mx, v[u].x, v[u].y), v[u].z, v[u].w);
     s += (v[u].x + v[u].y) + (v[u].z + v[u].w);
   }
   if (!small_policy(o)) return false;
   a.sum += s;
-  a.cnt += 4 * kTilesPerBatch;
+  a.cnt += 4 * kTiles;
   const unsigned mp1 = static_cast<unsigned>(mx) + 1u;
   a.maxp1 = mp1 > a.maxp1 ? mp1 : a.maxp1;
   return true;
@@ -367,7 +373,7 @@ __device__ __forceinline__ void acc_group(LaneAcc& a, const int4& q) {
   }
 }
 
-// Each warp owns a contiguous range of batches (kTilesPerBatch x 128 tokens) of
+// Each warp owns a contiguous range of batches (kTiles x 128 tokens) of
 // the flattened tag stream and walks the CSR offsets forward through it, so trajectories of
 // any length mix are balanced across warps.  The walk never leaves
 // [0, n_traj) and loads only tags[0, n_tokens), whatever the offsets hold;
@@ -456,12 +462,10 @@ __device__ void window_prep_block(int b, const WindowPrep& w) {
 // One warp's share of the stream (every warp of the first n_stream_blocks
 // blocks calls it; it returns early when the range is empty or the offsets end
 // before the tokens do).
-template <int kTilesPerBatch>
 __device__ __forceinline__ void stream_warp_range(const int32_t* __restrict__ tags,
                                                   const int64_t* __restrict__ offsets,
                                                   int64_t n_traj, int64_t n_tokens,
                                                   const TagTotals& tt, int n_stream_blocks) {
-  constexpr int64_t kBatchTokens = kTileTokens * kTilesPerBatch;
   const int lane = threadIdx.x & 31;
   const int64_t warp = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t n_warps = (static_cast<int64_t>(n_stream_blocks) * blockDim.x) >> 5;
@@ -476,9 +480,8 @@ __device__ __forceinline__ void stream_warp_range(const int32_t* __restrict__ ta
   const int64_t t_end = b_end * kBatchTokens < n_tokens ? b_end * kBatchTokens : n_tokens;
 
   // Start the stream before the search below: the warp's first batches are
-  // requested into L2 while the offsets are searched (lanes 0..kPrefetchAhead-1,
-  // one batch each; the pipeline then keeps kPrefetchAhead batches ahead).
-  if (lane < kPrefetchAhead) {
+  // requested into L2 while the offsets are searched (lanes 0.., one batch each).
+  if (lane < kFirstBatches) {
     const int64_t pf = b_begin + lane;
     if (pf < b_end && (pf + 1) * kBatchTokens <= n_tokens)
       l2_prefetch_bulk(tags + pf * kBatchTokens, static_cast<uint32_t>(kBatchTokens * 4));
@@ -503,58 +506,60 @@ __device__ __forceinline__ void stream_warp_range(const int32_t* __restrict__ ta
       lo = qj;
     }
   }
+  // Positions from here on are relative to the range (32 bits: a warp's share of the
+  // tags that fit a GPU's memory is far below 2^31), ends past it clamped.
+  const int len = static_cast<int>(t_end - t_begin);
+  const int32_t* base = tags + t_begin;
+  auto rel = [&](int64_t o) -> int {
+    const int64_t d = o - t_begin;
+    return d > len + 1 ? len + 1 : (d < 0 ? 0 : static_cast<int>(d));
+  };
   int64_t cur = lo;
-  int64_t cur_begin = offsets[cur];
-  int64_t cur_end = offsets[cur + 1];
   // the first trajectory began before this range: this warp's part of it is its
   // head slot; otherwise the head slot says there is none
-  const bool head_open = cur_begin < t_begin;
+  const bool head_open = offsets[cur] < t_begin;
+  bool cur_here = offsets[cur] < t_end;  // the current trajectory begins before t_end
+  int cur_end = rel(offsets[cur + 1]);
   if (!head_open && lane == 0) tt.head[warp].traj = -1;
   LaneAcc acc{0, 0u, 0u};
+  constexpr int kBatch = static_cast<int>(kBatchTokens);
 
-  auto load_batch = [&](int4 (&v)[kTilesPerBatch], int64_t b) {
-    const int64_t bt0 = b * kBatchTokens;
-    // ask L2 for a batch further ahead (no registers held while it is in flight)
-    const int64_t pf = b + kPrefetchAhead;
-    if (lane == 0 && pf < b_end && (pf + 1) * kBatchTokens <= n_tokens)
-      l2_prefetch_bulk(tags + pf * kBatchTokens, static_cast<uint32_t>(kBatchTokens * 4));
-    if (bt0 + kBatchTokens <= n_tokens) {
+  auto load_batch = [&](int4 (&v)[kTiles], int at) {
+    if (at + kBatch <= len) {
 #pragma unroll
-      for (int u = 0; u < kTilesPerBatch; ++u)
-        v[u] = ld_stream_v4(tags + bt0 + u * kTileTokens + lane * 4);
+      for (int u = 0; u < kTiles; ++u)
+        v[u] = ld_stream_v4(base + at + u * kTileTokens + lane * 4);
     } else {
 #pragma unroll
-      for (int u = 0; u < kTilesPerBatch; ++u) {
-        const int64_t t = bt0 + u * kTileTokens + lane * 4;
-        v[u].x = (t + 0 < n_tokens) ? tags[t + 0] : -1;
-        v[u].y = (t + 1 < n_tokens) ? tags[t + 1] : -1;
-        v[u].z = (t + 2 < n_tokens) ? tags[t + 2] : -1;
-        v[u].w = (t + 3 < n_tokens) ? tags[t + 3] : -1;
+      for (int u = 0; u < kTiles; ++u) {
+        const int t = at + u * kTileTokens + lane * 4;
+        v[u].x = (t + 0 < len) ? base[t + 0] : -1;
+        v[u].y = (t + 1 < len) ? base[t + 1] : -1;
+        v[u].z = (t + 2 < len) ? base[t + 2] : -1;
+        v[u].w = (t + 3 < len) ? base[t + 3] : -1;
       }
     }
   };
 
-  // Adds batch b to the running trajectory sums; false when the offsets end
+  // Adds the batch at `at` to the running trajectory sums; false when the offsets end
   // before the tokens do (inconsistent offsets: stop).
-  auto process = [&](const int4 (&v)[kTilesPerBatch], int64_t b) -> bool {
-    const int64_t bt0 = b * kBatchTokens;
-    const int64_t bt1 = (bt0 + kBatchTokens < n_tokens) ? bt0 + kBatchTokens : n_tokens;
-    int64_t pos = bt0;
+  auto process = [&](const int4 (&v)[kTiles], int at) -> bool {
+    const int end = at + kBatch < len ? at + kBatch : len;
+    int pos = at;
     while (true) {
-      const int64_t seg_hi = cur_end < bt1 ? cur_end : bt1;
-      if (pos == bt0 && seg_hi == bt0 + kBatchTokens) {
+      const int seg_hi = cur_end < end ? cur_end : end;
+      if (pos == at && seg_hi == at + kBatch) {
         // whole batch inside one trajectory: no position tests
-        if (!acc_batch_fast<kTilesPerBatch>(acc, v)) {
+        if (!acc_batch_fast(acc, v)) {
 #pragma unroll
-          for (int u = 0; u < kTilesPerBatch; ++u) acc_group(acc, v[u]);
+          for (int u = 0; u < kTiles; ++u) acc_group(acc, v[u]);
         }
       } else if (seg_hi > pos) {
-        // batch-relative bounds fit 32 bits; they are the same in every lane, so
-        // whole 128-token tiles outside [lo_r, hi_r) are skipped and tiles inside
-        // it need no position tests
-        const int lo_r = static_cast<int>(pos - bt0), hi_r = static_cast<int>(seg_hi - bt0);
+        // the bounds are the same in every lane, so whole 128-token tiles outside
+        // [lo_r, hi_r) are skipped and tiles inside it need no position tests
+        const int lo_r = pos - at, hi_r = seg_hi - at;
 #pragma unroll
-        for (int u = 0; u < kTilesPerBatch; ++u) {
+        for (int u = 0; u < kTiles; ++u) {
           const int t0 = u * kTileTokens;
           if (t0 + kTileTokens <= lo_r || t0 >= hi_r) continue;
           if (t0 >= lo_r && t0 + kTileTokens <= hi_r) {
@@ -568,34 +573,36 @@ __device__ __forceinline__ void stream_warp_range(const int32_t* __restrict__ ta
           }
         }
       }
-      if (cur_end > bt1) return true;  // trajectory continues into the next batch
+      if (cur_end > end) return true;  // trajectory continues into the next batch
       emit(acc, cur, false, head_open && cur == lo, warp, tt);
       if (seg_hi > pos) pos = seg_hi;
       ++cur;
       if (cur >= n_traj) return false;  // tokens past the last trajectory: offsets are bad
-      cur_begin = cur_end;
-      cur_end = offsets[cur + 1];
+      cur_here = cur_end < len;
+      cur_end = rel(offsets[cur + 1]);
       // the next trajectory starts at the batch edge: continue in the next batch;
       // otherwise loop (more of this batch, or empty trajectories to step over)
-      if (pos >= bt1 && cur_end > bt1) return true;
+      if (pos >= end && cur_end > end) return true;
     }
   };
 
   // two register sets: the next batch's loads are in flight while one is added up
-  int4 va[kTilesPerBatch], vb[kTilesPerBatch];
-  int64_t b = b_begin;
-  load_batch(va, b);
+  int4 va[kTiles], vb[kTiles];
+  int at = 0;
+  load_batch(va, at);
   while (true) {
-    if (b + 1 < b_end) load_batch(vb, b + 1);
-    if (!process(va, b)) return;
-    if (++b >= b_end) break;
-    if (b + 1 < b_end) load_batch(va, b + 1);
-    if (!process(vb, b)) return;
-    if (++b >= b_end) break;
+    if (at + kBatch < len) load_batch(vb, at + kBatch);
+    if (!process(va, at)) return;
+    at += kBatch;
+    if (at >= len) break;
+    if (at + kBatch < len) load_batch(va, at + kBatch);
+    if (!process(vb, at)) return;
+    at += kBatch;
+    if (at >= len) break;
   }
   // the trajectory still open continues past this range (one that begins at
   // t_end belongs to the next warp)
-  if (cur < n_traj && cur_begin < t_end) emit(acc, cur, true, head_open && cur == lo, warp, tt);
+  if (cur < n_traj && cur_here) emit(acc, cur, true, head_open && cur == lo, warp, tt);
 }
 
 struct FinalizeArgs {
@@ -929,8 +936,8 @@ __device__ __forceinline__ void fused_finalize(const int64_t* __restrict__ offse
       b_hi = S - 1;
     } else if (t1 > t0) {
       const StreamGeom& g = p.geom;
-      b_lo = warp_of_batch(g, t0 / g.batch_tokens) / (kReduceThreads / 32);
-      b_hi = warp_of_batch(g, (t1 - 1) / g.batch_tokens) / (kReduceThreads / 32);
+      b_lo = warp_of_batch(g, t0 / kBatchTokens) / (kReduceThreads / 32);
+      b_hi = warp_of_batch(g, (t1 - 1) / kBatchTokens) / (kReduceThreads / 32);
     }
     bool ok = true;
     const uint64_t start = global_timer_ns();
@@ -970,8 +977,8 @@ __device__ __forceinline__ void fused_finalize(const int64_t* __restrict__ offse
   }
 }
 
-template <int kTilesPerBatch, int kMinBlocks>
-__global__ void __launch_bounds__(kReduceThreads, kMinBlocks)
+template <bool kFused>
+__global__ void __launch_bounds__(kReduceThreads, kBlocksPerSm)
     tag_reduce_kernel(const int32_t* __restrict__ tags, const int64_t* __restrict__ offsets,
                       int64_t n_traj, int64_t n_tokens, TagTotals tt, int n_stream_blocks,
                       WindowPrep prep, FusedFinalize fz) {
@@ -979,8 +986,8 @@ __global__ void __launch_bounds__(kReduceThreads, kMinBlocks)
     window_prep_block(static_cast<int>(blockIdx.x) - n_stream_blocks, prep);
     return;
   }
-  stream_warp_range<kTilesPerBatch>(tags, offsets, n_traj, n_tokens, tt, n_stream_blocks);
-  if (fz.done) fused_finalize(offsets, n_tokens, n_stream_blocks, fz);
+  stream_warp_range(tags, offsets, n_traj, n_tokens, tt, n_stream_blocks);
+  if (kFused) fused_finalize(offsets, n_tokens, n_stream_blocks, fz);
 }
 
 // Stale-k admission (Sec. 2): kbar = sum (j - v_t) / T = (j T - sum v_t) / T in
@@ -1033,46 +1040,43 @@ ScoreWs carve_score_ws(Carver& cv, int64_t n_traj) {
   return w;
 }
 
-// Resident blocks per SM of a tag-reduction instance with the given dynamic
-// shared memory (cached per device, instance and size).
-template <int kTiles, int kBlocks>
+// Resident blocks per SM of the fused tag reduction with the given dynamic shared
+// memory (cached per device and size).
 pace_status reduce_blocks_per_sm(size_t smem, int* out) {
   constexpr int kMaxDevices = 64;
-  static int cache[kMaxDevices][2] = {};
-  static size_t cache_smem[kMaxDevices][2] = {};
+  static int cache[kMaxDevices] = {};
+  static size_t cache_smem[kMaxDevices] = {};
   static std::mutex mu;
   int dev = 0;
   PACE_TRY_CUDA(cudaGetDevice(&dev));
-  const int which = kTiles == kTilesSmall ? 0 : 1;
   std::lock_guard<std::mutex> g(mu);
-  if (dev >= 0 && dev < kMaxDevices && cache[dev][which] > 0 && cache_smem[dev][which] == smem) {
-    *out = cache[dev][which];
+  if (dev >= 0 && dev < kMaxDevices && cache[dev] > 0 && cache_smem[dev] == smem) {
+    *out = cache[dev];
     return PACE_OK;
   }
   int nb = 0;
   // above the default 48 KB (windows of more than ~2,000 values with their F
   // table) the kernel must be allowed the larger dynamic shared memory first
   if (smem > 48 * 1024)
-    PACE_TRY_CUDA(cudaFuncSetAttribute(tag_reduce_kernel<kTiles, kBlocks>,
+    PACE_TRY_CUDA(cudaFuncSetAttribute(tag_reduce_kernel<true>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
-  PACE_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &nb, tag_reduce_kernel<kTiles, kBlocks>, kReduceThreads, smem));
+  PACE_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tag_reduce_kernel<true>,
+                                                              kReduceThreads, smem));
   if (dev >= 0 && dev < kMaxDevices) {
-    cache[dev][which] = nb;
-    cache_smem[dev][which] = smem;
+    cache[dev] = nb;
+    cache_smem[dev] = smem;
   }
   *out = nb;
   return PACE_OK;
 }
 
-template <int kTiles, int kBlocks>
-pace_status launch_tag_reduce(unsigned grid, size_t smem, bool cooperative, cudaStream_t st,
+pace_status launch_tag_reduce(unsigned grid, size_t smem, bool fused, cudaStream_t st,
                               const int32_t* tags, const int64_t* offsets, int64_t n_traj,
                               int64_t n_tokens, const ScoreWs& ws, int stream_blocks,
                               const WindowPrep& prep, const FusedFinalize& fz) {
-  if (!cooperative) {
-    tag_reduce_kernel<kTiles, kBlocks><<<grid, kReduceThreads, smem, st>>>(
+  if (!fused) {
+    tag_reduce_kernel<false><<<grid, kReduceThreads, smem, st>>>(
         tags, offsets, n_traj, n_tokens, ws.tt, stream_blocks, prep, fz);
     return last_launch_status();
   }
@@ -1086,8 +1090,8 @@ pace_status launch_tag_reduce(unsigned grid, size_t smem, bool cooperative, cuda
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  PACE_TRY_CUDA(cudaLaunchKernelEx(&cfg, tag_reduce_kernel<kTiles, kBlocks>, tags, offsets,
-                                   n_traj, n_tokens, ws.tt, stream_blocks, prep, fz));
+  PACE_TRY_CUDA(cudaLaunchKernelEx(&cfg, tag_reduce_kernel<true>, tags, offsets, n_traj, n_tokens,
+                                   ws.tt, stream_blocks, prep, fz));
   return last_launch_status();
 }
 
@@ -1104,19 +1108,14 @@ pace_status run_tag_reduce(const int32_t* tags, const int64_t* offsets, int64_t 
   const unsigned prep_blocks = (prep.window && !fused) ? window_prep_blocks(prep.n) : 0u;
   size_t smem = prep_blocks ? window_prep_smem(prep.n) : 0;
   if (fused) smem = fused_smem;
-  const bool small = n_tokens <= kSmallPoolTokens;
-  const int tiles = small ? kTilesSmall : kTilesLarge;
-  int per_sm = small ? kBlocksSmall : kBlocksLarge;
+  int per_sm = kBlocksPerSm;
   if (fused) {
     int nb = 0;
-    const pace_status occ = small ? reduce_blocks_per_sm<kTilesSmall, kBlocksSmall>(smem, &nb)
-                                  : reduce_blocks_per_sm<kTilesLarge, kBlocksLarge>(smem, &nb);
-    if (occ != PACE_OK) return occ;
+    PACE_TRY(reduce_blocks_per_sm(smem, &nb));
     if (nb < 1) return PACE_ERR_UNSUPPORTED_SHAPE;
     per_sm = nb < per_sm ? nb : per_sm;
   }
-  const int64_t batch_tokens = static_cast<int64_t>(kTileTokens) * tiles;
-  const int64_t n_batches = (n_tokens + batch_tokens - 1) / batch_tokens;
+  const int64_t n_batches = (n_tokens + kBatchTokens - 1) / kBatchTokens;
   const int warps_per_block = kReduceThreads / 32;
   const int64_t per_block = warps_per_block * kMinBatchesPerWarp;
   int64_t blocks = (n_batches + per_block - 1) / per_block;
@@ -1124,7 +1123,6 @@ pace_status run_tag_reduce(const int32_t* tags, const int64_t* offsets, int64_t 
   if (cap > kMaxStreamBlocks) cap = kMaxStreamBlocks;
   if (blocks > cap) blocks = cap;
   if (fused && blocks < 1) blocks = 1;
-  geom->batch_tokens = batch_tokens;
   geom->n_batches = n_batches;
   geom->n_warps = blocks * warps_per_block;
   if (blocks == 0 && prep_blocks == 0) return PACE_OK;
@@ -1142,14 +1140,8 @@ pace_status run_tag_reduce(const int32_t* tags, const int64_t* offsets, int64_t 
   const int stream_blocks = static_cast<int>(blocks);
   const ProfileEvents& pe = profile_events(PACE_PROFILE_TAG_REDUCE);
   if (pe.begin) PACE_TRY_CUDA(cudaEventRecord(pe.begin, st));
-  if (small)
-    PACE_TRY((launch_tag_reduce<kTilesSmall, kBlocksSmall>(grid, smem, fused, st, tags, offsets,
-                                                            n_traj, n_tokens, ws, stream_blocks,
-                                                            prep, fz)));
-  else
-    PACE_TRY((launch_tag_reduce<kTilesLarge, kBlocksLarge>(grid, smem, fused, st, tags, offsets,
-                                                            n_traj, n_tokens, ws, stream_blocks,
-                                                            prep, fz)));
+  PACE_TRY(launch_tag_reduce(grid, smem, fused, st, tags, offsets, n_traj, n_tokens, ws,
+                             stream_blocks, prep, fz));
   if (pe.end) PACE_TRY_CUDA(cudaEventRecord(pe.end, st));
   return PACE_OK;
 }
