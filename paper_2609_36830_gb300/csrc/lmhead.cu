@@ -16,10 +16,10 @@
 //                     read straight from the caller's hidden-state tensor
 //                     through the compact-row index.  Per work item the warp
 //                     splits the block's 128 rows into runs of consecutive
-//                     source rows (plan_block_loads) and the runs into boxes of
-//                     1, 2, 4 or a multiple of 8 rows (one box for a block inside
-//                     a response; the first and last of several runs, rounded up
-//                     to one box, spill into 16 KB regions around the tile).  A block of more than 31 boxes is
+//                     source rows (plan_block_loads) and the runs into boxes
+//                     (Boxes; one for a block inside a response; the first and
+//                     last of several runs, rounded up to one box, spill into
+//                     16 KB regions around the tile).  A block of more than 31 boxes is
 //                     fetched by four-row TMA gathers (tile::gather4), one per
 //                     lane.  No copy of the rows is made.
 //   warp 1 / lane 0   MMA issuer, even CTA only: tcgen05.mma.cta_group::2
@@ -99,29 +99,40 @@ __host__ __device__ constexpr uint32_t a_tile_off(uint32_t s) {
   return kSpill + s * (kStageA + kSpill);
 }
 __host__ __device__ constexpr uint32_t b_tile_off(uint32_t s) { return kARegion + s * kStageB; }
-// Tensor maps of the hidden states with boxes of 1, 2, 4, 8, 16, 24, ..., 128 rows
-// (64 columns, 128-byte swizzle).  An SM takes in operand tiles at close to the
-// rate the tensor cores use them, so the rows a block's boxes load beyond its 128
-// cost their share of time: with heights of 2^j only, a block of two runs loaded 192
-// rows on average, with multiples of 8 it loads 135.  Micro-batches whose blocks
-// straddle two or three sequences (H 2048, V 151,936), one launch: 1,455 rows 605-654
-// -> 558-575 us, 2,582 rows 1135 -> 1054, 6,186 rows 2484 -> 2222; 37k rows of
-// multi-turn sequences (H 3584) 24.1 -> 23.7-24.1 ms (power-capped).
-constexpr int kBoxLevels = 19;
+// Tensor maps of the hidden states with boxes of several heights (64 columns, 128-byte
+// swizzle).  An SM takes in operand tiles at close to the rate the tensor cores use
+// them, so the rows a block's boxes load beyond its 128 cost their share of time, and
+// so do its boxes: with every block cut alike (19,456 rows, H 2048, V 151,936) one and
+// two boxes run at 1934 TFLOP/s, three at 1896, four at 1770, eight at 1344.
+//   Fine: 1, 2, ..., 128 rows, so every run is one box.  128 maps take 3.6 us of host
+//     time to encode and 16 KB of kernel parameters, so for large launches only
+//     (kFineFlops).
+//   Coarse: 1, 2, 4, 8, 16, 24, ..., 128 rows: the first and last run of a block are one
+//     box each, of at most 7 rows more than they have; a run in between takes up to four.
+// One launch, coarse and fine: 2,582 rows of eight sequences (H 2048 head) 1050 and 963
+// us where a block has three runs, 37k rows of multi-turn sequences (H 3584) 24.0 and
+// 23.5 ms; powers of two only were 7-12 % slower still on micro-batches.
+template <bool kFine>
+struct Boxes {
+  static constexpr int kLevels = kFine ? 128 : 19;
+  __host__ __device__ static constexpr int rows(int level) {
+    return kFine ? level + 1 : (level < 3 ? 1 << level : 8 * (level - 2));
+  }
+  // the lowest box of at least n rows, the tallest of at most n (n in 1..128)
+  __host__ __device__ static constexpr int covering(int n) {
+    return kFine || n <= 2 ? n - 1 : (n <= 4 ? 2 : 2 + (n + 7) / 8);
+  }
+  __host__ __device__ static constexpr int within(int n) {
+    return kFine ? n - 1 : (n >= 8 ? 2 + n / 8 : (n >= 4 ? 2 : (n >= 2 ? 1 : 0)));
+  }
+};
+static_assert(Boxes<false>::rows(18) == BM && Boxes<true>::rows(127) == BM,
+              "the tallest box is a block");
 constexpr int kMaxBoxes = 31;  // more boxes in a block: four-row gathers instead
-__host__ __device__ constexpr int box_rows(int level) {
-  return level < 3 ? 1 << level : 8 * (level - 2);
-}
-// the lowest box of at least n rows, the tallest of at most n (n in 1..128)
-__host__ __device__ constexpr int box_covering(int n) {
-  return n <= 2 ? n - 1 : (n <= 4 ? 2 : 2 + (n + 7) / 8);
-}
-__host__ __device__ constexpr int box_within(int n) {
-  return n >= 8 ? 2 + n / 8 : (n >= 4 ? 2 : n - 1 < 1 ? 0 : 1);
-}
-static_assert(box_rows(kBoxLevels - 1) == BM, "the tallest box is a block");
+constexpr double kFineFlops = 4e11;  // about 200 us
+template <bool kFine>
 struct AMaps {
-  CUtensorMap box[kBoxLevels];  // box[j]: box_rows(j) rows
+  CUtensorMap box[Boxes<kFine>::kLevels];  // box[j]: Boxes::rows(j) rows
 };
 constexpr int kMaxSplits = 8;
 constexpr int kMaxClusters = 76;  // clusters launched at most (bounds the tail's partials)
@@ -306,9 +317,10 @@ struct BlockLoads {
 // region before the tile), the last one such box starting at the run's start (its
 // later rows land in the spill region after the tile), and a run in between is
 // loaded exactly.  Boxes never overlap inside the tile, and no box is taller than
-// box_rows(max_level) (the tallest map the hidden-state tensor allows).  Writes the source rows to row_src[BM], the boxes to piece[] as
+// Boxes::rows(max_level) (the tallest map the hidden-state tensor allows).  Writes the source rows to row_src[BM], the boxes to piece[] as
 // (first source row, (first block row + 128) | level << 9), their number to
 // plan[0] and their bytes per K step to plan[1].  All 32 lanes call it.
+template <bool kFine>
 __device__ void plan_block_loads(const int32_t* __restrict__ rowidx, int64_t row0,
                                  int64_t n_valid, int max_level, int lane, int32_t* row_src,
                                  int2* piece, volatile int* plan) {
@@ -351,21 +363,21 @@ __device__ void plan_block_loads(const int32_t* __restrict__ rowidx, int64_t row
       }
       const int32_t s0 = row_src[r];
       const int len = e - r;
-      const int cl = box_covering(len);
+      const int cl = Boxes<kFine>::covering(len);
       if (m > 1 && (k == 0 || k == m - 1) && cl <= max_level) {
         // first or last of several runs: one box that covers it, ending at the
         // first run's end (spilling before the tile) or starting at the last
         // run's start (spilling after it)
-        const int at = k == 0 ? len - box_rows(cl) : r;
+        const int at = k == 0 ? len - Boxes<kFine>::rows(cl) : r;
         piece[n++] = make_int2(s0 + (at - r), (at + BM) | (cl << 9));
-        rows += box_rows(cl);
+        rows += Boxes<kFine>::rows(cl);
       } else {  // the only run, or one in between: exactly
         int at = r, left_rows = len;
         int32_t src = s0;
         while (left_rows > 0) {
-          int lev = box_within(left_rows);
+          int lev = Boxes<kFine>::within(left_rows);
           if (lev > max_level) lev = max_level;
-          const int h = box_rows(lev);
+          const int h = Boxes<kFine>::rows(lev);
           piece[n++] = make_int2(src, (at + BM) | (lev << 9));
           rows += h;
           at += h;
@@ -382,8 +394,9 @@ __device__ void plan_block_loads(const int32_t* __restrict__ rowidx, int64_t row
   __syncwarp();
 }
 
+template <bool kFine>
 __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
-    lmhead_lse_kernel(const __grid_constant__ AMaps am, const __grid_constant__ CUtensorMap tm_b,
+    lmhead_lse_kernel(const __grid_constant__ AMaps<kFine> am, const __grid_constant__ CUtensorMap tm_b,
                       LmArgs p) {
   extern __shared__ unsigned char smem_raw[];
   // the same offsets in both CTAs: the pair's MMA reads each CTA's operand
@@ -457,7 +470,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
     // more than kMaxBoxes boxes is gathered four rows a lane instead.
     const bool gather = p.gather != 0;
     if (lane == 0) tma_prefetch_desc(&tm_b);
-    if (gather ? lane < kBoxLevels : lane == kBoxLevels - 1) tma_prefetch_desc(&am.box[lane]);
+    if (lane == 1) tma_prefetch_desc(&am.box[Boxes<kFine>::kLevels - 1]);
     const uint64_t pol = make_policy_evict_normal();
     uint32_t it = 0;
     bool ok = true;
@@ -469,12 +482,12 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
       bl.a_bytes = kStageA;
       bl.psrc = static_cast<int32_t>(row0);
       bl.pdst = 0;
-      bl.plev = kBoxLevels - 1;
+      bl.plev = Boxes<kFine>::kLevels - 1;
 #pragma unroll
       for (int j = 0; j < 4; ++j) bl.g4[j] = 0;
       bl.scattered = false;
       if (!gather) return;
-      plan_block_loads(p.rowidx, row0, n_valid, p.max_level, lane, row_src, piece, plan);
+      plan_block_loads<kFine>(p.rowidx, row0, n_valid, p.max_level, lane, row_src, piece, plan);
       bl.n = plan[0];
       bl.scattered = bl.n > kMaxBoxes;
       if (!bl.scattered) {
@@ -787,6 +800,36 @@ struct LmLaunchInfo {
   int max_clusters = 0;
 };
 
+// Tensor maps, launch of one instance.
+struct LmLaunch {
+  const void* hidden;
+  int64_t n_rows;
+  int H;
+  bool compact;
+  CUtensorMap tm_b;
+  unsigned grid;
+};
+template <bool kFine>
+pace_status launch_lmhead(const LmLaunch& l, LmArgs a, cudaStream_t st) {
+  using B = Boxes<kFine>;
+  AMaps<kFine> am;
+  // boxes up to the tensor's height (at most 128 rows); taller levels repeat the
+  // tallest valid map and are never used, nor are the others without a row index
+  int max_level = 0;
+  while (max_level + 1 < B::kLevels && B::rows(max_level + 1) <= l.n_rows) ++max_level;
+  if (!l.compact && max_level != B::kLevels - 1) return PACE_ERR_INVALID_ARG;  // n_rows >= 128
+  PACE_TRY(encode_bf16_2d(&am.box[max_level], l.hidden, l.n_rows, l.H, l.H, BK, B::rows(max_level)));
+  for (int j = 0; j < B::kLevels; ++j) {
+    if (l.compact && j < max_level)
+      PACE_TRY(encode_bf16_2d(&am.box[j], l.hidden, l.n_rows, l.H, l.H, BK, B::rows(j)));
+    else
+      am.box[j] = am.box[max_level];
+  }
+  a.max_level = max_level;
+  lmhead_lse_kernel<kFine><<<l.grid, kThreads, kSmemBytes, st>>>(am, l.tm_b, a);
+  return last_launch_status();
+}
+
 // Dynamic shared memory opt-in and the number of 2-CTA clusters that can be
 // resident at once on the current device (cached per device).
 pace_status lm_launch_info(LmLaunchInfo* out) {
@@ -798,7 +841,10 @@ pace_status lm_launch_info(LmLaunchInfo* out) {
   if (dev < 0 || dev >= kMaxDevices) return PACE_ERR_CUDA;
   std::lock_guard<std::mutex> g(mu);
   if (info[dev].max_clusters == 0) {
-    PACE_TRY_CUDA(cudaFuncSetAttribute(lmhead_lse_kernel,
+    PACE_TRY_CUDA(cudaFuncSetAttribute(lmhead_lse_kernel<false>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(kSmemBytes)));
+    PACE_TRY_CUDA(cudaFuncSetAttribute(lmhead_lse_kernel<true>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kSmemBytes)));
     cudaLaunchConfig_t cfg = {};
@@ -813,7 +859,7 @@ pace_status lm_launch_info(LmLaunchInfo* out) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, lmhead_lse_kernel, &cfg) != cudaSuccess || n < 1)
+    if (cudaOccupancyMaxActiveClusters(&n, lmhead_lse_kernel<false>, &cfg) != cudaSuccess || n < 1)
       n = sm_count() / CLUSTER;
     info[dev].max_clusters = n < kMaxClusters ? n : kMaxClusters;
   }
@@ -879,21 +925,12 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   }
   if (n_rows == 0) return PACE_OK;
   const int n_vtiles = (V + BN - 1) / BN;
-  AMaps am;
-  CUtensorMap tm_b;
-  // boxes up to the tensor's height (at most 128 rows); taller levels repeat the
-  // tallest valid map and are never used, nor are the others without a row index
-  int max_level = 0;
-  while (max_level + 1 < kBoxLevels && box_rows(max_level + 1) <= n_rows) ++max_level;
-  if (!compact && max_level != kBoxLevels - 1) return PACE_ERR_INVALID_ARG;  // n_rows >= 128
-  PACE_TRY(encode_bf16_2d(&am.box[max_level], hidden, n_rows, H, H, BK, box_rows(max_level)));
-  for (int j = 0; j < kBoxLevels; ++j) {
-    if (compact && j < max_level)
-      PACE_TRY(encode_bf16_2d(&am.box[j], hidden, n_rows, H, H, BK, box_rows(j)));
-    else
-      am.box[j] = am.box[max_level];
-  }
-  PACE_TRY(encode_bf16_2d(&tm_b, w_vocab, V, H, H, BK, BN / CLUSTER));  // one CTA's half tile
+  LmLaunch l;
+  l.hidden = hidden;
+  l.n_rows = n_rows;
+  l.H = H;
+  l.compact = compact;
+  PACE_TRY(encode_bf16_2d(&l.tm_b, w_vocab, V, H, H, BK, BN / CLUSTER));  // one CTA's half tile
   LmLaunchInfo li;
   PACE_TRY(lm_launch_info(&li));
   LmArgs a;
@@ -907,7 +944,6 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   a.targets = targets;
   a.rowidx = rowidx;
   a.gather = compact ? 1 : 0;
-  a.max_level = max_level;
   a.part_m = ws.part_m;
   a.part_s = ws.part_s;
   a.tgt_logit = ws.tgt;
@@ -917,12 +953,13 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   // rows could make tiles
   const int64_t tiles = (rows_cap + 2 * BM - 1) / (2 * BM) * n_vtiles;
   const int64_t clusters = tiles < li.max_clusters ? tiles : li.max_clusters;
-  const int64_t grid = clusters * CLUSTER;
+  l.grid = static_cast<unsigned>(clusters * CLUSTER);
   if (!compact) PACE_TRY_CUDA(cudaMemsetAsync(ws.round_ctr, 0, sizeof(unsigned), st));
   const ProfileEvents& pe = profile_events(PACE_PROFILE_LMHEAD);
   if (pe.begin) PACE_TRY_CUDA(cudaEventRecord(pe.begin, st));
-  lmhead_lse_kernel<<<static_cast<unsigned>(grid), kThreads, kSmemBytes, st>>>(am, tm_b, a);
-  PACE_TRY(last_launch_status());
+  const bool fine =
+      compact && n_rows >= BM && 2.0 * H * V * static_cast<double>(n_rows) >= kFineFlops;
+  PACE_TRY(fine ? launch_lmhead<true>(l, a, st) : launch_lmhead<false>(l, a, st));
   if (pe.end) PACE_TRY_CUDA(cudaEventRecord(pe.end, st));
   int64_t mblocks = (rows_cap + 255) / 256;
   const int64_t cap = static_cast<int64_t>(sm_count()) * 8;

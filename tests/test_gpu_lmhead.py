@@ -113,27 +113,33 @@ def test_row_pairs_around_whole_rounds(pairs, extra, V):
         assert np.abs(lp - as_np(olp)).max() <= 2 * tol
 
 
+@pytest.mark.parametrize("H,V", [(64, 300), (1024, 12500)])
 @pytest.mark.parametrize("cut_len,n_rows_last", [(3, 128), (200, 77), (1, 1)])
-def test_blocks_cut_at_every_row(cut_len, n_rows_last):
-    """Block b of the rows in the loss is a run of b rows and one of 128 - b (every
-    height of box, at both ends of the tile), the last block short; the bound is that
-    of 32-bit sums of 64 products and V terms (|z| < 12)."""
-    H, V = 64, 300
+def test_blocks_cut_at_every_row(cut_len, n_rows_last, H, V):
+    """Blocks of a run of b rows and one of 128 - b, and of a run of b rows between two
+    others (every height of box at both ends of the tile and inside it), the last block
+    short; a launch small enough for the coarse set of boxes and one large enough for the
+    fine set.  The bound is that of 32-bit sums of H products and V terms (|z| < 12)."""
     parts = []
     for b in range(1, 128):
         parts += [np.ones(b), np.zeros(cut_len), np.ones(128 - b)]
         parts += [np.zeros(5)] if b % 3 == 0 else []
-    m = np.concatenate(parts + [np.ones(n_rows_last)]).astype(np.uint8)
+    for b in range(1, 127):
+        first = (127 - b) // 2 + 1 if b < 126 else 1
+        parts += [np.zeros(cut_len), np.ones(first), np.zeros(2), np.ones(b), np.zeros(1),
+                  np.ones(128 - first - b)]
+    m = np.concatenate(parts + [np.zeros(1), np.ones(n_rows_last)]).astype(np.uint8)
     g = torch.Generator(device=DEV)
     g.manual_seed(cut_len)
     h = torch.randn(m.size, H, device=DEV, generator=g).to(torch.bfloat16)
-    w = (torch.randn(V, H, device=DEV, generator=g) / 4).to(torch.bfloat16)
+    w = (torch.randn(V, H, device=DEV, generator=g) * 2 / math.sqrt(H)).to(torch.bfloat16)
     y = torch.randint(0, V, (m.size,), device=DEV, generator=g, dtype=torch.int32)
-    z = h.double() @ w.double().T
-    olse = as_np(torch.logsumexp(z, 1))
+    wd = w.double().T
+    olse = as_np(torch.cat([torch.logsumexp(h[i:i + 4096].double() @ wd, 1)
+                            for i in range(0, m.size, 4096)]))
     lp, lse = _run(h, w, y, mask=to_dev(m))
     sel = m.astype(bool)
-    assert np.abs(lse[sel] - olse[sel]).max() <= 12 * 64 * 2.0 ** -24 + 16 * 2.0 ** -22
+    assert np.abs(lse[sel] - olse[sel]).max() <= 12 * H * 2.0 ** -24 + 16 * 2.0 ** -22
     assert (lp[~sel] == 0).all() and (lse[~sel] == 0).all()
 
 
