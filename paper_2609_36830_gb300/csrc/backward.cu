@@ -627,24 +627,25 @@ struct GradArgs {
   const float* adv;
   int64_t n_seq, n_rows;
   RowGeom geom;
+  bool vec;
   float eps_low, eps_high, dual;
-  int agg;
   const long long* block_in;  // TOKEN_MEAN: rows in the loss per block of the count
   const unsigned long long* seq_in;  // SEQ_MEAN: rows in the loss per sequence,
   const int* n_used;                 // sequences that have any
   float* dlp;
 };
 
+template <bool kSeqMean>
 __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_kernel(GradArgs p) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int wid = threadIdx.x >> 5;
   const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * p.geom.per_warp;
   const int64_t w1 = w0 + p.geom.per_warp < p.geom.n_tiles ? w0 + p.geom.per_warp : p.geom.n_tiles;
   int64_t t0 = w0 * kRowTile;
   RowLoads cur, nxt;
   // the first rows' loads are in flight while the counts are added up
-  if (w0 < w1) cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows));
+  if (w0 < w1) cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows), p.vec);
   double scale = 0.0;
-  if (p.agg == PACE_AGG_TOKEN_MEAN) {
+  if (!kSeqMean) {
     __shared__ double s_scale;
     long long mine = 0, total = 0;
     for (int i = threadIdx.x; i < p.geom.blocks; i += kRowThreads) mine += p.block_in[i];
@@ -657,18 +658,16 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
   PieceWalker pw(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0);
   for (int64_t w = w0; w < w1; ++w) {
     const int64_t t1 = tile_end(t0, p.n_rows);
-    if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows));
+    if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
     unsigned in = 0u;
-    pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t) {
-      const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
-      in |= rows;
-      if (p.agg != PACE_AGG_TOKEN_MEAN)
-        scale = 1.0 / (static_cast<double>(*p.n_used) * static_cast<double>(p.seq_in[seq]));
+    float adv[kRowsPerLane];  // per row; derivatives once per tile, not per piece
+    auto derive = [&](unsigned rows) {
       const float s_hi = static_cast<float>(scale);
       const float s_lo = static_cast<float>(scale - static_cast<double>(s_hi));
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) {
         if (rows >> u & 1u) {
+          const float a = adv[u];
           const float d = cur.lp[u] - cur.bh[u];
           const float dc = fminf(fmaxf(d, -20.0f), 20.0f);
           const float rho = expf(dc);
@@ -681,12 +680,19 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
           cur.lp[u] = fmaf(x, s_hi, x * s_lo);  // the derivative, once the row is used
         }
       }
-    });
+    };
+    pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t) {
+      const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
+      in |= rows;
 #pragma unroll
-    for (int u = 0; u < kRowsPerLane; ++u) {
-      const int64_t r = t0 + 32 * u + lane;
-      if (r < t1) p.dlp[r] = in >> u & 1u ? cur.lp[u] : 0.0f;
-    }
+      for (int u = 0; u < kRowsPerLane; ++u) adv[u] = rows >> u & 1u ? a : adv[u];
+      if (kSeqMean) {
+        scale = 1.0 / (static_cast<double>(*p.n_used) * static_cast<double>(p.seq_in[seq]));
+        derive(rows);
+      }
+    });
+    if (!kSeqMean) derive(in);
+    store_rows(p.dlp, t0, t1, p.vec, in, cur.lp);
     cur = nxt;
     t0 = t1;
   }
@@ -837,15 +843,18 @@ extern "C" pace_status pace_surrogate_backward(const PaceBatch* batch, const flo
   a.n_seq = batch->n_seq;
   a.n_rows = batch->n_rows;
   a.geom = row_geom(batch->n_rows);
+  a.vec = rows_vec(logprob, loss->behav_lp, dlp, batch->mask);
   a.eps_low = loss->params.eps_low;
   a.eps_high = loss->params.eps_high;
   a.dual = loss->params.dual_clip;
-  a.agg = loss->params.agg;
   a.block_in = ws.counts.block;
   a.seq_in = ws.seq_in;
   a.n_used = ws.n_used;
   a.dlp = dlp;
-  surrogate_grad_kernel<<<static_cast<unsigned>(a.geom.blocks), kRowThreads, 0, st>>>(a);
+  if (seq_mean)
+    surrogate_grad_kernel<true><<<static_cast<unsigned>(a.geom.blocks), kRowThreads, 0, st>>>(a);
+  else
+    surrogate_grad_kernel<false><<<static_cast<unsigned>(a.geom.blocks), kRowThreads, 0, st>>>(a);
   return last_launch_status();
 }
 

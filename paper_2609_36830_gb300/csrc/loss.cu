@@ -168,7 +168,7 @@ struct SurrogateArgs {
   const float* adv;
   int64_t n_seq, n_rows;
   RowGeom geom;
-  int agg;
+  bool vec;
   float eps_low, eps_high, dual;
   float* ratio;
   SurrogateWs ws;
@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(kRowThreads) seq_mean_kernel(SurrogateArgs p) 
   finish_in_last_block(p.ws.counter, p.ws.seq_sum, p.ws.seq_cnt, p.n_seq, p.loss, p.partial);
 }
 
+template <bool kSeqMean>
 __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(SurrogateArgs p) {
   __shared__ double sh_sum[kRowWarps], sh_cnt[kRowWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -281,36 +282,37 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
   if (w0 < w1) {
     int64_t t0 = w0 * kRowTile;
     RowLoads cur, nxt;
-    cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows));
+    cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows), p.vec);
     PieceWalker pw(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0);
     for (int64_t w = w0; w < w1; ++w) {
       const int64_t t1 = tile_end(t0, p.n_rows);
-      if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows));
+      if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
       unsigned in = 0u;
-      double head_s = 0.0, head_c = 0.0;
-      pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t begin) {
-        const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
-        in |= rows;
+      float adv[kRowsPerLane];  // per row; the terms are computed once per tile, not per piece
+      // the terms of the given rows, added up
+      auto terms = [&](unsigned rows) -> double {
         Sum3 sum{0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int u = 0; u < kRowsPerLane; ++u) {
           if (rows >> u & 1u) {
             float rho;
-            const float x =
-                clipped_term(cur.lp[u], cur.bh[u], a, p.eps_low, p.eps_high, p.dual, &rho);
+            const float x = clipped_term(cur.lp[u], cur.bh[u], adv[u], p.eps_low, p.eps_high,
+                                         p.dual, &rho);
             cur.bh[u] = rho;  // the ratio, once the row is used
             sum.add(x);
           }
         }
-        double s = sum.value();
-        const int c = __popc(rows);
-        if (p.agg == PACE_AGG_TOKEN_MEAN) {
-          tot = __dadd_rn(tot, s);
-          cnt += c;
-          return;
-        }
-        s = warp_sum_fixed(s);
-        const double cd = static_cast<double>(__reduce_add_sync(0xffffffffu, c));
+        return sum.value();
+      };
+      double head_s = 0.0, head_c = 0.0;
+      pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t begin) {
+        const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
+        in |= rows;
+#pragma unroll
+        for (int u = 0; u < kRowsPerLane; ++u) adv[u] = rows >> u & 1u ? a : adv[u];
+        if (!kSeqMean) return;
+        const double s = warp_sum_fixed(terms(rows));
+        const double cd = static_cast<double>(__reduce_add_sync(0xffffffffu, __popc(rows)));
         if (begin < t0) {  // the sequence began in an earlier tile
           head_s = s;
           head_c = cd;
@@ -319,22 +321,21 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
           p.ws.seq_cnt[seq] = cd;
         }
       });
-      if (p.agg != PACE_AGG_TOKEN_MEAN && lane == 0) {
-        p.ws.head_sum[w] = head_s;
-        p.ws.head_cnt[w] = head_c;
-      }
-      if (p.ratio) {
-#pragma unroll
-        for (int u = 0; u < kRowsPerLane; ++u) {
-          const int64_t r = t0 + 32 * u + lane;
-          if (r < t1) p.ratio[r] = in >> u & 1u ? cur.bh[u] : 0.0f;
+      if (kSeqMean) {
+        if (lane == 0) {
+          p.ws.head_sum[w] = head_s;
+          p.ws.head_cnt[w] = head_c;
         }
+      } else {
+        tot = __dadd_rn(tot, terms(in));
+        cnt += __popc(in);
       }
+      if (p.ratio) store_rows(p.ratio, t0, t1, p.vec, in, cur.bh);
       cur = nxt;
       t0 = t1;
     }
   }
-  if (p.agg != PACE_AGG_TOKEN_MEAN) return;
+  if (kSeqMean) return;
   tot = warp_sum_fixed(tot);
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   if (lane == 0) {
@@ -425,7 +426,7 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
   a.n_seq = b->n_seq;
   a.n_rows = b->n_rows;
   a.geom = row_geom(b->n_rows);
-  a.agg = l->params.agg;
+  a.vec = rows_vec(logprob, l->behav_lp, l->ratio, b->mask);
   a.eps_low = l->params.eps_low;
   a.eps_high = l->params.eps_high;
   a.dual = l->params.dual_clip;
@@ -433,10 +434,13 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
   a.ws = ws;
   a.loss = l->loss;
   a.partial = l->partial;
-  surrogate_kernel<<<static_cast<unsigned>(a.geom.blocks > 0 ? a.geom.blocks : 1), kRowThreads, 0,
-                     st>>>(a);
+  const unsigned grid = static_cast<unsigned>(a.geom.blocks > 0 ? a.geom.blocks : 1);
+  if (l->params.agg == PACE_AGG_TOKEN_MEAN) {
+    surrogate_kernel<false><<<grid, kRowThreads, 0, st>>>(a);
+    return last_launch_status();
+  }
+  surrogate_kernel<true><<<grid, kRowThreads, 0, st>>>(a);
   PACE_TRY(last_launch_status());
-  if (a.agg == PACE_AGG_TOKEN_MEAN) return PACE_OK;
   int64_t blocks = (b->n_seq + kRowWarps - 1) / kRowWarps;
   const int64_t most = static_cast<int64_t>(sm_count()) * 8;
   if (blocks > most) blocks = most;
@@ -454,7 +458,7 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
 __global__ void __launch_bounds__(kRowThreads)
     count_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
-                      int64_t n_seq, int64_t n_rows, RowGeom geom, RowCounts counts,
+                      int64_t n_seq, int64_t n_rows, RowGeom geom, bool vec, RowCounts counts,
                       unsigned long long* __restrict__ seq_in, int* __restrict__ n_used,
                       AdvJob adv, unsigned* counter0, unsigned* counter1, int32_t* status) {
   if (static_cast<int>(blockIdx.x) >= geom.blocks) {
@@ -478,7 +482,7 @@ __global__ void __launch_bounds__(kRowThreads)
     PieceWalker pw(seq_offsets, seq_accepted, nullptr, n_seq, w0 * kRowTile);
     for (int64_t w = w0; w < w1; ++w) {
       const int64_t t0 = w * kRowTile, t1 = tile_end(t0, n_rows);
-      const unsigned bits = load_mask_bits(mask, t0, t1);
+      const unsigned bits = load_mask_bits(mask, t0, t1, vec);
       pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float, int64_t) {
         const int k = __reduce_add_sync(0xffffffffu, __popc(piece_bits(t0, lo, hi) & bits));
         if (lane == 0 && k > 0 && atomicAdd(seq_in + seq, static_cast<unsigned long long>(k)) == 0)
@@ -487,7 +491,7 @@ __global__ void __launch_bounds__(kRowThreads)
       });
     }
   } else {
-    walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1,
+    walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1, vec,
                       [&](int64_t, int64_t, unsigned in) { c += __popc(in); });
     c = __reduce_add_sync(0xffffffffu, c);
   }
@@ -510,7 +514,7 @@ __global__ void __launch_bounds__(kRowThreads)
 __global__ void __launch_bounds__(kRowThreads)
     write_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
-                      int64_t n_seq, int64_t n_rows, RowGeom geom, RowCounts counts,
+                      int64_t n_seq, int64_t n_rows, RowGeom geom, bool vec, RowCounts counts,
                       int32_t* __restrict__ rowidx, long long* __restrict__ total,
                       float* __restrict__ lp, float* __restrict__ lse) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -526,12 +530,14 @@ __global__ void __launch_bounds__(kRowThreads)
   if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1)
     *total = before + counts.block[blockIdx.x];
   before += __reduce_add_sync(0xffffffffu, wc);
-  walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1,
+  walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1, vec,
                     [&](int64_t t0, int64_t t1, unsigned in) {
+    // 32 rows at a time, lane l row l of them (held by lane l / 8 of four), so that the
+    // warp's stores are consecutive
 #pragma unroll
-    for (int u = 0; u < kRowsPerLane; ++u) {
+    for (int u = 0; u < kRowTile / 32; ++u) {
       const int64_t r = t0 + 32 * u + lane;
-      const bool k = in >> u & 1u;
+      const bool k = __shfl_sync(0xffffffffu, in, 4 * u + (lane >> 3)) >> (lane & 7) & 1u;
       const unsigned bal = __ballot_sync(0xffffffffu, k);
       if (k) {
         rowidx[before + __popc(bal & ((1u << lane) - 1u))] = static_cast<int32_t>(r);
@@ -580,7 +586,8 @@ pace_status launch_count_rows(const PaceBatch* b, RowCounts counts, unsigned lon
                               unsigned* counter1, int32_t* status, cudaStream_t st) {
   const RowGeom g = row_geom(b->n_rows);
   count_rows_kernel<<<static_cast<unsigned>(g.blocks + adv.blocks), kRowThreads, 0, st>>>(
-      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, counts, seq_in, n_used,
+      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, aligned(b->mask, 8), counts,
+      seq_in, n_used,
       adv, counter0, counter1, status);
   return last_launch_status();
 }
@@ -599,7 +606,8 @@ pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob
   PACE_TRY(launch_count_rows(b, ws.counts, nullptr, nullptr, adv, counter0, counter1, status, st));
   const RowGeom g = row_geom(b->n_rows);
   write_rows_kernel<<<static_cast<unsigned>(g.blocks), kRowThreads, 0, st>>>(
-      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, ws.counts, ws.rowidx,
+      b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, aligned(b->mask, 8),
+      ws.counts, ws.rowidx,
       ws.total, lp, lse);
   return last_launch_status();
 }

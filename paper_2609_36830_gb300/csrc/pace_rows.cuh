@@ -17,8 +17,9 @@ constexpr int kRowsPerLane = kRowTile / 32;
 constexpr int kRowThreads = 256;
 constexpr int kRowWarps = kRowThreads / 32;
 // Three blocks an SM (80 registers), one wave: the loss and its derivative over 5.4M
-// rows took 83 us (graph replay) with a tile a warp in four waves of blocks, 72 with a
-// range a warp; four blocks an SM spill (109), 512-row tiles as a range do no better.
+// rows took 83 us (graph replay) with a tile a warp in four waves of blocks and 66 with
+// a range a warp, 58 with 32-byte accesses and each tile's terms computed once whatever
+// its sequences; four blocks an SM spill (109).
 constexpr int kRowMinBlocks = 3;
 constexpr int kMaxRowBlocks = 152 * kRowMinBlocks;
 
@@ -118,15 +119,32 @@ struct PieceWalker {
   }
 };
 
-// A lane's rows of a tile: row t0 + 32 u + lane for u = 0 .. kRowsPerLane - 1.
-// The mask of them as bits (rows at or past t1: 0).
+// A lane's rows of a tile: row t0 + 8 lane + u for u = 0 .. 7, so that aligned arrays
+// are read and written as 32 bytes a lane (`vec`: every array of the launch is aligned
+// for that) and a piece of the tile is a range of each lane's rows.
+__device__ __forceinline__ int row_in_tile(int u) {
+  return kRowsPerLane * static_cast<int>(threadIdx.x & 31) + u;
+}
+
+inline bool rows_vec(const void* a, const void* b, const void* c, const uint8_t* mask) {
+  return aligned(a, 32) && aligned(b, 32) && aligned(c, 32) && aligned(mask, 8);
+}
+
+// The mask of the lane's rows as bits (rows at or past t1: 0).
 __device__ __forceinline__ unsigned load_mask_bits(const uint8_t* __restrict__ mask, int64_t t0,
-                                                   int64_t t1) {
-  const int lane = threadIdx.x & 31;
+                                                   int64_t t1, bool vec) {
+  if (vec && t1 - t0 == kRowTile) {
+    if (!mask) return 0xffu;
+    const uint2 q = *(reinterpret_cast<const uint2*>(mask + t0) + (threadIdx.x & 31));
+    uint32_t x = __vcmpne4(q.x, 0u) & 0x08040201u;  // byte k's bit k
+    x |= __vcmpne4(q.y, 0u) & 0x80402010u;          // byte k's bit 4 + k
+    x |= x >> 16;
+    return (x | x >> 8) & 0xffu;
+  }
   uint8_t m[kRowsPerLane];
 #pragma unroll
   for (int u = 0; u < kRowsPerLane; ++u) {
-    const int64_t r = t0 + 32 * u + lane;
+    const int64_t r = t0 + row_in_tile(u);
     m[u] = r < t1 ? (mask ? mask[r] : 1) : 0;
   }
   unsigned bits = 0u;
@@ -135,13 +153,49 @@ __device__ __forceinline__ unsigned load_mask_bits(const uint8_t* __restrict__ m
   return bits;
 }
 
+__device__ __forceinline__ void load_rows(const float* __restrict__ a, int64_t t0, int64_t t1,
+                                          bool vec, float (&x)[kRowsPerLane]) {
+  if (vec && t1 - t0 == kRowTile) {
+    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]),
+                   "=f"(x[6]), "=f"(x[7])
+                 : "l"(a + t0 + row_in_tile(0)));
+    return;
+  }
+#pragma unroll
+  for (int u = 0; u < kRowsPerLane; ++u) {
+    const int64_t r = t0 + row_in_tile(u);
+    x[u] = r < t1 ? a[r] : 0.0f;
+  }
+}
+
+// x of the rows whose bit is set, 0 of the tile's others.
+__device__ __forceinline__ void store_rows(float* __restrict__ a, int64_t t0, int64_t t1, bool vec,
+                                           unsigned bits, const float (&x)[kRowsPerLane]) {
+  float y[kRowsPerLane];
+#pragma unroll
+  for (int u = 0; u < kRowsPerLane; ++u) y[u] = bits >> u & 1u ? x[u] : 0.0f;
+  if (vec && t1 - t0 == kRowTile) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(a + t0 +
+                                                                                 row_in_tile(0)),
+                 "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]),
+                 "f"(y[7])
+                 : "memory");
+    return;
+  }
+#pragma unroll
+  for (int u = 0; u < kRowsPerLane; ++u) {
+    const int64_t r = t0 + row_in_tile(u);
+    if (r < t1) a[r] = y[u];
+  }
+}
+
 // The lane's rows that lie in [lo, hi) of the tile at t0, as bits.
 __device__ __forceinline__ unsigned piece_bits(int64_t t0, int64_t lo, int64_t hi) {
-  const int lane = threadIdx.x & 31;
-  const int a = static_cast<int>(lo - t0), b = static_cast<int>(hi - t0);
-  const int u0 = a > lane ? (a - lane + 31) >> 5 : 0;
-  const int u1 = b > lane ? (b - lane + 31) >> 5 : 0;
-  return (1u << u1) - (1u << u0);
+  const int first = row_in_tile(0);
+  const int a = min(max(static_cast<int>(lo - t0) - first, 0), kRowsPerLane);
+  const int b = min(max(static_cast<int>(hi - t0) - first, 0), kRowsPerLane);
+  return (1u << b) - (1u << a);
 }
 
 __device__ __forceinline__ int64_t tile_end(int64_t t0, int64_t n_rows) {
@@ -155,15 +209,15 @@ __device__ __forceinline__ void walk_rows_in_loss(const int64_t* __restrict__ of
                                                   const uint8_t* __restrict__ accepted,
                                                   const uint8_t* __restrict__ mask, int64_t n_seq,
                                                   int64_t n_rows, int64_t tile0, int64_t tile1,
-                                                  F f) {
+                                                  bool vec, F f) {
   if (tile0 >= tile1) return;
   int64_t t0 = tile0 * kRowTile;
-  unsigned bits = load_mask_bits(mask, t0, tile_end(t0, n_rows));
+  unsigned bits = load_mask_bits(mask, t0, tile_end(t0, n_rows), vec);
   PieceWalker pw(offsets, accepted, nullptr, n_seq, t0);
   for (int64_t w = tile0; w < tile1; ++w) {
     const int64_t t1 = tile_end(t0, n_rows);
     unsigned next = 0u;
-    if (w + 1 < tile1) next = load_mask_bits(mask, t1, tile_end(t1, n_rows));
+    if (w + 1 < tile1) next = load_mask_bits(mask, t1, tile_end(t1, n_rows), vec);
     unsigned in = 0u;
     pw.walk(t0, t1, [&](int64_t, int64_t lo, int64_t hi, float, int64_t) {
       in |= piece_bits(t0, lo, hi);
@@ -180,15 +234,11 @@ struct RowLoads {
   unsigned mask;
   __device__ __forceinline__ void load(const float* __restrict__ logprob,
                                        const float* __restrict__ behav,
-                                       const uint8_t* __restrict__ mask_, int64_t t0, int64_t t1) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int u = 0; u < kRowsPerLane; ++u) {
-      const int64_t r = t0 + 32 * u + lane;
-      lp[u] = r < t1 ? logprob[r] : 0.0f;
-      bh[u] = r < t1 ? behav[r] : 0.0f;
-    }
-    mask = load_mask_bits(mask_, t0, t1);
+                                       const uint8_t* __restrict__ mask_, int64_t t0, int64_t t1,
+                                       bool vec) {
+    load_rows(logprob, t0, t1, vec, lp);
+    load_rows(behav, t0, t1, vec, bh);
+    mask = load_mask_bits(mask_, t0, t1, vec);
   }
 };
 

@@ -170,3 +170,40 @@ def test_row_tiles_of_any_layout(kind, G, agg, masked):
     assert abs(float(loss.item()) - oloss) <= unit * max(np.abs(oterm).max(initial=0.0), 1e-30)
     assert (np.abs(as_np(ratio) - oratio) <= unit * oratio).all()
     assert (np.abs(as_np(dlp) - odlp) <= unit * np.abs(odlp)).all()
+
+
+@pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
+@pytest.mark.parametrize("n", [8 * 256, 10_000])
+def test_rows_at_any_alignment(agg, n):
+    """Arrays that begin off the 32-byte (masks: 8-byte) boundary are read row by row;
+    every output has the same bits as from aligned ones, and rows around are not touched."""
+    rng = np.random.default_rng(n)
+    lens = rng.multinomial(n, np.ones(16) / 16)
+    so = to_dev(np.concatenate([[0], np.cumsum(lens)]).astype(np.int64))
+    lp, behav = (torch.from_numpy(rng.standard_normal(n).astype(np.float32)) for _ in range(2))
+    mask = torch.from_numpy((rng.random(n) < 0.7).astype(np.uint8))
+    reward = to_dev(rng.random(16).astype(np.float32))
+
+    def run(shift):
+        def at(x):
+            y = torch.full((n + 16,), 9, dtype=x.dtype, device=DEV)
+            y[shift:shift + n] = x.to(DEV)
+            return y[shift:shift + n]
+        loss = torch.zeros(1, dtype=torch.float64, device=DEV)
+        ratio, dlp = (torch.full((n + 16,), 5.0, dtype=torch.float32, device=DEV)
+                      for _ in range(2))
+        la = pace.make_loss_args(at(behav), reward, 8, pace.loss_params(agg=agg), loss,
+                                 ratio_out=ratio[shift:shift + n])
+        b = pace.make_batch(so, n, mask=at(mask))
+        x = at(lp)
+        pace.surrogate_loss(b, x, la)
+        pace.surrogate_backward(b, x, la, dlp=dlp[shift:shift + n])
+        torch.cuda.synchronize()
+        for y in (ratio, dlp):
+            assert (y[:shift] == 5.0).all() and (y[shift + n:] == 5.0).all()
+        return loss, ratio[shift:shift + n], dlp[shift:shift + n]
+
+    want = run(0)
+    for shift in (1, 2, 4, 7, 8):
+        for a, b in zip(run(shift), want):
+            assert torch.equal(a, b), shift
