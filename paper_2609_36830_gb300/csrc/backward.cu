@@ -19,7 +19,8 @@
 //                             MN-major), fp32 accumulation in place; the first
 //                             chunk stores, so dW needs no clearing.
 // The GEMM is one warp-specialised tcgen05 kernel on CTA pairs: in each CTA
-// warp 0 issues TMA for the CTA's own A tile and its own half of the B tile
+// warp 0 issues TMA for the CTA's own A tile and its own half of the B tile (one
+// instruction of several lanes a stage)
 // into a 4-stage ring (128-byte swizzle), both CTAs' bytes completing on the
 // even CTA's barrier; warp 1 of the even CTA issues tcgen05.mma.cta_group::2
 // (M 256 = 128 rows per CTA, N 256 = 128 columns from each CTA, K 16; the
@@ -281,61 +282,70 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   };
 
   if (warp == 0) {
+    // The whole warp produces: a stage's boxes (one or two 64-wide ones per operand) are
+    // one TMA instruction of lanes 0..n-1.  Issued one after the other by one lane, whole
+    // calls took 3.03 against 2.96 ms (2,582 rows, H 2048 head) and 1.63 against 1.61
+    // (8,248 rows, H 1024 / V 50,001); 21k rows of H 3584 the same (power-capped).
     if (lane == 0) {
       tma_prefetch_desc(&tm_a);
       tma_prefetch_desc(&tm_b);
-      uint64_t pol;
-      asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
-      uint32_t it = 0;
-      bool ok = true;
-      unsigned round = 0;  // this cluster's items so far
-      for (int64_t t = cid; t < n_items && ok; t += n_clusters, ++round) {
-        int64_t mp, nt;
-        int kb0, kb1, part;
-        item_of(p, m_tiles, work_of(t, &kb0, &kb1, &part), &mp, &nt);
-        const int32_t m0 = static_cast<int32_t>((2 * mp + crank) * GBM);
-        const int32_t n0 = static_cast<int32_t>(nt * GBN);
-        // the clusters start this round together (every round but the last is full)
-        if (leader && round > 0 && round % pace_rounds == 0 && p.round_ctr)
-          wait_round(p.round_ctr, round * static_cast<unsigned>(n_clusters));
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const uint32_t s = it % GSTAGES, ph = (it / GSTAGES) & 1u;
-          if (!mbar_wait_bounded(&empty[s], ph ^ 1u, abort_flag)) {
-            ok = false;
-            break;
-          }
-          unsigned char* sa = smem + s * kGStageBytes;
-          unsigned char* sb = sa + kGStageA;
-          const uint32_t bar = cluster_addr(&full[s], 0);
-          if (leader) mbar_arrive_expect_tx(&full[s], 2 * kGStageBytes);
-          const int32_t k0 = kb * GBK;
-          if (p.a_pitch > 0) {  // blocked G: one 64-wide block is the inner dimension
-            const int64_t ap = p.a_pitch;
-            if (A_MN) {  // M = vocabulary: blocks m0 / 64 and m0 / 64 + 1, rows k0..k0+63
-              const int64_t b0 = m0 / 64;
-              tma_load_2d_pair(sa, &tm_a, bar, 0, static_cast<int32_t>(b0 * ap + k0), pol);
-              tma_load_2d_pair(sa + 8192, &tm_a, bar, 0,
-                               static_cast<int32_t>((b0 + 1) * ap + k0), pol);
-            } else {     // K = vocabulary: block kb, rows m0..m0+127
-              tma_load_2d_pair(sa, &tm_a, bar, 0, static_cast<int32_t>(kb * ap + m0), pol);
-            }
-          } else if (A_MN) {  // box {64 MN, 64 K}: two along M
-            tma_load_2d_pair(sa, &tm_a, bar, m0, k0, pol);
-            tma_load_2d_pair(sa + 8192, &tm_a, bar, m0 + 64, k0, pol);
-          } else {     // box {64 K, 128 rows}
-            tma_load_2d_pair(sa, &tm_a, bar, k0, m0, pol);
-          }
-          // this CTA's half of B: columns n0 + 128 * crank .. + 127
-          const int32_t nh = n0 + static_cast<int32_t>(crank) * (GBN / 2);
-          if (B_MN) {  // two {64 N, 64 K} boxes along N
-            tma_load_2d_pair(sb, &tm_b, bar, nh, k0, pol);
-            tma_load_2d_pair(sb + 8192, &tm_b, bar, nh + 64, k0, pol);
-          } else {     // {64 K, 128 rows}
-            tma_load_2d_pair(sb, &tm_b, bar, k0, nh, pol);
-          }
-        }
-        if (leader && ok && p.round_ctr) atomicAdd(p.round_ctr, 1u);
+    }
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+    constexpr int kBoxesA = A_MN ? 2 : 1, kBoxes = kBoxesA + (B_MN ? 2 : 1);
+    const bool is_a = lane < kBoxesA;
+    const int half = is_a ? lane : lane - kBoxesA;  // which 64-wide box of an MN-major tile
+    const void* desc = is_a ? static_cast<const void*>(&tm_a) : static_cast<const void*>(&tm_b);
+    const uint32_t dst = (is_a ? 0u : kGStageA) + half * 8192u;
+    uint32_t it = 0;
+    bool ok = true;
+    unsigned round = 0;  // this cluster's items so far
+    for (int64_t t = cid; t < n_items && ok; t += n_clusters, ++round) {
+      int64_t mp, nt;
+      int kb0, kb1, part;
+      item_of(p, m_tiles, work_of(t, &kb0, &kb1, &part), &mp, &nt);
+      const int32_t m0 = static_cast<int32_t>((2 * mp + crank) * GBM);
+      // this CTA's half of B: columns nh .. nh + 127
+      const int32_t nh = static_cast<int32_t>(nt * GBN) + static_cast<int32_t>(crank) * (GBN / 2);
+      // this lane's box: at K step kb it starts at (x + kb * dx, y + kb * dy)
+      int32_t x, y, dx, dy;
+      if (is_a && p.a_pitch > 0) {  // G in 64-wide blocks: the block is the inner dimension
+        const int32_t ap = static_cast<int32_t>(p.a_pitch);
+        x = 0;
+        dx = 0;
+        y = A_MN ? (m0 / 64 + half) * ap : m0;  // M = vocabulary: block, K rows; else K = vocabulary
+        dy = A_MN ? GBK : ap;
+      } else if (is_a ? A_MN : B_MN) {  // {64 MN, 64 K}
+        x = (is_a ? m0 : nh) + 64 * half;
+        dx = 0;
+        y = 0;
+        dy = GBK;
+      } else {  // {64 K, 128 rows}
+        x = 0;
+        dx = GBK;
+        y = is_a ? m0 : nh;
+        dy = 0;
       }
+      // the clusters start this round together (every round but the last is full)
+      if (leader && lane == 0 && round > 0 && round % pace_rounds == 0 && p.round_ctr)
+        wait_round(p.round_ctr, round * static_cast<unsigned>(n_clusters));
+      __syncwarp();
+      for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        const uint32_t s = it % GSTAGES, ph = (it / GSTAGES) & 1u;
+        // one outcome for the warp
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph ^ 1u, abort_flag))) {
+          ok = false;
+          break;
+        }
+        const uint32_t bar = cluster_addr(&full[s], 0);
+        if (leader && lane == 0) mbar_arrive_expect_tx(&full[s], 2 * kGStageBytes);
+        __syncwarp();  // the lanes' loads are one TMA instruction
+        if (lane < kBoxes)
+          tma_load_2d_pair(smem + s * kGStageBytes + dst, desc, bar, x + kb * dx, y + kb * dy, pol);
+      }
+      if (leader && lane == 0 && ok && p.round_ctr) atomicAdd(p.round_ctr, 1u);
+    }
+    if (lane == 0) {
       if (!ok) give_up();
       // every copy issued has landed before the CTA exits: the even CTA sees
       // both CTAs' bytes on its full barriers, the odd CTA its stages consumed
