@@ -154,7 +154,8 @@ def test_quantile_admit_sizes(capacity, filled, n_cand, batch):
 
 @pytest.mark.parametrize("lo,hi,n_bins", [(0.0, 32.0, 1000), (0.1, 0.7, 77), (-3.0, 1e-3, 4096),
                                           (0.0, 5e-324, 3), (-1e308, 1.5e308, 10),
-                                          (1e-310, 1e-308, 50), (0.3, np.nextafter(0.3, 1), 2)])
+                                          (1e-310, 1e-308, 50), (0.3, np.nextafter(0.3, 1), 2),
+                                          (0.0, 10.0, 10), (0.0, 1e-280, 7), (0.0, 3e290, 9)])
 def test_histogram_at_bin_edges(lo, hi, n_bins):
     """Values at every bin edge and a few ulps around it, on ranges up to the smallest and
     largest that doubles hold, where a shorter computation of the bin could go astray;
