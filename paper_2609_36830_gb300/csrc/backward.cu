@@ -670,25 +670,24 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
     const int64_t t1 = tile_end(t0, p.n_rows);
     if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
     unsigned in = 0u;
-    float adv[kRowsPerLane];  // per row; derivatives once per tile, not per piece
+    float adv[kRowsPerLane] = {};  // per row; derivatives once per tile, not per piece
     auto derive = [&](unsigned rows) {
       const float s_hi = static_cast<float>(scale);
       const float s_lo = static_cast<float>(scale - static_cast<double>(s_hi));
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) {
-        if (rows >> u & 1u) {
-          const float a = adv[u];
-          const float d = cur.lp[u] - cur.bh[u];
-          const float dc = fminf(fmaxf(d, -20.0f), 20.0f);
-          const float rho = expf(dc);
-          const float rc = fminf(fmaxf(rho, 1.0f - p.eps_low), 1.0f + p.eps_high);
-          const float p1 = -a * rho, p2 = -a * rc;
-          const float lm = fmaxf(p1, p2);
-          float x = 0.0f;
-          if (d > -20.0f && d < 20.0f && p1 >= p2) x = -a * rho;
-          if (a < 0.0f && -p.dual * a < lm) x = 0.0f;
-          cur.lp[u] = fmaf(x, s_hi, x * s_lo);  // the derivative, once the row is used
-        }
+        if (kSeqMean && !(rows >> u & 1u)) continue;
+        const float a = adv[u];
+        const float d = cur.lp[u] - cur.bh[u];
+        const float dc = fminf(fmaxf(d, -20.0f), 20.0f);
+        const float rho = expf(dc);
+        const float rc = fminf(fmaxf(rho, 1.0f - p.eps_low), 1.0f + p.eps_high);
+        const float p1 = -a * rho, p2 = -a * rc;
+        const float lm = fmaxf(p1, p2);
+        float x = 0.0f;
+        if (d > -20.0f && d < 20.0f && p1 >= p2) x = -a * rho;
+        if (a < 0.0f && -p.dual * a < lm) x = 0.0f;
+        cur.lp[u] = fmaf(x, s_hi, x * s_lo);  // the derivative, once the row is used
       }
     };
     pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t) {
@@ -701,7 +700,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
         derive(rows);
       }
     });
-    if (!kSeqMean) derive(in);
+    if (!kSeqMean && __any_sync(0xffffffffu, in != 0u)) derive(in);
     store_rows(p.dlp, t0, t1, p.vec, in, cur.lp);
     cur = nxt;
     t0 = t1;

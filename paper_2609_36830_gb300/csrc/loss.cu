@@ -288,19 +288,20 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
       const int64_t t1 = tile_end(t0, p.n_rows);
       if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
       unsigned in = 0u;
-      float adv[kRowsPerLane];  // per row; the terms are computed once per tile, not per piece
-      // the terms of the given rows, added up
+      float adv[kRowsPerLane] = {};  // per row; the terms are computed once per tile, not per piece
+      // the terms of the given rows, added up: every row's is computed, without a branch,
+      // so that the eight rows' chains of latencies overlap
       auto terms = [&](unsigned rows) -> double {
         Sum3 sum{0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int u = 0; u < kRowsPerLane; ++u) {
-          if (rows >> u & 1u) {
-            float rho;
-            const float x = clipped_term(cur.lp[u], cur.bh[u], adv[u], p.eps_low, p.eps_high,
-                                         p.dual, &rho);
-            cur.bh[u] = rho;  // the ratio, once the row is used
-            sum.add(x);
-          }
+          const bool take = rows >> u & 1u;
+          if (kSeqMean && !take) continue;
+          float rho;
+          const float x = clipped_term(cur.lp[u], cur.bh[u], adv[u], p.eps_low, p.eps_high,
+                                       p.dual, &rho);
+          cur.bh[u] = rho;  // the ratio, once the row is used
+          sum.add(take ? x : 0.0f);
         }
         return sum.value();
       };
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
           p.ws.head_sum[w] = head_s;
           p.ws.head_cnt[w] = head_c;
         }
-      } else {
+      } else if (__any_sync(0xffffffffu, in != 0u)) {
         tot = __dadd_rn(tot, terms(in));
         cnt += __popc(in);
       }
