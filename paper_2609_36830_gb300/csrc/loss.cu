@@ -508,6 +508,29 @@ __global__ void __launch_bounds__(kRowThreads)
   }
 }
 
+// A tile's rows in the loss (the lanes' bits) into the list from entry `before` on; lp
+// and lse (or null) of its other rows are set to 0.
+__device__ __forceinline__ void list_tile(int64_t t0, int64_t t1, unsigned in, long long& before,
+                                          int32_t* __restrict__ rowidx, float* __restrict__ lp,
+                                          float* __restrict__ lse) {
+  const int lane = threadIdx.x & 31;
+  // 32 rows at a time, lane l row l of them (held by lane l / 8 of four), so that the
+  // warp's stores are consecutive
+#pragma unroll
+  for (int u = 0; u < kRowTile / 32; ++u) {
+    const int64_t r = t0 + 32 * u + lane;
+    const bool k = __shfl_sync(0xffffffffu, in, 4 * u + (lane >> 3)) >> (lane & 7) & 1u;
+    const unsigned bal = __ballot_sync(0xffffffffu, k);
+    if (k) {
+      rowidx[before + __popc(bal & ((1u << lane) - 1u))] = static_cast<int32_t>(r);
+    } else if (r < t1) {
+      if (lp) lp[r] = 0.0f;
+      if (lse) lse[r] = 0.0f;
+    }
+    before += __popc(bal);
+  }
+}
+
 // The row indices of the rows in the loss, in row order; their number in *total.
 // Every block adds up the counts of the blocks before it itself (at most
 // kMaxRowBlocks of them), so there is no launch for a scan.  lp and lse (or null) of
@@ -533,22 +556,62 @@ __global__ void __launch_bounds__(kRowThreads)
   before += __reduce_add_sync(0xffffffffu, wc);
   walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1, vec,
                     [&](int64_t t0, int64_t t1, unsigned in) {
-    // 32 rows at a time, lane l row l of them (held by lane l / 8 of four), so that the
-    // warp's stores are consecutive
-#pragma unroll
-    for (int u = 0; u < kRowTile / 32; ++u) {
-      const int64_t r = t0 + 32 * u + lane;
-      const bool k = __shfl_sync(0xffffffffu, in, 4 * u + (lane >> 3)) >> (lane & 7) & 1u;
-      const unsigned bal = __ballot_sync(0xffffffffu, k);
-      if (k) {
-        rowidx[before + __popc(bal & ((1u << lane) - 1u))] = static_cast<int32_t>(r);
-      } else if (r < t1) {
-        if (lp) lp[r] = 0.0f;
-        if (lse) lse[r] = 0.0f;
-      }
-      before += __popc(bal);
-    }
-  });
+                      list_tile(t0, t1, in, before, rowidx, lp, lse);
+                    });
+}
+
+// Up to kFewRows rows: the count and the list in one launch, whose blocks (32 tiles each,
+// one a warp) count the tiles before theirs again.  Bound by latency and the launch: a
+// log-prob call (H 64, V 64, one graph replay of ten) took 30 us in two launches and 25
+// in one at 200 rows, 38 and 34 at 4,096, 39 and 37 at 10,000, 39.6 and 39.6 at 16,384,
+// 39.7 and 41.7 at 24,576, where the line could lie no higher.
+constexpr int kFewThreads = 1024;
+constexpr int kFewWarps = kFewThreads / 32;
+constexpr int64_t kFewRows = 2 * kFewWarps * kRowTile;
+
+__global__ void __launch_bounds__(kFewThreads)
+    list_few_rows_kernel(const int64_t* __restrict__ seq_offsets,
+                         const uint8_t* __restrict__ seq_accepted,
+                         const uint8_t* __restrict__ mask, int64_t n_seq, int64_t n_rows,
+                         int blocks, bool vec, int32_t* __restrict__ rowidx,
+                         long long* __restrict__ total, float* __restrict__ lp,
+                         float* __restrict__ lse, AdvJob adv, unsigned* counter0,
+                         unsigned* counter1, int32_t* status) {
+  if (static_cast<int>(blockIdx.x) >= blocks) {
+    adv_block(adv, blockIdx.x - blocks);
+    return;
+  }
+  __shared__ int sh_before[kFewWarps], sh_own[kFewWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * kFewThreads + threadIdx.x;
+  if (t == 0) {
+    if (counter0) *counter0 = 0u;
+    if (counter1) *counter1 = 0u;
+  }
+  for (int64_t i = t; i < n_seq; i += static_cast<int64_t>(blocks) * kFewThreads)
+    check_seq(seq_offsets, i, n_rows, status);
+  // block b's 32 warps share the 32 b tiles before its own, b each
+  const int64_t b = blockIdx.x, n_tiles = (n_rows + kRowTile - 1) / kRowTile;
+  int c = 0;
+  walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, wid * b, (wid + 1) * b, vec,
+                    [&](int64_t, int64_t, unsigned in) { c += __popc(in); });
+  const int64_t w = b * kFewWarps + wid;
+  unsigned own = 0u;
+  walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w, w < n_tiles ? w + 1 : w,
+                    vec, [&](int64_t, int64_t, unsigned in) { own = in; });
+  c = __reduce_add_sync(0xffffffffu, c);
+  const int n_own = __reduce_add_sync(0xffffffffu, __popc(own));
+  if (lane == 0) {
+    sh_before[wid] = c;
+    sh_own[wid] = n_own;
+  }
+  __syncthreads();
+  long long before = __reduce_add_sync(0xffffffffu, sh_before[lane] + (lane < wid ? sh_own[lane] : 0));
+  if (b == blocks - 1 && wid == kFewWarps - 1 && lane == 0) *total = before + n_own;
+  if (w < n_tiles) {
+    const int64_t t0 = w * kRowTile;
+    list_tile(t0, tile_end(t0, n_rows), own, before, rowidx, lp, lse);
+  }
 }
 
 // Copy the hidden rows listed in rowidx into a dense buffer, one warp per row,
@@ -603,6 +666,14 @@ pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob
     if (lse && bytes) PACE_TRY_CUDA(cudaMemsetAsync(lse, 0, bytes, st));
     if (counter1) PACE_TRY_CUDA(cudaMemsetAsync(counter1, 0, sizeof(unsigned), st));
     return launch_group_adv(adv, b, counter0, status, st);
+  }
+  if (b->n_rows <= kFewRows) {
+    const int blocks = static_cast<int>((b->n_rows + kFewWarps * kRowTile - 1) /
+                                        (kFewWarps * kRowTile));
+    list_few_rows_kernel<<<static_cast<unsigned>(blocks + adv.blocks), kFewThreads, 0, st>>>(
+        b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, blocks,
+        aligned(b->mask, 8), ws.rowidx, ws.total, lp, lse, adv, counter0, counter1, status);
+    return last_launch_status();
   }
   PACE_TRY(launch_count_rows(b, ws.counts, nullptr, nullptr, adv, counter0, counter1, status, st));
   const RowGeom g = row_geom(b->n_rows);

@@ -363,27 +363,33 @@ def test_concurrent_launches_on_two_streams():
         np.testing.assert_array_equal(as_np(lp), r)
 
 
-def test_row_list_of_several_tiles_a_warp():
-    """A million rows (more than one 256-row tile a warp of the row walk), masked at
-    random and in runs, over sequences of many lengths: every row in the loss gets its
-    own log-prob and the others 0.  Bound: 32-bit sums of 64 products (|z| < 12)."""
-    H, V, n = 64, 96, 1_000_003
+@pytest.mark.parametrize("n,shift", [(1_000_003, 0), (1, 0), (255, 1), (8192, 0), (8193, 3),
+                                     (16_383, 0), (16_384, 1), (16_385, 0)])
+def test_row_lists(n, shift):
+    """Row counts around one block, the one-launch list and more than one 256-row tile a
+    warp of the row walk, masked (at any alignment) at random and in runs, over sequences
+    of many lengths: every row in the loss gets its own log-prob and the others 0.
+    Bound: 32-bit sums of 64 products (|z| < 12)."""
+    H, V = 64, 96
     g = torch.Generator(device=DEV)
     g.manual_seed(9)
     h = torch.randn(n, H, device=DEV, generator=g).to(torch.bfloat16)
     w = (torch.randn(V, H, device=DEV, generator=g) / 4).to(torch.bfloat16)
     y = torch.randint(0, V, (n,), device=DEV, generator=g, dtype=torch.int32)
     rng = np.random.default_rng(2)
-    cuts = np.sort(rng.choice(n, size=3000, replace=False))
+    cuts = np.sort(rng.choice(n, size=min(3000, n // 4), replace=False))
     so = to_dev(np.concatenate([[0], cuts, [n]]).astype(np.int64))
-    acc = to_dev((rng.random(3001) < 0.8).astype(np.uint8))
-    mask = torch.rand(n, device=DEV, generator=g) < 0.9
-    mask[400_000:600_000] = True
-    lp, _ = _run(h, w, y, seq_offsets=so, seq_accepted=acc, mask=mask.to(torch.uint8))
+    acc = to_dev((rng.random(cuts.size + 1) < 0.8).astype(np.uint8))
+    mask = torch.rand(n + shift, device=DEV, generator=g) < 0.9
+    mask = mask[shift:]
+    mask[n * 2 // 5:n * 3 // 5] = True
+    bytes_ = torch.zeros(n + shift, dtype=torch.uint8, device=DEV)
+    bytes_[shift:] = mask
+    lp, _ = _run(h, w, y, seq_offsets=so, seq_accepted=acc, mask=bytes_[shift:])
     sel = mask & (torch.repeat_interleave(acc, torch.diff(so)) == 1)
     z = h.float() @ w.float().T
     ref = as_np(z.gather(1, y.long()[:, None])[:, 0] - torch.logsumexp(z, 1))
     sel = as_np(sel)
     tol = 4 * 12 * 64 * 2.0 ** -24
-    assert np.abs(lp - ref)[sel].max() <= tol
+    assert np.abs(lp - ref)[sel].max(initial=0.0) <= tol
     assert (lp[~sel] == 0).all()
