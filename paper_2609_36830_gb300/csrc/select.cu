@@ -5,7 +5,7 @@
 // Order: score descending, then unit id ascending.  The k first units in that
 // order are rejected; outputs list trajectory ids ascending.
 //
-//   small pools (U <= 288): one block ranks every unit against every other
+//   small pools (U <= 256): one block ranks every unit against every other
 //     unit in shared memory and compacts the ids (one launch).
 //   mid-size pools (U <= 131,072): one cluster of up to 8 CTAs holds every key
 //     in shared memory (16,384 per CTA), finds the pivot by a radix select that
@@ -37,10 +37,10 @@ namespace {
 namespace cg = cooperative_groups;
 
 // Ranking takes U^2 comparisons on one SM, the radix select a nearly constant time: per
-// call (graph of 20) 128 units 3.7 against 7.2 us, 256 units 6.5 / 8.2, 320 units 9.1 /
-// 8.3, 512 units 15.8 / 8.7.
-constexpr int kSmallMax = 288;
-constexpr int kSmallThreads = 288;
+// call (graph of 20) 128 units 3.7 against 6.3 us, 256 units 6.7 / 6.9, 288 units 8.6 /
+// 7.1, 512 units 15.8 / 7.3.
+constexpr int kSmallMax = 256;
+constexpr int kSmallThreads = 256;
 // Pools up to this size take one CTA whatever their outputs and stay within the shared
 // memory that needs no attribute, so their first call may be inside a stream capture.
 constexpr int kOneCtaMax = 512;
@@ -216,23 +216,27 @@ __global__ void __launch_bounds__(kSmallThreads)
 // shared memory instead (the kMulti = false instance).
 constexpr int kSelCtaUnits = 16384;  // units per CTA at most
 constexpr int kSelThreads = 1024;
-constexpr int kSelPer = kSelCtaUnits / kSelThreads;  // units per thread at most
 constexpr int kSelMaxCluster = 8;
 constexpr int64_t kSelMaxUnits = int64_t(kSelCtaUnits) * kSelMaxCluster;
-constexpr int kSelRow = kSelThreads + 1;  // keys per slot row (one pad key)
-static_assert(kSelPer * kSelThreads == kSelCtaUnits, "whole units per thread");
+// One CTA with few units runs 512 threads: its steps are short chains between barriers,
+// which half as many warps pass sooner.  Per call (graph replay), 1,024 and 512 threads:
+// 320 units 8.2 and 6.9 us, 1,024 9.7 and 8.4, 2,048 11.2 and 9.8, 4,096 14.1 and 13.2,
+// 6,000 and 8,192 the same.
+constexpr int kSelFewThreads = 512;
+constexpr int kSelFewUnits = 4096;
 static_assert(kSelCtaUnits <= 65536, "a CTA's unit numbers are stored in 16 bits");
 
 // log2 of the units per thread: the smallest power of two that covers b units.
-__host__ __device__ inline int sel_per_log2(int b) {
+__host__ __device__ inline int sel_per_log2(int b, int threads) {
   int lg = 0;
-  while ((kSelThreads << lg) < b) ++lg;
+  while ((threads << lg) < b) ++lg;
   return lg;
 }
 
-// Dynamic shared memory of a CTA holding b units: keys, unit order, rejected bytes.
-__host__ __device__ inline size_t sel_smem_bytes(int b) {
-  return static_cast<size_t>(1 << sel_per_log2(b)) * kSelRow * sizeof(uint64_t) +
+// Dynamic shared memory of a CTA holding b units: keys (a row of `threads` and a pad key
+// per slot), unit order, rejected bytes.
+__host__ __device__ inline size_t sel_smem_bytes(int b, int threads) {
+  return static_cast<size_t>(1 << sel_per_log2(b, threads)) * (threads + 1) * sizeof(uint64_t) +
          static_cast<size_t>(b) * (sizeof(uint16_t) + 1);
 }
 
@@ -249,9 +253,10 @@ __device__ __forceinline__ void cta_min_max_to_slot(uint64_t lo, uint64_t hi, ui
     s_whi[wid] = hi;
   }
   __syncthreads();
-  if (wid == 0) {  // one warp folds the 32 warp results into this CTA's slot
-    lo = warp_min_u64(s_wlo[lane]);
-    hi = warp_max_u64(s_whi[lane]);
+  if (wid == 0) {  // one warp folds the warps' results into this CTA's slot
+    const bool have = lane < static_cast<int>(blockDim.x >> 5);
+    lo = warp_min_u64(have ? s_wlo[lane] : ~0ull);
+    hi = warp_max_u64(have ? s_whi[lane] : 0ull);
     if (lane == 0) {
       s_mm[0] = lo;
       s_mm[1] = hi;
@@ -337,14 +342,14 @@ __device__ __forceinline__ void finish_list(cg::cluster_group& cluster, uint64_t
 
 // kMulti = false: a cluster of one CTA, with block barriers and plain shared
 // memory in place of cluster barriers and distributed shared memory.
-template <bool kMulti>
-__global__ void __launch_bounds__(kSelThreads, 1)
+template <bool kMulti, int kT>
+__global__ void __launch_bounds__(kT, 1)
     select_cluster_kernel(const double* __restrict__ score, int n_units, int G, long long k,
                           int32_t* accepted_ids, int32_t* rejected_ids, uint8_t* flags,
                           int32_t* status, int vec4) {
   extern __shared__ __align__(16) unsigned char sel_smem[];
   __shared__ unsigned hist[kHistBins];
-  __shared__ uint64_t s_wlo[kSelThreads / 32], s_whi[kSelThreads / 32];
+  __shared__ uint64_t s_wlo[kT / 32], s_whi[kT / 32];
   __shared__ uint64_t s_mm[2], s_g[2];
   __shared__ long long s_cnt[2];  // this CTA's keys equal to / above the pivot (peers read)
   __shared__ long long s_off[2];  // ties and rejections in lower-ranked CTAs
@@ -359,26 +364,26 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   const int B = (n_units + nc - 1) / nc;
   const int base = rank * B;                        // first unit of this CTA
   const int nb = max(0, min(B, n_units - base));    // units of this CTA
-  const int lg = sel_per_log2(B);
+  const int lg = sel_per_log2(B, kT);
   const int per = 1 << lg;
   uint64_t* keys = reinterpret_cast<uint64_t*>(sel_smem);
-  uint16_t* order = reinterpret_cast<uint16_t*>(sel_smem + static_cast<size_t>(per) * kSelRow *
+  uint16_t* order = reinterpret_cast<uint16_t*>(sel_smem + static_cast<size_t>(per) * (kT + 1) *
                                                                sizeof(uint64_t));
   uint8_t* rej_u = reinterpret_cast<uint8_t*>(order + B);
   const int u0 = t * per;
   const int n_mine = max(0, min(per, nb - u0));
 
-  // coalesced loads: unit v (read by thread v % 1024) belongs to thread v / per,
+  // coalesced loads: unit v (read by thread v % kT) belongs to thread v / per,
   // slot v % per; the padded rows make this scatter at most two-way conflicted
-  for (int v = t; v < nb; v += kSelThreads) {
+  for (int v = t; v < nb; v += kT) {
     const double x = score[base + v];
     if (isnan(x)) report(status, PACE_ERR_NAN_INPUT);
-    keys[(v & (per - 1)) * kSelRow + (v >> lg)] = order_key(x);
+    keys[(v & (per - 1)) * (kT + 1) + (v >> lg)] = order_key(x);
   }
   __syncthreads();
   uint64_t lo = ~0ull, hi = 0ull;
   for (int i = 0; i < n_mine; ++i) {
-    const uint64_t key = keys[i * kSelRow + t];
+    const uint64_t key = keys[i * (kT + 1) + t];
     lo = key < lo ? key : lo;
     hi = key > hi ? key : hi;
   }
@@ -407,58 +412,57 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     const int nbins = 1 << (d - shift + 1);
     mask = d == 63 ? 0ull : (~0ull << (d + 1));
     prefix = lo & mask;
-    for (int b = t; b < nbins; b += kSelThreads) hist[b] = 0u;
+    for (int b = t; b < nbins; b += kT) hist[b] = 0u;
     if (t == 0) {
       s_digit = -1;
       s_n_list = 0;
     }
     __syncthreads();
     for (int i = 0; i < n_mine; ++i) {
-      const uint64_t key = keys[i * kSelRow + t];
+      const uint64_t key = keys[i * (kT + 1) + t];
       if ((key & mask) == prefix)
         atomicAdd(&hist[static_cast<unsigned>(key >> shift) & (nbins - 1)], 1u);
     }
     if (kMulti) cluster.sync();  // every CTA's histogram is complete
     else __syncthreads();
-    // thread t owns digits nbins-1-2t and nbins-2-2t, summed over the cluster: an
+    // thread t owns the kOwn digits from nbins-1-kOwn t down, summed over the cluster: an
     // exclusive scan in thread order counts the candidates with larger digits
     // (the loads of all peers are issued together: a fixed-bound loop the
     // compiler unrolls, one distributed-shared-memory round trip per round)
-    const int top = nbins - 1 - 2 * t;
-    long long h0 = 0, h1 = 0;
+    constexpr int kOwn = kHistBins / kT;
+    const int top = nbins - 1 - kOwn * t;
+    unsigned own[kOwn] = {};
     if (kMulti) {
-      unsigned c0[kSelMaxCluster], c1[kSelMaxCluster];
+      unsigned c[kSelMaxCluster][kOwn];
 #pragma unroll
       for (int r = 0; r < kSelMaxCluster; ++r) {
-        c0[r] = 0u;
-        c1[r] = 0u;
-        if (r < nc) {
-          const unsigned* ph = cluster.map_shared_rank(hist, static_cast<unsigned>(r));
-          if (top >= 0) c0[r] = ph[top];
-          if (top >= 1) c1[r] = ph[top - 1];
-        }
+        const unsigned* ph =
+            r < nc ? cluster.map_shared_rank(hist, static_cast<unsigned>(r)) : nullptr;
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i) c[r][i] = ph && top >= i ? ph[top - i] : 0u;
       }
 #pragma unroll
-      for (int r = 0; r < kSelMaxCluster; ++r) {
-        h0 += c0[r];
-        h1 += c1[r];
-      }
+      for (int r = 0; r < kSelMaxCluster; ++r)
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i) own[i] += c[r][i];
     } else {
-      if (top >= 0) h0 = hist[top];
-      if (top >= 1) h1 = hist[top - 1];
+#pragma unroll
+      for (int i = 0; i < kOwn; ++i)
+        if (top >= i) own[i] = hist[top - i];
     }
     // every count fits 32 bits (at most kSelMaxUnits keys in the cluster)
-    long long run = block_exclusive_scan<unsigned>(static_cast<unsigned>(h0 + h1), nullptr);
-    if (top >= 0 && run < k_rem && k_rem <= run + h0) {
-      s_digit = top;
-      s_left = k_rem - run;
-      s_here = static_cast<int>(h0);
-    }
-    run += h0;
-    if (top >= 1 && run < k_rem && k_rem <= run + h1) {
-      s_digit = top - 1;
-      s_left = k_rem - run;
-      s_here = static_cast<int>(h1);
+    unsigned sum = 0u;
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) sum += own[i];
+    long long run = block_exclusive_scan<unsigned>(sum, nullptr);
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) {
+      if (top >= i && run < k_rem && k_rem <= run + own[i]) {
+        s_digit = top - i;
+        s_left = k_rem - run;
+        s_here = static_cast<int>(own[i]);
+      }
+      run += own[i];
     }
     __syncthreads();  // s_digit and s_left are set
     if (s_digit < 0) {  // the same in every CTA: the histograms summed are the same
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     k_rem = s_left;
     if (s_here <= kSelList) {  // the same in every CTA
       for (int i = 0; i < n_mine; ++i) {
-        const uint64_t key = keys[i * kSelRow + t];
+        const uint64_t key = keys[i * (kT + 1) + t];
         if ((key & mask) == prefix) s_list[atomicAdd(&s_n_list, 1)] = key;
       }
       if (kMulti) cluster.sync();  // every CTA's list is complete
@@ -484,7 +488,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     lo = ~0ull;
     hi = 0ull;
     for (int i = 0; i < n_mine; ++i) {
-      const uint64_t key = keys[i * kSelRow + t];
+      const uint64_t key = keys[i * (kT + 1) + t];
       if ((key & mask) == prefix) {
         lo = key < lo ? key : lo;
         hi = key > hi ? key : hi;
@@ -502,7 +506,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   // carries into the other
   unsigned eqgt = 0u;
   for (int i = 0; i < n_mine; ++i) {
-    const uint64_t key = keys[i * kSelRow + t];
+    const uint64_t key = keys[i * (kT + 1) + t];
     eqgt += (key == pivot ? 0x10000u : 0u) + (key > pivot ? 1u : 0u);
   }
   unsigned cta_eqgt = 0u;
@@ -546,7 +550,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   int nrej = 0;
   long long tie = tie0;
   for (int i = 0; i < n_mine; ++i) {
-    const uint64_t key = keys[i * kSelRow + t];
+    const uint64_t key = keys[i * (kT + 1) + t];
     nrej += key > pivot || (key == pivot && (tie++) < k_rem);
   }
   unsigned cta_rej32 = 0u;
@@ -555,7 +559,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   const long long n_acc_cta = nb - cta_rej;
   tie = tie0;
   for (int i = 0; i < n_mine; ++i) {
-    const uint64_t key = keys[i * kSelRow + t];
+    const uint64_t key = keys[i * (kT + 1) + t];
     const bool r = key > pivot || (key == pivot && (tie++) < k_rem);
     const int u = u0 + i;
     order[r ? n_acc_cta + lrpos : u - lrpos] = static_cast<uint16_t>(u);
@@ -567,7 +571,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   // this CTA's runs: accepted ids from position (base - rej_off) * G, rejected
   // ids from rej_off * G, flags from base * G.  Local position p of the CTA's
   // [accepted | rejected] list holds trajectory (base + order[p / G]) * G + p % G;
-  // (q, r) = (p / G, p % G) is advanced by 1024 per step without dividing.
+  // (q, r) = (p / G, p % G) is advanced by kT per step without dividing.
   const int64_t n_out = static_cast<int64_t>(nb) * G;
   const int64_t acc_end = n_acc_cta * G;
   int32_t* acc_run = accepted_ids + (static_cast<int64_t>(base) - rej_off) * G;
@@ -582,9 +586,9 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     const int64_t acc_end4 = n_acc_cta * G4;
     int4* acc4 = reinterpret_cast<int4*>(acc_run);
     int4* rej4 = reinterpret_cast<int4*>(rej_run);
-    const int sq4 = kSelThreads / G4, sr4 = kSelThreads % G4;
+    const int sq4 = kT / G4, sr4 = kT % G4;
     int q = t / G4, r = t % G4;
-    for (int64_t p = t; p < n_out4; p += kSelThreads) {
+    for (int64_t p = t; p < n_out4; p += kT) {
       const int32_t id = (base + static_cast<int32_t>(order[q])) * G + 4 * r;
       const int4 v = make_int4(id, id + 1, id + 2, id + 3);
       if (p < acc_end4) acc4[p] = v;
@@ -600,7 +604,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
       uint32_t* f4 = reinterpret_cast<uint32_t*>(flags + static_cast<int64_t>(base) * G);
       q = t / G4;
       r = t % G4;
-      for (int64_t p = t; p < n_out4; p += kSelThreads) {
+      for (int64_t p = t; p < n_out4; p += kT) {
         f4[p] = rej_u[q] ? 0u : 0x01010101u;
         q += sq4;
         r += sr4;
@@ -612,9 +616,9 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     }
     return;
   }
-  const int sq = kSelThreads / G, sr = kSelThreads % G;
+  const int sq = kT / G, sr = kT % G;
   int q = t / G, r = t % G;
-  for (int64_t p = t; p < n_out; p += kSelThreads) {
+  for (int64_t p = t; p < n_out; p += kT) {
     const int32_t id = (base + static_cast<int32_t>(order[q])) * G + r;
     if (p < acc_end) acc_run[p] = id;
     else if (rej_run) rej_run[p - acc_end] = id;
@@ -629,7 +633,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     uint8_t* f_run = flags + static_cast<int64_t>(base) * G;
     q = t / G;
     r = t % G;
-    for (int64_t p = t; p < n_out; p += kSelThreads) {
+    for (int64_t p = t; p < n_out; p += kT) {
       f_run[p] = rej_u[q] ? 0 : 1;
       q += sq;
       r += sr;
@@ -843,13 +847,16 @@ pace_status sel_cluster_limit(int* out) {
   if (dev < 0 || dev >= kMaxDevices) return PACE_ERR_CUDA;
   std::lock_guard<std::mutex> g(mu);
   if (limit[dev] == 0) {
-    const size_t smem = sel_smem_bytes(kSelCtaUnits);
-    PACE_TRY_CUDA(cudaFuncSetAttribute(select_cluster_kernel<true>,
+    const size_t smem = sel_smem_bytes(kSelCtaUnits, kSelThreads);
+    PACE_TRY_CUDA(cudaFuncSetAttribute(select_cluster_kernel<true, kSelThreads>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
-    PACE_TRY_CUDA(cudaFuncSetAttribute(select_cluster_kernel<false>,
+    PACE_TRY_CUDA(cudaFuncSetAttribute(select_cluster_kernel<false, kSelThreads>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
+    PACE_TRY_CUDA(cudaFuncSetAttribute(
+        select_cluster_kernel<false, kSelFewThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        static_cast<int>(sel_smem_bytes(kSelFewUnits, kSelFewThreads))));
     int c = kSelMaxCluster;
     for (; c > 1; c /= 2) {
       cudaLaunchConfig_t cfg = {};
@@ -864,7 +871,8 @@ pace_status sel_cluster_limit(int* out) {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, select_cluster_kernel<true>, &cfg) == cudaSuccess &&
+      if (cudaOccupancyMaxActiveClusters(&n, select_cluster_kernel<true, kSelThreads>, &cfg) ==
+              cudaSuccess &&
           n >= 1)
         break;
       (void)cudaGetLastError();  // a refused size is not an error of this call
@@ -896,8 +904,10 @@ pace_status launch_select_cluster(const double* unit_score, int n_units, int G, 
                                   uint8_t* flags, int32_t* status, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(c), 1, 1);
-  cfg.blockDim = dim3(kSelThreads, 1, 1);
-  cfg.dynamicSmemBytes = sel_smem_bytes((n_units + c - 1) / c);
+  const bool few = c == 1 && n_units <= kSelFewUnits;
+  const int threads = few ? kSelFewThreads : kSelThreads;
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+  cfg.dynamicSmemBytes = sel_smem_bytes((n_units + c - 1) / c, threads);
   cfg.stream = st;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeClusterDimension;
@@ -908,13 +918,11 @@ pace_status launch_select_cluster(const double* unit_score, int n_units, int G, 
   cfg.numAttrs = 1;
   const int vec4 = G % 4 == 0 && aligned(accepted_ids, 16) &&
                    (!rejected_ids || aligned(rejected_ids, 16)) && (!flags || aligned(flags, 4));
-  if (c > 1) {
-    PACE_TRY_CUDA(cudaLaunchKernelEx(&cfg, select_cluster_kernel<true>, unit_score, n_units, G,
-                                     k, accepted_ids, rejected_ids, flags, status, vec4));
-  } else {
-    PACE_TRY_CUDA(cudaLaunchKernelEx(&cfg, select_cluster_kernel<false>, unit_score, n_units, G,
-                                     k, accepted_ids, rejected_ids, flags, status, vec4));
-  }
+  const auto kernel = few     ? select_cluster_kernel<false, kSelFewThreads>
+                      : c > 1 ? select_cluster_kernel<true, kSelThreads>
+                              : select_cluster_kernel<false, kSelThreads>;
+  PACE_TRY_CUDA(cudaLaunchKernelEx(&cfg, kernel, unit_score, n_units, G, k, accepted_ids,
+                                   rejected_ids, flags, status, vec4));
   return last_launch_status();
 }
 

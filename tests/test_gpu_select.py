@@ -255,7 +255,7 @@ def test_candidate_list_sizes(U, m, dist):
         _check_k(s, 8, k)
 
 
-@pytest.mark.parametrize("U", [31, 32, 33, 287, 288, 289, 511, 512, 513])
+@pytest.mark.parametrize("U", [31, 32, 33, 255, 256, 257, 288, 289, 511, 512, 513])
 @pytest.mark.parametrize("G", [1, 3, 8, 100])
 def test_small_pools_around_the_rank_kernel(U, G):
     """Pools around the largest that are ranked all against all and the largest that take
