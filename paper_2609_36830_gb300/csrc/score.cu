@@ -7,10 +7,11 @@
 //                       tag (+1, for the Lemma 1 premise check).
 //                       On pools of 8k trajectories and more the same launch
 //                       also prepares the prefix-score window (extra blocks
-//                       after the streaming ones, run in its tail): one sorts W,
-//                       the others tabulate F = phi(count / |W|) (Eqs. 9-10)
-//                       for every possible count 0..|W| (F depends on s only
-//                       through the count).
+//                       after the streaming ones, run in its tail): each puts a
+//                       part of W in its sorted places and tabulates a part
+//                       of F = phi(count / |W|) (Eqs. 9-10) for every
+//                       possible count 0..|W| (F depends on s only through
+//                       the count).
 //   score_finalize_kernel  one thread per trajectory: K_gen, K_wait, the ECDF
 //                       count of s against the window (binary search in the
 //                       sorted window, or a direct count on small pools), F
@@ -393,13 +394,17 @@ __device__ __forceinline__ double sharpen(double q, int gamma) {
 // The prefix-score window's preparation, done by extra blocks of the tag
 // reduction's launch (the blocks after its streaming blocks): they are
 // scheduled as the streaming blocks retire, so the preparation runs in the
-// reduction's ragged tail instead of as a launch of its own.  Prep block 0
-// sorts the window ascending (bitonic, in dynamic shared memory, padded to a
-// power of two with +inf, which sorts last and is never read back); the other
-// prep blocks tabulate F[c] = phi_gamma(c / n) for c = 0..n, kFPerBlock entries
-// each, so the table's fp64 divisions and products run on many SMs instead of
-// queueing on one SM's fp64 units.  NaN in the window is a data error.
-constexpr int kFPerBlock = 32;
+// reduction's ragged tail instead of as a launch of its own.  Every prep block
+// tabulates F[c] = phi_gamma(c / n) for kPrepPerBlock of c = 0..n and puts as many
+// window values in their places of the ascending order, each by counting the values
+// before it (ties by index), so that neither the table's fp64 divisions nor the order
+// wait for one SM.  A bitonic sort by one block (45 to 78 steps behind barriers) held
+// short streams' launches open: whole calls (graph replay) 20k trajectories with a window
+// of 777 65.0 and now 62.2 us, 32k with 4,096 91.5 and 65.7 (128 values a block 79.1, 64
+// 69.9), 128k with 4,096 303 and 284, 300k 378 and 364, 16k with 512 52.9 both.  NaN in the window is a data error.
+constexpr int kPrepPerBlock = 32;
+constexpr int kPrepParts = kReduceThreads / kPrepPerBlock;  // threads a value, each for a
+                                                            // part of the window
 
 struct WindowPrep {
   const float* window;  // null: no preparation blocks
@@ -411,27 +416,31 @@ struct WindowPrep {
 };
 
 inline unsigned window_prep_blocks(int64_t n) {
-  return 1u + static_cast<unsigned>((n + 1 + kFPerBlock - 1) / kFPerBlock);
+  return static_cast<unsigned>((n + 1 + kPrepPerBlock - 1) / kPrepPerBlock);
 }
 
 inline size_t window_prep_smem(int64_t n) {
-  size_t np2 = 1;
-  while (np2 < static_cast<size_t>(n)) np2 <<= 1;
-  return np2 * sizeof(float);
+  return static_cast<size_t>((n + 3) / 4 * 4) * sizeof(float);
+}
+
+// The values of sw[a, b) (both multiples of 4) that lie before v.
+template <bool kOrEqual>
+__device__ __forceinline__ int count_before(const float* sw, int a, int b, float v) {
+  int c = 0;
+#pragma unroll 4
+  for (int k = a; k < b; k += 4) {
+    const float4 y = *reinterpret_cast<const float4*>(sw + k);
+    c += kOrEqual ? (y.x <= v) + (y.y <= v) + (y.z <= v) + (y.w <= v)
+                  : (y.x < v) + (y.y < v) + (y.z < v) + (y.w < v);
+  }
+  return c;
 }
 
 __device__ void window_prep_block(int b, const WindowPrep& w) {
-  const int n = w.n;
-  if (b > 0) {
-    const int c = (b - 1) * kFPerBlock + static_cast<int>(threadIdx.x);
-    if (threadIdx.x < kFPerBlock && c <= n)
-      w.f_table[c] = sharpen(__ddiv_rn(static_cast<double>(c), static_cast<double>(n)), w.gamma);
-    return;
-  }
-  extern __shared__ float sw[];
-  int np2 = 1;
-  while (np2 < n) np2 <<= 1;
-  for (int k = threadIdx.x; k < np2; k += blockDim.x) {
+  extern __shared__ __align__(16) float sw[];  // the window, padded with +inf to a multiple of 4
+  __shared__ int s_rank[kPrepParts][kPrepPerBlock];
+  const int n = w.n, n4 = (n + 3) & ~3;
+  for (int k = threadIdx.x; k < n4; k += blockDim.x) {
     float v = k < n ? w.window[k] : __int_as_float(0x7f800000);
     if (isnan(v)) {
       report(w.status, PACE_ERR_NAN_INPUT);
@@ -439,24 +448,29 @@ __device__ void window_prep_block(int b, const WindowPrep& w) {
     }
     sw[k] = v;
   }
-  // Each step compares the pairs (lo, lo + stride): pair i puts a zero bit at
-  // the stride's position of i, so every thread has work on every step.
-  for (int size = 2; size <= np2; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      __syncthreads();
-      for (int i = threadIdx.x; i < (np2 >> 1); i += blockDim.x) {
-        const int lo = ((i & ~(stride - 1)) << 1) | (i & (stride - 1));
-        const int hi = lo | stride;
-        const float a = sw[lo], c = sw[hi];
-        if ((a > c) == ((lo & size) == 0)) {
-          sw[lo] = c;
-          sw[hi] = a;
-        }
-      }
-    }
-  }
   __syncthreads();
-  for (int k = threadIdx.x; k < n; k += blockDim.x) w.sorted[k] = sw[k];
+  const int e = static_cast<int>(threadIdx.x) % kPrepPerBlock;
+  const int part = static_cast<int>(threadIdx.x) / kPrepPerBlock;
+  const int c0 = b * kPrepPerBlock, i = c0 + e;  // value i, table entry i
+  const int per = (n4 / 4 + kPrepParts - 1) / kPrepParts * 4;
+  const int from = min(part * per, n4), to = min(from + per, n4);
+  int rank = 0;
+  if (i < n) {
+    const float v = sw[i];
+    rank = count_before<true>(sw, from, min(to, c0), v);  // equal ones of lower index: before
+    for (int k = max(from, c0); k < min(to, c0 + kPrepPerBlock); ++k)
+      rank += sw[k] < v || (sw[k] == v && k < i);
+    rank += count_before<false>(sw, max(from, c0 + kPrepPerBlock), to, v);
+  }
+  s_rank[part][e] = rank;
+  __syncthreads();
+  if (part == 0 && i < n) {
+#pragma unroll
+    for (int q = 1; q < kPrepParts; ++q) rank += s_rank[q][e];
+    w.sorted[rank] = sw[i];
+  } else if (part == 1 && i <= n) {
+    w.f_table[i] = sharpen(__ddiv_rn(static_cast<double>(i), static_cast<double>(n)), w.gamma);
+  }
 }
 
 // One warp's share of the stream (every warp of the first n_stream_blocks
@@ -883,8 +897,8 @@ struct FusedFinalize {
 
 // Run by every block once its own warps have streamed: publish that, take a
 // finishing ticket (the first finishers, idle in the reduction's ragged tail,
-// run the window's preparation tasks: task 0 sorts W, task 1 + k tabulates F
-// for 32 counts), then finalise this block's slice of the groups,
+// run the window's preparation tasks: each sorts in 32 values of W and tabulates
+// F for 32 counts), then finalise this block's slice of the groups,
 // [U b / S, U (b + 1) / S), once the stream blocks covering those groups'
 // tokens and the preparation are done.  Each block thus finalises in the tail
 // as soon as its neighbourhood of the stream is complete, and no launch of its

@@ -225,6 +225,28 @@ def test_window_shapes_and_ties(n_traj, wlen, gamma):
         _check(g, o, f"w{wlen}/g{gamma}/{mode}")
 
 
+@pytest.mark.parametrize("wlen", [2, 3, 31, 33, 63, 255, 257, 4095])
+@pytest.mark.parametrize("kind", ["equal", "descending", "two values", "signed zeros"])
+def test_window_order(wlen, kind):
+    """The sorted window where equal values lie on both sides of the blocks and parts that
+    place them, s_pre on, just above and just below every value; bits as the oracle's."""
+    rng = np.random.default_rng(wlen)
+    window = {"equal": np.full(wlen, 0.25), "descending": np.arange(wlen, 0, -1) / 64.0,
+              "two values": np.where(np.arange(wlen) % 3 == 0, 0.5, 0.125),
+              "signed zeros": np.where(np.arange(wlen) % 2 == 0, -0.0, 0.0)}[kind]
+    window = window.astype(np.float32)
+    lens = rng.integers(1, 6, size=8192)
+    tags, offsets, c, _, j, _ = _mk_fast(lens, rng)
+    s_pre = rng.choice(window, size=len(lens))
+    step = rng.integers(-1, 2, size=len(lens))
+    s_pre = np.where(step == 0, s_pre,
+                     np.nextafter(s_pre, np.where(step > 0, np.inf, -np.inf).astype(np.float32)))
+    s_pre = s_pre.astype(np.float32)
+    g = gpu_score(tags, offsets, c, s_pre, j, window, gamma=3, min_obs=1, group_size=4)
+    o = oracle_score(tags, offsets, c, s_pre, j, window, gamma=3, min_obs=1, group_size=4)
+    _check(g, o, f"{kind} {wlen}")
+
+
 @pytest.mark.parametrize("n_traj,n_tok,wlen", [(64, 0, 512), (8192, 0, 4096), (8192, 1500, 4096),
                                                 (16384, 70000, 512)])
 def test_short_streams(n_traj, n_tok, wlen):
