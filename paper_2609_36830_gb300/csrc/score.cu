@@ -5,8 +5,8 @@
 //                       bound): per trajectory the count T of policy tokens,
 //                       the exact integer sum of their tags and the largest
 //                       tag (+1, for the Lemma 1 premise check).
-//                       On pools of 8k trajectories and more the same launch
-//                       also prepares the prefix-score window (extra blocks
+//                       The same launch also prepares the
+//                       prefix-score window (extra blocks
 //                       after the streaming ones, run in its tail): each puts a
 //                       part of W in its sorted places and tabulates a part
 //                       of F = phi(count / |W|) (Eqs. 9-10) for every
@@ -14,8 +14,7 @@
 //                       the count).
 //   score_finalize_kernel  one thread per trajectory: K_gen, K_wait, the ECDF
 //                       count of s against the window (binary search in the
-//                       sorted window, or a direct count on small pools), F
-//                       (from the table, or computed), the mode's score
+//                       sorted window), F from the table, the mode's score
 //                       (Eqs. 7-8), and the mean of each group of G in fixed
 //                       left-to-right order.
 #include <cuda_runtime.h>
@@ -78,7 +77,6 @@ bool cooperative_launch_ok() {
   }
   return c == 1;
 }
-constexpr int64_t kTableMinTraj = 8192;  // pools from this size sort W and tabulate F
 
 __device__ __forceinline__ int4 ld_stream_v4(const int32_t* p) {
   int4 v;
@@ -623,9 +621,8 @@ struct FinalizeArgs {
   const int64_t* offsets;
   const int32_t* c_version;
   const float* s_pre;
-  const float* window;           // W as given (used when window_sorted is null)
-  const float* window_sorted;   // ascending, window_len values, or null
-  const double* f_table;        // F for counts 0..window_len (with window_sorted)
+  const float* window_sorted;   // ascending, window_len values (with window_ready)
+  const double* f_table;        // F for counts 0..window_len (with window_ready)
   TagTotals tt;
   StreamGeom geom;
   int64_t n_traj;
@@ -637,7 +634,6 @@ struct FinalizeArgs {
   int32_t gamma;
   int32_t group_size;
   double inv_group;             // 1 / G for G a power of two (exact), else 0
-  int32_t lanes;                // threads per trajectory for the direct count
   double f_missing;
   double* kgen;
   double* kwait;
@@ -647,65 +643,50 @@ struct FinalizeArgs {
   int32_t* status;
 };
 
-// Shared memory of one finalisation pass: the window (padded to a multiple of
-// 4 floats), optionally the F table, the scores of the pass's trajectories and
-// the partial counts.
+// Shared memory of one finalisation pass: the sorted window (padded to a multiple of
+// 4 floats), the F table and the scores of the pass's trajectories.
 struct FinalizeSmem {
   float* swin;
-  double* ftab;    // [window_len + 1] or null (then F is read from global memory)
+  double* ftab;    // [window_len + 1]
   double* sscore;  // [tpb]
-  int* pcount;     // [lanes][tpb]
 };
 
-__host__ __device__ inline size_t finalize_smem_bytes(int64_t window_len, int tpb, int threads,
-                                                      bool table_in_smem) {
+__host__ __device__ inline size_t finalize_smem_bytes(int64_t window_len, int tpb) {
   return align_up(static_cast<size_t>((window_len + 3) & ~3) * sizeof(float), 16) +
-         (table_in_smem ? static_cast<size_t>(window_len + 1) * sizeof(double) : 0) +
-         static_cast<size_t>(tpb) * sizeof(double) + static_cast<size_t>(threads) * sizeof(int);
+         static_cast<size_t>(window_len + 1) * sizeof(double) +
+         static_cast<size_t>(tpb) * sizeof(double);
 }
 
-__device__ __forceinline__ FinalizeSmem finalize_smem(unsigned char* raw, int window_len, int tpb,
-                                                      bool table_in_smem) {
+__device__ __forceinline__ FinalizeSmem finalize_smem(unsigned char* raw, int window_len) {
   FinalizeSmem m;
   const int wpad = (window_len + 3) & ~3;
   m.swin = reinterpret_cast<float*>(raw);
-  double* d = reinterpret_cast<double*>(raw + align_up(wpad * sizeof(float), 16));
-  m.ftab = table_in_smem ? d : nullptr;
-  m.sscore = table_in_smem ? d + window_len + 1 : d;
-  m.pcount = reinterpret_cast<int*>(m.sscore + tpb);
+  m.ftab = reinterpret_cast<double*>(raw + align_up(wpad * sizeof(float), 16));
+  m.sscore = m.ftab + window_len + 1;
   return m;
 }
 
-// The window into shared memory: the sorted window, or the raw one NaN-padded
-// to a multiple of 4 (NaN never counts as <= s); four loads per thread in
-// flight at a time; with m.ftab set, the F table too.  L2 loads: the sorted
-// window and the table may have been written by another block of the same
-// launch.  Every thread of the block calls it.
+// The sorted window and the F table into shared memory, four loads of each per thread in
+// flight at a time.  L2 loads: another block of the same launch may have written them.
+// Every thread of the block calls it.
 __device__ void finalize_load_window(const FinalizeArgs& p, const FinalizeSmem& m) {
   if (p.window_ready) {
-    const bool sorted = p.window_sorted != nullptr;
-    const bool table = m.ftab && sorted;
-    const int wpad = (p.window_len + 3) & ~3;
-    const int tlen = table ? p.window_len + 1 : 0;
-    const int span = wpad > tlen ? wpad : tlen;
-    const float* src = sorted ? p.window_sorted : p.window;
+    const int tlen = p.window_len + 1;
     const int nb = static_cast<int>(blockDim.x);
-    // four window values and four table entries per thread in flight at once
-    for (int k0 = threadIdx.x; k0 < span; k0 += 4 * nb) {
+    for (int k0 = threadIdx.x; k0 < tlen; k0 += 4 * nb) {
       float w[4];
       double f[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int k = k0 + j * nb;
-        w[j] = k < p.window_len ? __ldcg(src + k) : __int_as_float(0x7fc00000);
+        w[j] = k < p.window_len ? __ldcg(p.window_sorted + k) : 0.0f;
         f[j] = k < tlen ? __ldcg(p.f_table + k) : 0.0;
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int k = k0 + j * nb;
-        if (k < wpad) m.swin[k] = w[j];
+        if (k < p.window_len) m.swin[k] = w[j];
         if (k < tlen) m.ftab[k] = f[j];
-        if (!sorted && k < p.window_len && isnan(w[j])) report(p.status, PACE_ERR_NAN_INPUT);
       }
     }
   }
@@ -725,12 +706,11 @@ struct TrajIn {
 };
 
 __device__ __forceinline__ void load_traj_inputs(const FinalizeArgs& p, int64_t i0, int64_t i_end,
-                                                 int tpb, int lanes, TrajIn& in) {
+                                                 int tpb, TrajIn& in) {
   const int tid = static_cast<int>(threadIdx.x);
-  const int64_t i = i0 + tid % tpb;
-  const bool valid = tid < tpb * lanes && i < i_end;
-  in.s = (valid && p.s_pre) ? p.s_pre[i] : __int_as_float(0x7fc00000);
+  const int64_t i = i0 + tid;
   if (tid < tpb && i < i_end) {
+    in.s = p.s_pre ? p.s_pre[i] : __int_as_float(0x7fc00000);
     in.c = p.c_version[i];
     in.o0 = p.offsets[i];
     in.o1 = p.offsets[i + 1];
@@ -758,37 +738,15 @@ __device__ __forceinline__ void load_traj_acc(const FinalizeArgs& p, int64_t i0,
 }
 
 // One pass over trajectories [i0, i0 + tpb) clipped to i_end (i0 and tpb whole
-// groups), from what load_traj_inputs and load_traj_acc read: thread t <
-// tpb * lanes counts for trajectory slot t % tpb (on the direct-count path
-// `lanes` threads per trajectory each count one strided share of the window;
-// lanes = 1 with the sorted window); threads t < tpb then do that trajectory's
-// fp64 work, and the first thread of each group its mean in fixed left-to-right
+// groups), from what load_traj_inputs and load_traj_acc read: threads t < tpb do
+// trajectory i0 + t, then consecutive threads the groups' means in fixed left-to-right
 // order.  Every thread of the block calls it.
 __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, int tpb,
-                              int lanes, const FinalizeSmem& m, const TrajIn& in) {
-  const bool sorted = p.window_sorted != nullptr;
-  const int wpad = (p.window_len + 3) & ~3;
+                              const FinalizeSmem& m, const TrajIn& in) {
   const int tid = static_cast<int>(threadIdx.x);
-  const bool active = tid < tpb * lanes;
-  const int slot = tid % tpb;
-  const int64_t i = i0 + slot;
-  const bool lead = tid < tpb;  // owns trajectory i's results
-  const float s = in.s;
-  if (p.window_ready && !sorted) {
-    // direct count of window values <= s, one strided share of the window per lane
-    int count = 0;
-    if (active && !isnan(s)) {
-      const float4* w4 = reinterpret_cast<const float4*>(m.swin);
-      for (int k = tid / tpb; k < wpad / 4; k += lanes) {
-        const float4 w = w4[k];
-        count += (w.x <= s) + (w.y <= s) + (w.z <= s) + (w.w <= s);
-      }
-    }
-    if (active) m.pcount[tid] = count;
-    __syncthreads();
-  }
-
-  if (lead && i < i_end) {
+  const int64_t i = i0 + tid;
+  if (tid < tpb && i < i_end) {
+    const float s = in.s;
     const int64_t o0 = in.o0, o1 = in.o1;
     if (o1 < o0 || (i == 0 && o0 != 0) || (i == p.n_traj - 1 && o1 != p.n_tokens))
       report(p.status, PACE_ERR_INVALID_ARG);
@@ -810,7 +768,7 @@ __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, 
       f = 1.0;
     } else if (isnan(s)) {
       f = p.f_missing;
-    } else if (sorted) {
+    } else {
       // count of window values <= s: the first index of the sorted window
       // holding a value > s
       int lo = 0, hi = p.window_len;
@@ -819,12 +777,7 @@ __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, 
         if (m.swin[mid] <= s) lo = mid + 1;
         else hi = mid;
       }
-      f = m.ftab ? m.ftab[lo] : __ldcg(p.f_table + lo);
-    } else {  // small pools: F from the summed partial counts
-      int count = 0;
-      for (int l = 0; l < lanes; ++l) count += m.pcount[l * tpb + slot];
-      f = sharpen(__ddiv_rn(static_cast<double>(count), static_cast<double>(p.window_len)),
-                  p.gamma);
+      f = m.ftab[lo];
     }
     double sc;
     if (p.mode == PACE_SCORE_EFF) sc = __dadd_rn(kwait, __dmul_rn(f, kgen));
@@ -834,7 +787,7 @@ __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, 
     if (p.kwait) p.kwait[i] = kwait;
     if (p.weight) p.weight[i] = f;
     p.score[i] = sc;
-    m.sscore[slot] = sc;
+    m.sscore[tid] = sc;
   }
   __syncthreads();
   // The groups' means, a thread per group, the groups in consecutive threads: a chain of
@@ -859,21 +812,21 @@ __device__ void finalize_pass(const FinalizeArgs& p, int64_t i0, int64_t i_end, 
   }
 }
 
-// The finalisation as a launch of its own (groups of more than 256): blockDim.x
-// = tpb * lanes, tpb trajectories (whole groups) per block.
+// The finalisation as a launch of its own: blockDim.x trajectories (whole groups) per
+// block.
 __global__ void score_finalize_kernel(FinalizeArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int tpb = static_cast<int>(blockDim.x) / p.lanes;
-  const FinalizeSmem m = finalize_smem(smem_raw, p.window_len, tpb, p.window_sorted != nullptr);
+  const int tpb = static_cast<int>(blockDim.x);
+  const FinalizeSmem m = finalize_smem(smem_raw, p.window_len);
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * tpb;
   // the inputs, the slot and the window are in flight together; the head slots
   // of continuing trajectories are loaded once the window is in place
   TrajIn in;
-  load_traj_inputs(p, i0, p.n_traj, tpb, p.lanes, in);
+  load_traj_inputs(p, i0, p.n_traj, tpb, in);
   load_traj_slot(p, i0, p.n_traj, tpb, in);
   finalize_load_window(p, m);
   load_traj_acc(p, i0, p.n_traj, tpb, in);
-  finalize_pass(p, i0, p.n_traj, tpb, p.lanes, m, in);
+  finalize_pass(p, i0, p.n_traj, tpb, m, in);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
@@ -889,8 +842,8 @@ struct FusedFinalize {
   unsigned* done;       // [stream blocks] set once a block's warps have all streamed; null: off
   unsigned* ticket;     // counts the blocks that have finished streaming
   unsigned* prep_done;  // counts the finished preparation tasks
-  int prep_tasks;       // window sort + F-table slices (0: no table)
-  int tpb, lanes;       // trajectories per finalisation pass, threads per trajectory
+  int prep_tasks;       // parts of the sorted window and the F table (0: no window)
+  int tpb;              // trajectories per finalisation pass
   WindowPrep prep;
   FinalizeArgs fin;
 };
@@ -933,11 +886,10 @@ __device__ __forceinline__ void fused_finalize(const int64_t* __restrict__ offse
   if (u_lo >= u_hi) return;
   const int64_t i_lo = u_lo * G, i_hi = u_hi * G;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const bool sorted = p.window_sorted != nullptr;
-  const FinalizeSmem m = finalize_smem(smem_raw, p.window_len, fz.tpb, sorted);
+  const FinalizeSmem m = finalize_smem(smem_raw, p.window_len);
   // the first pass's inputs are in flight while the waits below run
   TrajIn cur;
-  load_traj_inputs(p, i_lo, i_hi, fz.tpb, fz.lanes, cur);
+  load_traj_inputs(p, i_lo, i_hi, fz.tpb, cur);
   if (tid < 32) {
     const int lane = tid;
     // stream blocks holding the tokens of trajectories [i_lo, i_hi): the warp of
@@ -981,11 +933,11 @@ __device__ __forceinline__ void fused_finalize(const int64_t* __restrict__ offse
     TrajIn nxt;
     const int64_t i1 = i0 + fz.tpb;
     if (i1 < i_hi) {
-      load_traj_inputs(p, i1, i_hi, fz.tpb, fz.lanes, nxt);
+      load_traj_inputs(p, i1, i_hi, fz.tpb, nxt);
       load_traj_slot(p, i1, i_hi, fz.tpb, nxt);
       load_traj_acc(p, i1, i_hi, fz.tpb, nxt);
     }
-    finalize_pass(p, i0, i_hi, fz.tpb, fz.lanes, m, cur);
+    finalize_pass(p, i0, i_hi, fz.tpb, m, cur);
     __syncthreads();  // the pass's shared scores and counts are reused
     cur = nxt;
   }
@@ -1252,11 +1204,12 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
   const bool window_ready = window_len > 0 && window_len >= params->min_obs;
   // With the sorted window and the F table the finalisation takes one binary
   // search and one table read per trajectory; their preparation runs inside the
-  // tag reduction's launch.  Small pools count against the raw window instead
-  // (the same bits either way).
-  const bool use_table = window_ready && n_traj >= kTableMinTraj;
+  // tag reduction's launch.  (Small pools counted against the raw window instead, eight
+  // threads a trajectory, while one block sorted it; whole calls by graph replay that way
+  // and now: 64 trajectories 17.8 and 16.4 us, 1,024 22.6 and 21.2, 4,096 28.8 and 27.8,
+  // 2,048 with a window of 4,096 34.9 and 31.5, 6,000 with 1,024 32.8 and 31.3.)
   WindowPrep prep{};
-  if (use_table) {
+  if (window_ready) {
     prep.window = window;
     prep.n = static_cast<int>(window_len);
     prep.gamma = params->gamma;
@@ -1268,15 +1221,14 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
   a.offsets = offsets;
   a.c_version = c_version;
   a.s_pre = s_pre;
-  a.window = window;
-  a.window_sorted = use_table ? wws.sorted : nullptr;
-  a.f_table = use_table ? wws.f_table : nullptr;
+  a.window_sorted = wws.sorted;
+  a.f_table = wws.f_table;
   a.tt = ws.tt;
   a.geom = StreamGeom{};
   a.n_traj = n_traj;
   a.n_tokens = n_tokens;
   a.j = trainer_version;
-  a.window_len = static_cast<int32_t>(window_len);
+  a.window_len = window_ready ? static_cast<int32_t>(window_len) : 0;
   a.window_ready = window_ready ? 1 : 0;
   a.mode = params->mode;
   a.gamma = params->gamma;
@@ -1297,24 +1249,15 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
     // hides (1M sweep pool: 2.31 -> 2.28 ms per call).  On small pools the chain
     // after the last stream block (flags, waits, one pass) costs more than a
     // launch of its own (16k: 65.6 -> 71 us), so they keep that launch.  Passes
-    // of whole groups over the block's 256 threads; on the direct-count path
-    // up to 8 threads per trajectory share the count.
-    int lanes = 1;
-    if (!use_table && window_ready) {
-      lanes = 8;
-      while (lanes > 1 && G * lanes > kReduceThreads) lanes /= 2;
-    }
+    // of whole groups over the block's 256 threads.
     FusedFinalize fz{};
-    fz.lanes = lanes;
-    fz.tpb = (kReduceThreads / lanes / G) * G;
-    a.lanes = lanes;
+    fz.tpb = (kReduceThreads / G) * G;
     fz.fin = a;
-    if (use_table) {
+    if (window_ready) {
       fz.prep = prep;
       fz.prep_tasks = static_cast<int>(window_prep_blocks(prep.n));
     }
-    size_t smem = finalize_smem_bytes(window_len, fz.tpb, kReduceThreads, use_table);
-    if (use_table && window_prep_smem(prep.n) > smem) smem = window_prep_smem(prep.n);
+    const size_t smem = finalize_smem_bytes(a.window_len, fz.tpb);  // at least the preparation's
     StreamGeom geom{};
     return run_tag_reduce(tags, offsets, n_traj, n_tokens, ws, WindowPrep{}, fz, true, smem, &geom,
                           st);
@@ -1322,40 +1265,24 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
 
   PACE_TRY(run_tag_reduce(tags, offsets, n_traj, n_tokens, ws, prep, FusedFinalize{}, false, 0,
                           &a.geom, st));
-  // A launch of its own: whole groups per block.  With the sorted window: one
-  // thread per trajectory, 256 threads (whole groups) per block, so that one
-  // round of loads brings the window and the F table into shared memory.
-  // Otherwise small pools take fewer groups per block so that the
-  // per-trajectory fp64 work of F (GB300's fp64 rate is low) is spread over
-  // about two blocks per SM instead of queueing on a few SMs; with the direct
-  // count, up to 8 threads per trajectory share the count so its chain is 8
-  // times shorter.
+  // A launch of its own: whole groups per block, one thread per trajectory.  With the
+  // window, 256 threads per block, so that one round of loads brings it and the F table
+  // into shared memory; without, about 64, so that the little fp64 work left is spread
+  // over more SMs.
   const int max_units = G >= 256 ? 1 : 256 / G;
   const int64_t n_units = n_traj / G;
   const int64_t spread = 2 * static_cast<int64_t>(sm_count());
+  const int min_units = window_ready ? max_units : (G >= 64 ? 1 : (64 + G - 1) / G);
   int64_t want = (n_units + spread - 1) / spread;
-  int min_units = 1;
-  int lanes = 1;
-  if (use_table) {
-    min_units = max_units;
-  } else if (window_ready) {
-    lanes = 8;
-  } else {
-    min_units = G >= 64 ? 1 : (64 + G - 1) / G;
-  }
   want = want < min_units ? min_units : want;
-  const int units_per_block = want > max_units ? max_units : static_cast<int>(want);
-  const int tpb = units_per_block * G;
-  while (lanes > 1 && tpb * lanes > 1024) lanes /= 2;
-  a.lanes = lanes;
-  const int threads = tpb * lanes;
+  const int tpb = (want > max_units ? max_units : static_cast<int>(want)) * G;
   const int64_t blocks = (n_traj + tpb - 1) / tpb;
-  const size_t smem = finalize_smem_bytes(window_len, tpb, threads, use_table);
+  const size_t smem = finalize_smem_bytes(a.window_len, tpb);
   if (smem > 48 * 1024)
     PACE_TRY_CUDA(cudaFuncSetAttribute(score_finalize_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
-  score_finalize_kernel<<<static_cast<unsigned>(blocks), threads, smem, st>>>(a);
+  score_finalize_kernel<<<static_cast<unsigned>(blocks), tpb, smem, st>>>(a);
   return last_launch_status();
 }
 
