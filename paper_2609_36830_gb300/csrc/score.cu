@@ -1245,10 +1245,10 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
   if (G <= kReduceThreads && n_traj >= fused_min_traj().load() && cooperative_launch_ok()) {
     // Large pools whose groups fit one block: the finalisation runs inside the
     // tag reduction's launch, each stream block finalising its slice of the
-    // groups in the stream's ragged tail, where most of the per-trajectory work
-    // hides (1M sweep pool: 2.31 -> 2.28 ms per call).  On small pools the chain
-    // after the last stream block (flags, waits, one pass) costs more than a
-    // launch of its own (16k: 65.6 -> 71 us), so they keep that launch.  Passes
+    // groups in the stream's ragged tail.  The chain after the last stream block
+    // (flags, waits, one pass) costs more than a launch of its own (16k 55.2 against
+    // 51.8 us per call, 128k 282.8 / 278.7), on large pools hardly more (1M 2142 /
+    // 2138), where it saves the launch.  Passes
     // of whole groups over the block's 256 threads.
     FusedFinalize fz{};
     fz.tpb = (kReduceThreads / G) * G;
