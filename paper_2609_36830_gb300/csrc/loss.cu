@@ -289,8 +289,9 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
       if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
       unsigned in = 0u;
       float adv[kRowsPerLane] = {};  // per row; the terms are computed once per tile, not per piece
-      // the terms of the given rows, added up: every row's is computed, without a branch,
-      // so that the eight rows' chains of latencies overlap
+      // the terms of the given rows, added up; under TOKEN_MEAN every row's is computed,
+      // without a branch, so that the eight rows' chains of latencies overlap (loss and
+      // derivative over 5.4M rows 58.0 -> 55.6 us; SEQ_MEAN, per piece, spills that way)
       auto terms = [&](unsigned rows) -> double {
         Sum3 sum{0.0f, 0.0f, 0.0f};
 #pragma unroll

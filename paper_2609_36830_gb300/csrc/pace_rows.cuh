@@ -19,7 +19,8 @@ constexpr int kRowWarps = kRowThreads / 32;
 // Three blocks an SM (80 registers), one wave: the loss and its derivative over 5.4M
 // rows took 83 us (graph replay) with a tile a warp in four waves of blocks and 66 with
 // a range a warp, 58 with 32-byte accesses and each tile's terms computed once whatever
-// its sequences; four blocks an SM spill (109).
+// its sequences, 55.6 without a branch per row; four blocks an SM spill (109).  Staging
+// two tiles a warp in shared memory needs fewer registers and took 64 to 67.
 constexpr int kRowMinBlocks = 3;
 constexpr int kMaxRowBlocks = 152 * kRowMinBlocks;
 
