@@ -440,7 +440,9 @@ PACE_API size_t pace_stale_k_workspace_size(int64_t n_traj);
  * for rejected and accepted units, as in the paper's retained-vs-rejected
  * admission analysis.  n_bins (1..4096) equal-width bins over [lo, hi): the bin
  * of x is floor((x - lo) / (hi - lo) * n_bins) in fp64, values below lo count
- * in the first bin and values at or above hi in the last.  hist is device
+ * in the first bin and values at or above hi in the last.  Where hi - lo
+ * overflows, so that the quotient is 0 or NaN, every value below hi counts in
+ * the first bin.  hist is device
  * uint32 [2 * n_bins] (output): [0, n_bins) rejected (flag 0), [n_bins,
  * 2 n_bins) accepted; with flags NULL every value counts in the first half.
  * Exact integer counts; NaN values are skipped and reported as

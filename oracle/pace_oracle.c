@@ -531,7 +531,8 @@ int oracle_stale_k(const int32_t* tags, const int64_t* offsets, int64_t n_traj, 
  * analysis): counts of values in n_bins equal-width bins over [lo, hi), values
  * below lo in the first bin and at or above hi in the last; hist[0..n_bins) for
  * rejected entries (flag 0), hist[n_bins..2 n_bins) for accepted (flag != 0).
- * The bin of x is floor((x - lo) / (hi - lo) * n_bins), computed in fp64. */
+ * The bin of x is floor((x - lo) / (hi - lo) * n_bins), computed in fp64; where hi - lo
+ * overflows that is bin 0 (the quotient is 0, or NaN where x - lo overflows too). */
 int oracle_histogram(const double* values, const uint8_t* flags, int64_t n, double lo,
                      double hi, int32_t n_bins, uint32_t* hist) {
   if (n < 0 || n_bins < 1 || !(hi > lo)) return OR_ERR_INVALID_ARG;
@@ -543,8 +544,8 @@ int oracle_histogram(const double* values, const uint8_t* flags, int64_t n, doub
     if (x < lo) b = 0;
     else if (x >= hi) b = n_bins - 1;
     else {
-      b = (int64_t)floor((x - lo) / (hi - lo) * (double)n_bins);
-      if (b > n_bins - 1) b = n_bins - 1;
+      const double f = floor((x - lo) / (hi - lo) * (double)n_bins);
+      b = !(f > 0.0) ? 0 : (f > (double)(n_bins - 1) ? n_bins - 1 : (int64_t)f);
     }
     hist[(flags && flags[i] ? n_bins : 0) + b] += 1;
   }

@@ -1288,7 +1288,9 @@ __global__ void staleness_hist_kernel(const double* __restrict__ values,
           per_bin == 0.0 || frac < 0x3DB0000000000000ll || frac > 0x3FEFFFFFFFFE0000ll;
       if (__any_sync(__activemask(), edge))  // the vote keeps it a branch, not predicates
         b = hist_bin(d, width, inv_width, bins);
-      if (b > n_bins - 1) b = n_bins - 1;
+      // hi - lo may overflow: the quotient is then 0 or, where x - lo overflows too, NaN,
+      // whose conversion is the smallest integer
+      b = min(max(b, 0), n_bins - 1);
     }
     atomicAdd(&h[(flags && flags[i] ? n_bins : 0) + b], 1u);
   }

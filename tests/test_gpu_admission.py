@@ -179,3 +179,16 @@ def test_histogram_at_bin_edges(lo, hi, n_bins):
     st, oh = oracle.histogram(x, flags, lo, hi, n_bins)
     assert st == 0
     np.testing.assert_array_equal(as_np(hist).astype(np.uint32), oh)
+
+
+def test_histogram_where_the_width_overflows():
+    """lo and hi are finite, hi - lo is not: x - lo overflows for the larger values below hi
+    and their quotient is NaN.  They count in the first bin, none outside the histogram."""
+    lo, hi, n_bins = -1e308, 1.5e308, 10
+    x = np.array([0.9e308, 1.2e308, 1.49e308, -0.9e308, 0.0, 1.5e308, 1.7e308, -1.7e308])
+    flags = np.array([0, 1, 0, 1, 0, 1, 0, 1], np.uint8)
+    want = np.zeros((2, n_bins), np.uint32)
+    want[0, [0, n_bins - 1]] = 3, 1
+    want[1, [0, n_bins - 1]] = 3, 1
+    hist = pace.staleness_histogram(to_dev(x), to_dev(flags), lo, hi, n_bins)
+    np.testing.assert_array_equal(as_np(hist).astype(np.uint32), want)

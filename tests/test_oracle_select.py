@@ -152,3 +152,11 @@ def test_quantile_admit_rank_is_the_real_number_rank():
     w.count, w.head = 189, 189
     st, _, kappa = oracle.quantile_admit(np.zeros(0), 1 / 3, 0, w, min_obs=1)
     assert st == 0 and kappa == 126.0
+
+
+def test_histogram_where_the_width_overflows():
+    """x - lo and hi - lo overflow: the quotient is NaN and counts in the first bin."""
+    x = np.array([0.9e308, 1.2e308, -0.9e308, 0.0, 1.5e308])
+    st, h = oracle.histogram(x, np.zeros(5, np.uint8), -1e308, 1.5e308, 4)
+    assert st == 0
+    np.testing.assert_array_equal(h, [[4, 0, 0, 1], [0, 0, 0, 0]])
