@@ -366,9 +366,9 @@ __global__ void loss_from_partial_kernel(const double* __restrict__ partial,
 }
 
 void carve_surrogate_ws(Carver& cv, int64_t n_rows, int64_t n_seq, SurrogateWs* w) {
-  const RowGeom g = row_geom(n_rows);
-  const size_t blocks = g.blocks > 0 ? g.blocks : 1;
-  const size_t tiles = g.n_tiles > 0 ? static_cast<size_t>(g.n_tiles) : 1;
+  const size_t blocks = row_blocks_bound(n_rows);
+  const int64_t n_tiles = row_geom(n_rows).n_tiles;
+  const size_t tiles = n_tiles > 0 ? static_cast<size_t>(n_tiles) : 1;
   w->seq_sum = cv.take<double>(n_seq > 0 ? n_seq : 1);
   w->seq_cnt = cv.take<double>(n_seq > 0 ? n_seq : 1);
   w->head_sum = cv.take<double>(tiles);
@@ -632,8 +632,7 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ hidden, int64_t row
 }
 
 RowCounts carve_row_counts(Carver& cv, int64_t n_rows) {
-  const RowGeom g = row_geom(n_rows);
-  const size_t blocks = g.blocks > 0 ? g.blocks : 1;
+  const size_t blocks = row_blocks_bound(n_rows);
   RowCounts c;
   c.block = cv.take<long long>(blocks);
   c.warp = cv.take<int>(blocks * kRowWarps);

@@ -43,6 +43,15 @@ inline RowGeom row_geom(int64_t n_rows) {
   return g;
 }
 
+// Blocks that a workspace for n_rows rows holds.  A launch's own count falls where
+// per_warp steps up; this one never does, so a workspace made for the largest batch
+// serves every smaller one.
+inline size_t row_blocks_bound(int64_t n_rows) {
+  const int64_t n_tiles = (n_rows + kRowTile - 1) / kRowTile;
+  const int64_t b = (n_tiles + kRowWarps - 1) / kRowWarps;
+  return static_cast<size_t>(b < 1 ? 1 : (b < kMaxRowBlocks ? b : kMaxRowBlocks));
+}
+
 // Reports offsets that do not partition the rows (any thread of a grid: sequence i).
 __device__ __forceinline__ void check_seq(const int64_t* __restrict__ offsets, int64_t i,
                                           int64_t n_rows, int32_t* status) {

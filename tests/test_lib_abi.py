@@ -168,3 +168,42 @@ def test_shard_selection_argument_checks_return_before_launch(pace):
     assert L.pace_loss_from_partial(None, fake, None) == pace.ERR_INVALID_ARG
     assert L.pace_div_selftest(None, None, -1, None, None, None, None, None) == \
         pace.ERR_INVALID_ARG
+
+
+def test_workspaces_never_shrink_as_batches_grow(pace):
+    """A workspace made for the largest batch serves every smaller one: no size query falls
+    as rows, sequences, trajectories or units grow, around every multiple at which the row
+    walk's launches change shape and at each power of two."""
+    L = pace.lib()
+    step = 256 * 8 * 456  # rows of one tile a warp in a full launch
+    rows = sorted({max(0, k * r + d) for k in (1, 2, 3) for d in (-1, 0, 1, 255, 256, 257, 4096)
+                   for r in (step, step // 2, 16384, 32768)}
+                  | {max(0, 2 ** e + d) for e in range(0, 23) for d in (-1, 0, 1)}
+                  | {610_000, 1_000_000, 1_200_000, 5_400_000})
+    seqs = [0, 1, 7, 8, 9, 64, 1000, 1024, 100_000]
+    heads = ((64, 64), (256, 2048), (64, 4033), (1024, 50_001), (3584, 152_064))
+
+    def nondecreasing(f, xs):
+        sizes = [f(x) for x in xs]
+        assert all(a <= b for a, b in zip(sizes, sizes[1:])), \
+            [(x, a, b) for x, a, b in zip(xs, sizes, sizes[1:]) if a > b][:3]
+
+    for f in (L.pace_surrogate_loss_workspace_size, L.pace_surrogate_backward_workspace_size):
+        for s in seqs:
+            nondecreasing(lambda n: f(n, s), rows)
+        for n in rows[::5]:
+            nondecreasing(lambda s: f(n, s), seqs)
+    for f in (L.pace_token_logprob_workspace_size, L.pace_prefix_score_workspace_size,
+              L.pace_token_logprob_backward_workspace_size):
+        for H, V in heads:
+            for s in (1, 1024):
+                nondecreasing(lambda n: f(n, s, H, V), rows)
+            for n in rows[::9]:
+                nondecreasing(lambda s: f(n, s, H, V), seqs)
+    for w in (0, 1, 512, 4096):
+        nondecreasing(lambda n: L.pace_score_pool_workspace_size(n, w), rows)
+    for n in rows[::5]:
+        nondecreasing(lambda w: L.pace_score_pool_workspace_size(n, w), [0, 1, 511, 512, 4096])
+    nondecreasing(L.pace_stale_k_workspace_size, rows)
+    nondecreasing(L.pace_select_workspace_size, rows)
+    nondecreasing(L.pace_select_shard_workspace_size, rows)
