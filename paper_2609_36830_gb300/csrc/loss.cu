@@ -401,9 +401,14 @@ pace_status check_loss_args(const PaceBatch* b, const PaceLossArgs* l) {
 
 pace_status launch_group_adv(const AdvJob& j, const PaceBatch* b, unsigned* counter,
                              int32_t* status, cudaStream_t st) {
-  if (j.blocks == 0 && !counter) return PACE_OK;
-  group_adv_kernel<<<static_cast<unsigned>(j.blocks > 0 ? j.blocks : 1), kAdvThreads, 0, st>>>(
-      j, b ? b->seq_offsets : nullptr, b ? b->n_seq : 0, b ? b->n_rows : 0, counter, status);
+  const int64_t n_seq = b ? b->n_seq : 0;
+  // the offsets are checked whether or not there are advantages to compute
+  int64_t blocks = (n_seq + kAdvThreads - 1) / kAdvThreads;
+  if (blocks > 1024) blocks = 1024;
+  if (blocks < j.blocks) blocks = j.blocks;
+  if (blocks == 0 && !counter) return PACE_OK;
+  group_adv_kernel<<<static_cast<unsigned>(blocks > 0 ? blocks : 1), kAdvThreads, 0, st>>>(
+      j, b ? b->seq_offsets : nullptr, n_seq, b ? b->n_rows : 0, counter, status);
   return last_launch_status();
 }
 

@@ -111,6 +111,52 @@ def test_empty_loss_is_zero_and_bad_offsets_reported():
     assert int(status.item()) == pace.ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("call", ["logprob", "logprob_with_loss", "prefix", "loss", "derivative"])
+def test_bad_offsets_of_an_empty_batch_reported(call):
+    """No rows, offsets that name some: every call says so."""
+    b = pace.make_batch(to_dev(np.array([0, 2, 5, 9], np.int64)), 0)
+    status = pace.new_status(DEV)
+    hidden = torch.empty(0, 64, dtype=torch.bfloat16, device=DEV)
+    w = torch.zeros(64, 64, dtype=torch.bfloat16, device=DEV)
+    y = torch.empty(0, dtype=torch.int32, device=DEV)
+    empty = torch.empty(0, device=DEV)
+    loss = torch.full((1,), 7.0, dtype=torch.float64, device=DEV)
+    la = pace.make_loss_args(torch.zeros(1, device=DEV), to_dev(np.ones(3, np.float32)), 3,
+                             pace.loss_params(), loss)
+    if call == "prefix":
+        pace.prefix_score(b, hidden, w, y, torch.zeros(1, device=DEV), status=status)
+    elif call == "loss":
+        pace.surrogate_loss(b, empty, la, status=status)
+    elif call == "derivative":
+        pace.surrogate_backward(b, empty, la, status=status)
+    else:
+        pace.token_logprob(b, hidden, w, y, loss=la if call == "logprob_with_loss" else None,
+                           status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == pace.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
+def test_workspace_of_a_larger_batch_serves_a_smaller_one(agg):
+    """933,888 rows are one tile a warp of a full launch, 1,200,000 two (in half the blocks)."""
+    most, rows, n_seq = 1_200_000, 933_888, 16
+    L = pace.lib()
+    ws = pace.workspace(L.pace_surrogate_loss_workspace_size(most, n_seq), DEV)
+    ws_b = pace.workspace(L.pace_surrogate_backward_workspace_size(most, n_seq), DEV)
+    so = np.linspace(0, rows, n_seq + 1).astype(np.int64)
+    b = pace.make_batch(to_dev(so), rows)
+    lp = torch.zeros(rows, device=DEV)
+    reward = (np.arange(n_seq) % 2).astype(np.float32)
+    loss = torch.zeros(1, dtype=torch.float64, device=DEV)
+    la = pace.make_loss_args(torch.zeros(rows, device=DEV), to_dev(reward), n_seq,
+                             pace.loss_params(agg=agg), loss)
+    status = pace.new_status(DEV)
+    pace.surrogate_loss(b, lp, la, ws=ws, status=status)
+    pace.surrogate_backward(b, lp, la, ws=ws_b, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+
+
 def _layout(kind, rng):
     if kind == "short":      # more sequences than a walker holds, in every tile, and empty ones
         return rng.integers(0, 6, size=1200)
