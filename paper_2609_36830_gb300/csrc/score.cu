@@ -1006,6 +1006,31 @@ ScoreWs carve_score_ws(Carver& cv, int64_t n_traj) {
   return w;
 }
 
+// The two kernels that hold the sorted window and the F table are allowed the shared
+// memory of the largest window once per device, whatever window a call has: a limit set
+// per call could be lowered by another thread between its setting and the launch.
+// (Below kPlainSmem no permission is needed, the kernels' static shared memory included.)
+constexpr size_t kPlainSmem = 40 * 1024;
+
+pace_status allow_window_smem() {
+  constexpr int kMaxDevices = 64;
+  static bool done[kMaxDevices] = {};
+  static std::mutex mu;
+  int dev = 0;
+  PACE_TRY_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) return PACE_ERR_CUDA;
+  std::lock_guard<std::mutex> g(mu);
+  if (done[dev]) return PACE_OK;
+  PACE_TRY_CUDA(cudaFuncSetAttribute(score_finalize_kernel,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(finalize_smem_bytes(kMaxWindow, 1024))));
+  PACE_TRY_CUDA(cudaFuncSetAttribute(
+      tag_reduce_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      static_cast<int>(finalize_smem_bytes(kMaxWindow, kReduceThreads))));
+  done[dev] = true;
+  return PACE_OK;
+}
+
 // Resident blocks per SM of the fused tag reduction with the given dynamic shared
 // memory (cached per device and size).
 pace_status reduce_blocks_per_sm(size_t smem, int* out) {
@@ -1021,12 +1046,6 @@ pace_status reduce_blocks_per_sm(size_t smem, int* out) {
     return PACE_OK;
   }
   int nb = 0;
-  // above the default 48 KB (windows of more than ~2,000 values with their F
-  // table) the kernel must be allowed the larger dynamic shared memory first
-  if (smem > 48 * 1024)
-    PACE_TRY_CUDA(cudaFuncSetAttribute(tag_reduce_kernel<true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem)));
   PACE_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tag_reduce_kernel<true>,
                                                               kReduceThreads, smem));
   if (dev >= 0 && dev < kMaxDevices) {
@@ -1076,6 +1095,7 @@ pace_status run_tag_reduce(const int32_t* tags, const int64_t* offsets, int64_t 
   if (fused) smem = fused_smem;
   int per_sm = kBlocksPerSm;
   if (fused) {
+    if (smem > kPlainSmem) PACE_TRY(allow_window_smem());
     int nb = 0;
     PACE_TRY(reduce_blocks_per_sm(smem, &nb));
     if (nb < 1) return PACE_ERR_UNSUPPORTED_SHAPE;
@@ -1278,10 +1298,7 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
   const int tpb = (want > max_units ? max_units : static_cast<int>(want)) * G;
   const int64_t blocks = (n_traj + tpb - 1) / tpb;
   const size_t smem = finalize_smem_bytes(a.window_len, tpb);
-  if (smem > 48 * 1024)
-    PACE_TRY_CUDA(cudaFuncSetAttribute(score_finalize_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem)));
+  if (smem > kPlainSmem) PACE_TRY(allow_window_smem());
   score_finalize_kernel<<<static_cast<unsigned>(blocks), tpb, smem, st>>>(a);
   return last_launch_status();
 }

@@ -3,6 +3,7 @@
 import ctypes
 import json
 import os
+import threading
 
 import numpy as np
 import pytest
@@ -223,6 +224,54 @@ def test_window_shapes_and_ties(n_traj, wlen, gamma):
         o = oracle_score(tags, offsets, c, s_pre, j, window, mode=mode, gamma=gamma, min_obs=1,
                          group_size=4)
         _check(g, o, f"w{wlen}/g{gamma}/{mode}")
+
+
+@pytest.mark.parametrize("wlen", [3320, 3420, 3838, 3880, 3924, 3925])
+def test_windows_around_the_plain_shared_memory(wlen):
+    """Windows whose sorted copy and table of F need a little less or more shared memory
+    than a kernel has without asking, in either launch that holds them (the first calls of
+    a process; later ones find it asked for)."""
+    rng = np.random.default_rng(wlen)
+    window = rng.random(wlen).astype(np.float32)
+    tags, offsets, c, s_pre, j, _ = _mk_fast(rng.integers(1, 30, size=512), rng)
+    g = gpu_score(tags, offsets, c, s_pre, j, window, min_obs=1)
+    o = oracle_score(tags, offsets, c, s_pre, j, window, min_obs=1)
+    _check(g, o, f"w{wlen}")
+
+
+def test_threads_with_different_large_windows():
+    """Two host threads, a stream each, score with windows of different sizes that both
+    need more than the plain shared memory: every call launches and gives its own bits."""
+    rng = np.random.default_rng(5)
+    tags, offsets, c, s_pre, j, _ = _mk_fast(rng.integers(1, 30, size=256), rng)
+    sizes = (3925, 4096)
+    want, args, errors = [], [], []
+    for w in sizes:
+        window = rng.random(w).astype(np.float32)
+        want.append(oracle_score(tags, offsets, c, s_pre, j, window, min_obs=1))
+        args.append([to_dev(x) for x in (tags, offsets, c, s_pre)] + [j, to_dev(window)])
+    got = [None, None]
+
+    def work(i):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for _ in range(300):
+                    got[i] = pace.score_pool(*args[i], pace.score_params(min_obs=1),
+                                             stream=stream)
+            stream.synchronize()
+        except Exception as e:  # the other thread goes on
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(i,)) for i in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+    for i in (0, 1):
+        _check({k: as_np(v) for k, v in got[i].items()}, want[i], f"w{sizes[i]}")
 
 
 @pytest.mark.parametrize("wlen", [2, 3, 31, 33, 63, 255, 257, 4095])
