@@ -624,10 +624,8 @@ __global__ void zero_tail_rows_kernel(uint4* __restrict__ buf, int64_t row_vecs,
 
 // dLoss/dlp per row of the clipped surrogate (oracle: oracle_surrogate_grad), 0
 // outside the loss.  The scale (1 / rows in the loss, or 1 / (sequences x rows of
-// the sequence)) is an fp64 quotient; a row's product with it is rounded once to
-// fp32 as g * hi + g * lo, scale = hi + lo in two floats (48 bits), because one
-// conversion to fp64, product and conversion back per row would bound the kernel on
-// GB300's narrow fp64 pipe.
+// the sequence)) is an fp64 quotient and a row's product with it is taken in fp64 and
+// rounded to fp32 (quick_product does without where it can).
 struct GradArgs {
   const int64_t* seq_offsets;
   const uint8_t* seq_accepted;
@@ -644,6 +642,21 @@ struct GradArgs {
   const int* n_used;                 // sequences that have any
   float* dlp;
 };
+
+// x * scale rounded to fp64 and then to fp32, without the fp64 pipe, which a conversion,
+// a product and a conversion back per row would keep busy for most of the kernel (derivative
+// of 5.4M rows by graph replay 42.6 us that way, 24.5 so).  scale = s_hi + s_lo to 2^-49; the two partial products give
+// x * scale to 2^-45, and Ziv's test (ACM TOMS 17, 1991) says whether that decides the
+// rounding.  Where it does not (2^-18 of all products), or where the product is so small
+// that a partial product is subnormal, `sure` is false and the result is to be computed.
+__device__ __forceinline__ float quick_product(float x, float s_hi, float s_lo, bool* sure) {
+  const float q = __fmul_rn(x, s_hi);
+  const float t = __fmaf_rn(x, s_lo, __fmaf_rn(x, s_hi, -q));
+  const float r = __fadd_rn(q, t);
+  const float low = __fsub_rn(t, __fsub_rn(r, q));  // r + low = q + t
+  *sure = x == 0.0f || (r == __fmaf_rn(low, 1.0f + 0x1p-18f, r) && fabsf(r) > 0x1p-90f);
+  return r;
+}
 
 template <bool kSeqMean>
 __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_kernel(GradArgs p) {
@@ -674,6 +687,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
     auto derive = [&](unsigned rows) {
       const float s_hi = static_cast<float>(scale);
       const float s_lo = static_cast<float>(scale - static_cast<double>(s_hi));
+      unsigned unsure = 0u;
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) {
         if (kSeqMean && !(rows >> u & 1u)) continue;
@@ -687,7 +701,17 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
         float x = 0.0f;
         if (d > -20.0f && d < 20.0f && p1 >= p2) x = -a * rho;
         if (a < 0.0f && -p.dual * a < lm) x = 0.0f;
-        cur.lp[u] = fmaf(x, s_hi, x * s_lo);  // the derivative, once the row is used
+        bool sure;
+        cur.lp[u] = quick_product(x, s_hi, s_lo, &sure);  // the derivative, once the row is used
+        cur.bh[u] = x;
+        if (!sure) unsure |= 1u << u;
+      }
+      unsure &= rows;
+      if (__any_sync(0xffffffffu, unsure != 0u)) {  // the vote keeps it a branch
+#pragma unroll
+        for (int u = 0; u < kRowsPerLane; ++u)
+          if (unsure >> u & 1u)
+            cur.lp[u] = static_cast<float>(static_cast<double>(cur.bh[u]) * scale);
       }
     };
     pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t) {

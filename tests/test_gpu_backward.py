@@ -74,6 +74,45 @@ def test_surrogate_backward_matches_oracle(rows_spec, agg):
     assert (gg[og == 0] == 0).sum() >= (og == 0).sum() - near.sum()
 
 
+@pytest.mark.parametrize("adv_eps", [1e-6, 1e30, 1e34])
+@pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
+def test_derivative_is_the_fp64_product_rounded(agg, adv_eps):
+    """dlp of every row to the bit: the fp32 derivative of its term (from the ratios and
+    advantages that the loss returns) times the fp64 scale, rounded to fp64 and to fp32.
+    A large adv_eps makes the products small, down to subnormal results."""
+    rng = np.random.default_rng(23)
+    n_seq, G = 96, 8
+    lens = rng.integers(1, 60_000, size=n_seq)
+    so = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    n = int(so[-1])
+    lp = rng.uniform(-3, 0, size=n).astype(np.float32)
+    behav = (lp - rng.normal(0, 0.3, size=n)).astype(np.float32)
+    mask = (rng.random(n) < 0.8).astype(np.uint8)
+    loss = torch.zeros(1, dtype=torch.float64, device=DEV)
+    adv = torch.empty(n_seq, device=DEV)
+    ratio = torch.empty(n, device=DEV)
+    la = pace.make_loss_args(to_dev(behav), to_dev(rng.random(n_seq).astype(np.float32)), G,
+                             pace.loss_params(agg=agg, adv_eps=adv_eps), loss, adv_out=adv,
+                             ratio_out=ratio)
+    b = pace.make_batch(to_dev(so), n, mask=to_dev(mask))
+    pace.surrogate_loss(b, to_dev(lp), la)
+    dlp = as_np(pace.surrogate_backward(b, to_dev(lp), la))
+    a, rho = np.repeat(as_np(adv), lens), as_np(ratio)
+    one = np.float32(1.0)
+    rc = np.minimum(np.maximum(rho, one - np.float32(0.2)), one + np.float32(0.28))
+    p1, p2 = -a * rho, -a * rc
+    low = np.maximum(p1, p2)
+    x = np.where((p1 >= p2) & ~((a < 0) & (np.float32(-10.0) * a < low)), p1, np.float32(0.0))
+    inn = np.add.reduceat(mask.astype(np.int64), so[:-1])
+    if agg == pace.AGG_TOKEN_MEAN:
+        scale = np.full(n, 1.0 / float(mask.sum()))
+    else:
+        scale = np.repeat(1.0 / (float((inn > 0).sum()) * np.maximum(inn, 1)), lens)
+    want = np.where(mask == 1, (x.astype(np.float64) * scale).astype(np.float32),
+                    np.float32(0.0))
+    assert (dlp == want).all(), (int((dlp != want).sum()), np.nonzero(dlp != want)[0][:5])
+
+
 @pytest.mark.parametrize("rows,H,V,masked", [(100, 64, 256, False), (300, 128, 1000, True),
                                              (1000, 256, 2048, False), (700, 192, 4099, True),
                                              (3000, 512, 2304, True), (600, 2048, 1000, True),
