@@ -513,8 +513,11 @@ PACE_API size_t pace_surrogate_backward_workspace_size(int64_t n_rows, int64_t n
  * chunks of up to 32,768: logits are recomputed on the tensor cores, G is held
  * in bf16 in the workspace for the chunk (in 64-column blocks), then two
  * tensor-core GEMMs form G W and G^T H.  Chunks past the rows in the loss (a
- * count known only on the device) cost no tensor-core work.  Returns
- * PACE_ERR_UNSUPPORTED_SHAPE when ceil(V / 64) x the chunk's rows exceeds
+ * count known only on the device) cost no tensor-core work.  The workspace holds
+ * the gathered rows (2 H bytes a row), one chunk of G (2 V bytes a row of the
+ * chunk) and, for V above 4,032, partial tiles of G W: at most 75 tiles of 256 KB,
+ * and no more than the chunk has, in min(8, floor(ceil(V / 64) / 32)) parts, up
+ * to 157 MB.  Returns PACE_ERR_UNSUPPORTED_SHAPE when ceil(V / 64) x the chunk's rows exceeds
  * 2^31 - 1 (V above about 4.2M at full chunks).  Other arguments and errors as
  * for pace_token_logprob. */
 PACE_API pace_status pace_token_logprob_backward(const PaceBatch* batch, const void* hidden,

@@ -138,16 +138,21 @@ struct TailSplit {
   int splits;
 };
 
+// Parts that a tile of nkb K steps may be split into: each has at least 32 of them.
+__host__ __device__ inline int max_k_splits(int nkb) {
+  return nkb / 32 < kMaxKSplits ? nkb / 32 : kMaxKSplits;
+}
+
 __host__ __device__ inline TailSplit tail_split(int64_t items, int n_clusters, int nkb) {
   TailSplit s;
   s.full = items / n_clusters * n_clusters;
   s.tail = static_cast<int>(items - s.full);
   s.splits = 1;
   int best = nkb;  // the tail's K steps
-  for (int k = 2; k <= kMaxKSplits; ++k) {
+  for (int k = 2; k <= max_k_splits(nkb); ++k) {
     const int rounds = (s.tail * k + n_clusters - 1) / n_clusters;
     const int steps = rounds * ((nkb + k - 1) / k);
-    if (nkb >= 32 * k && steps < best) {
+    if (steps < best) {
       best = steps;
       s.splits = k;
     }
@@ -793,12 +798,13 @@ void carve_bw_ws(Carver& cv, int64_t n_rows, int64_t n_seq, int H, int V, BwWs* 
   const int64_t g_cols = (static_cast<int64_t>(V) + 63) / 64 * 64;
   w->g = cv.take<uint16_t>(static_cast<size_t>(chunk_rows(n_rows > 0 ? n_rows : 1)) * g_cols);
   w->round_ctr = cv.take<unsigned>(1);
-  // a tail of R < kMaxGemmClusters tiles in kMaxKSplits parts at most, and no more
-  // tiles than the rows have
+  // a tail of R < kMaxGemmClusters tiles, and no more tiles than the rows have, in as many
+  // parts as the vocabulary's K steps allow (none below 64 K steps: no tile is split then)
   const int64_t tiles = (chunk_rows(n_rows > 0 ? n_rows : 1) + 2 * GBM - 1) / (2 * GBM) *
                         ((H + GBN - 1) / GBN);
   const int64_t tail = tiles < kMaxGemmClusters ? tiles : kMaxGemmClusters - 1;
-  w->part = cv.take<float>(static_cast<size_t>(tail) * kMaxKSplits * 2 * GBM * GBN);
+  const int parts = max_k_splits(static_cast<int>((V + GBK - 1) / GBK));
+  w->part = parts > 1 ? cv.take<float>(static_cast<size_t>(tail) * parts * 2 * GBM * GBN) : nullptr;
 }
 
 }  // namespace

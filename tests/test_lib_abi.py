@@ -207,3 +207,19 @@ def test_workspaces_never_shrink_as_batches_grow(pace):
     nondecreasing(L.pace_stale_k_workspace_size, rows)
     nondecreasing(L.pace_select_workspace_size, rows)
     nondecreasing(L.pace_select_shard_workspace_size, rows)
+
+
+@pytest.mark.parametrize("n,H,V,parts", [(16384, 256, 2048, 0), (65536, 64, 4032, 0),
+                                         (16384, 1024, 4033, 2), (2582, 2048, 12288, 6),
+                                         (2582, 2048, 151936, 8)])
+def test_backward_workspace_holds_what_the_vocabulary_needs(pace, n, H, V, parts):
+    """Gathered rows, one chunk of G, and dH's partial tiles: at most 75 tiles of 256 x 256
+    floats in `parts` parts, one per 32 K steps of 64 vocabulary entries and at most 8, none
+    where that is below 2; the rest (row lists, log-prob partials) is below 128 bytes a row
+    and 1 MB."""
+    chunk = min(n, 32768)
+    chunk = (chunk + 127) // 128 * 128
+    tiles = min((chunk + 255) // 256 * ((H + 255) // 256), 75)
+    need = 2 * n * H + 2 * chunk * ((V + 63) // 64 * 64) + tiles * parts * 256 * 256 * 4
+    got = pace.lib().pace_token_logprob_backward_workspace_size(n, 8, H, V)
+    assert need <= got <= need + 128 * n + (1 << 20)
