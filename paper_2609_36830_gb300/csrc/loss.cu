@@ -16,7 +16,7 @@ namespace pace {
 
 // ------------------------------------------------------------ advantages
 
-// Prompt groups of at most 32: L = 2^m >= G lanes per group (32 / L groups a warp),
+// L = 2^m >= G lanes per group (32 / L groups a warp),
 // lane k holding member k.  Mean and standard deviation of the accepted members'
 // rewards in fp64, summed from the lowest index up (the same order as one thread
 // would take), then A_i = (R_i - mean) / (std + eps), each lane its own division:
@@ -57,7 +57,7 @@ __device__ void group_adv_lanes(const float* __restrict__ reward,
   if (mine) adv[i] = static_cast<float>(in && d != 0.0 ? __ddiv_rn(d, den) : 0.0);
 }
 
-// Larger groups: a thread per group, in the same order.
+// A thread per group, in the same order.
 __device__ void group_adv_thread(const float* __restrict__ reward,
                                  const uint8_t* __restrict__ accepted, int64_t g, int G, double eps,
                                  int unbiased, float* __restrict__ adv) {
@@ -89,9 +89,16 @@ __device__ void group_adv_thread(const float* __restrict__ reward,
   }
 }
 
+// Lanes or threads: the lanes of a group share its chain of loads and divisions, but each
+// repeats its sums and root, about G times the fp64 work, so they win while the groups are
+// few enough for latency to count.  pace_group_advantages, a thread and lanes per group:
+// G 2, 16,000 sequences 4.5 and 3.7 us, 32,000 4.5 and 4.8; G 8, 32,000 8.2 and 5.7,
+// 64,000 8.3 and 9.1, 1M 44 and 105; G 16, 64,000 14.1 and 11.4, 128,000 14.0 and 20.3;
+// G 32, 1M 47 and 198.  (One member has no work to repeat: lanes at any size.)
+constexpr int64_t kLaneGroups = 6144, kLanes = 65536;
+
 constexpr int kAdvThreads = 32;  // a warp: the groups' fp64 divisions spread over the SMs
 
-// The advantages a launch computes, by `blocks` of its blocks (0: none).
 AdvJob adv_job(const float* reward, const uint8_t* accepted, int64_t n_seq, int G, float eps,
                int unbiased, float* adv) {
   AdvJob j{};
@@ -101,23 +108,32 @@ AdvJob adv_job(const float* reward, const uint8_t* accepted, int64_t n_seq, int 
   j.G = G;
   j.L = 1;
   while (j.L < G && j.L < 32) j.L *= 2;
+  if (G > 32 || (G > 1 && (j.n_groups > kLaneGroups || j.n_groups * j.L > kLanes))) j.L = 0;
   j.eps = static_cast<double>(eps);
   j.unbiased = unbiased;
   j.adv = adv;
-  // warps (or threads, for groups of more than 32) over the groups
-  const int64_t per_block = G <= 32 ? kAdvThreads / j.L : kAdvThreads;
-  j.blocks = static_cast<int>((j.n_groups + per_block - 1) / per_block);
   return j;
 }
 
-// Block b of the job's blocks (threads from kAdvThreads on have no part in it).
+// Blocks of `threads` threads that compute the advantages: with lanes, one warp each
+// (their other threads have no part in it); with a thread per group, up to 128 threads.
+__host__ __device__ inline int adv_threads(const AdvJob& j, int threads) {
+  return j.L > 0 ? kAdvThreads : (threads < 128 ? threads : 128);
+}
+
+int adv_blocks(const AdvJob& j, int threads) {
+  const int64_t per_block = adv_threads(j, threads) / (j.L > 0 ? j.L : 1);
+  return static_cast<int>((j.n_groups + per_block - 1) / per_block);
+}
+
+// Block b of the job's blocks.
 __device__ void adv_block(const AdvJob& j, int64_t b) {
-  if (threadIdx.x >= kAdvThreads) return;
-  if (j.G <= 32) {
-    group_adv_lanes(j.reward, j.accepted, j.n_groups, j.G, j.L, j.eps, j.unbiased, j.adv,
-                    b * (kAdvThreads / 32) + (threadIdx.x >> 5));
+  const int threads = adv_threads(j, blockDim.x);
+  if (static_cast<int>(threadIdx.x) >= threads) return;
+  if (j.L > 0) {
+    group_adv_lanes(j.reward, j.accepted, j.n_groups, j.G, j.L, j.eps, j.unbiased, j.adv, b);
   } else {
-    const int64_t g = b * kAdvThreads + threadIdx.x;
+    const int64_t g = b * threads + threadIdx.x;
     if (g < j.n_groups) group_adv_thread(j.reward, j.accepted, g, j.G, j.eps, j.unbiased, j.adv);
   }
 }
@@ -132,7 +148,7 @@ __global__ void __launch_bounds__(kAdvThreads)
   if (seq_offsets)
     for (int64_t i = t; i < n_seq; i += static_cast<int64_t>(gridDim.x) * blockDim.x)
       check_seq(seq_offsets, i, n_rows, status);
-  if (blockIdx.x < static_cast<unsigned>(j.blocks)) adv_block(j, blockIdx.x);
+  adv_block(j, blockIdx.x);  // past the job's blocks: none of the groups
 }
 
 // ------------------------------------------------------------ surrogate
@@ -405,7 +421,7 @@ pace_status launch_group_adv(const AdvJob& j, const PaceBatch* b, unsigned* coun
   // the offsets are checked whether or not there are advantages to compute
   int64_t blocks = (n_seq + kAdvThreads - 1) / kAdvThreads;
   if (blocks > 1024) blocks = 1024;
-  if (blocks < j.blocks) blocks = j.blocks;
+  if (blocks < adv_blocks(j, kAdvThreads)) blocks = adv_blocks(j, kAdvThreads);
   if (blocks == 0 && !counter) return PACE_OK;
   group_adv_kernel<<<static_cast<unsigned>(blocks > 0 ? blocks : 1), kAdvThreads, 0, st>>>(
       j, b ? b->seq_offsets : nullptr, n_seq, b ? b->n_rows : 0, counter, status);
@@ -654,7 +670,7 @@ pace_status launch_count_rows(const PaceBatch* b, RowCounts counts, unsigned lon
                               int* n_used, const AdvJob& adv, unsigned* counter0,
                               unsigned* counter1, int32_t* status, cudaStream_t st) {
   const RowGeom g = row_geom(b->n_rows);
-  count_rows_kernel<<<static_cast<unsigned>(g.blocks + adv.blocks), kRowThreads, 0, st>>>(
+  count_rows_kernel<<<static_cast<unsigned>(g.blocks + adv_blocks(adv, kRowThreads)), kRowThreads, 0, st>>>(
       b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, aligned(b->mask, 8), counts,
       seq_in, n_used,
       adv, counter0, counter1, status);
@@ -675,7 +691,7 @@ pace_status run_compaction(const PaceBatch* b, const CompactWs& ws, const AdvJob
   if (b->n_rows <= kFewRows) {
     const int blocks = static_cast<int>((b->n_rows + kFewWarps * kRowTile - 1) /
                                         (kFewWarps * kRowTile));
-    list_few_rows_kernel<<<static_cast<unsigned>(blocks + adv.blocks), kFewThreads, 0, st>>>(
+    list_few_rows_kernel<<<static_cast<unsigned>(blocks + adv_blocks(adv, kFewThreads)), kFewThreads, 0, st>>>(
         b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, blocks,
         aligned(b->mask, 8), ws.rowidx, ws.total, lp, lse, adv, counter0, counter1, status);
     return last_launch_status();

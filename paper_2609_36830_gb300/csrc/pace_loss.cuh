@@ -28,16 +28,16 @@ struct CompactWs {
   int32_t* rowidx;      // [n_rows]: compact row -> original row
 };
 
-// The group advantages of a call, computed by `blocks` blocks of some launch.
+// The group advantages of a call, computed by some blocks of a launch (adv_blocks).
 struct AdvJob {
   const float* reward;
   const uint8_t* accepted;
-  int64_t n_groups;
-  int G, L;
+  int64_t n_groups;  // 0: none
+  int G;
+  int L;             // lanes per group, or 0: a thread per group
   double eps;
   int unbiased;
   float* adv;
-  int blocks;
 };
 
 // Workspace of the log-prob pipeline (compaction, gathered rows, split partials).

@@ -16,8 +16,28 @@ from paper_2609_36830_gb300 import pace, workloads
 pytestmark = pytest.mark.gpu
 
 
+def test_advantages_of_few_and_of_many_groups_cost_alike():
+    """Whatever the number of groups, the time per group does not grow with it: lanes per
+    group repeat its fp64 sums, so they may not be used where throughput counts (1M
+    sequences in groups of 32 took 198 us that way, 47 with a thread per group)."""
+    n, G = 1 << 20, 32
+    r, out = torch.rand(n, device=DEV), torch.empty(n, device=DEV)
+    times = []
+    for _ in range(8):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            pace.group_advantages(r, G, out=out)
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) / 20)
+    assert min(times) < 0.1  # ms
+
+
+# the last four: around the number of groups from which a thread takes each
 @pytest.mark.parametrize("G,n_seq,p_acc", [(8, 64, 1.0), (8, 512, 0.75), (12, 1200, 0.5),
-                                           (1, 300, 0.8), (16, 16, 0.3)])
+                                           (1, 300, 0.8), (16, 16, 0.3), (2, 12288, 0.6),
+                                           (2, 12290, 0.6), (12, 49152, 0.6), (12, 49164, 0.6)])
 @pytest.mark.parametrize("unbiased", [True, False])
 def test_advantages_bitwise(G, n_seq, p_acc, unbiased):
     rng = np.random.default_rng(G * 1000 + n_seq)
