@@ -82,18 +82,15 @@ struct PieceWalker {
     j = 0;
   }
 
-  // to the last sequence in [0, n_seq) that begins at or before t0, else the first
+  // to the last sequence from lo on that begins at or before t, else to lo
   // (a 32-way search: two rounds at 1,024 sequences)
-  __device__ PieceWalker(const int64_t* offsets_, const uint8_t* accepted_, const float* per_seq_,
-                         int64_t n_seq_, int64_t t0)
-      : offsets(offsets_), accepted(accepted_), per_seq(per_seq_), n_seq(n_seq_), base(0), j(0),
-        o(0), v(0.0f), acc_bits(0u) {
+  __device__ void seek(int64_t lo, int64_t t) {
     const int lane = threadIdx.x & 31;
-    int64_t lo = 0, hi = n_seq;
+    int64_t hi = n_seq;
     while (hi - lo > 1) {
       const int64_t span = hi - lo;
       const int64_t q = lo + 1 + ((span - 1) * lane) / 32;  // in [lo + 1, hi - 1], nondecreasing
-      const unsigned bal = __ballot_sync(0xffffffffu, offsets[q] <= t0);
+      const unsigned bal = __ballot_sync(0xffffffffu, offsets[q] <= t);
       if (bal == 0u) {
         hi = lo + 1;
       } else {
@@ -104,7 +101,14 @@ struct PieceWalker {
       }
     }
     base = lo;
-    if (n_seq > 0) load();
+    load();
+  }
+
+  __device__ PieceWalker(const int64_t* offsets_, const uint8_t* accepted_, const float* per_seq_,
+                         int64_t n_seq_, int64_t t0)
+      : offsets(offsets_), accepted(accepted_), per_seq(per_seq_), n_seq(n_seq_), base(0), j(0),
+        o(0), v(0.0f), acc_bits(0u) {
+    if (n_seq > 0) seek(0, t0);
   }
 
   // Calls f(seq, lo, hi, value, begin) for every piece [lo, hi) of an accepted sequence
@@ -123,7 +127,12 @@ struct PieceWalker {
       if (o1 >= t1) return;  // (o1 == t1: the next tile steps over it)
       if (++j == 31) {
         base += 31;
-        if (base < n_seq) load();
+        if (base < n_seq) {
+          load();
+          // a run of empty sequences is searched over, not walked (100,000 of them between
+          // two sequences of 150,000 rows: loss 11.5 ms walked, 20 us searched)
+          if (__shfl_sync(full, o, 31) <= o1) seek(base, o1);
+        }
       }
     }
   }

@@ -186,6 +186,10 @@ def _layout(kind, rng):
         return np.array([1])
     if kind == "gap":        # long sequences between short ones
         return np.array([0, 3000, 1, 5000, 0, 1, 2, 4097, 31, 0])
+    if kind == "empties":    # runs of empty sequences around the 31 that a walker holds
+        runs = [np.zeros(k, np.int64) for k in (40, 30, 31, 32, 61, 62, 63, 93, 3000, 125)]
+        full = [3, 253, 1, 300, 7, 2000, 1, 200, 12]
+        return np.concatenate([x for r, f in zip(runs, full) for x in (r, [f])] + runs[-1:])
     return rng.integers(0, 4000, size=608)  # several tiles a warp
 
 
@@ -236,6 +240,42 @@ def test_row_tiles_of_any_layout(kind, G, agg, masked):
     assert abs(float(loss.item()) - oloss) <= unit * max(np.abs(oterm).max(initial=0.0), 1e-30)
     assert (np.abs(as_np(ratio) - oratio) <= unit * oratio).all()
     assert (np.abs(as_np(dlp) - odlp) <= unit * np.abs(odlp)).all()
+
+
+@pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
+@pytest.mark.parametrize("masked", [False, True])
+def test_runs_of_empty_sequences(agg, masked):
+    assert _layout("empties", None).size == 3546
+    test_row_tiles_of_any_layout("empties", 9, agg, masked)
+
+
+@pytest.mark.parametrize("call", ["loss", "derivative", "list"])
+def test_runs_of_empty_sequences_are_not_walked(call):
+    """200,000 empty sequences between two of 5,000 rows: walked one by one they took 23 ms
+    in the loss's launch and 42 in the derivative's two."""
+    n, E = 10_000, 200_000
+    so = np.full(E + 3, 5000, np.int64)
+    so[0], so[-1] = 0, n
+    b = pace.make_batch(to_dev(so), n)
+    lp = torch.zeros(n, device=DEV)
+    loss = torch.zeros(1, dtype=torch.float64, device=DEV)
+    la = pace.make_loss_args(lp, torch.ones(E + 2, device=DEV), 2, pace.loss_params(), loss)
+    acc = torch.ones(E + 2, dtype=torch.uint8, device=DEV)
+    hidden = torch.zeros((n, 64), dtype=torch.bfloat16, device=DEV)
+    w, y = hidden[:64], torch.zeros(n, dtype=torch.int32, device=DEV)
+    masked = pace.make_batch(to_dev(so), n, seq_accepted=acc)
+    run = {"loss": lambda: pace.surrogate_loss(b, lp, la),
+           "derivative": lambda: pace.surrogate_backward(b, lp, la),
+           "list": lambda: pace.token_logprob(masked, hidden, w, y)}[call]
+    times = []
+    for _ in range(8):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        run()
+        e1.record()
+        torch.cuda.synchronize()
+        times.append(e0.elapsed_time(e1))
+    assert min(times) < 3.0  # ms
 
 
 @pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
