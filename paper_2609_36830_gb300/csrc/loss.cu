@@ -153,17 +153,18 @@ __global__ void __launch_bounds__(kAdvThreads)
 
 // ------------------------------------------------------------ surrogate
 
-__device__ __forceinline__ float clipped_term(float lp, float behav, float a, float eps_low,
-                                              float eps_high, float dual, float* rho_out) {
-  float d = lp - behav;
-  d = fminf(fmaxf(d, -20.0f), 20.0f);
-  const float rho = expf(d);
+__device__ __forceinline__ float clamped_ratio(float lp, float behav) {
+  const float d = lp - behav;
+  return expf(fminf(fmaxf(d, -20.0f), 20.0f));
+}
+
+__device__ __forceinline__ float clipped_term(float rho, float a, float eps_low, float eps_high,
+                                              float dual) {
   const float rc = fminf(fmaxf(rho, 1.0f - eps_low), 1.0f + eps_high);
   const float p1 = -a * rho;
   const float p2 = -a * rc;
   float l = fmaxf(p1, p2);
   if (a < 0.0f) l = fminf(l, -dual * a);
-  *rho_out = rho;
   return l;
 }
 
@@ -287,7 +288,9 @@ __global__ void __launch_bounds__(kRowThreads) seq_mean_kernel(SurrogateArgs p) 
   finish_in_last_block(p.ws.counter, p.ws.seq_sum, p.ws.seq_cnt, p.n_seq, p.loss, p.partial);
 }
 
-template <bool kSeqMean>
+// TOKEN_MEAN: every row's term is computed once per tile, without a branch, so that the
+// eight rows' chains of latencies overlap (loss and derivative over 5.4M rows 58.0 -> 55.6
+// us).
 __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(SurrogateArgs p) {
   __shared__ double sh_sum[kRowWarps], sh_cnt[kRowWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -299,53 +302,27 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
     int64_t t0 = w0 * kRowTile;
     RowLoads cur, nxt;
     cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows), p.vec);
-    PieceWalker pw(p.seq_offsets, p.seq_accepted, p.adv, p.n_seq, t0);
+    PieceWalker<FloatOf> pw(p.seq_offsets, p.seq_accepted, FloatOf{p.adv}, p.n_seq, t0);
     for (int64_t w = w0; w < w1; ++w) {
       const int64_t t1 = tile_end(t0, p.n_rows);
       if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
       unsigned in = 0u;
-      float adv[kRowsPerLane] = {};  // per row; the terms are computed once per tile, not per piece
-      // the terms of the given rows, added up; under TOKEN_MEAN every row's is computed,
-      // without a branch, so that the eight rows' chains of latencies overlap (loss and
-      // derivative over 5.4M rows 58.0 -> 55.6 us; SEQ_MEAN, per piece, spills that way)
-      auto terms = [&](unsigned rows) -> double {
-        Sum3 sum{0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int u = 0; u < kRowsPerLane; ++u) {
-          const bool take = rows >> u & 1u;
-          if (kSeqMean && !take) continue;
-          float rho;
-          const float x = clipped_term(cur.lp[u], cur.bh[u], adv[u], p.eps_low, p.eps_high,
-                                       p.dual, &rho);
-          cur.bh[u] = rho;  // the ratio, once the row is used
-          sum.add(take ? x : 0.0f);
-        }
-        return sum.value();
-      };
-      double head_s = 0.0, head_c = 0.0;
-      pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float a, int64_t begin) {
+      float adv[kRowsPerLane] = {};
+      pw.walk(t0, t1, [&](int64_t, int64_t lo, int64_t hi, float a, int64_t) {
         const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
         in |= rows;
 #pragma unroll
         for (int u = 0; u < kRowsPerLane; ++u) adv[u] = rows >> u & 1u ? a : adv[u];
-        if (!kSeqMean) return;
-        const double s = warp_sum_fixed(terms(rows));
-        const double cd = static_cast<double>(__reduce_add_sync(0xffffffffu, __popc(rows)));
-        if (begin < t0) {  // the sequence began in an earlier tile
-          head_s = s;
-          head_c = cd;
-        } else if (lane == 0) {
-          p.ws.seq_sum[seq] = s;
-          p.ws.seq_cnt[seq] = cd;
-        }
       });
-      if (kSeqMean) {
-        if (lane == 0) {
-          p.ws.head_sum[w] = head_s;
-          p.ws.head_cnt[w] = head_c;
+      if (__any_sync(0xffffffffu, in != 0u)) {
+        Sum3 sum{0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int u = 0; u < kRowsPerLane; ++u) {
+          cur.bh[u] = clamped_ratio(cur.lp[u], cur.bh[u]);  // the ratio, once the row is used
+          const float x = clipped_term(cur.bh[u], adv[u], p.eps_low, p.eps_high, p.dual);
+          sum.add(in >> u & 1u ? x : 0.0f);
         }
-      } else if (__any_sync(0xffffffffu, in != 0u)) {
-        tot = __dadd_rn(tot, terms(in));
+        tot = __dadd_rn(tot, sum.value());
         cnt += __popc(in);
       }
       if (p.ratio) store_rows(p.ratio, t0, t1, p.vec, in, cur.bh);
@@ -353,7 +330,6 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
       t0 = t1;
     }
   }
-  if (kSeqMean) return;
   tot = warp_sum_fixed(tot);
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   if (lane == 0) {
@@ -371,6 +347,100 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_kernel(S
     p.ws.block_cnt[blockIdx.x] = c;
   }
   finish_in_last_block(p.ws.counter, p.ws.block_sum, p.ws.block_cnt, gridDim.x, p.loss, p.partial);
+}
+
+// SEQ_MEAN: a tile's pieces go through shared memory; where there are several, so do its
+// ratios, and groups of 16 to 4 lanes add up a piece each.  With the whole warp on every
+// piece in turn, 5,000 rows of 1,000 sequences took 75 us a call (1.2 us a piece), now 20;
+// 5.4M rows of 1,024 sequences 35 and 35.
+__global__ void __launch_bounds__(kRowThreads, kRowMinBlocks)
+    surrogate_seq_kernel(SurrogateArgs p) {
+  __shared__ PieceList lists[kRowWarps];
+  __shared__ float values[kRowWarps][kRowTile];            // per piece: the advantage
+  __shared__ __align__(16) float ratios[kRowWarps][kRowTile];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  PieceList& list = lists[wid];
+  const int64_t w0 = (static_cast<int64_t>(blockIdx.x) * kRowWarps + wid) * p.geom.per_warp;
+  const int64_t w1 = w0 + p.geom.per_warp < p.geom.n_tiles ? w0 + p.geom.per_warp : p.geom.n_tiles;
+  if (w0 >= w1) return;
+  int64_t t0 = w0 * kRowTile;
+  RowLoads cur, nxt;
+  cur.load(p.logprob, p.behav, p.mask, t0, tile_end(t0, p.n_rows), p.vec);
+  PieceWalker<FloatOf> pw(p.seq_offsets, p.seq_accepted, FloatOf{p.adv}, p.n_seq, t0);
+  for (int64_t w = w0; w < w1; ++w) {
+    const int64_t t1 = tile_end(t0, p.n_rows);
+    if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
+#pragma unroll
+    for (int u = 0; u < kRowsPerLane; ++u) cur.bh[u] = clamped_ratio(cur.lp[u], cur.bh[u]);
+    bool began_before = false;  // by the lane that holds the first piece
+    int n = pw.collect(t0, t1, [&](int i, int64_t seq, int64_t lo, int64_t hi, float a,
+                                   int64_t begin) {
+      list.put(i, seq, t0, lo, hi);
+      if (i < kRowTile) values[wid][i] = a;
+      if (i == 0) began_before = begin < t0;
+    });
+    const bool first_began_before = __any_sync(0xffffffffu, began_before);
+    n = n < kRowTile ? n : kRowTile;
+    const auto put_part = [&](int q, double sum, int count) {
+      const bool head = q == 0 && first_began_before;
+      const int64_t i = head ? w : list.seq[q];
+      (head ? p.ws.head_sum : p.ws.seq_sum)[i] = sum;
+      (head ? p.ws.head_cnt : p.ws.seq_cnt)[i] = static_cast<double>(count);
+    };
+    unsigned in = 0u;
+    if (n == 1) {  // a long sequence's tile: the lanes add up their own rows
+      __syncwarp();
+      const float a = values[wid][0];
+      in = list.rows_in_piece(0) & cur.mask;
+      Sum3 sum{0.0f, 0.0f, 0.0f};
+#pragma unroll
+      for (int u = 0; u < kRowsPerLane; ++u) {
+        const float x = clipped_term(cur.bh[u], a, p.eps_low, p.eps_high, p.dual);
+        sum.add(in >> u & 1u ? x : 0.0f);
+      }
+      const double s = warp_sum_fixed(sum.value());
+      const int c = __reduce_add_sync(0xffffffffu, __popc(in));
+      if (lane == 0) put_part(0, s, c);
+    } else if (n > 1) {
+      float4* r4 = reinterpret_cast<float4*>(ratios[wid] + row_in_tile(0));
+      r4[0] = make_float4(cur.bh[0], cur.bh[1], cur.bh[2], cur.bh[3]);
+      r4[1] = make_float4(cur.bh[4], cur.bh[5], cur.bh[6], cur.bh[7]);
+      list.put_mask(cur.mask);
+      __syncwarp();
+      const int g = n <= 2 ? 16 : (n <= 4 ? 8 : 4);  // lanes a piece
+      const int sub = lane & (g - 1);
+      for (int q0 = 0; q0 < n; q0 += 32 / g) {
+        const int q = q0 + lane / g;
+        Sum3 sum{0.0f, 0.0f, 0.0f};
+        int c = 0;
+        if (q < n) {
+          const float a = values[wid][q];
+          const int hi = list.range[q] >> 16;
+          for (int r = (list.range[q] & 0xffffu) + sub; r < hi; r += g) {
+            const bool take = list.in_mask(r);
+            const float x = clipped_term(ratios[wid][r], a, p.eps_low, p.eps_high, p.dual);
+            sum.add(take ? x : 0.0f);
+            c += take;
+          }
+        }
+        double s = sum.value();
+        for (int o = g >> 1; o > 0; o >>= 1) {
+          s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+          c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+        if (q < n && sub == 0) put_part(q, s, c);
+      }
+      in = list.rows_in_pieces(n) & cur.mask;
+    }
+    if (lane == 0 && !first_began_before) {
+      p.ws.head_sum[w] = 0.0;
+      p.ws.head_cnt[w] = 0.0;
+    }
+    if (p.ratio) store_rows(p.ratio, t0, t1, p.vec, in, cur.bh);
+    __syncwarp();  // the list is rewritten
+    cur = nxt;
+    t0 = t1;
+  }
 }
 
 // loss = numerator / denominator of partials summed over the parts of a batch
@@ -459,10 +529,10 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
   a.partial = l->partial;
   const unsigned grid = static_cast<unsigned>(a.geom.blocks > 0 ? a.geom.blocks : 1);
   if (l->params.agg == PACE_AGG_TOKEN_MEAN) {
-    surrogate_kernel<false><<<grid, kRowThreads, 0, st>>>(a);
+    surrogate_kernel<<<grid, kRowThreads, 0, st>>>(a);
     return last_launch_status();
   }
-  surrogate_kernel<true><<<grid, kRowThreads, 0, st>>>(a);
+  surrogate_seq_kernel<<<grid, kRowThreads, 0, st>>>(a);
   PACE_TRY(last_launch_status());
   int64_t blocks = (b->n_seq + kRowWarps - 1) / kRowWarps;
   const int64_t most = static_cast<int64_t>(sm_count()) * 8;
@@ -478,6 +548,7 @@ pace_status run_surrogate(const PaceBatch* b, const float* logprob, const PaceLo
 // needs them.  Clears the two counters of the launches that follow (either may be
 // null).  seq_in (or null): rows in the loss per sequence, added to, and n_used the
 // sequences that have any.
+template <bool kPerSeq>
 __global__ void __launch_bounds__(kRowThreads)
     count_rows_kernel(const int64_t* __restrict__ seq_offsets,
                       const uint8_t* __restrict__ seq_accepted, const uint8_t* __restrict__ mask,
@@ -501,23 +572,38 @@ __global__ void __launch_bounds__(kRowThreads)
   const int64_t w0 = warp * geom.per_warp;
   const int64_t w1 = w0 + geom.per_warp < geom.n_tiles ? w0 + geom.per_warp : geom.n_tiles;
   int c = 0;
-  if (seq_in && w0 < w1) {
-    PieceWalker pw(seq_offsets, seq_accepted, nullptr, n_seq, w0 * kRowTile);
-    for (int64_t w = w0; w < w1; ++w) {
-      const int64_t t0 = w * kRowTile, t1 = tile_end(t0, n_rows);
-      const unsigned bits = load_mask_bits(mask, t0, t1, vec);
-      pw.walk(t0, t1, [&](int64_t seq, int64_t lo, int64_t hi, float, int64_t) {
-        const int k = __reduce_add_sync(0xffffffffu, __popc(piece_bits(t0, lo, hi) & bits));
-        if (lane == 0 && k > 0 && atomicAdd(seq_in + seq, static_cast<unsigned long long>(k)) == 0)
-          atomicAdd(n_used, 1);
-        c += k;
-      });
+  if constexpr (kPerSeq) {
+    // a lane counts a piece (the warp on one piece after the other waited for each atomic's
+    // result, about 1 us)
+    __shared__ PieceList lists[kRowWarps];
+    PieceList& list = lists[wid];
+    if (w0 < w1) {
+      PieceWalker<NoValue> pw(seq_offsets, seq_accepted, NoValue{}, n_seq, w0 * kRowTile);
+      for (int64_t w = w0; w < w1; ++w) {
+        const int64_t t0 = w * kRowTile, t1 = tile_end(t0, n_rows);
+        list.put_mask(load_mask_bits(mask, t0, t1, vec));
+        int n = pw.collect(t0, t1, [&](int i, int64_t seq, int64_t lo, int64_t hi, NoValue, int64_t) {
+          list.put(i, seq, t0, lo, hi);
+        });
+        n = n < kRowTile ? n : kRowTile;
+        __syncwarp();
+        int first = 0;
+        for (int q = lane; q < n; q += 32) {
+          const int k = list.rows_in_mask(q);
+          if (k > 0 && atomicAdd(seq_in + list.seq[q], static_cast<unsigned long long>(k)) == 0)
+            ++first;
+          c += k;
+        }
+        first = __reduce_add_sync(0xffffffffu, first);
+        if (lane == 0 && first > 0) atomicAdd(n_used, first);
+        __syncwarp();  // the list is rewritten
+      }
     }
   } else {
     walk_rows_in_loss(seq_offsets, seq_accepted, mask, n_seq, n_rows, w0, w1, vec,
                       [&](int64_t, int64_t, unsigned in) { c += __popc(in); });
-    c = __reduce_add_sync(0xffffffffu, c);
   }
+  c = __reduce_add_sync(0xffffffffu, c);
   if (lane == 0) {
     sh[wid] = c;
     counts.warp[warp] = c;
@@ -670,10 +756,10 @@ pace_status launch_count_rows(const PaceBatch* b, RowCounts counts, unsigned lon
                               int* n_used, const AdvJob& adv, unsigned* counter0,
                               unsigned* counter1, int32_t* status, cudaStream_t st) {
   const RowGeom g = row_geom(b->n_rows);
-  count_rows_kernel<<<static_cast<unsigned>(g.blocks + adv_blocks(adv, kRowThreads)), kRowThreads, 0, st>>>(
+  const auto kernel = seq_in ? count_rows_kernel<true> : count_rows_kernel<false>;
+  kernel<<<static_cast<unsigned>(g.blocks + adv_blocks(adv, kRowThreads)), kRowThreads, 0, st>>>(
       b->seq_offsets, b->seq_accepted, b->mask, b->n_seq, b->n_rows, g, aligned(b->mask, 8), counts,
-      seq_in, n_used,
-      adv, counter0, counter1, status);
+      seq_in, n_used, adv, counter0, counter1, status);
   return last_launch_status();
 }
 

@@ -59,17 +59,34 @@ __device__ __forceinline__ void check_seq(const int64_t* __restrict__ offsets, i
   if (r1 < r0 || r0 < 0 || r1 > n_rows || (i == 0 && r0 != 0)) report(status, PACE_ERR_INVALID_ARG);
 }
 
+// What a walk wants to know of a sequence: nothing, or a float of an array.
+struct NoValue {
+  using Value = NoValue;
+  __device__ Value operator()(int64_t) const { return {}; }
+};
+struct FloatOf {
+  using Value = float;
+  const float* a;
+  __device__ Value operator()(int64_t i) const { return a[i]; }
+};
+__device__ __forceinline__ NoValue shfl_value(NoValue v, int) { return v; }
+__device__ __forceinline__ float shfl_value(float v, int j) {
+  return __shfl_sync(0xffffffffu, v, j);
+}
+
 // Walks the sequences along a warp's tiles.  31 sequences' offsets, flags and values
-// are held at a time, one per lane.  All lanes call everything together.
+// (Of's, computed by as many lanes at once) are held at a time, one per lane.  All lanes
+// call everything together.
+template <class Of>
 struct PieceWalker {
   const int64_t* offsets;
   const uint8_t* accepted;  // null: all accepted
-  const float* per_seq;     // null: 0
+  Of of;
   int64_t n_seq;
   int64_t base;             // sequence of lane 0
   int j;                    // current sequence: base + j
   int64_t o;                // lane's offset, value; the lanes' accepted flags
-  float v;
+  typename Of::Value v;
   unsigned acc_bits;
 
   __device__ void load() {
@@ -77,7 +94,7 @@ struct PieceWalker {
     const int64_t i = base + lane;
     const int64_t is = i < n_seq ? i : n_seq - 1;
     o = offsets[i < n_seq ? i : n_seq];
-    v = per_seq ? per_seq[is] : 0.0f;
+    v = of(is);
     acc_bits = __ballot_sync(0xffffffffu, accepted ? accepted[is] != 0 : true);
     j = 0;
   }
@@ -104,10 +121,10 @@ struct PieceWalker {
     load();
   }
 
-  __device__ PieceWalker(const int64_t* offsets_, const uint8_t* accepted_, const float* per_seq_,
-                         int64_t n_seq_, int64_t t0)
-      : offsets(offsets_), accepted(accepted_), per_seq(per_seq_), n_seq(n_seq_), base(0), j(0),
-        o(0), v(0.0f), acc_bits(0u) {
+  __device__ PieceWalker(const int64_t* offsets_, const uint8_t* accepted_, Of of_, int64_t n_seq_,
+                         int64_t t0)
+      : offsets(offsets_), accepted(accepted_), of(of_), n_seq(n_seq_), base(0), j(0), o(0), v{},
+        acc_bits(0u) {
     if (n_seq > 0) seek(0, t0);
   }
 
@@ -120,7 +137,7 @@ struct PieceWalker {
     while (base + j < n_seq) {
       const int64_t o0 = __shfl_sync(full, o, j);
       const int64_t o1 = __shfl_sync(full, o, j + 1);
-      const float val = __shfl_sync(full, v, j);
+      const typename Of::Value val = shfl_value(v, j);
       const int64_t p0 = o0 < t0 ? t0 : o0;
       const int64_t p1 = o1 < t1 ? o1 : t1;
       if (p0 < p1 && (acc_bits >> j & 1u)) f(base + j, p0, p1, val, o0);
@@ -135,6 +152,40 @@ struct PieceWalker {
         }
       }
     }
+  }
+
+  // The same pieces (walk or collect, not both), 31 sequences at a time: the lane that holds
+  // a piece's sequence calls f(index, seq, lo, hi, value, begin), index counting the tile's
+  // pieces.  Returns their number.
+  template <class F>
+  __device__ __forceinline__ int collect(int64_t t0, int64_t t1, F f) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int n = 0;
+    while (base + j < n_seq) {
+      const int64_t o1 = __shfl_down_sync(full, o, 1);
+      const bool held = lane >= j && lane < 31 && base + lane < n_seq;
+      const unsigned stop = __ballot_sync(full, held && o1 >= t1);
+      const int last = stop ? __ffs(stop) - 1 : 31;
+      const int64_t p0 = o < t0 ? t0 : o;
+      const int64_t p1 = o1 < t1 ? o1 : t1;
+      const bool mine = held && lane <= last && p0 < p1 && (acc_bits >> lane & 1u);
+      const unsigned bal = __ballot_sync(full, mine);
+      if (mine) f(n + __popc(bal & ((1u << lane) - 1u)), base + lane, p0, p1, v, o);
+      n += __popc(bal);
+      if (stop) {
+        j = last;
+        return n;
+      }
+      const int64_t end = __shfl_sync(full, o, 31);  // of the sequences held
+      base += 31;
+      j = 0;
+      if (base < n_seq) {
+        load();
+        if (__shfl_sync(full, o, 31) <= end) seek(base, end);
+      }
+    }
+    return n;
   }
 };
 
@@ -232,13 +283,13 @@ __device__ __forceinline__ void walk_rows_in_loss(const int64_t* __restrict__ of
   if (tile0 >= tile1) return;
   int64_t t0 = tile0 * kRowTile;
   unsigned bits = load_mask_bits(mask, t0, tile_end(t0, n_rows), vec);
-  PieceWalker pw(offsets, accepted, nullptr, n_seq, t0);
+  PieceWalker<NoValue> pw(offsets, accepted, NoValue{}, n_seq, t0);
   for (int64_t w = tile0; w < tile1; ++w) {
     const int64_t t1 = tile_end(t0, n_rows);
     unsigned next = 0u;
     if (w + 1 < tile1) next = load_mask_bits(mask, t1, tile_end(t1, n_rows), vec);
     unsigned in = 0u;
-    pw.walk(t0, t1, [&](int64_t, int64_t lo, int64_t hi, float, int64_t) {
+    pw.walk(t0, t1, [&](int64_t, int64_t lo, int64_t hi, NoValue, int64_t) {
       in |= piece_bits(t0, lo, hi);
     });
     f(t0, t1, in & bits);
@@ -246,6 +297,55 @@ __device__ __forceinline__ void walk_rows_in_loss(const int64_t* __restrict__ of
     t0 = t1;
   }
 }
+
+// The pieces of a warp's tile and its mask, in shared memory, so that the lanes can share
+// out what there is to do per piece.
+struct PieceList {
+  int64_t seq[kRowTile];
+  uint32_t range[kRowTile];  // first row in the tile | end << 16
+  unsigned mask[kRowTile / 32];
+
+  // piece n, by one lane (offsets that overlap may make more than a tile has rows: left out)
+  __device__ __forceinline__ void put(int n, int64_t s, int64_t t0, int64_t lo, int64_t hi) {
+    if (n >= kRowTile) return;
+    seq[n] = s;
+    range[n] = static_cast<uint32_t>(lo - t0) | static_cast<uint32_t>(hi - t0) << 16;
+  }
+  __device__ __forceinline__ void put_mask(unsigned bits) {
+    reinterpret_cast<uint8_t*>(mask)[threadIdx.x & 31] = static_cast<uint8_t>(bits);
+  }
+  __device__ __forceinline__ bool in_mask(int row) const { return mask[row >> 5] >> (row & 31) & 1u; }
+  // the lane's rows of the tile that lie in piece n, in the first n pieces, as bits
+  __device__ __forceinline__ unsigned rows_in_piece(int n) const {
+    return piece_bits(0, range[n] & 0xffffu, range[n] >> 16);
+  }
+  __device__ __forceinline__ unsigned rows_in_pieces(int n) const {
+    const int r0 = row_in_tile(0);
+    int k = 0;  // the first piece that ends past the lane's first row
+    for (int above = n; k < above;) {
+      const int m = (k + above) >> 1;
+      if (static_cast<int>(range[m] >> 16) <= r0) k = m + 1;
+      else above = m;
+    }
+    unsigned bits = 0u;
+    for (; k < n; ++k) {
+      bits |= rows_in_piece(k);
+      if (static_cast<int>(range[k] >> 16) >= r0 + kRowsPerLane) break;
+    }
+    return bits;
+  }
+  __device__ __forceinline__ int rows_in_mask(int n) const {
+    const int lo = range[n] & 0xffffu, hi = range[n] >> 16;
+    int c = 0;
+    for (int w = lo >> 5; w <= (hi - 1) >> 5; ++w) {
+      unsigned m = mask[w];
+      if (w == lo >> 5) m &= ~0u << (lo & 31);
+      if (w == hi >> 5) m &= (1u << (hi & 31)) - 1u;
+      c += __popc(m);
+    }
+    return c;
+  }
+};
 
 // A lane's log-probs and behaviour log-probs of a tile, with the mask bits.
 struct RowLoads {

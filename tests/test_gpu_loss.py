@@ -278,6 +278,37 @@ def test_runs_of_empty_sequences_are_not_walked(call):
     assert min(times) < 3.0  # ms
 
 
+def test_short_sequences_share_a_tile():
+    """The sequence mean over 5,000 rows of 1,000 sequences: with a tile's pieces taken one
+    by one the loss took 75 us and the derivative 95, shared out among the lanes 20 and 17."""
+    n, n_seq = 5000, 1000
+    so = to_dev(np.arange(n_seq + 1, dtype=np.int64) * (n // n_seq))
+    b = pace.make_batch(so, n)
+    lp, dlp = torch.zeros(n, device=DEV), torch.empty(n, device=DEV)
+    loss = torch.zeros(1, dtype=torch.float64, device=DEV)
+    la = pace.make_loss_args(lp, torch.rand(n_seq, device=DEV), 8,
+                             pace.loss_params(agg=pace.AGG_SEQ_MEAN_TOKEN_MEAN), loss)
+    L = pace.lib()
+    ws = pace.workspace(L.pace_surrogate_loss_workspace_size(n, n_seq), DEV)
+    ws_b = pace.workspace(L.pace_surrogate_backward_workspace_size(n, n_seq), DEV)
+    pace.surrogate_loss(b, lp, la, ws=ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(10):
+            pace.surrogate_loss(b, lp, la, ws=ws)
+            pace.surrogate_backward(b, lp, la, dlp=dlp, ws=ws_b)
+    times = []
+    for _ in range(8):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        graph.replay()
+        e1.record()
+        torch.cuda.synchronize()
+        times.append(e0.elapsed_time(e1) / 10)
+    assert min(times) < 0.09  # ms
+
+
 @pytest.mark.parametrize("agg", [pace.AGG_TOKEN_MEAN, pace.AGG_SEQ_MEAN_TOKEN_MEAN])
 @pytest.mark.parametrize("n", [8 * 256, 10_000])
 def test_rows_at_any_alignment(agg, n):
