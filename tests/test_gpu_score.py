@@ -296,6 +296,22 @@ def test_window_order(wlen, kind):
     _check(g, o, f"{kind} {wlen}")
 
 
+@pytest.mark.parametrize("wlen", [2015, 2016, 4096])
+@pytest.mark.parametrize("n_tok", [456 * 8 * 4 * 512, 456 * 8 * 12 * 512, 456 * 8 * 12 * 512 + 1])
+def test_large_windows_beside_short_streams(n_tok, wlen):
+    """Streams up to the length that leaves a large window's preparation room in its wave
+    (12 batches of 512 tags for each of 8 warps of 456 blocks), and one tag past it, with
+    windows on both sides of the size from which it does."""
+    rng = np.random.default_rng(n_tok + wlen)
+    n_traj = 4096
+    lens = np.bincount(rng.integers(0, n_traj, size=n_tok), minlength=n_traj)
+    tags, offsets, c, s_pre, j, _ = _mk_fast(lens, rng)
+    window = rng.random(wlen).astype(np.float32)
+    g = gpu_score(tags, offsets, c, s_pre, j, window, min_obs=1)
+    o = oracle_score(tags, offsets, c, s_pre, j, window, min_obs=1)
+    _check(g, o, f"{n_tok}/w{wlen}")
+
+
 @pytest.mark.parametrize("n_traj,n_tok,wlen", [(64, 0, 512), (8192, 0, 4096), (8192, 1500, 4096),
                                                 (16384, 70000, 512)])
 def test_short_streams(n_traj, n_tok, wlen):
