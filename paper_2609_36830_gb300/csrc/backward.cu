@@ -149,10 +149,12 @@ __host__ __device__ inline TailSplit tail_split(int64_t items, int n_clusters, i
   s.tail = static_cast<int>(items - s.full);
   s.splits = 1;
   int best = nkb;  // the tail's K steps
-  for (int k = 2; k <= max_k_splits(nkb); ++k) {
+  const int most = max_k_splits(nkb);
+#pragma unroll
+  for (int k = 2; k <= kMaxKSplits; ++k) {  // (unrolled: the divisions' latencies overlap)
     const int rounds = (s.tail * k + n_clusters - 1) / n_clusters;
     const int steps = rounds * ((nkb + k - 1) / k);
-    if (steps < best) {
+    if (k <= most && steps < best) {
       best = steps;
       s.splits = k;
     }

@@ -768,49 +768,70 @@ inline Float2x float2x(double x) {
 // 64 bits in units of the last place, with exact logits (0.29 is a correctly rounded
 // result), of a plain sum and lg2.approx, and so: 200 rows of V 4,096 0.51 and 0.29,
 // 20,000 rows of V 20,000 0.56 and 0.32, 2,582 rows of V 151,936 0.41 and 0.30.
-__global__ void lse_merge_kernel(int64_t rows_cap, const long long* __restrict__ n_valid_dev,
-                                 int lm_clusters, int n_vtiles, int split_pref, int32_t V,
-                                 Float2x inv_temp, Float2x max_unit,
-                                 const float* __restrict__ part_m, const float* __restrict__ part_s,
-                                 const float* __restrict__ tgt_logit,
-                                 const int32_t* __restrict__ targets,
-                                 const int32_t* __restrict__ rowidx, float* __restrict__ logprob,
-                                 float* __restrict__ lse_out, int32_t* status) {
+// Where the tail's rows have more than kMergeLanes partials, as many lanes take each row:
+// one thread's chain of 78 was 4 us of a call of 200 rows (H 1,024 / V 50,001 62.4 us with a
+// plain sum, 65.6 with its errors, 57.9 so).  Otherwise a thread a row (9,000 rows of V 64
+// 16.8 us, 17.9 with eight lanes).
+constexpr int kMergeLanes = 8;
+constexpr int kMergeThreads = 256;
+
+// sum += x; the addition's error goes to err (Knuth's two-sum).
+__device__ __forceinline__ void add_with_error(float& sum, float& err, float x) {
+  const float t = __fadd_rn(sum, x);
+  const float z = __fsub_rn(t, sum);
+  err = __fadd_rn(err, __fadd_rn(__fsub_rn(sum, __fsub_rn(t, z)), __fsub_rn(x, z)));
+  sum = t;
+}
+
+__global__ void __launch_bounds__(kMergeThreads)
+    lse_merge_kernel(int64_t rows_cap, const long long* __restrict__ n_valid_dev, int lm_clusters,
+                     int n_vtiles, int split_pref, int32_t V, Float2x inv_temp, Float2x max_unit,
+                     const float* __restrict__ part_m, const float* __restrict__ part_s,
+                     const float* __restrict__ tgt_logit, const int32_t* __restrict__ targets,
+                     const int32_t* __restrict__ rowidx, float* __restrict__ logprob,
+                     float* __restrict__ lse_out, int32_t* status) {
+  const unsigned full = 0xffffffffu;
   const int64_t n_valid = n_valid_dev ? static_cast<int64_t>(*n_valid_dev) : rows_cap;
   // how the LM head dealt these rows
   const LmPlan plan = lm_plan((n_valid + 2 * BM - 1) / (2 * BM), lm_clusters, n_vtiles, split_pref);
   const int64_t tail_row0 = plan.rounds_rp * (2 * BM);
-  for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < n_valid;
-       r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t orig = rowidx ? static_cast<int64_t>(rowidx[r]) : r;
+  const int64_t threads = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + (threadIdx.x & ~31u);
+  const int lanes = plan.tail_slots > kMergeLanes ? kMergeLanes : 1;
+  const int lane = threadIdx.x & 31, sub = lane & (lanes - 1);
+  for (int64_t t = t0; t < n_valid * lanes; t += threads) {  // lanes * the warp's first row
+    const int64_t r = (t + lane) / lanes;
+    const bool valid = r < n_valid;
     int64_t o = r * plan.splits;
     int splits = plan.splits;
     if (r >= tail_row0) {  // the clusters whose stretch meets the row pair's
       o = tail_row0 * plan.splits + (r - tail_row0) * plan.tail_slots;
-      const int i = static_cast<int>((r - tail_row0) / (2 * BM));
-      const int64_t x1 = static_cast<int64_t>(i + 1) * lm_clusters - 1;
-      splits = static_cast<int>(x1 / plan.tail_rp) -
-               tail_first_cluster(i, plan.tail_rp, lm_clusters) + 1;
+      if (valid) {
+        const int i = static_cast<int>((r - tail_row0) / (2 * BM));
+        const int64_t x1 = static_cast<int64_t>(i + 1) * lm_clusters - 1;
+        splits = static_cast<int>(x1 / plan.tail_rp) -
+                 tail_first_cluster(i, plan.tail_rp, lm_clusters) + 1;
+      }
     }
+    if (!valid) splits = 0;
     float mm = -INFINITY;
-    for (int s = 0; s < splits; ++s) mm = fmaxf(mm, part_m[o + s]);
-    float ss = 0.0f, se = 0.0f;  // the sum and its additions' errors (Knuth's two-sum)
-    for (int s = 0; s < splits; ++s) {
-      const float x = part_s[o + s] * ex2_approx(part_m[o + s] - mm);
-      const float t = __fadd_rn(ss, x);
-      const float z = __fsub_rn(t, ss);
-      se = __fadd_rn(se, __fadd_rn(__fsub_rn(ss, __fsub_rn(t, z)), __fsub_rn(x, z)));
-      ss = t;
+    for (int s = sub; s < splits; s += lanes) mm = fmaxf(mm, part_m[o + s]);
+    for (int x = lanes >> 1; x > 0; x >>= 1) mm = fmaxf(mm, __shfl_xor_sync(full, mm, x));
+    float ss = 0.0f, se = 0.0f;  // the sum and its additions' errors
+    for (int s = sub; s < splits; s += lanes)
+      add_with_error(ss, se, part_s[o + s] * ex2_approx(part_m[o + s] - mm));
+    for (int x = lanes >> 1; x > 0; x >>= 1) {
+      const float s2 = __shfl_xor_sync(full, ss, x);
+      se = __fadd_rn(se, __shfl_xor_sync(full, se, x));
+      add_with_error(ss, se, s2);
     }
+    if (!valid || sub != 0) continue;
     // lse = (largest logit) / tau + ln(sum): mm counts in units of 1 / (tau scale_log2)
     const float a = __fmul_rn(mm, max_unit.hi);
-    const float a_lo = __fmaf_rn(mm, max_unit.lo, __fmaf_rn(mm, max_unit.hi, -a));
-    const float l = logf(ss);
-    const float h = __fadd_rn(a, l);
-    const float z = __fsub_rn(h, a);
-    const float h_lo = __fadd_rn(__fadd_rn(__fsub_rn(a, __fsub_rn(h, z)), __fsub_rn(l, z)),
-                                 __fadd_rn(a_lo, __fdividef(se, ss)));
-    const float lse = __fadd_rn(h, h_lo);
+    float h = a, h_lo = __fadd_rn(__fmaf_rn(mm, max_unit.lo, __fmaf_rn(mm, max_unit.hi, -a)),
+                                  __fdividef(se, ss));
+    add_with_error(h, h_lo, logf(ss));
+    const int64_t orig = rowidx ? static_cast<int64_t>(rowidx[r]) : r;
     const int32_t y = targets[orig];
     float lp;
     if (y < 0 || y >= V) {
@@ -822,7 +843,7 @@ __global__ void lse_merge_kernel(int64_t rows_cap, const long long* __restrict__
       lp = __fadd_rn(__fmaf_rn(zy, inv_temp.hi, -h), low);
     }
     logprob[orig] = lp;
-    if (lse_out) lse_out[orig] = lse;
+    if (lse_out) lse_out[orig] = __fadd_rn(h, h_lo);
   }
 }
 
@@ -993,10 +1014,11 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
       compact && n_rows >= BM && 2.0 * H * V * static_cast<double>(n_rows) >= kFineFlops;
   PACE_TRY(fine ? launch_lmhead<true>(l, a, st) : launch_lmhead<false>(l, a, st));
   if (pe.end) PACE_TRY_CUDA(cudaEventRecord(pe.end, st));
-  int64_t mblocks = (rows_cap + 255) / 256;
+  const int64_t per_block = kMergeThreads / kMergeLanes;
+  int64_t mblocks = (rows_cap + per_block - 1) / per_block;
   const int64_t cap = static_cast<int64_t>(sm_count()) * 8;
   if (mblocks > cap) mblocks = cap;
-  lse_merge_kernel<<<static_cast<unsigned>(mblocks), 256, 0, st>>>(
+  lse_merge_kernel<<<static_cast<unsigned>(mblocks), kMergeThreads, 0, st>>>(
       rows_cap, n_valid_dev, static_cast<int>(clusters), n_vtiles, a.split_pref, V,
       float2x(1.0 / temperature),
       float2x(1.0 / (static_cast<double>(temperature) * a.scale_log2)), ws.part_m, ws.part_s,
