@@ -1435,6 +1435,7 @@ __global__ void __launch_bounds__(kAdmitThreads)
     // the ring's newest n values, in any order (one thread does the fp64 work: GB300's
     // fp64 pipe is narrow)
     if (t == 0) {
+      s_kappa = -0.0;
       const long long k = static_cast<long long>(
           ceil(__dsub_rn(__dmul_rn(__dsub_rn(1.0, r), static_cast<double>(n)), 1e-9)));
       s_kth = k < 1 ? 1 : (k > n ? n : k);
@@ -1451,11 +1452,14 @@ __global__ void __launch_bounds__(kAdmitThreads)
     const uint64_t pivot =
         block_kth_smallest(key, static_cast<int>(n), static_cast<int>(s_kth));
 #pragma unroll
-    for (int s = 0; s < kAdmitSlots; ++s) {  // a value with that key (either zero has it)
+    for (int s = 0; s < kAdmitSlots; ++s) {  // the value with that key; of the two zeros, +0
       const int i = t + s * kAdmitThreads;
       long long at = head - n + i;
       if (at < 0) at += capacity;
-      if (i < n && key[s] == pivot) s_kappa = window[at];
+      if (i < n && key[s] == pivot) {
+        const long long bits = __double_as_longlong(window[at]);
+        if (bits != static_cast<long long>(1ull << 63)) s_kappa = __longlong_as_double(bits);
+      }
     }
     __syncthreads();
     kappa = s_kappa;

@@ -192,3 +192,19 @@ def test_histogram_where_the_width_overflows():
     want[1, [0, n_bins - 1]] = 3, 1
     hist = pace.staleness_histogram(to_dev(x), to_dev(flags), lo, hi, n_bins)
     np.testing.assert_array_equal(as_np(hist).astype(np.uint32), want)
+
+
+@pytest.mark.parametrize("order", ["-+", "+-", "--", "++"])
+@pytest.mark.parametrize("at", [(10, 11), (10, 40), (10, 590)])  # one warp, two, two passes
+def test_kappa_of_both_zeros(at, order):
+    """A threshold of zero is +0 where the window holds one, whichever thread has it, and
+    -0 where every zero in it is."""
+    zeros = {"-": -0.0, "+": 0.0}
+    win = pace.ScoreWindow(600, DEV)
+    vals = np.full(600, 5.0)
+    vals[at[0]], vals[at[1]] = zeros[order[0]], zeros[order[1]]  # the two smallest
+    win.values.copy_(to_dev(vals))
+    win.state[0] = 600
+    _, kappa = pace.quantile_admit(to_dev(np.ones(3)), 1.0 - 1.0 / 600, 0, win)
+    got = as_np(kappa)[0]
+    assert got == 0.0 and np.signbit(got) == ("+" not in order)
