@@ -112,8 +112,8 @@ PACE_API void pace_score_params_default(PaceScoreParams* p);
  * S = sum (c - v_t) summed exactly in integers (0 when T = 0); q = count of
  * window values <= s_pre (float32 compare) / |W|; integer powers by repeated
  * multiplication; no fused multiply-add anywhere.
- * Launches: the tag stream (one wave, whose blocks also sort the window and
- * tabulate F on pools of 8,192 trajectories and more) and a finalisation
+ * Launches: the tag stream (one wave of blocks, after them blocks that sort the
+ * window and tabulate F where it is long enough to count) and a finalisation
  * launch; from 2^18 trajectories (pace_set_score_fused_min_traj) the stream is
  * a cooperative launch that also finalises, each block waiting (bounded) for
  * the blocks that streamed its groups' tokens.
@@ -589,7 +589,7 @@ PACE_API pace_status pace_set_profile_events(int32_t kernel, void* begin, void* 
  *   q_fp64[i] = the same quotient from the fp64 pipe, __ll2double_rn(S[i]) then
  *               a correctly rounded division (the rounding the oracle's
  *               (double)S / (double)T performs),
- *   c_int[i], c_fp64[i] = (double)S[i] both ways.
+ *   c_int[i], c_fp64[i] = (double)S[i] both ways (c_int as the quotient by 1).
  * The two must agree bit for bit.  All arrays are device arrays of n entries.
  * Returns PACE_ERR_INVALID_ARG for n < 0 or a NULL array when n > 0. */
 PACE_API pace_status pace_div_selftest(const int64_t* S, const uint32_t* T, int64_t n,

@@ -32,9 +32,10 @@ constexpr int kReduceThreads = 256;  // 8 warps
 constexpr int kTileTokens = 128;     // one int4 per lane
 // Tiles of a warp's batch (128 tokens each), two register sets of them in flight in
 // turn, and resident blocks per SM: 24 warps with 80 registers keep 48-96 KB of loads
-// in flight per SM, which is what the memory needs.  No L2 prefetch runs beside them:
-// one of four batches ahead held every pool back (the prefetched lines compete with the
-// loads).  Whole scoring + selection calls, graph replay: 20k pool 72.0 -> 66.7 us, 128k
+// in flight per SM, which is what the memory needs.  No L2 prefetch runs beside them (only
+// a range's first two batches are asked for early, before the search for its first
+// trajectory): one of four batches ahead held every pool back (the prefetched lines compete
+// with the loads).  Whole scoring + selection calls, graph replay: 20k pool 72.0 -> 66.7 us, 128k
 // 316 -> 282, 1M 2203 -> 2129; pace_stale_k on 128k 293 -> 257.  Measured without the
 // prefetch (tiles x blocks per SM, 128k / 1M pool): 8 x 2 337 us / 2.51 ms, 6 x 3 288 /
 // 2.13, 4 x 4 296 / 2.16 (spills), 3 x 4 289 / 2.13, 2 x 6 367 / 3.0, one register set
@@ -103,36 +104,10 @@ constexpr int64_t kRoomBatches = 12;
 
 // ---- exact integer quotients without the fp64 pipe
 //
-// GB300's fp64 pipe is narrow.  The functions below build the same doubles from
-// integer arithmetic: the result of __ddiv_rn(__ll2double_rn(S), T) for 64-bit S and
-// 32-bit T > 0, and of __ll2double_rn(x), bit for bit.  pace_stale_k's quotients are
-// built this way (as fast as in fp64 there); the scores' finalisation divides in fp64.
-
-// (double)x rounded to nearest even, from its bits (every int64 is in range).
-__device__ __forceinline__ double i64_to_double_rn(long long x) {
-  if (x == 0) return 0.0;
-  const unsigned long long sign = x < 0 ? (1ull << 63) : 0ull;
-  unsigned long long a = x < 0 ? 0ull - static_cast<unsigned long long>(x)
-                               : static_cast<unsigned long long>(x);
-  int top = 63 - __clzll(static_cast<long long>(a));  // leading bit position
-  unsigned long long mant;
-  if (top <= 52) {
-    mant = a << (52 - top);
-  } else {
-    const int sh = top - 52;  // bits dropped, 1..11
-    mant = a >> sh;
-    const unsigned long long rem = a & ((1ull << sh) - 1);
-    const unsigned long long half = 1ull << (sh - 1);
-    if (rem > half || (rem == half && (mant & 1ull))) ++mant;
-    if (mant >> 53) {  // carried into a new bit: 2^53 -> 2^52 one binade up
-      mant >>= 1;
-      ++top;
-    }
-  }
-  const unsigned long long bits = sign | (static_cast<unsigned long long>(top + 1023) << 52) |
-                                  (mant & ((1ull << 52) - 1));
-  return __longlong_as_double(static_cast<long long>(bits));
-}
+// GB300's fp64 pipe is narrow.  The function below builds the same double from integer
+// arithmetic: the result of __ddiv_rn(__ll2double_rn(S), T) for 64-bit S and 32-bit T > 0,
+// bit for bit.  pace_stale_k's quotients are built this way (as fast as in fp64 there); the
+// scores' finalisation divides in fp64.
 
 // RN(RN53(S) / T): exactly __ddiv_rn(__ll2double_rn(S), (double)T), T >= 1.
 // |S| is first rounded to 53 significant bits (a * 2^e, a < 2^53) as the
@@ -377,11 +352,6 @@ __device__ __forceinline__ void acc_group(LaneAcc& a, const int4& q) {
   }
 }
 
-// Each warp owns a contiguous range of batches (kTiles x 128 tokens) of
-// the flattened tag stream and walks the CSR offsets forward through it, so trajectories of
-// any length mix are balanced across warps.  The walk never leaves
-// [0, n_traj) and loads only tags[0, n_tokens), whatever the offsets hold;
-// inconsistent offsets are reported by the finalize kernel.
 // phi_gamma(q) of Eq. 10 with integer gamma, powers by repeated
 // multiplication, every operation rounded once (no FMA).
 __device__ __forceinline__ double sharpen(double q, int gamma) {
@@ -476,6 +446,12 @@ __device__ void window_prep_block(int b, const WindowPrep& w) {
   }
 }
 
+// Each warp owns a contiguous range of batches (kTiles x 128 tokens) of
+// the flattened tag stream and walks the CSR offsets forward through it, so trajectories of
+// any length mix are balanced across warps.  The walk never leaves
+// [0, n_traj) and loads only tags[0, n_tokens), whatever the offsets hold;
+// inconsistent offsets are reported by the finalize kernel.
+//
 // One warp's share of the stream (every warp of the first n_stream_blocks
 // blocks calls it; it returns early when the range is empty or the offsets end
 // before the tokens do).
@@ -636,7 +612,6 @@ struct FinalizeArgs {
   int32_t window_len;
   int32_t window_ready;
   int32_t mode;
-  int32_t gamma;
   int32_t group_size;
   double inv_group;             // 1 / G for G a power of two (exact), else 0
   double f_missing;
@@ -1265,7 +1240,6 @@ extern "C" pace_status pace_score_pool(const int32_t* tags, const int64_t* offse
   a.window_len = window_ready ? static_cast<int32_t>(window_len) : 0;
   a.window_ready = window_ready ? 1 : 0;
   a.mode = params->mode;
-  a.gamma = params->gamma;
   a.group_size = G;
   a.inv_group = (G & (G - 1)) == 0 ? 1.0 / static_cast<double>(G) : 0.0;
   a.f_missing = params->f_missing;
@@ -1329,7 +1303,7 @@ __global__ void div_selftest_kernel(const long long* __restrict__ S,
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     q_int[i] = i64_div_u32_rn(S[i], T[i]);
     q_fp64[i] = __ddiv_rn(__ll2double_rn(S[i]), __ull2double_rn(T[i]));
-    c_int[i] = i64_to_double_rn(S[i]);
+    c_int[i] = i64_div_u32_rn(S[i], 1u);
     c_fp64[i] = __ll2double_rn(S[i]);
   }
 }

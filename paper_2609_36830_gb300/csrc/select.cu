@@ -187,10 +187,10 @@ __global__ void __launch_bounds__(kSmallThreads)
 }
 
 // kSmallMax < U <= 131,072: one launch of one thread-block cluster of C CTAs (1, 2,
-// 4 or 8; 1024 threads each).  CTA r owns the contiguous units
-// [r * B, r * B + B) with B = ceil(U / C) <= 16,384; its thread t owns the
-// contiguous units t * per .. t * per + per - 1 of that range (per, a power of
-// two, <= 16), whose order keys sit in shared memory at [i * (1024 + 1) + t], so
+// 4 or 8; kT threads each: 512 where one CTA has up to 4,096 units, else 1,024).  CTA r
+// owns the contiguous units [r * B, r * B + B) with B = ceil(U / C) <= 16,384; its
+// thread t owns the contiguous units t * per .. t * per + per - 1 of that range (per, a
+// power of two, <= 16), whose order keys sit in shared memory at [i * (kT + 1) + t], so
 // a warp's accesses are conflict-free.
 //
 // The k-th largest key (the pivot) is found by a radix select that adapts to
@@ -200,10 +200,10 @@ __global__ void __launch_bounds__(kSmallThreads)
 // each CTA counts its own keys and sums the C histograms through distributed
 // shared memory.  Once the pivot's digit holds at most kSelList candidates (after one
 // round, on spread-out scores), no further round is taken: every CTA lists its own,
-// and one warp of each ranks them all against each other (finish_list).  Candidates in one round share every bit above that one, so a
-// round fixes at least one bit and there are at most 64 rounds.  Every CTA computes the same values from the same shared
-// data, so all of them take the same branches and pass the same sequence of
-// cluster barriers.
+// and one warp of each ranks them all against each other (finish_list).  Candidates in
+// one round share every bit above that one, so a round fixes at least one bit and there
+// are at most 64 rounds.  Every CTA computes the same values from the same shared data,
+// so all of them take the same branches and pass the same sequence of cluster barriers.
 //
 // Then each CTA counts its keys above and equal to the pivot, learns the
 // counts of the lower-ranked CTAs (ties are rejected lowest id first), lists
