@@ -750,24 +750,10 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();  // the collective release is complete in both CTAs
 }
 
-// x in two floats: hi + lo is x to about 48 bits.
-struct Float2x {
-  float hi, lo;
-};
-inline Float2x float2x(double x) {
-  Float2x f;
-  f.hi = static_cast<float>(x);
-  f.lo = static_cast<float>(x - static_cast<double>(f.hi));
-  return f;
-}
-
 // Per row in the loss: log-sum-exp from the split partials, then
 // lp = z_y / tau - lse, scattered back to the original row.  Up to 78 partials a row are
-// merged, so the sum keeps its additions' errors, and the result is put together in two
-// floats (the largest logit is not scaled to base 2 and back).  Rms error of lse against
-// 64 bits in units of the last place, with exact logits (0.29 is a correctly rounded
-// result), of a plain sum and lg2.approx, and so: 200 rows of V 4,096 0.51 and 0.29,
-// 20,000 rows of V 20,000 0.56 and 0.32, 2,582 rows of V 151,936 0.41 and 0.30.
+// merged, so the sum keeps its additions' errors: a plain sum drops each partial below half
+// a last place of the sum so far, 75 of them 4e-6 in all, where sums of 8 partials kept most.
 // Where the tail's rows have more than kMergeLanes partials, as many lanes take each row:
 // one thread's chain of 78 was 4 us of a call of 200 rows (H 1,024 / V 50,001 62.4 us with a
 // plain sum, 65.6 with its errors, 57.9 so).  Otherwise a thread a row (9,000 rows of V 64
@@ -785,7 +771,7 @@ __device__ __forceinline__ void add_with_error(float& sum, float& err, float x) 
 
 __global__ void __launch_bounds__(kMergeThreads)
     lse_merge_kernel(int64_t rows_cap, const long long* __restrict__ n_valid_dev, int lm_clusters,
-                     int n_vtiles, int split_pref, int32_t V, Float2x inv_temp, Float2x max_unit,
+                     int n_vtiles, int split_pref, int32_t V, float inv_temp,
                      const float* __restrict__ part_m, const float* __restrict__ part_s,
                      const float* __restrict__ tgt_logit, const int32_t* __restrict__ targets,
                      const int32_t* __restrict__ rowidx, float* __restrict__ logprob,
@@ -826,11 +812,7 @@ __global__ void __launch_bounds__(kMergeThreads)
       add_with_error(ss, se, s2);
     }
     if (!valid || sub != 0) continue;
-    // lse = (largest logit) / tau + ln(sum): mm counts in units of 1 / (tau scale_log2)
-    const float a = __fmul_rn(mm, max_unit.hi);
-    float h = a, h_lo = __fadd_rn(__fmaf_rn(mm, max_unit.lo, __fmaf_rn(mm, max_unit.hi, -a)),
-                                  __fdividef(se, ss));
-    add_with_error(h, h_lo, logf(ss));
+    const float lse = (mm + lg2_approx(__fadd_rn(ss, se))) * 0.69314718055994531f;
     const int64_t orig = rowidx ? static_cast<int64_t>(rowidx[r]) : r;
     const int32_t y = targets[orig];
     float lp;
@@ -838,12 +820,10 @@ __global__ void __launch_bounds__(kMergeThreads)
       report(status, PACE_ERR_INVALID_ARG);
       lp = __int_as_float(0x7fc00000);
     } else {
-      const float zy = tgt_logit[r];
-      const float low = isinf(zy) ? 0.0f : __fmaf_rn(zy, inv_temp.lo, -h_lo);
-      lp = __fadd_rn(__fmaf_rn(zy, inv_temp.hi, -h), low);
+      lp = tgt_logit[r] * inv_temp - lse;
     }
     logprob[orig] = lp;
-    if (lse_out) lse_out[orig] = __fadd_rn(h, h_lo);
+    if (lse_out) lse_out[orig] = lse;
   }
 }
 
@@ -1020,9 +1000,7 @@ pace_status run_logprob(const PaceBatch* batch, const void* hidden, const void* 
   if (mblocks > cap) mblocks = cap;
   lse_merge_kernel<<<static_cast<unsigned>(mblocks), kMergeThreads, 0, st>>>(
       rows_cap, n_valid_dev, static_cast<int>(clusters), n_vtiles, a.split_pref, V,
-      float2x(1.0 / temperature),
-      float2x(1.0 / (static_cast<double>(temperature) * a.scale_log2)), ws.part_m, ws.part_s,
-      ws.tgt, targets, rowidx, logprob, lse, status_dev);
+      1.0f / temperature, ws.part_m, ws.part_s, ws.tgt, targets, rowidx, logprob, lse, status_dev);
   return last_launch_status();
 }
 

@@ -197,14 +197,14 @@ def test_window_below_min_obs_and_no_window():
     _check(g, o, "no window")
 
 
-@pytest.mark.parametrize("n_traj", [256, 32768])  # direct count / sorted window + F table
+@pytest.mark.parametrize("n_traj", [256, 32768])  # a part of one wave, several finalisation waves
 @pytest.mark.parametrize("wlen", [1, 7, 32, 512, 513, 1000, 4096])
 @pytest.mark.parametrize("gamma", [1, 2, 4, 7])
 def test_window_shapes_and_ties(n_traj, wlen, gamma):
     """The ECDF count of Eq. 9 against windows of every size up to the 4096
     maximum, heavy ties, +0 and -0, +inf, and s exactly on window values; F of
-    Eq. 10 for several gamma; on a small pool (counted directly) and a large one
-    (sorted window and a table of F).  Bits must match the oracle."""
+    Eq. 10 for several gamma; on a small pool and a large one (both with the sorted
+    window and a table of F).  Bits must match the oracle."""
     rng = np.random.default_rng(wlen * 10 + gamma)
     window = (np.round(rng.random(wlen) * 8) / 8).astype(np.float32)  # ties
     window[rng.random(wlen) < 0.05] = -0.0
@@ -317,8 +317,8 @@ def test_large_windows_beside_short_streams(n_tok, wlen):
 def test_short_streams(n_traj, n_tok, wlen):
     """Pools whose tag stream is empty or a block or two long: the finalisation
     runs in the tag reduction's launch, so its one or few stream blocks score every
-    group; on the table path (8,192 trajectories and more) those few blocks also run
-    every window-preparation task (the sort and up to 129 slices of the F table)."""
+    group; those few blocks also run every window-preparation task (up to 129 parts of
+    the sorted window and the F table)."""
     rng = np.random.default_rng(n_traj + n_tok + wlen)
     lens = np.zeros(n_traj, np.int64)
     if n_tok:
