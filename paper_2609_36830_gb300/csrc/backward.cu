@@ -150,8 +150,7 @@ __host__ __device__ inline TailSplit tail_split(int64_t items, int n_clusters, i
   s.splits = 1;
   int best = nkb;  // the tail's K steps
   const int most = max_k_splits(nkb);
-#pragma unroll
-  for (int k = 2; k <= kMaxKSplits; ++k) {  // (unrolled: the divisions' latencies overlap)
+  for (int k = 2; k <= kMaxKSplits; ++k) {  // (constant bounds: the divisions' latencies overlap)
     const int rounds = (s.tail * k + n_clusters - 1) / n_clusters;
     const int steps = rounds * ((nkb + k - 1) / k);
     if (k <= most && steps < best) {
@@ -652,17 +651,23 @@ struct GradArgs {
 
 // x * scale rounded to fp64 and then to fp32, without the fp64 pipe, which a conversion,
 // a product and a conversion back per row would keep busy for most of the kernel (derivative
-// of 5.4M rows by graph replay 42.6 us that way, 24.5 so).  scale = s_hi + s_lo to 2^-49; the two partial products give
-// x * scale to 2^-45, and Ziv's test (ACM TOMS 17, 1991) says whether that decides the
-// rounding.  Where it does not (2^-18 of all products), or where the product is so small
-// that a partial product is subnormal, `sure` is false and the result is to be computed.
+// of 5.4M rows by graph replay 42.6 us that way, 23.2 so).  scale = s_hi + s_lo to 2^-49, and
+// q + t is x * scale to 2^-45.  Where t moved by 2^-18 of itself both ways rounds to the same
+// float, so does the product (after Ziv, ACM TOMS 17, 1991: |t| is at least 2^-26 |q| where
+// q + t is near the middle of two floats); otherwise `sure` is false and the result is to be
+// computed.  The partial products must not be subnormal: see products_fit.
 __device__ __forceinline__ float quick_product(float x, float s_hi, float s_lo, bool* sure) {
   const float q = __fmul_rn(x, s_hi);
   const float t = __fmaf_rn(x, s_lo, __fmaf_rn(x, s_hi, -q));
-  const float r = __fadd_rn(q, t);
-  const float low = __fsub_rn(t, __fsub_rn(r, q));  // r + low = q + t
-  *sure = x == 0.0f || (r == __fmaf_rn(low, 1.0f + 0x1p-18f, r) && fabsf(r) > 0x1p-90f);
+  const float r = __fmaf_rn(t, 1.0f - 0x1p-18f, q);
+  *sure = r == __fmaf_rn(t, 1.0f + 0x1p-18f, q);
   return r;
+}
+
+// A row's derivative is 0 or at least |a| e^-20 in magnitude, so its product with the scale is
+// 0 or above 2^-90, which keeps every bit of the partial products in the normal range.
+__device__ __forceinline__ bool products_fit(float a, double scale) {
+  return (a == 0.0f || fabsf(a) >= 0x1p-20f) && scale >= 0x1p-40;
 }
 
 // A sequence's advantage and, under SEQ_MEAN, its rows' scale.
@@ -720,17 +725,17 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
   for (int64_t w = w0; w < w1; ++w) {
     const int64_t t1 = tile_end(t0, p.n_rows);
     if (w + 1 < w1) nxt.load(p.logprob, p.behav, p.mask, t1, tile_end(t1, p.n_rows), p.vec);
-    unsigned in = 0u;
+    unsigned in = 0u, unsure = 0u;
     float adv[kRowsPerLane] = {};
     pw.walk(t0, t1, [&](int64_t, int64_t lo, int64_t hi, float a, int64_t) {
       const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
       in |= rows;
+      if (!products_fit(a, scale)) unsure |= rows;
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) adv[u] = rows >> u & 1u ? a : adv[u];
     });
     if (__any_sync(0xffffffffu, in != 0u)) {
       const float s_hi = scale_hi(scale), s_lo = scale_lo(scale);
-      unsigned unsure = 0u;
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) {
         const float x = term_derivative(p, cur.lp[u], cur.bh[u], adv[u]);
@@ -757,7 +762,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
 // have divided for, go through shared memory; a lane then finds the piece of each of its
 // rows.  (All lanes on every piece in turn, each with its own division, and the count's
 // atomics one by one took 1 to 2 us a piece: 5,000 rows of 1,000 sequences 95 us a call,
-// now 17; 300 rows of 8 20.7 and 14.1, 5.4M rows of 1,024 39.9 and 38.)
+// now 17; 300 rows of 8 19.1 and 12.5, 5.4M rows of 1,024 37.3 and 37.5.)
 struct PieceScales {
   double scale[kRowTile];
   float a[kRowTile];
@@ -800,6 +805,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks)
     const int k0 = k;
     int begin = kRowTile, end = kRowTile;
     float a = 0.0f, s_hi = 0.0f, s_lo = 0.0f;
+    bool fit = true;
     auto fetch = [&]() {
       const bool any = k < n;
       begin = any ? list.begin[k] : kRowTile;
@@ -808,6 +814,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks)
       const double sc = any ? list.scale[k] : 0.0;
       s_hi = scale_hi(sc);
       s_lo = scale_lo(sc);
+      fit = !any || products_fit(a, sc);
     };
     fetch();
     unsigned in = 0u, unsure = 0u;
@@ -822,7 +829,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks)
       bool sure;
       cur.lp[u] = quick_product(x, s_hi, s_lo, &sure);
       cur.bh[u] = x;
-      if (!sure) unsure |= 1u << u;
+      if (!sure || !fit) unsure |= 1u << u;
     }
     in &= cur.mask;
     unsure &= in;
