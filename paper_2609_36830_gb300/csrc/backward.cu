@@ -666,8 +666,8 @@ __device__ __forceinline__ float quick_product(float x, float s_hi, float s_lo, 
 
 // A row's derivative is 0 or at least |a| e^-20 in magnitude, so its product with the scale is
 // 0 or above 2^-90, which keeps every bit of the partial products in the normal range.
-__device__ __forceinline__ bool products_fit(float a, double scale) {
-  return (a == 0.0f || fabsf(a) >= 0x1p-20f) && scale >= 0x1p-40;
+__device__ __forceinline__ bool products_fit(float a, float s_hi) {
+  return (a == 0.0f || fabsf(a) >= 0x1p-20f) && s_hi >= 0x1p-40f;
 }
 
 // A sequence's advantage and, under SEQ_MEAN, its rows' scale.
@@ -717,9 +717,14 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
   long long mine = 0, total = 0;
   for (int i = threadIdx.x; i < p.geom.blocks; i += kRowThreads) mine += p.block_in[i];
   block_exclusive_scan<long long>(mine, &total);
-  if (threadIdx.x == 0) s_scale = 1.0 / static_cast<double>(total);
+  __shared__ float s_part[2];
+  if (threadIdx.x == 0) {
+    s_scale = 1.0 / static_cast<double>(total);
+    s_part[0] = scale_hi(s_scale);
+    s_part[1] = scale_lo(s_scale);
+  }
   __syncthreads();
-  const double scale = s_scale;
+  const float s_hi = s_part[0], s_lo = s_part[1];
   if (w0 >= w1) return;
   PieceWalker<FloatOf> pw(p.seq_offsets, p.seq_accepted, FloatOf{p.adv}, p.n_seq, t0);
   for (int64_t w = w0; w < w1; ++w) {
@@ -730,12 +735,11 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
     pw.walk(t0, t1, [&](int64_t, int64_t lo, int64_t hi, float a, int64_t) {
       const unsigned rows = piece_bits(t0, lo, hi) & cur.mask;
       in |= rows;
-      if (!products_fit(a, scale)) unsure |= rows;
+      if (!products_fit(a, s_hi)) unsure |= rows;
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) adv[u] = rows >> u & 1u ? a : adv[u];
     });
     if (__any_sync(0xffffffffu, in != 0u)) {
-      const float s_hi = scale_hi(scale), s_lo = scale_lo(scale);
 #pragma unroll
       for (int u = 0; u < kRowsPerLane; ++u) {
         const float x = term_derivative(p, cur.lp[u], cur.bh[u], adv[u]);
@@ -749,7 +753,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) surrogate_grad_ker
 #pragma unroll
         for (int u = 0; u < kRowsPerLane; ++u)
           if (unsure >> u & 1u)
-            cur.lp[u] = static_cast<float>(static_cast<double>(cur.bh[u]) * scale);
+            cur.lp[u] = static_cast<float>(static_cast<double>(cur.bh[u]) * s_scale);
       }
     }
     store_rows(p.dlp, t0, t1, p.vec, in, cur.lp);
@@ -814,7 +818,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks)
       const double sc = any ? list.scale[k] : 0.0;
       s_hi = scale_hi(sc);
       s_lo = scale_lo(sc);
-      fit = !any || products_fit(a, sc);
+      fit = !any || products_fit(a, s_hi);
     };
     fetch();
     unsigned in = 0u, unsure = 0u;
