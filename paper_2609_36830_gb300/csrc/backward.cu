@@ -651,7 +651,7 @@ struct GradArgs {
 
 // x * scale rounded to fp64 and then to fp32, without the fp64 pipe, which a conversion,
 // a product and a conversion back per row would keep busy for most of the kernel (derivative
-// of 5.4M rows by graph replay 42.6 us that way, 23.2 so).  scale = s_hi + s_lo to 2^-49, and
+// of 5.4M rows by graph replay 42.6 us that way, 23.0 so).  scale = s_hi + s_lo to 2^-49, and
 // q + t is x * scale to 2^-45.  Where t moved by 2^-18 of itself both ways rounds to the same
 // float, so does the product (after Ziv, ACM TOMS 17, 1991: |t| is at least 2^-26 |q| where
 // q + t is near the middle of two floats); otherwise `sure` is false and the result is to be
