@@ -52,6 +52,34 @@ def test_advantages_bitwise(G, n_seq, p_acc, unbiased):
     np.testing.assert_array_equal(as_np(adv), oadv.astype(np.float32))
 
 
+@pytest.mark.parametrize("G,groups", [(8, 6144), (8, 6145), (32, 2049), (1, 9000), (40, 300)])
+@pytest.mark.parametrize("call", ["derivative", "few rows", "rows"])
+def test_advantages_in_other_launches(G, groups, call):
+    """The advantages that the count's or the list's launch computes in its extra blocks, on
+    both sides of the number of groups from which a thread takes each, have the bits of a
+    launch of their own."""
+    rng = np.random.default_rng(G + groups)
+    n_seq = G * groups
+    n = {"derivative": 20_000, "few rows": 3000, "rows": 20_000}[call]
+    so = np.sort(rng.integers(0, n + 1, size=n_seq + 1)).astype(np.int64)
+    so[0], so[-1] = 0, n
+    acc = to_dev((rng.random(n_seq) < 0.7).astype(np.uint8))
+    reward = to_dev(rng.random(n_seq).astype(np.float32))
+    want = as_np(pace.group_advantages(reward, G, seq_accepted=acc))
+    adv = torch.full((n_seq,), 7.0, device=DEV)
+    la = pace.make_loss_args(torch.zeros(n, device=DEV), reward, G, pace.loss_params(),
+                             torch.zeros(1, dtype=torch.float64, device=DEV), adv_out=adv)
+    b = pace.make_batch(to_dev(so), n, seq_accepted=acc)
+    if call == "derivative":
+        pace.surrogate_backward(b, torch.zeros(n, device=DEV), la)
+    else:
+        hidden = torch.zeros((n, 64), dtype=torch.bfloat16, device=DEV)
+        pace.token_logprob(b, hidden, hidden[:64], torch.zeros(n, dtype=torch.int32, device=DEV),
+                           loss=la)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(as_np(adv), want)
+
+
 def _batch(rows, seed, accept_p=0.75):
     pool = workloads.make_pool(*rows)
     rw = workloads.make_rows(pool)
